@@ -7,8 +7,8 @@
 //   zero     local expansions and dependency counters of every system
 //   up       P2M of every leaf, then M2M from the deepest level up (per-warp
 //            items; an M2M item waits, bounded, until the level below is done)
-//   pad      multipole rows padded to whole k-blocks (tensor-core M2L)
-//   M2L      same-level pairs on the tensor cores, persistent over (system, tile)
+//   split    FP16 (hi, lo) multipole rows of the tensor-core M2L
+//   M2L      same-level pairs on the tensor cores, persistent over (system, tile, range)
 //   M2L'     pairs across levels of adaptive trees, one block per target cell
 //   down     L2L from the top level down, then L2P (bounded waits per level)
 //   P2P      persistent over (system, target leaf), on a second stream
@@ -151,13 +151,15 @@ int fmm_batch_create(const fmm_handle *handles, int nsys, void *const *phi, void
             maxdepth = std::max(maxdepth, h->depth);
             // same-level M2L: the system's tiles in the persistent tensor-core launch
             if (h->depth >= 2) {
-                M2LJob j = m2l_tensor_job(h, S.L, S.M, s);
-                if (j.mrow != S.M) S.mpad = const_cast<float *>(j.mrow);
+                M2LJob j = m2l_tensor_job(h, S.L);
+                S.rows = const_cast<unsigned char *>(j.mrow);
+                S.m2l_ws = const_cast<unsigned *>(j.lmax);
+                S.ws_words = j.ws_words;
                 int nt = 0;
                 FMM_CUDA_TRY(cudaMemcpy(&nt, j.ntiles, sizeof(int), cudaMemcpyDeviceToHost));
                 j.item0 = item0;
-                j.count = nt;
-                item0 += nt;
+                j.count = nt * j.nsplit;
+                item0 += j.count;
                 if (nt > 0) jobs.push_back(j);
             }
             // tree structure for the work lists
@@ -250,7 +252,7 @@ int fmm_batch_evaluate(fmm_batch b, void *stream)
         FMM_CUDA_TRY(cudaEventRecord(b->join, b->side));
         batch_zero(b->p, sys, b->nsys, s);
         batch_up(b->p, b->nsm, sys, b->up.as<int4>(), b->n_up, misc + BQ_UP, h0->m2m_mat.as<float>(), misc + BE_DEP, s);
-        batch_mpad(b->p, sys, b->nsys, s);
+        batch_split(b->p, sys, b->nsys, s);
         if (b->n_jobs > 0)
             m2l_tensor_jobs(b->p, b->nsm, b->jobs.as<M2LJob>(), b->n_jobs, misc + BQ_M2L, misc + BE_M2L, s);
         batch_m2lx(b->p, sys, b->mx.as<int2>(), b->n_mx, s);
@@ -276,7 +278,7 @@ int fmm_batch_status(fmm_batch b, int *async_error, int64_t *kernel_launches)
         FMM_CUDA_TRY(cudaDeviceSynchronize());
         FMM_CUDA_TRY(cudaMemcpy(e, b->misc.as<int>() + BE_DEP, sizeof(e), cudaMemcpyDeviceToHost));
         *async_error = (e[0] ? 1 : 0) | (e[1] ? 2 : 0) | (e[2] ? 4 : 0);
-        if (kernel_launches) *kernel_launches = 6 + (b->n_mx > 0 ? 1 : 0) + (b->p * b->p % 32 != 0 ? 1 : 0);
+        if (kernel_launches) *kernel_launches = 6 + (b->n_jobs > 0 ? 1 : 0) + (b->n_mx > 0 ? 1 : 0);
         return FMM_OK;
     } catch (const Error &e) {
         set_error(e.msg);

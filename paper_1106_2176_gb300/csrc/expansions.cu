@@ -30,6 +30,7 @@
 #include <tuple>
 
 #include "fmm_internal.cuh"
+#include "m2l_norm.cuh"
 #include "m2lx_layout.cuh"
 
 namespace fmm {
@@ -1401,7 +1402,8 @@ void stencil_update(fmm_ctx *h)
 void stencil_levels(fmm_ctx *h, cudaStream_t s)
 {
     const int ne = h->st_off[9];
-    std::vector<int> cnt(9 * (FMM_MAXLEVEL + 1));
+    std::vector<int> &cnt = h->st_cnt;
+    cnt.assign(9 * (FMM_MAXLEVEL + 1), 0);
     int ecum = -1;
     for (int l = 0; l <= FMM_MAXLEVEL; l++) {
         // no extent known: every entry; an empty level (-1): none
@@ -1717,6 +1719,7 @@ __global__ void __launch_bounds__(32 * MV_WARPS) batch_up_k(const BatchSys *__re
             m2m_parent_warp<NR>(item.z, lane, P * P, S.child, S.nchild, S.xyz, mat, S.M, sx[w]);
         }
         __syncwarp();
+        if (S.m2l_ws) m2l_row_max(S.M + (size_t)item.z * P * P, P * P, lane, S.m2l_ws + item.w);
         if (lane == 0) batch_done(S.cnt_up + item.w);
     }
 }

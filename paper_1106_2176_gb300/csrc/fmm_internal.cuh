@@ -23,6 +23,7 @@
 #include <cstdint>
 #include <cstring>
 #include <cstdio>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -112,7 +113,7 @@ struct M2LTile {
 
 // One system's share of a persistent tensor-core M2L launch: its tile list
 // and the arrays the tiles read and write. Queue items item0 .. item0 + count
-// - 1 are its tiles (count < 0: *ntiles tiles, read on the device).
+// - 1 are its (tile, range) pairs, tile-major (count < 0: *ntiles tiles, read on the device).
 struct M2LJob {
     const M2LTile *tiles;
     const int *ntiles;
@@ -123,16 +124,35 @@ struct M2LJob {
     const int *map_pool;
     const int4 *st;
     const int *st_off;
-    const float *mrow;
-    const unsigned char *ttab;
+    const unsigned char *mrow;  // FP16 (hi, lo) rows of M~ by cell
+    const unsigned char *ttab;  // operator image
+    const int *rowexp;          // its power of two per output coefficient: L~ = 2^(rowexp - e) sums
     float *L;
+    const unsigned *lmax;       // per level: the bits of its largest coefficient (sets the rows' scale)
+    unsigned *tcnt;             // per tile: ranges finished (nsplit > 1)
+    float2 *part;               // per (tile, range): its (hi, lo) sums (nsplit > 1)
     // complete levels whose sources come by TMA tile loads from the lattice
     // copy of M~ (bit l: level l); lat_maps holds a 128-byte tensor map per level
     const unsigned char *lat_maps;
     unsigned lat_levels;
+    int nsplit;                 // ranges the vectors of a tile are cut into, one CTA each
+    int ws_words;               // words of the workspace at lmax (maxima, counters) to zero per evaluation
     int item0;
     int count;
 };
+
+// first cell of every level (levels past the depth: the number of cells)
+struct M2LLevels {
+    int start[FMM_MAXLEVEL + 2];
+};
+
+// levels with a lattice copy of their rows (bit l), and each one's first row in it
+struct M2LLattice {
+    unsigned levels;
+    long long off[FMM_MAXLEVEL + 1];
+};
+
+struct TcImage;  // operator image of the tensor-core M2L on one device (m2l_tc.cu)
 
 // One system of a batched evaluation (mixed precision, FP32 inputs): the
 // arrays of its handle that the batch kernels read and write, its output
@@ -152,7 +172,9 @@ struct BatchSys {
     const int2 *runs_pr;
     float *phi, *grad;              // caller's order
     unsigned *cnt_up, *cnt_dn;      // per level: cells whose M (up) / L (down) is final
-    float *mpad;                    // M rows zero-padded to whole k-blocks (tensor-core M2L), or null
+    unsigned char *rows;            // FP16 (hi, lo) rows of the tensor-core M2L, or null (no same-level M2L)
+    unsigned *m2l_ws;               // its per-level maxima, then tile counters: ws_words words
+    int ws_words;
     int n, ncells, nleaves, depth, c0;  // c0: first cell of level 2
     int lvl_start[FMM_MAXLEVEL + 2];
 };
@@ -224,18 +246,20 @@ struct fmm_ctx {
     int st_R = 0;               // offsets |v_k| <= st_R are in the stencil
     fmm::DevBuf rtab64, rtab32; // R_n^m(t_o), 8 child offsets, full complex storage of degree < p
     fmm::DevBuf m2m_mat, l2l_mat; // FP32 p^2 x p^2 real maps of M2M and L2L per child octant, [o][in][out]
-    fmm::DevBuf ttab;           // tensor-core M2L operators (split TF32 images), per vector
-    size_t ttab_stride = 0;     // bytes per vector in ttab
+    std::shared_ptr<fmm::TcImage> ttab;  // tensor-core M2L operators (split FP16 images), per vector
     int ttab_nv = -1;           // stencil vectors the operator images were made for
+    std::vector<int> st_cnt;    // per set (octants, union) and level: entries that can reach a cell
     fmm::DevBuf rot_tab;        // rotation M2L maps per vector ([A | B], FP32 or FP64)
     int rot_nv = -1, rot_kind = 0;  // vectors and precision (1 FP32, 2 FP64) of rot_tab
-    fmm::DevBuf msplit;         // M~ split into TF32 (hi, lo) rows for the tensor-core M2L
-    // tensor-core M2L on complete levels: M~ of each such level in lattice
+    fmm::DevBuf msplit;         // M~ split into FP16 (hi, lo) rows for the tensor-core M2L
+    fmm::DevBuf m2l_ws, m2l_part;  // its level maxima and tile counters; sums of the ranges of split tiles
+    int m2l_nsplit = 1;         // ranges per tile (m2l_plan)
+    // tensor-core M2L on complete levels: the rows of each such level in lattice
     // order (octant bits, then z, y, x of the halved position), one TMA tensor
     // map per level (device copy and its pinned staging)
     bool lattice_req = true;    // fmm_set_m2l_lattice
     unsigned lat_levels = 0;    // bit l: level l reads its sources from the lattice copy
-    long long lat_off[FMM_MAXLEVEL + 1] = {};  // float offset of level l in mlat
+    long long lat_off[FMM_MAXLEVEL + 1] = {};  // first row of level l in mlat
     fmm::DevBuf mlat, lat_maps;
     fmm::PinnedBuf lat_host;
 
@@ -334,14 +358,14 @@ void cell_geometry(fmm_ctx *h, cudaStream_t s);  // h->cgeo: centre and 1 / widt
 void tensor_tables_init(fmm_ctx *h);
 bool tensor_m2l_supported(fmm_ctx *h);
 void m2l_tensor(fmm_ctx *h, float *L, const float *M);
-// the same-level M2L of several systems (same p; mrow already padded to
-// whole k-blocks where p^2 is not a multiple of 32) in one persistent launch
+// the same-level M2L of several systems (same p; rows already split) in one persistent launch
 void m2l_tensor_jobs(int p, int nsm, const M2LJob *jobs_dev, int njobs, int *queue, int *err, cudaStream_t s);
-M2LJob m2l_tensor_job(fmm_ctx *h, float *L, const float *M, cudaStream_t s);  // pads M if needed
+M2LJob m2l_tensor_job(fmm_ctx *h, float *L);  // the handle's arrays; allocates its workspaces
+void m2l_plan(fmm_ctx *h);                     // (build) ranges per tile
 // (build) which complete levels the tensor-core M2L reads through TMA tile
 // loads: their lattice buffer and tensor maps
 void lattice_prepare(fmm_ctx *h, cudaStream_t s);
-void batch_mpad(int p, const BatchSys *sys, int nsys, cudaStream_t s);  // every system's padded M rows
+void batch_split(int p, const BatchSys *sys, int nsys, cudaStream_t s);  // every system's FP16 rows
 
 // p2p.cu
 void near_field(fmm_ctx *h, cudaStream_t s);  // P2P into h->near

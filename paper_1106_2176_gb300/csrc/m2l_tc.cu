@@ -9,36 +9,54 @@
 // all levels needs no synchronisation between levels: one launch covers every
 // level's tiles.
 //
-// Precision: A = M~ and B = T_v are split into two TF32 values each, hi and
-// lo (round to nearest), and the MMAs compute A_hi [T_hi ; T_lo] (N = 2 NP)
-// plus A_lo T_hi, accumulating in FP32 in tensor memory: the main sum in
-// columns [0, NP), the small correction terms in [NP, 2 NP). Every GV vectors
-// the accumulator is drained into per-thread FP32 (hi, lo) TwoSum registers;
-// two TMEM buffers alternate so the drain overlaps the next MMAs.
+// Precision: A = M~ and B = T_v are split into two FP16 values each, hi and
+// lo = x - hi (both rounded to nearest: 22 bits, an error below 2^-23 of x),
+// and the MMAs compute A_hi [T_hi ; T_lo] plus A_lo T_hi, accumulating in
+// FP32 in tensor memory: the main sum in columns [0, NP), the small
+// correction terms in [NP, 2 NP). FP16's 11-bit significand is TF32's, at
+// twice the MMA rate and half the operand bytes; what it lacks is exponent
+// range, so the operands are brought into range by powers of two (exact):
+//   - coefficient (n, m) of M~ is multiplied and that of L~ divided by
+//     2^round(log2 sqrt((n+m)! (n-m)!)), which takes the factorials out of the
+//     solid harmonics; the powers of the distance in T are then balanced by
+//     2^-n on M~ and one power of two per degree of L~, so that the largest
+//     entries of every degree's rows lie in [2^13, 2^14);
+//   - a level's rows are multiplied by 2^e so that the largest coefficient of
+//     the level lies in [2^14, 2^15) (e from a maximum taken each evaluation).
+// FP16's subnormals end 2^-39 below that maximum, 15 bits below the rounding
+// of the FP32 sums. Every GV vectors the accumulator is drained into
+// per-thread FP32 (hi, lo) TwoSum registers; two TMEM buffers alternate so
+// the drain overlaps the next MMAs.
 //
-// Per CTA (320 threads: two groups of 4 worker warps, 1 MMA warp, 1 operator
-// warp), for every unit (v, k-block) of 32 coefficients, taken by the group
-// u % 2:
-//   - the group gathers the unit's raw FP32 multipole rows with cp.async into
-//     a 128B-swizzled stage of its A ring; each warp fills its own 32 rows,
-//     eight lanes per row, so that one copy instruction covers four whole
-//     rows (sources found by lattice lookups fetched ahead into a ring; zero
-//     fill where a cell is absent);
-//   - once the stage is full, each thread splits its row into TF32 hi and lo
-//     (lo = a - hi), stores both in the unit's compute stage in tensor memory
-//     and issues the copies of its group's next unit;
-//   - the operator warp bulk-copies the pre-split, pre-swizzled [T_hi ; T_lo]
-//     operator: for p <= 8 the blocks of a whole vector into a ring of its
-//     own, several vectors ahead; otherwise one block into the unit's
-//     compute stage;
-//   - the MMA warp issues the tcgen05.mma (A from tensor memory, the operator
-//     from shared memory) and commits; for p <= 8 it takes one whole vector
-//     per iteration, waiting once on a barrier that both worker groups and the
-//     operator warp arrive on, because every wait and commit costs the issuing
-//     thread a few hundred cycles.
+// Per CTA (320 threads: two groups of 4 worker warps, an MMA warp and a
+// producer warp) a ring of NS stages, one unit (vector v, k-block of 64
+// coefficients) each: 128 rows of A_hi and A_lo and the operator block
+// [T_hi ; T_lo], all 128B-swizzled in shared memory, where the MMAs read both
+// operands.
+//   - the producer brings the operator block with one bulk copy and, on
+//     complete levels (lattice tiles), A_hi and A_lo with one TMA tile load
+//     each; the workers then only drain.
+//   - on other levels the worker group u % 2 gathers the unit's rows with
+//     cp.async straight into the stage (sources found by lattice lookups
+//     fetched ahead into a ring; zero fill where a cell is absent). The
+//     copies' completion arrives on the stage's mbarrier; the MMA thread
+//     orders them before its asynchronous reads with a proxy fence.
+//   - the MMA warp issues the tcgen05.mma of a unit and commits it to the
+//     stage's "empty" barrier.
+// The rows are split into FP16 once per evaluation (m2l_split_k) and not once
+// per vector, so nothing but copies and MMAs is left per vector.
+// Bound: the copies into shared memory (48 KB per vector and tile at p = 8,
+// MEASURED_BOUND).
+//
+// A tree with few tiles (5 at N = 16,384) would leave most SMs idle: the
+// vectors of every tile are then cut into nsplit ranges, one CTA each
+// (m2l_plan). Each CTA writes its (hi, lo) sums and the last one of a tile to
+// finish adds the ranges in order, so results do not depend on scheduling.
+//
 // Every wait is bounded; on a timeout the kernel records an error code and
 // leaves after its copies have landed and its TMEM is released.
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -47,8 +65,10 @@
 #include <tuple>
 
 #include <cuda.h>  // CUtensorMap and its encoding enums (the encoder comes from the runtime's driver entry point)
+#include <cuda_fp16.h>
 
 #include "fmm_internal.cuh"
+#include "m2l_norm.cuh"
 #include "ptx_sm100.cuh"
 
 namespace fmm {
@@ -61,141 +81,167 @@ __device__ int g_no_cell = -1;
 // ---------------------------------------------------------------------------
 // tile geometry
 // ---------------------------------------------------------------------------
-// Warp roles: warps 0-7 form two groups of four (group g = warps 4g .. 4g+3,
-// thread row r = tid % 128, in its warp's TMEM lane quarter); group g takes
-// the units u with u % 2 == g, so the latency of one group's hand-offs is
-// hidden behind the other's. Warp 8 issues the MMAs; warp 9 copies the
-// operator blocks.
-//   A raw rings (RSG stages per group, shared memory): the gathered FP32
-//     multipoles of a unit, 128 B per row, 128B-swizzled. A warp copies and
-//     reads only its own 32 rows, so it refills a stage right after the
-//     warp's split.
-//   compute stages (CS): A_hi, A_lo in tensor memory (written by the unit's
-//     group with tcgen05.st, read by the MMA as its A operand), freed by the
-//     MMA commit of the unit (or of its vector).
-//   operator blocks in shared memory: VEC (p <= 8) a ring of OSV whole
-//     vectors; otherwise one block in each compute stage.
-// Tensor memory: AC accumulator buffers of 2 NP columns (main | correction)
-// followed by the CS A stages of 64 columns (hi 32 | lo 32). Thread (r, g)
-// drains output columns [g HN, (g + 1) HN) of row r.
-template <int NP, int KB>
+// NP: p^2 padded to a multiple of 16 (the MMA's N). A cell's row is KB blocks
+// of 64 coefficients, each 128 bytes of hi and 128 bytes of lo; with NP <= 32
+// both halves fit one 128-byte row (PACK: hi in the first 64 bytes, lo in the
+// last), and so do T_hi and T_lo.
+// Tensor memory: two accumulator buffers of 2 NP columns (main | correction).
+// Thread (r, g) drains output columns [g HN, (g + 1) HN) of row r.
+template <int NP>
 struct TcCfg {
     static constexpr int M = 128;                  // target rows per tile
     static constexpr int NW = 8;                   // worker warps
     static constexpr int NG = 2;                   // worker groups
-    static constexpr int MMA_WARP = NW, B_WARP = NW + 1;
-    static constexpr int NT = NW * 32 + 64;        // threads (workers, MMA warp, operator warp)
-    static constexpr int A_RAW = M * 128;          // raw A k-block (FP32, swizzled)
-    static constexpr int B_RAW = 2 * NP * 128;     // [T_hi ; T_lo] k-block (TF32 pair, swizzled)
-    static constexpr int ACOLS = 64;               // TMEM columns of one A stage (hi, lo)
-    // accumulator buffers: two (the drain overlaps the next MMAs) when the
-    // compute stages of at least one whole vector (KB) still fit beside them
-    static constexpr int CS2 = (512 - 4 * NP) / ACOLS >= 4 ? 4 : (512 - 4 * NP) / ACOLS;
-    static constexpr int AC = CS2 >= KB && CS2 >= 2 ? 2 : 1;
-    static constexpr int CS = AC == 2 ? CS2 : ((512 - 2 * NP) / ACOLS >= 4 ? 4 : (512 - 2 * NP) / ACOLS);
-    static constexpr int ACC_COLS = AC * 2 * NP;
-    static constexpr int TCOLS = 512;
+    static constexpr int MMA_WARP = NW, P_WARP = NW + 1;
+    static constexpr int NT = NW * 32 + 64;        // threads (workers, MMA warp, producer warp)
+    static constexpr bool PACK = NP <= 32;
+    static constexpr int KB = (NP + 63) / 64;      // k-blocks per vector
+    static constexpr int ROWB = PACK ? 128 : 256;  // bytes of a row's k-block (hi and lo)
+    static constexpr int A_BYTES = M * ROWB;
+    static constexpr int B_BYTES = (PACK ? 1 : 2) * NP * 128;
+    static constexpr int STAGE = A_BYTES + B_BYTES;
     static constexpr int QU = 8;                   // lookahead of the source lookups (units of the group)
     static constexpr int RINGU = 2 * QU;
     static constexpr int RING = NG * RINGU * M * 4;
-    // VEC (p <= 8): the MMA warp takes one stencil vector (KB units) per
-    // iteration, and the operator blocks of whole vectors sit in a ring of
-    // their own (OSV slots), filled up to OSV vectors ahead and freed by one
-    // commit per vector (VR "vector done" barriers). Otherwise the operator
-    // block of a unit travels in that unit's compute stage.
-    static constexpr bool VEC = KB <= 2 && CS >= 2 * KB;
-    static constexpr int OPV = KB * B_RAW;         // operator bytes of one vector
-    static constexpr int VR = 8;
-    static constexpr int RSG_V = 2;
     static constexpr int BAR = 768;                // mbarriers (first 512 bytes), then the CTA's job
-    static constexpr int OSV_FIT = (220 * 1024 - RING - BAR - 1024 - NG * RSG_V * A_RAW) / OPV;
-    static constexpr int OSV = OSV_FIT > 6 ? 6 : OSV_FIT;
-    static constexpr int BUDGET = 220 * 1024 - RING - BAR - 1024 - CS * B_RAW;
-    static constexpr int RSG_U = BUDGET / (NG * A_RAW) >= 3 ? 3 : BUDGET / (NG * A_RAW);
-    static constexpr int RSG = VEC ? RSG_V : RSG_U;  // raw stages per group
-    static constexpr int OPB = VEC ? OSV * OPV : CS * B_RAW;  // operator bytes in shared memory
-    static constexpr int SMEM = NG * RSG * A_RAW + OPB + RING + BAR + 1024;
-    static_assert(!VEC || (OSV >= 2 && OSV <= VR), "operator ring");
-    static_assert(RSG >= 2 && RSG <= 3 && CS >= 2 && CS >= KB && QU >= RSG && ACC_COLS + CS * ACOLS <= TCOLS &&
-                      SMEM <= 227 * 1024,
-                  "stage budget");
+    static constexpr int NS_FIT = (226 * 1024 - RING - BAR - 1024) / STAGE;
+    static constexpr int NS = NS_FIT > 6 ? 6 : NS_FIT;
+    static constexpr int SMEM = NS * STAGE + RING + BAR + 1024;
+    static constexpr int TCOLS = 512;
     static constexpr int GV = 8;                   // vectors per accumulator drain
     static constexpr int HN = NP / 2;              // output coefficients per thread
-    static constexpr int DRAIN_AT = AC == 2 ? 2 : 0;  // vectors into group gg + 1 at which group gg is drained
+    // vectors into group gg + 1 at which a gathering worker drains group gg:
+    // its units have then been consumed (the ring is NS units deep)
+    static constexpr int DRAIN_AT = (NS + KB - 1) / KB;
+    static_assert(NP % 16 == 0 && STAGE % 1024 == 0 && NS >= 3 && DRAIN_AT < GV && 4 * NP <= TCOLS &&
+                      SMEM <= 227 * 1024 && 2 * QU >= NS,
+                  "stage budget");
 };
 
-// Zero-padded copy of the scaled multipoles: out[c][KB * 32] (only when p^2 is
-// not a multiple of 32; otherwise the kernel reads M~ directly).
-__global__ void mpad_k(const float *__restrict__ M, int PP, int KP, int c0, int nc, float *__restrict__ out)
+// ---------------------------------------------------------------------------
+// operand rows
+// ---------------------------------------------------------------------------
+// Largest |M~ a| (a: m2l_norm) of every level from 2 on, as FP32 bits (the order of
+// non-negative floats), over the finite coefficients; lmax starts at zero.
+// grid.y: levels; a warp walks cells, lane i holds coefficients i, i + 32, ...
+__global__ void __launch_bounds__(256) m2l_lmax_k(const float *__restrict__ M, int PP, const __grid_constant__ M2LLevels lv,
+                                                  unsigned *__restrict__ lmax)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)(nc - c0) * KP) return;
-    const int c = c0 + (int)(i / KP), k = (int)(i % KP);
-    out[(size_t)c * KP + k] = k < PP ? M[(size_t)c * PP + k] : 0.f;
+    const int l = 2 + blockIdx.y, lane = threadIdx.x & 31;
+    const int c1 = lv.start[l + 1];
+    float a[4];
+#pragma unroll
+    for (int r = 0; r < 4; r++) a[r] = m2l_norm(lane + 32 * r);
+    unsigned best = 0;
+    for (int c = lv.start[l] + (int)(blockIdx.x * 8 + (threadIdx.x >> 5)); c < c1; c += (int)gridDim.x * 8) {
+        const float *Mc = M + (size_t)c * PP;
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+            if (lane + 32 * r < PP) best = max(best, m2l_mag(Mc[lane + 32 * r] * a[r]));
+    }
+    best = __reduce_max_sync(0xffffffffu, best);
+    __shared__ unsigned sb[8];
+    if (lane == 0) sb[threadIdx.x >> 5] = best;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; w++) best = max(best, sb[w]);
+        if (best > *(volatile unsigned *)(lmax + l)) atomicMax(lmax + l, best);
+    }
 }
 
-// Lattice copy of a complete level's M~ for the TMA tile loads of the
-// tensor-core M2L: the row of the cell at lattice position (x, y, z) goes to
-// ((b H + z/2) H + y/2) H + x/2, b = (x & 1) | (y & 1) << 1 | (z & 1) << 2 its
-// octant bits and H = 2^(l-1), zero-padded to KP coefficients. The cells of
-// one octant then form an H^3 block in x, y, z order, so the sources of a
-// block of targets under one translation are a shifted block.
-__global__ void lattice_fill_k(const float *__restrict__ M, int PP, int KP, const int4 *__restrict__ xyz, int c0, int c1,
-                               int l, float *__restrict__ out)
+// coefficients 8 ch .. 8 ch + 7 of one cell as FP16 (hi, lo): M~ a 2^e
+template <int NP>
+__device__ __forceinline__ void m2l_split_chunk(const float *__restrict__ Mc, int PP, int ch, int e,
+                                                unsigned char *__restrict__ row)
 {
+    using C = TcCfg<NP>;
+    float v[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++) v[i] = 0.f;
+    const int k0 = 8 * ch;
+    if ((PP & 3) == 0) {  // rows start on 16-byte boundaries
+        if (k0 < PP) *reinterpret_cast<float4 *>(v) = *reinterpret_cast<const float4 *>(Mc + k0);
+        if (k0 + 4 < PP) *reinterpret_cast<float4 *>(v + 4) = *reinterpret_cast<const float4 *>(Mc + k0 + 4);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; i++)
+            if (k0 + i < PP) v[i] = Mc[k0 + i];
+    }
+    // 2^e in two factors: e may lie outside the exponent range of one float
+    const float s1 = m2l_pow2(e >> 1), s2 = m2l_pow2(e - (e >> 1));
+    __half h[8], w[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        const float x = (v[i] * m2l_norm(k0 + i)) * s1 * s2;
+        h[i] = __float2half_rn(x);
+        w[i] = __float2half_rn(x - __half2float(h[i]));
+    }
+    const int off = C::PACK ? ch * 16 : (ch >> 3) * 256 + (ch & 7) * 16;
+    *reinterpret_cast<uint4 *>(row + off) = *reinterpret_cast<const uint4 *>(h);
+    *reinterpret_cast<uint4 *>(row + off + (C::PACK ? 64 : 128)) = *reinterpret_cast<const uint4 *>(w);
+}
+
+// FP16 rows of the cells from level 2 on. A cell of a lattice level (bit l of
+// lat.levels) goes to the lattice copy of its level: the row of position (x, y,
+// z) at ((b H + z/2) H + y/2) H + x/2, b = (x & 1) | (y & 1) << 1 | (z & 1) << 2
+// its octant bits and H = 2^(l-1), so that the cells of one octant form an H^3
+// block in x, y, z order and the sources of a block of targets under one
+// translation are a shifted block. Other cells go to row c of `rows`.
+template <int NP>
+__global__ void __launch_bounds__(256) m2l_split_k(const float *__restrict__ M, int PP, const int4 *__restrict__ xyz, int c0,
+                                                   int nc, const unsigned *__restrict__ lmax,
+                                                   const __grid_constant__ M2LLattice lat, unsigned char *__restrict__ rows,
+                                                   unsigned char *__restrict__ mlat)
+{
+    using C = TcCfg<NP>;
+    constexpr int NCH = NP / 8, RB = C::KB * C::ROWB;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)(c1 - c0) * KP) return;
-    const int c = c0 + (int)(i / KP), k = (int)(i % KP);
+    if (i >= (int64_t)(nc - c0) * NCH) return;
+    const int c = c0 + (int)(i / NCH), ch = (int)(i % NCH);
     const int4 a = xyz[c];
-    const int sh = FMM_MAXLEVEL - l;
-    const int64_t H = 1ll << (l - 1);
-    const int x = a.x >> sh, y = a.y >> sh, z = a.z >> sh;
-    const int b = (x & 1) | ((y & 1) << 1) | ((z & 1) << 2);
-    const int64_t r = ((b * H + (z >> 1)) * H + (y >> 1)) * H + (x >> 1);
-    out[r * KP + k] = k < PP ? M[(size_t)c * PP + k] : 0.f;
+    const int l = a.w;
+    unsigned char *row = rows + (size_t)c * RB;
+    if ((lat.levels >> l) & 1u) {
+        const int sh = FMM_MAXLEVEL - l;
+        const int64_t H = 1ll << (l - 1);
+        const int x = a.x >> sh, y = a.y >> sh, z = a.z >> sh;
+        const int b = (x & 1) | ((y & 1) << 1) | ((z & 1) << 2);
+        row = mlat + (lat.off[l] + ((b * H + (z >> 1)) * H + (y >> 1)) * H + (x >> 1)) * RB;
+    }
+    m2l_split_chunk<NP>(M + (size_t)c * PP, PP, ch, m2l_exponent(lmax[l]), row);
 }
 
-template <int NP, int KB, bool PERSIST>
-__global__ void __launch_bounds__(TcCfg<NP, KB>::NT, 1)
+template <int NP, bool PERSIST>
+__global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     m2l_tc_k(int p, const __grid_constant__ M2LJob one, const M2LJob *__restrict__ jobs, int njobs,
              int *__restrict__ queue, int *__restrict__ err)
 {
     // PERSIST (many systems: jobs[], njobs entries sorted by item0): each CTA
-    // takes tiles from the queue until it is empty. Otherwise CTA b computes
-    // tile b of the single job `one`, read from the parameter space, which
-    // measured faster for one system than the persistent loop (25.1 vs
-    // 27.7 ms at N = 1e7).
-    using C = TcCfg<NP, KB>;
-    constexpr int RSG = C::RSG, CS = C::CS, AC = C::AC, NG = C::NG, QU = C::QU, RINGU = C::RINGU, KP = KB * 32;
+    // takes (tile, range) items from the queue until it is empty. Otherwise
+    // CTA b computes item b of the single job `one`, read from the parameter
+    // space, which measured faster for one system than the persistent loop.
+    using C = TcCfg<NP>;
+    constexpr int NS = C::NS, QU = C::QU, RINGU = C::RINGU, KB = C::KB;
+    constexpr bool PACK = C::PACK;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    unsigned char *araw = base;                           // NG x RSG x A_RAW
-    constexpr bool VEC = C::VEC;
-    constexpr int NB = VEC ? C::OSV : CS;     // operator slots
-    constexpr int NF = VEC ? C::VR : CS;      // "free" barriers: per vector (VEC) or per compute stage
-    unsigned char *bops = araw + NG * RSG * C::A_RAW;     // operator slots (VEC: OSV x OPV; else CS x B_RAW)
-    int *ring = reinterpret_cast<int *>(bops + C::OPB);  // NG x RINGU x M
+    int *ring = reinterpret_cast<int *>(base + NS * C::STAGE);  // NG x RINGU x M
     uint64_t *bar = reinterpret_cast<uint64_t *>(reinterpret_cast<unsigned char *>(ring) + C::RING);
-    uint64_t *a_full = bar;                   // NG x RSG: cp.async arrivals of the group's 128 threads
-    uint64_t *b_full = a_full + NG * RSG;     // NB: operator copies (transaction bytes)
-    uint64_t *cmp_full = b_full + NB;         // CS: one arrival per warp of the unit's group
-    uint64_t *cmp_free = cmp_full + CS;       // NF: MMA commits (VEC: vector w done, slot w % VR)
-    uint64_t *acc_full = cmp_free + NF;       // AC: MMA commits at the end of a group of vectors
-    uint64_t *acc_empty = acc_full + AC;      // AC: one arrival per worker warp after a drain
-    uint64_t *fin = acc_empty + AC;           // 1
-    uint64_t *ready = fin + 1;                // VEC, VR: vector w ready (its KB units split, its operator landed)
-    uint64_t *a_lat = ready + C::VR;          // NG x RSG x 4: TMA tile loads of one warp's 32 rows (lattice tiles)
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(a_lat + NG * RSG * 4);
+    uint64_t *full = bar;                     // NS: bytes of the producer's copies
+    uint64_t *gfull = full + NS;              // NS: cp.async arrivals of a group's 128 threads (gathered tiles)
+    uint64_t *empty = gfull + NS;             // NS: MMA commits
+    uint64_t *acc_full = empty + NS;          // 2: MMA commits at the end of a group of vectors
+    uint64_t *acc_empty = acc_full + 2;       // 2: one arrival per worker warp after a drain
+    uint64_t *fin = acc_empty + 2;            // 1
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(fin + 1);
     int *abort_flag = reinterpret_cast<int *>(tmem_slot + 1);
-    int *s_tile = abort_flag + 1;                 // this CTA's current tile (-1: none left)
+    int *s_item = abort_flag + 1;                 // this CTA's current item (-1: none left)
+    int *s_last = s_item + 1;                     // this CTA finished its tile last
     M2LJob *s_job = reinterpret_cast<M2LJob *>(reinterpret_cast<unsigned char *>(bar) + 512);  // its job
-    static_assert(sizeof(uint64_t) * (NG * RSG + NB + CS + NF + 2 * AC + 1 + C::VR + NG * RSG * 4) + 16 <= 512 &&
-                      512 + sizeof(M2LJob) <= C::BAR,
-                  "barrier area");
+    static_assert(sizeof(uint64_t) * (3 * NS + 5) + 16 <= 512 && 512 + sizeof(M2LJob) <= C::BAR, "barrier area");
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const bool worker = warp < C::NW;
-    const int row = tid & 127, grp = (tid >> 7) & 1;  // worker: target row and group
+    if (!PERSIST && (int)blockIdx.x >= *one.ntiles * one.nsplit) return;
     if (warp == C::MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(C::TCOLS));
@@ -218,109 +264,89 @@ __global__ void __launch_bounds__(TcCfg<NP, KB>::NT, 1)
             }
             *s_job = jobs[lo];
             const int t = it - s_job->item0;
-            *s_tile = (t >= 0 && t < s_job->count) ? t : -1;
+            *s_item = (t >= 0 && t < s_job->count) ? t : -1;
         } else {
-            *s_tile = (int)blockIdx.x < *one.ntiles ? (int)blockIdx.x : -1;
+            *s_item = (int)blockIdx.x;
         }
-        // the tile's barriers start from phase 0 (the previous tile left
+        // the item's barriers start from phase 0 (the previous item left
         // every barrier idle: all its waits, copies and commits completed)
-        for (int s = 0; s < NG * RSG; s++) mbar_init(&a_full[s], 128);
-        for (int s = 0; s < NB; s++) mbar_init(&b_full[s], 1);
-        for (int s = 0; s < CS; s++) mbar_init(&cmp_full[s], C::NW / C::NG);
-        for (int s = 0; s < NF; s++) mbar_init(&cmp_free[s], 1);
-        for (int b = 0; b < AC; b++) {
+        for (int s = 0; s < NS; s++) {
+            mbar_init(&full[s], 1);
+            mbar_init(&gfull[s], 128);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < 2; b++) {
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], C::NW);
         }
         mbar_init(fin, 1);
-        // per vector: one arrival per warp of the groups that split its KB
-        // units, and one from the operator warp once the operator landed
-        for (int s = 0; s < C::VR; s++) mbar_init(&ready[s], 4 * KB + 1);
-        for (int s = 0; s < NG * RSG * 4; s++) mbar_init(&a_lat[s], 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    const int tile = *s_tile;
-    if (tile < 0) break;
+    const int item = *s_item;
+    if (item < 0) break;
     const M2LJob &J = PERSIST ? *s_job : one;
-    const M2LTile *__restrict__ tiles = J.tiles;
-    const int *__restrict__ tgt = J.tgt;
-    const int4 *__restrict__ xyz = J.xyz;
-    const uint64_t *__restrict__ anchor = J.anchor;
-    const LevelDesc *__restrict__ ld = J.ld;
-    const int *__restrict__ map_pool = J.map_pool;
-    const int4 *__restrict__ st = J.st;
-    const int *__restrict__ st_off = J.st_off;
-    const float *__restrict__ mrow = J.mrow;
-    const unsigned char *__restrict__ ttab = J.ttab;
-    float *__restrict__ L = J.L;
-    const M2LTile td = tiles[tile];
+    const int nsplit = J.nsplit, tile = item / nsplit, split = item - tile * nsplit;
+    const M2LTile td = J.tiles[tile];
     const int PP = p * p;
     const int l = td.level;
-    // this row's cell, its level, lattice position and octant (a pooled tile
-    // mixes levels and octants)
-    int px = 0, py = 0, pz = 0, cell = -1, rl = l, ro = 0;
-    if (worker && row < td.count) {
-        cell = tgt[td.start + row];
-        const int4 a = xyz[cell];
-        rl = a.w;
-        const int sh = FMM_MAXLEVEL - rl;
-        px = a.x >> sh;
-        py = a.y >> sh;
-        pz = a.z >> sh;
-        ro = (px & 1) | ((py & 1) << 1) | ((pz & 1) << 2);
-    }
-    const LevelDesc LD = ld[rl];
-    // the set's entries are sorted by reach: only a prefix can hit a cell
-    const int e0 = st_off[td.octant], nv = st_off[10 + td.octant * (FMM_MAXLEVEL + 1) + l];
+    const int4 *__restrict__ st = J.st;
+    // the set's entries are sorted by reach: only a prefix can hit a cell;
+    // this CTA's range of it
+    const int nvt = J.st_off[10 + td.octant * (FMM_MAXLEVEL + 1) + l];
+    const int w0 = (int)((long long)nvt * split / nsplit), w1 = (int)((long long)nvt * (split + 1) / nsplit);
+    const int e0 = J.st_off[td.octant] + w0, nv = w1 - w0;
     const int nunits = nv * KB;
     const int ngroups = (nv + C::GV - 1) / C::GV;
+    // Lattice tile (a complete level with a lattice copy of M~): the tile is
+    // an 8 x 4 x 4 block of its octant's sub-lattice with rows in x, y, z
+    // order, and for every vector the sources form the same block shifted, in
+    // the sub-lattice of the source octant; positions outside the level
+    // arrive as zeros, as absent cells do.
+    // (persistent launches serve the batch engine, which gathers everywhere)
+    const bool lat = !PERSIST && J.lat_maps != nullptr && td.octant < 8 && ((J.lat_levels >> l) & 1u);
 
     if (warp == C::MMA_WARP) {
         // ------------------------------------------------------------ MMA warp
-        // VEC: one iteration per stencil vector (its KB compute stages and its
-        // operator slot), so the waits and commits, a few hundred cycles each
-        // on the issuing thread, are paid once per vector. Otherwise one
-        // iteration per unit. The whole warp runs the loop; lane 0 issues.
-        const uint32_t id_full = idesc_tf32(128, 2 * NP), id_half = idesc_tf32(128, NP);
-        constexpr int STEP = VEC ? KB : 1;
-        for (int u0 = 0; u0 < nunits; u0 += STEP) {
-            const int vi = u0 / KB, g = vi / C::GV, b = g % AC;
-            bool ok = true;
-#pragma unroll
-            for (int kb = 0; kb < (VEC ? 0 : STEP); kb++) ok = ok && mbar_wait(&cmp_full[(u0 + kb) % CS], (uint32_t)(((u0 + kb) / CS) & 1));
-            if (VEC) ok = mbar_wait(&ready[vi % C::VR], (uint32_t)((vi / C::VR) & 1));
-            if (ok && u0 % KB == 0 && vi % C::GV == 0 && g >= AC) ok = mbar_wait(&acc_empty[b], (uint32_t)(((g - AC) / AC) & 1));
+        // one iteration per unit; the whole warp runs the loop, lane 0 issues
+        const uint32_t id_full = idesc_f16(128, 2 * NP), id_half = idesc_f16(128, NP);
+        for (int u = 0; u < nunits; u++) {
+            const int s = u % NS, vi = u / KB, kb = u % KB, g = vi / C::GV, b = g & 1;
+            const uint32_t ph = (uint32_t)((u / NS) & 1);
+            bool ok = mbar_wait(&full[s], ph);
+            if (!lat) ok = ok && mbar_wait(&gfull[s], ph);
+            if (ok && kb == 0 && vi % C::GV == 0 && g >= 2) ok = mbar_wait(&acc_empty[b], (uint32_t)(((g - 2) >> 1) & 1));
             ok = __all_sync(0xffffffffu, ok) && !*(volatile int *)abort_flag;
             if (!ok) {
                 if (lane == 0) atomicExch(abort_flag, 1);
                 break;
             }
+            if (!lat) fence_proxy_async();  // the gathered rows (generic proxy) before the MMA's reads
             tc_fence_after();
             if (lane == 0) {
                 const uint32_t dmain = tmem + (uint32_t)(b * 2 * NP), dcorr = dmain + NP;
-                const bool first = vi % C::GV == 0;
+                const uint32_t first = (vi % C::GV == 0 && kb == 0) ? 0u : 1u;
+                const uint32_t ahi = smem_u32(base + s * C::STAGE), alo = ahi + (PACK ? 64u : 16384u);
+                const uint32_t bb = ahi + C::A_BYTES;
+                // k-steps of 16 coefficients holding any of the p^2 real ones
+                constexpr int KS = PACK ? NP / 16 : 4;
+                const int ks = min(KS, (PP - kb * 64 + 15) >> 4);
 #pragma unroll
-                for (int kk = 0; kk < STEP; kk++) {
-                    const int u = u0 + kk, c = u % CS, kb = u % KB;
-                    const uint32_t ahi = tmem + (uint32_t)(C::ACC_COLS + c * C::ACOLS), alo = ahi + 32;
-                    const uint32_t bb = VEC ? smem_u32(bops + (vi % NB) * C::OPV + kb * C::B_RAW) : smem_u32(bops + c * C::B_RAW);
-                    // k-steps of 8 coefficients holding any of the p^2 real ones: the
-                    // rest of a padded k-block is zero in A and in the operator and
-                    // would add exactly zero (p = 6: 5 of 8 k-steps; p = 8: all)
-                    const int ks = min(4, (PP - kb * 32 + 7) >> 3);
-#pragma unroll
-                    for (int k = 0; k < 4; k++) {
-                        if (k >= ks) break;
-                        // A_hi [T_hi ; T_lo] -> main | correction, then A_lo T_hi -> correction
-                        mma_tf32_ta(dmain, ahi + 8 * k, sdesc(bb + 32 * k), id_full, (first && kb == 0 && k == 0) ? 0u : 1u);
-                        mma_tf32_ta(dcorr, alo + 8 * k, sdesc(bb + 32 * k), id_half, 1u);
+                for (int k = 0; k < KS; k++) {
+                    if (k >= ks) break;
+                    const uint32_t acc = k == 0 ? first : 1u;
+                    // A_hi [T_hi ; T_lo] -> main | correction, then A_lo T_hi -> correction
+                    if (PACK) {
+                        mma_f16(dmain, sdesc(ahi + 32 * k), sdesc(bb + 32 * k), id_half, acc);
+                        mma_f16(dcorr, sdesc(ahi + 32 * k), sdesc(bb + 64 + 32 * k), id_half, acc);
+                    } else {
+                        mma_f16(dmain, sdesc(ahi + 32 * k), sdesc(bb + 32 * k), id_full, acc);
                     }
+                    mma_f16(dcorr, sdesc(alo + 32 * k), sdesc(bb + 32 * k), id_half, 1u);
                 }
-                if (VEC) mma_commit(&cmp_free[vi % NF]);
-                else mma_commit(&cmp_free[u0 % CS]);
-                if ((u0 + STEP) % KB == 0 && ((vi % C::GV == C::GV - 1) || vi == nv - 1)) mma_commit(&acc_full[b]);
+                mma_commit(&empty[s]);
+                if (kb == KB - 1 && ((vi % C::GV == C::GV - 1) || vi == nv - 1)) mma_commit(&acc_full[b]);
             }
             __syncwarp();
         }
@@ -328,176 +354,79 @@ __global__ void __launch_bounds__(TcCfg<NP, KB>::NT, 1)
             // every commit has arrived before the shared memory goes away
             mma_commit(fin);
             mbar_wait(fin, 0);
-            if (VEC)
-                for (int w = max(0, nv - NF); w < nv; w++) mbar_wait(&cmp_free[w % NF], (uint32_t)((w / NF) & 1));
-            else
-                for (int u = max(0, nunits - CS); u < nunits; u++) mbar_wait(&cmp_free[u % CS], (uint32_t)((u / CS) & 1));
         }
         __syncwarp();
-    } else if (warp == C::B_WARP) {
-        // ------------------------------------------------------- operator warp
-        // VEC: the vector's KB operator blocks (contiguous in the image) in one
-        // bulk copy into slot w % OSV, once vector w - OSV is done. Otherwise
-        // one block per unit into its compute stage, once that stage is free.
-        if (lane == 0) {
+    } else if (warp == C::P_WARP) {
+        // ------------------------------------------------------- producer warp
+        if (lane == 0 && nunits > 0) {
+            int ox = 0, oy = 0, oz = 0;  // tile origin in halved coordinates
+            const int obx = td.octant & 1, oby = (td.octant >> 1) & 1, obz = (td.octant >> 2) & 1;
+            const void *lmap = nullptr;
+            if (lat) {
+                const int4 a = J.xyz[J.tgt[td.start]];
+                const int sh = FMM_MAXLEVEL - l + 1;
+                ox = a.x >> sh;
+                oy = a.y >> sh;
+                oz = a.z >> sh;
+                lmap = (const void *)(J.lat_maps + 128 * l);
+            }
+            const unsigned char *ttab = J.ttab;
             int issued = 0;
-            const int nitems = VEC ? nv : nunits;
-            for (int w = 0; w < nitems; w++) {
+            int4 vn = st[e0];
+            for (int u = 0; u < nunits; u++) {
+                const int s = u % NS, kb = u % KB, w = u / KB;
                 if (*(volatile int *)abort_flag) break;
-                bool ok = true;
-                if (VEC) {
-                    if (w >= NB) ok = mbar_wait(&cmp_free[(w - NB) % NF], (uint32_t)(((w - NB) / NF) & 1));
-                } else if (w >= CS) {
-                    ok = mbar_wait(&cmp_free[w % CS], (uint32_t)(((w - CS) / CS) & 1));
-                }
-                if (!ok) {
+                if (u >= NS && !mbar_wait(&empty[s], (uint32_t)((u / NS - 1) & 1))) {
                     atomicExch(abort_flag, 1);
                     break;
                 }
-                const int bs = w % NB;
-                if (VEC) {
-                    const int4 v = st[e0 + w];
-                    mbar_arrive_tx(&b_full[bs], C::OPV);
-                    bulk_g2s(smem_u32(bops + bs * C::OPV), ttab + (size_t)(v.w & 0xffff) * C::OPV, C::OPV, &b_full[bs]);
-                    // vector w - 1's operator has landed: its readiness
-                    if (w >= 1) {
-                        if (!mbar_wait(&b_full[(w - 1) % NB], (uint32_t)(((w - 1) / NB) & 1))) {
-                            atomicExch(abort_flag, 1);
-                            issued = w + 1;
-                            break;
-                        }
-                        mbar_arrive(&ready[(w - 1) % C::VR]);
-                    }
-                } else {
-                    const int4 v = st[e0 + w / KB];
-                    mbar_arrive_tx(&b_full[bs], C::B_RAW);
-                    bulk_g2s(smem_u32(bops + bs * C::B_RAW), ttab + ((size_t)(v.w & 0xffff) * KB + w % KB) * C::B_RAW,
-                             C::B_RAW, &b_full[bs]);
-                }
-                issued = w + 1;
-            }
-            if (VEC && issued == nitems && nitems > 0 && !*(volatile int *)abort_flag) {
-                if (mbar_wait(&b_full[(nitems - 1) % NB], (uint32_t)(((nitems - 1) / NB) & 1)))
-                    mbar_arrive(&ready[(nitems - 1) % C::VR]);
-                else
-                    atomicExch(abort_flag, 1);
-            }
-            // copies still in flight when the pipeline stopped early land
-            // before the shared memory goes away (bounded waits)
-            if (*(volatile int *)abort_flag)
-                for (int w = max(0, issued - NB); w < issued; w++) mbar_wait(&b_full[w % NB], (uint32_t)((w / NB) & 1));
-        }
-    } else {
-        // ---------------------------------------------------------- worker warps
-        constexpr int HN = C::HN;
-        float acc_hi[HN], acc_lo[HN];
-#pragma unroll
-        for (int k = 0; k < HN; k++) acc_hi[k] = acc_lo[k] = 0.f;
-        const uint32_t tlane = (uint32_t)((warp & 3) * 32) << 16;  // this warp's TMEM lane quarter
-        const int g = grp;
-        const int nown = nunits > g ? (nunits - g + 1) / 2 : 0;  // units u = g, g + 2, ... of this group
-        int *myring = ring + g * RINGU * C::M;
-        const bool dense = LD.map_off >= 0;  // the level has a lattice map: lookups arrive by cp.async
-        const bool full = rl <= 10 && LD.end - LD.start == (1 << (3 * rl));  // every lattice cell present
-        // Lattice tile (a complete level with a lattice copy of M~): the tile
-        // is an 8 x 4 x 4 block of its octant's sub-lattice with rows in x, y,
-        // z order, and for every vector the sources form the same block
-        // shifted, in the sub-lattice of the source octant. Each warp brings
-        // its 32 rows (one z slice) with one TMA tile load; positions outside
-        // the level arrive as zeros, like absent cells.
-        // (persistent launches serve the batch engine, which gathers everywhere)
-        const bool lat = !PERSIST && J.lat_maps != nullptr && td.octant < 8 && ((J.lat_levels >> l) & 1u);
-        const int q = warp & 3;
-        const int obx = td.octant & 1, oby = (td.octant >> 1) & 1, obz = (td.octant >> 2) & 1;
-        // tile origin in halved coordinates (from row 32 q = (0, 0, q), this warp's lane 0)
-        const int ox = (px >> 1) - (row & 7), oy = (py >> 1) - ((row >> 3) & 3), oz = (pz >> 1) - (row >> 5);
-        const void *lmap = lat ? (const void *)(J.lat_maps + 128 * l) : nullptr;
-        int lat_issued = 0, lat_done = 0;  // this warp's TMA loads issued / waited for
-
-        // source cell of this row for the group's unit j, looked up QU units
-        // ahead into ring slot j % RINGU (cp.async of the lattice-map entry, or
-        // a search of the level's keys); only this thread reads the slot, after
-        // the raw-stage barrier that its own later copies arrive on
-        // stencil entry of the group's unit j; the next call's entry is
-        // loaded one call ahead (calls come in order), so its latency is hidden
-        int4 st_next = make_int4(0, 0, 0, 0);
-        int st_next_j = -1;
-        auto fetch = [&](int j) {
-            if (lat || j >= nown) return;
-            const int4 v = st_next_j == j ? st_next : st[e0 + (2 * j + g) / KB];
-            if (j + 1 < nown) {
-                st_next = st[e0 + (2 * (j + 1) + g) / KB];
-                st_next_j = j + 1;
-            }
-            const uint32_t slot = smem_u32(myring + (j % RINGU) * C::M + row);
-            int r = -1;
-            if (cell >= 0) {
-                const int x = px + v.x, y = py + v.y, z = pz + v.z, side = 1 << rl;
-                if (((v.w >> (16 + ro)) & 1) && x >= 0 && y >= 0 && z >= 0 && x < side && y < side && z < side) {
-                    // a complete level holds every lattice cell in Morton order:
-                    // the index follows from the position
-                    if (full) {
-                        myring[(j % RINGU) * C::M + row] = LD.start + (int)morton3_10((uint32_t)x, (uint32_t)y, (uint32_t)z);
-                        return;
-                    }
-                    if (dense) {
-                        cp_async4(slot, map_pool + LD.map_off + (long long)morton3((uint32_t)x, (uint32_t)y, (uint32_t)z));
-                        return;
-                    }
-                    r = level_lookup(LD, map_pool, anchor, rl, x, y, z);
-                }
-            }
-            if (dense && !full) cp_async4(slot, &g_no_cell);
-            else myring[(j % RINGU) * C::M + row] = r;
-        };
-        // copy the group's unit j into its raw stage j % RSG. The warp fills
-        // its own 32 rows: in copy i, lanes 8s .. 8s+7 take the eight 16-byte
-        // chunks of row 4i + s, so one warp instruction reads 4 whole rows
-        // (4 cache lines, not 32); the source of each row comes from the lane
-        // that looked it up
-        auto load_unit = [&](int j) {
-            const int u = 2 * j + g, kb = u % KB;
-            if (lat) {
-                // the stencil entry of this call is loaded one call ahead (the
-                // lookahead registers of the lookups, which lattice tiles skip)
-                if (lane == 0) {
-                    const int4 v = st_next_j == j ? st_next : st[e0 + u / KB];
-                    if (j + 1 < nown) {
-                        st_next = st[e0 + (u + 2) / KB];
-                        st_next_j = j + 1;
-                    }
+                const int4 v = vn;
+                if (kb == KB - 1 && w + 1 < nv) vn = st[e0 + w + 1];
+                const uint32_t sa = smem_u32(base + s * C::STAGE);
+                mbar_arrive_tx(&full[s], C::B_BYTES + (lat ? C::A_BYTES : 0));
+                if (lat) {
                     // source octant bits and the block's shift in halved
                     // coordinates (arithmetic shifts: floor division by 2)
                     const int sx = obx + v.x, sy = oby + v.y, sz = obz + v.z;
                     const int ps = (sx & 1) | ((sy & 1) << 1) | ((sz & 1) << 2);
-                    uint64_t *b = &a_lat[(g * RSG + j % RSG) * 4 + q];
-                    // the warp's generic reads of this stage precede the async-proxy writes
-                    fence_proxy_async();
-                    mbar_arrive_tx(b, 32 * 128);
-                    tma_load_5d(smem_u32(araw + (g * RSG + j % RSG) * C::A_RAW + q * 32 * 128), lmap, kb * 32,
-                                ox + (sx >> 1), oy + (sy >> 1), oz + q + (sz >> 1), ps, b);
+                    const int x = ox + (sx >> 1), y = oy + (sy >> 1), z = oz + (sz >> 1);
+                    tma_load_5d(sa, lmap, kb * (C::ROWB / 2), x, y, z, ps, &full[s]);
+                    if (!PACK) tma_load_5d(sa + 16384, lmap, kb * (C::ROWB / 2) + 64, x, y, z, ps, &full[s]);
                 }
-                lat_issued = j + 1;
-                return;
+                bulk_g2s(sa + C::A_BYTES, ttab + ((size_t)(v.w & 0xffff) * KB + kb) * C::B_BYTES, C::B_BYTES, &full[s]);
+                issued = u + 1;
             }
-            const int src = myring[(j % RINGU) * C::M + row];
-            fetch(j + QU);
-            const uint32_t ab = smem_u32(araw + (g * RSG + j % RSG) * C::A_RAW);
-            const int ch = lane & 7, sub = lane >> 3, r0 = row - lane;  // r0: the warp's first row
+            // copies still in flight when the pipeline stopped early land
+            // before the shared memory goes away (bounded waits)
+            if (*(volatile int *)abort_flag)
+                for (int u = max(0, issued - NS); u < issued; u++) mbar_wait(&full[u % NS], (uint32_t)((u / NS) & 1));
+        }
+    } else {
+        // ---------------------------------------------------------- worker warps
+        constexpr int HN = C::HN;
+        const int row = tid & 127, g = (tid >> 7) & 1;  // target row and group
+        float acc_hi[HN], acc_lo[HN];
 #pragma unroll
-            for (int i = 0; i < 8; i++) {
-                const int rr = r0 + 4 * i + sub;
-                const int s = __shfl_sync(0xffffffffu, src, 4 * i + sub);
-                const float *gs = mrow + ((size_t)(s >= 0 ? s : 0) * KP + kb * 32) + ch * 4;
-                cp_async16(ab + (uint32_t)rr * 128u + ((((uint32_t)ch) ^ ((uint32_t)rr & 7u)) << 4), gs, s >= 0 ? 16u : 0u);
-            }
-            cp_async_arrive_noinc(&a_full[g * RSG + j % RSG]);
-        };
+        for (int k = 0; k < HN; k++) acc_hi[k] = acc_lo[k] = 0.f;
+        const uint32_t tlane = (uint32_t)((warp & 3) * 32) << 16;  // this warp's TMEM lane quarter
+        // this row's cell, its level, lattice position and octant (a pooled
+        // tile mixes levels and octants)
+        int px = 0, py = 0, pz = 0, cell = -1, rl = l, ro = 0;
+        if (row < td.count) {
+            cell = J.tgt[td.start + row];
+            const int4 a = J.xyz[cell];
+            rl = a.w;
+            const int sh = FMM_MAXLEVEL - rl;
+            px = a.x >> sh;
+            py = a.y >> sh;
+            pz = a.z >> sh;
+            ro = (px & 1) | ((py & 1) << 1) | ((pz & 1) << 2);
+        }
 
         auto drain = [&](int gg) {
-            const int b = gg % AC;
+            const int b = gg & 1;
             __syncwarp();
-            const bool ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (uint32_t)((gg / AC) & 1)));
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (uint32_t)((gg >> 1) & 1)));
             if (!ok) {
                 atomicExch(abort_flag, 1);
                 return;
@@ -523,95 +452,148 @@ __global__ void __launch_bounds__(TcCfg<NP, KB>::NT, 1)
             if (lane == 0) mbar_arrive(&acc_empty[b]);
         };
 
-        for (int j = 0; j < QU; j++) fetch(j);
-        cp_async_commit();
-        cp_async_wait_all();
-        for (int j = 0; j < RSG && j < nown; j++) load_unit(j);
         int drained = 0;
-        for (int j = 0; j < nown; j++) {
-            if (*(volatile int *)abort_flag) break;
-            const int u = 2 * j + g, c = u % CS, vi = u / KB;
-            // one accumulator buffer: group gg is drained before group gg + 1 starts
-            if (AC == 1 && vi / C::GV > drained) {
-                drain(drained);
-                drained++;
-                if (*(volatile int *)abort_flag) break;
-            }
-            // the compute stage is free once the unit that used it last (u - CS)
-            // is done: its vector's commit (VEC) or its own (otherwise)
-            const int wprev = max(u - CS, 0) / KB;
-            uint64_t *araw_bar = lat ? &a_lat[(g * RSG + j % RSG) * 4 + q] : &a_full[g * RSG + j % RSG];
-            const bool ok = VEC ? mbar_wait2(u >= CS ? 3u : 1u, araw_bar, (uint32_t)((j / RSG) & 1),
-                                             &cmp_free[wprev % NF], (uint32_t)((wprev / NF) & 1))
-                                : mbar_wait2(u >= CS ? 3u : 1u, araw_bar, (uint32_t)((j / RSG) & 1),
-                                             &cmp_free[c], (uint32_t)((max(u - CS, 0) / CS) & 1));
-            if (!ok) {
-                atomicExch(abort_flag, 1);
-                break;
-            }
-            lat_done = j + 1;
-            tc_fence_after();
-            // split this row's raw FP32 k-block into TF32 (hi, lo): hi rounded to
-            // nearest, lo = a - hi (exact in FP32; the MMA reads its leading 11
-            // bits, an error below 2^-21 of a); both go to the A stage in TMEM
-            const unsigned char *rs = araw + (g * RSG + j % RSG) * C::A_RAW + row * 128;
-            const uint32_t ta = tmem + tlane + (uint32_t)(C::ACC_COLS + c * C::ACOLS);
-            // the second half of a k-block that holds only padding is never read
-            // by the MMAs (they skip its k-steps)
-            const int nh = (u % KB) * 32 + 16 < PP ? 2 : 1;
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                if (h >= nh) break;
-                float hi[16], lo[16];
-#pragma unroll
-                for (int q = 0; q < 4; q++) {
-                    const int ch = 4 * h + q;
-                    const float4 a = *reinterpret_cast<const float4 *>(rs + ((ch ^ (row & 7)) << 4));
-                    hi[4 * q + 0] = tf32_rn(a.x); lo[4 * q + 0] = a.x - hi[4 * q + 0];
-                    hi[4 * q + 1] = tf32_rn(a.y); lo[4 * q + 1] = a.y - hi[4 * q + 1];
-                    hi[4 * q + 2] = tf32_rn(a.z); lo[4 * q + 2] = a.z - hi[4 * q + 2];
-                    hi[4 * q + 3] = tf32_rn(a.w); lo[4 * q + 3] = a.w - hi[4 * q + 3];
+        if (!lat) {
+            const LevelDesc LD = J.ld[rl];
+            const int *__restrict__ map_pool = J.map_pool;
+            const unsigned char *__restrict__ mrow = J.mrow;
+            const int nown = nunits > g ? (nunits - g + 1) / 2 : 0;  // units u = g, g + 2, ... of this group
+            int *myring = ring + g * RINGU * C::M;
+            const bool dense = LD.map_off >= 0;  // the level has a lattice map: lookups arrive by cp.async
+            const bool whole = rl <= 10 && LD.end - LD.start == (1 << (3 * rl));  // every lattice cell present
+            // source cell of this row for the group's unit j, looked up QU units
+            // ahead into ring slot j % RINGU (cp.async of the lattice-map entry,
+            // or a search of the level's keys); only this thread reads the slot
+            // stencil entry of the group's unit j; the next call's entry is
+            // loaded one call ahead (calls come in order), so its latency is hidden
+            int4 st_next = make_int4(0, 0, 0, 0);
+            int st_next_j = -1;
+            auto fetch = [&](int j) {
+                if (j >= nown) return;
+                const int4 v = st_next_j == j ? st_next : st[e0 + (2 * j + g) / KB];
+                if (j + 1 < nown) {
+                    st_next = st[e0 + (2 * (j + 1) + g) / KB];
+                    st_next_j = j + 1;
                 }
-                tmem_st16(ta + 16 * h, hi);
-                tmem_st16(ta + 32 + 16 * h, lo);
-            }
-            // every lane of the warp has read its row of the raw stage: the
-            // next unit's copies may overwrite it while the stores complete
-            __syncwarp();
-            if (j + RSG < nown) load_unit(j + RSG);
-            tmem_wait_st();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) {
-                // (per unit) the group's first warp also waits for the operator block
-                if (!VEC && (warp & 3) == 0 && !mbar_wait(&b_full[c], (uint32_t)((u / CS) & 1))) atomicExch(abort_flag, 1);
-                mbar_arrive(VEC ? &ready[(u / KB) % C::VR] : &cmp_full[c]);
-            }
-            // two accumulator buffers: drain group gg once group gg + 1 is well under way
-            if (AC == 2 && vi >= C::DRAIN_AT && (vi - C::DRAIN_AT) / C::GV > drained) {
-                drain(drained);
-                drained++;
-            }
-        }
-        cp_async_wait_all();
-        // tile loads still in flight when the loop stopped early land before
-        // the shared memory is reused or released (bounded waits)
-        if (lat && lane == 0)
-            for (int jj = lat_done; jj < lat_issued; jj++)
-                mbar_wait(&a_lat[(g * RSG + jj % RSG) * 4 + q], (uint32_t)((jj / RSG) & 1));
-        __syncwarp();
-        if (!*(volatile int *)abort_flag) {
-            while (drained < ngroups) {
-                drain(drained);
-                drained++;
+                int *const slot = myring + (j % RINGU) * C::M + row;
+                int r = -1;
+                if (cell >= 0) {
+                    const int x = px + v.x, y = py + v.y, z = pz + v.z, side = 1 << rl;
+                    if (((v.w >> (16 + ro)) & 1) && x >= 0 && y >= 0 && z >= 0 && x < side && y < side && z < side) {
+                        // a complete level holds every lattice cell in Morton order:
+                        // the index follows from the position
+                        if (whole) {
+                            *slot = LD.start + (int)morton3_10((uint32_t)x, (uint32_t)y, (uint32_t)z);
+                            return;
+                        }
+                        if (dense) {
+                            cp_async4(smem_u32(slot), map_pool + LD.map_off + (long long)morton3((uint32_t)x, (uint32_t)y, (uint32_t)z));
+                            return;
+                        }
+                        r = level_lookup(LD, map_pool, J.anchor, rl, x, y, z);
+                    }
+                }
+                if (dense && !whole) cp_async4(smem_u32(slot), &g_no_cell);
+                else *slot = r;
+            };
+            for (int j = 0; j < QU; j++) fetch(j);
+            cp_async_commit();
+            cp_async_wait_all();
+            for (int j = 0; j < nown; j++) {
                 if (*(volatile int *)abort_flag) break;
-            }
-        }
-        if (cell >= 0 && !*(volatile int *)abort_flag) {
-            float *Lc = L + (size_t)cell * PP + g * HN;
+                const int u = 2 * j + g, s = u % NS, kb = u % KB, vi = u / KB;
+                const bool ok = u < NS || mbar_wait(&empty[s], (uint32_t)((u / NS - 1) & 1));
+                if (!__all_sync(0xffffffffu, ok)) {
+                    atomicExch(abort_flag, 1);
+                    break;
+                }
+                // slot j was fetched with the copies of unit j - QU: all but the
+                // QU - 1 latest groups of copies are complete
+                cp_async_wait<QU - 1>();
+                const int src = myring[(j % RINGU) * C::M + row];
+                // The warp fills its own 32 rows: in copy i, groups of CL lanes
+                // take the CL 16-byte chunks of consecutive rows, so one warp
+                // instruction reads whole rows; the source of each row comes from
+                // the lane that looked it up
+                constexpr int CL = C::ROWB / 16;  // 16 (hi 8 | lo 8), PACK: 8
+                const uint32_t sa = smem_u32(base + s * C::STAGE);
+                const int ch = lane % CL, sub = lane / CL, r0 = row - lane;  // r0: the warp's first row
+                const uint32_t part = sa + (uint32_t)((ch >> 3) * 16384);
+                const unsigned char *colp = mrow + kb * C::ROWB + ch * 16;
 #pragma unroll
-            for (int k = 0; k < HN; k++)
-                if (g * HN + k < PP) Lc[k] += acc_hi[k] + acc_lo[k];
+                for (int i = 0; i < CL; i++) {
+                    const int rr = r0 + (32 / CL) * i + sub;
+                    const int sc = __shfl_sync(0xffffffffu, src, (32 / CL) * i + sub);
+                    cp_async16(part + (uint32_t)rr * 128u + ((((uint32_t)ch & 7u) ^ ((uint32_t)rr & 7u)) << 4),
+                               colp + (size_t)(sc >= 0 ? sc : 0) * (KB * C::ROWB), sc >= 0 ? 16u : 0u);
+                }
+                fetch(j + QU);
+                cp_async_arrive_noinc(&gfull[s]);
+                cp_async_commit();
+                // drain group gg once group gg + 1 is well under way
+                if (vi >= C::DRAIN_AT && (vi - C::DRAIN_AT) / C::GV > drained) {
+                    drain(drained);
+                    drained++;
+                }
+            }
+            cp_async_wait_all();
+            __syncwarp();
+        }
+        while (drained < ngroups && !*(volatile int *)abort_flag) {
+            drain(drained);
+            drained++;
+        }
+        // once every worker warp is here the flag is final: either a wait has
+        // failed, or the last drain saw the last MMA and nothing is waiting
+        named_barrier_sync(1, C::NW * 32);
+        if (!*(volatile int *)abort_flag) {
+            bool write = true;
+            if (nsplit > 1) {
+                // the range's sums, [item][coefficient][row]; the tile's last
+                // range to finish adds them all in order
+                const size_t rng = (size_t)PP * C::M;
+                float2 *pt = J.part + (size_t)item * rng + row;
+#pragma unroll
+                for (int k = 0; k < HN; k++)
+                    if (g * HN + k < PP) __stcg(&pt[(size_t)(g * HN + k) * C::M], make_float2(acc_hi[k], acc_lo[k]));
+                __threadfence();
+                named_barrier_sync(1, C::NW * 32);
+                if (tid == 0) {
+                    const bool last = atomicAdd(&J.tcnt[tile], 1u) == (unsigned)(nsplit - 1);
+                    if (last) J.tcnt[tile] = 0u;
+                    *s_last = last;
+                    __threadfence();
+                }
+                named_barrier_sync(1, C::NW * 32);
+                write = *(volatile int *)s_last != 0;
+                if (write) {
+                    pt = J.part + (size_t)tile * nsplit * rng + row;
+#pragma unroll
+                    for (int k = 0; k < HN; k++) acc_hi[k] = acc_lo[k] = 0.f;
+                    for (int r = 0; r < nsplit; r++, pt += rng) {
+                        float2 v[HN];
+#pragma unroll
+                        for (int k = 0; k < HN; k++)
+                            v[k] = g * HN + k < PP ? __ldcg(&pt[(size_t)(g * HN + k) * C::M]) : make_float2(0.f, 0.f);
+#pragma unroll
+                        for (int k = 0; k < HN; k++) {
+                            two_sum_acc(acc_hi[k], acc_lo[k], v[k].x);
+                            acc_lo[k] += v[k].y;
+                        }
+                    }
+                }
+            }
+            if (write && cell >= 0) {
+                // back from the operands' powers of two
+                const int e = m2l_exponent(J.lmax[rl]);
+                float *Lc = J.L + (size_t)cell * PP + g * HN;
+#pragma unroll
+                for (int k = 0; k < HN; k++)
+                    if (g * HN + k < PP) {
+                        const int t = J.rowexp[g * HN + k] - e;
+                        Lc[k] += ((acc_hi[k] + acc_lo[k]) * m2l_pow2(t >> 1)) * m2l_pow2(t - (t >> 1));
+                    }
+            }
         }
     }
     tc_fence_before();
@@ -619,9 +601,9 @@ __global__ void __launch_bounds__(TcCfg<NP, KB>::NT, 1)
     tc_fence_after();
     const bool aborted = *(volatile int *)abort_flag != 0;
     if (tid == 0 && aborted) atomicExch(err, 1);
-    __syncthreads();  // every thread has read the flag before the next tile resets it
+    __syncthreads();  // every thread has read the flag before the next item resets it
     if (aborted) break;
-    }  // tiles
+    }  // items
     tc_fence_before();
     __syncthreads();
     if (warp == C::MMA_WARP) {
@@ -632,40 +614,21 @@ __global__ void __launch_bounds__(TcCfg<NP, KB>::NT, 1)
 // ---------------------------------------------------------------------------
 // host
 // ---------------------------------------------------------------------------
-struct TcShape {
-    int NP, KB;
-};
-
-static TcShape tc_shape(int p)
+// p^2 padded to the MMA's N; 0: not supported
+static int tc_np(int p)
 {
     const int PP = p * p;
-    if (PP <= 16) return {16, 1};
-    if (PP <= 32) return {32, 1};
-    if (PP <= 48) return {48, 2};
-    if (PP <= 64) return {64, 2};
-    if (PP <= 96) return {96, 3};
-    if (PP <= 112) return {112, 4};
-    if (PP <= 128) return {128, 4};
-    return {0, 0};
+    for (int np : {16, 32, 48, 64, 96, 112, 128})
+        if (PP <= np) return np;
+    return 0;
 }
+static int tc_kb(int p) { return (tc_np(p) + 63) / 64; }                      // k-blocks of 64 coefficients
+static size_t tc_row_bytes(int p) { return (size_t)tc_kb(p) * (tc_np(p) <= 32 ? 128 : 256); }
+static size_t tc_op_bytes(int p) { return (size_t)tc_kb(p) * (tc_np(p) <= 32 ? 1 : 2) * tc_np(p) * 128; }
 
-bool tensor_m2l_supported(fmm_ctx *h) { return h->p >= 2 && tc_shape(h->p).NP > 0 && h->cc_major == 10; }
+bool tensor_m2l_supported(fmm_ctx *h) { return h->p >= 2 && tc_np(h->p) > 0 && h->cc_major == 10; }
 
 void tensor_tables_init(fmm_ctx *) {}
-
-// T_v for every stencil vector: the real p^2 x p^2 map of M2L in the packed
-// layout, L~_n^m = (-1)^n sum_{j,k} M~_j^k I_{j+n}^{k+m}(u), u = -v; split into
-// TF32 (hi, lo) and laid out as the 128B-swizzled shared-memory image of the
-// B operand: per k-block, rows 0..NP-1 = T_hi, rows NP..2NP-1 = T_lo.
-static float tf32_rn_host(float a)
-{
-    uint32_t u;
-    memcpy(&u, &a, 4);
-    if ((u & 0x7f800000u) != 0x7f800000u) u = (u + 0x1000u) & 0xffffe000u;
-    float r;
-    memcpy(&r, &u, 4);
-    return r;
-}
 
 // I_n^m(x) in full storage (n*n + n + m), degrees < Q, from the Cartesian
 // recurrences of the irregular solid harmonics
@@ -708,42 +671,42 @@ static void build_irregular_full(int Q, double x, double y, double z, std::vecto
     }
 }
 
-// The operator image depends only on p and the stencil, which the MAC
-// constant and the stencil bound fix (vectors are numbered in a fixed order):
-// handles with the same three share one host image, built once per process.
-static std::mutex g_img_mu;
-static std::map<std::tuple<int, double, int>, std::shared_ptr<const std::vector<unsigned char>>> g_img_cache;
+// The operators of every stencil vector: the real p^2 x p^2 map of M2L in the
+// packed layout, L~_n^m = (-1)^n sum_{j,k} M~_j^k I_{j+n}^{k+m}(u), u = -v,
+// its columns divided by m2l_norm and its rows multiplied by 2^-rowexp (a
+// factorial part as for the columns, and a part per degree that brings the
+// largest entries of the degree into [2^13, 2^14)), then split into FP16 (hi,
+// lo) and laid out as the 128B-swizzled shared-memory image of the B operand:
+// per k-block of 64 columns, rows 0..NP-1 = T_hi, rows NP..2NP-1 = T_lo (NP <=
+// 32: rows of T_hi | T_lo). The rowexp of the coefficients follow the vectors.
+// It depends only on p and the stencil, which the MAC constant and the
+// stencil bound fix (vectors are numbered in a fixed order): the host image is
+// built once per process, and the handles of one device that use it share one
+// device copy, which lives as long as the last of them (a batch's tiles then
+// find the operators of every system in L2).
+struct TcImage {
+    DevBuf buf;
+    ~TcImage() { buf.release(); }
+};
+using HostImage = std::vector<unsigned char>;
 
-void tensor_tables_update(fmm_ctx *h)
+static std::mutex g_img_mu;
+static std::map<std::tuple<int, double, int>, std::shared_ptr<const HostImage>> g_img_cache;
+static std::map<std::tuple<int, double, int, int>, std::weak_ptr<TcImage>> g_dev_img;
+
+static std::shared_ptr<const HostImage> build_image(fmm_ctx *h)
 {
-    const TcShape sh = tc_shape(h->p);
-    if (!sh.NP) return;
-    if (h->ttab_nv == h->nV && h->ttab.p) return;
-    const auto key = std::make_tuple(h->p, h->cmac, h->st_R);
-    {
-        std::lock_guard<std::mutex> lk(g_img_mu);
-        auto it = g_img_cache.find(key);
-        if (it != g_img_cache.end()) {
-            h->ttab.ensure(it->second->size());
-            FMM_CUDA_TRY(cudaMemcpy(h->ttab.p, it->second->data(), it->second->size(), cudaMemcpyHostToDevice));
-            h->ttab_stride = (size_t)tc_shape(h->p).KB * 2 * tc_shape(h->p).NP * 128;
-            h->ttab_nv = h->nV;
-            return;
-        }
-    }
-    const int p = h->p, PP = p * p, Q = 2 * p - 1, NP = sh.NP, KB = sh.KB;
-    const size_t bbytes = (size_t)2 * NP * 128;  // one k-block of [T_hi ; T_lo]
-    const size_t per_v = (size_t)KB * bbytes;
-    std::vector<unsigned char> img((size_t)h->nV * per_v, 0);
+    const int p = h->p, PP = p * p, Q = 2 * p - 1, NP = tc_np(p);
+    const bool pack = NP <= 32;
+    const size_t per_v = tc_op_bytes(p), bbytes = per_v / tc_kb(p);
+    auto img = std::make_shared<HostImage>();
+    img->assign((size_t)h->nV * per_v + sizeof(int) * M2L_NORM_N, 0);
     std::vector<int> seen(h->nV, 0);
     std::vector<double> Ire, Iim, T((size_t)PP * PP);
     auto re_i = [](int n, int m) { return n * n + (m == 0 ? 0 : 2 * m - 1); };
     auto im_i = [](int n, int m) { return n * n + 2 * m; };
     const int ne = h->st_off[8];
-    for (int e = 0; e < ne; e++) {
-        const int vx = h->st_host[4 * e], vy = h->st_host[4 * e + 1], vz = h->st_host[4 * e + 2], id = h->st_host[4 * e + 3] & 0xffff;
-        if (seen[id]) continue;
-        seen[id] = 1;
+    auto make = [&](int vx, int vy, int vz) {
         build_irregular_full(Q, -(double)vx, -(double)vy, -(double)vz, Ire, Iim);
         auto I = [&](int n, int m, double &r, double &i) {
             r = Ire[n * n + n + m];
@@ -778,77 +741,155 @@ void tensor_tables_update(fmm_ctx *h)
                             if (m) T[(size_t)im_i(n, m) * PP + col] = si;
                         }
                 }
-        // per k-block the 128B-swizzled image of [T_hi ; T_lo]: rows 0..NP-1
-        // hold hi = TF32(T) (round to nearest), rows NP..2NP-1 lo = T - hi
-        unsigned char *dst = img.data() + (size_t)id * per_v;
+        for (int r = 0; r < PP; r++)
+            for (int c = 0; c < PP; c++)
+                T[(size_t)r * PP + c] = std::ldexp(T[(size_t)r * PP + c], -(m2l_fact_exp(r) + m2l_norm_exp(c)));
+    };
+    // the entries decay with the distance: a degree's largest belongs to the
+    // shortest vectors (with the factor of 4 that [2^13, 2^14) leaves to FP16's
+    // largest value, beyond which the build of the image would fail)
+    double d2min = 1e300, big[FMM_MAXP] = {};
+    auto d2 = [&](int e) {
+        const int *v = &h->st_host[4 * (size_t)e];
+        return (double)v[0] * v[0] + (double)v[1] * v[1] + (double)v[2] * v[2];
+    };
+    for (int e = 0; e < ne; e++) d2min = std::min(d2min, d2(e));
+    for (int e = 0; e < ne; e++) {
+        const int *v = &h->st_host[4 * (size_t)e];
+        if (seen[v[3] & 0xffff] || d2(e) > 2.0 * d2min) continue;
+        seen[v[3] & 0xffff] = 1;
+        make(v[0], v[1], v[2]);
+        for (int n = 0; n < p; n++)
+            for (size_t i = (size_t)n * n * PP; i < (size_t)(n + 1) * (n + 1) * PP; i++) big[n] = std::max(big[n], std::fabs(T[i]));
+    }
+    std::fill(seen.begin(), seen.end(), 0);
+    std::vector<int> rexp(M2L_NORM_N, 0), rowexp(M2L_NORM_N, 0);
+    for (int n = 0; n < p; n++)
+        for (int r = n * n; r < (n + 1) * (n + 1); r++) {
+            rexp[r] = big[n] > 0 ? 13 - std::ilogb(big[n]) : 0;
+            rowexp[r] = m2l_fact_exp(r) - rexp[r];
+        }
+    memcpy(img->data() + (size_t)h->nV * per_v, rowexp.data(), sizeof(int) * M2L_NORM_N);
+    for (int e = 0; e < ne; e++) {
+        const int *v = &h->st_host[4 * (size_t)e];
+        const int id = v[3] & 0xffff;
+        if (seen[id]) continue;
+        seen[id] = 1;
+        make(v[0], v[1], v[2]);
+        unsigned char *dst = img->data() + (size_t)id * per_v;
         for (int r = 0; r < PP; r++)
             for (int c = 0; c < PP; c++) {
-                const double t = T[(size_t)r * PP + c];
-                const float hi = tf32_rn_host((float)t);
-                const float lo = (float)(t - (double)hi);
-                const int kb = c >> 5, cc = c & 31;
+                const double t = std::ldexp(T[(size_t)r * PP + c], rexp[r]);
+                if (!(std::fabs(t) < 65504.0)) throw Error{FMM_EINVAL, "tensor-core M2L: operator entry beyond FP16"};
+                const __half hi = __float2half_rn((float)t);
+                const __half lo = __float2half_rn((float)(t - (double)__half2float(hi)));
+                const int kb = pack ? 0 : c >> 6;
                 for (int part = 0; part < 2; part++) {
-                    const int row = r + part * NP;
-                    const size_t off = (size_t)kb * bbytes + (size_t)row * 128 + (size_t)((((cc >> 2) ^ (row & 7)) << 4) + (cc & 3) * 4);
-                    const float v = part ? lo : hi;
-                    memcpy(dst + off, &v, 4);
+                    const int row = pack ? r : r + part * NP, cc = pack ? c + 32 * part : c & 63;
+                    const size_t off = (size_t)kb * bbytes + (size_t)row * 128 + (size_t)((((cc >> 3) ^ (row & 7)) << 4) + (cc & 7) * 2);
+                    const __half x = part ? lo : hi;
+                    memcpy(dst + off, &x, 2);
                 }
             }
     }
-    h->ttab.ensure(img.size());
-    FMM_CUDA_TRY(cudaMemcpy(h->ttab.p, img.data(), img.size(), cudaMemcpyHostToDevice));
-    h->ttab_stride = per_v;
-    h->ttab_nv = h->nV;
-    std::lock_guard<std::mutex> lk(g_img_mu);
-    g_img_cache[key] = std::make_shared<const std::vector<unsigned char>>(std::move(img));
+    return img;
 }
 
-template <int NP, int KB>
+void tensor_tables_update(fmm_ctx *h)
+{
+    if (!tc_np(h->p)) return;
+    if (h->ttab_nv == h->nV && h->ttab) return;
+    std::lock_guard<std::mutex> lk(g_img_mu);
+    auto &dev = g_dev_img[std::make_tuple(h->p, h->cmac, h->st_R, h->dev)];
+    std::shared_ptr<TcImage> img = dev.lock();
+    if (!img) {
+        auto &host = g_img_cache[std::make_tuple(h->p, h->cmac, h->st_R)];
+        if (!host) host = build_image(h);
+        img = std::make_shared<TcImage>();
+        img->buf.ensure(host->size());
+        FMM_CUDA_TRY(cudaMemcpy(img->buf.p, host->data(), host->size(), cudaMemcpyHostToDevice));
+        // handles on other streams may read the copy as soon as it is shared
+        FMM_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));
+        dev = img;
+    }
+    h->ttab = img;
+    h->ttab_nv = h->nV;
+}
+
+template <int NP>
 static void launch_tc(int p, int grid, const M2LJob &one, const M2LJob *jobs, int njobs, int *queue, int *err,
                       cudaStream_t s)
 {
-    using C = TcCfg<NP, KB>;
-    // grid: one CTA per SM with a job list (persistent), else one per tile
+    using C = TcCfg<NP>;
+    // grid: one CTA per SM with a job list (persistent), else one per item
     if (jobs) {
-        ensure_smem((const void *)m2l_tc_k<NP, KB, true>, C::SMEM);
+        ensure_smem((const void *)m2l_tc_k<NP, true>, C::SMEM);
         FMM_CUDA_TRY(cudaMemsetAsync(queue, 0, sizeof(int), s));
-        m2l_tc_k<NP, KB, true><<<grid, C::NT, C::SMEM, s>>>(p, one, jobs, njobs, queue, err);
+        m2l_tc_k<NP, true><<<grid, C::NT, C::SMEM, s>>>(p, one, jobs, njobs, queue, err);
     } else {
-        ensure_smem((const void *)m2l_tc_k<NP, KB, false>, C::SMEM);
-        m2l_tc_k<NP, KB, false><<<grid, C::NT, C::SMEM, s>>>(p, one, jobs, njobs, queue, err);
+        ensure_smem((const void *)m2l_tc_k<NP, false>, C::SMEM);
+        m2l_tc_k<NP, false><<<grid, C::NT, C::SMEM, s>>>(p, one, jobs, njobs, queue, err);
     }
 }
 
-static void launch_tc_p(int p, int nsm, const M2LJob &one, const M2LJob *jobs, int njobs, int *queue, int *err,
+#define FMM_TC_SWITCH(np, CALL)                                            \
+    switch (np) {                                                          \
+    case 16: CALL(16); break;                                              \
+    case 32: CALL(32); break;                                              \
+    case 48: CALL(48); break;                                              \
+    case 64: CALL(64); break;                                              \
+    case 96: CALL(96); break;                                              \
+    case 112: CALL(112); break;                                            \
+    case 128: CALL(128); break;                                            \
+    default: throw Error{FMM_EINVAL, "tensor-core M2L: unsupported p"};    \
+    }
+
+static void launch_tc_p(int p, int grid, const M2LJob &one, const M2LJob *jobs, int njobs, int *queue, int *err,
                         cudaStream_t s)
 {
-    switch (tc_shape(p).NP) {
-    case 16: launch_tc<16, 1>(p, nsm, one, jobs, njobs, queue, err, s); break;
-    case 32: launch_tc<32, 1>(p, nsm, one, jobs, njobs, queue, err, s); break;
-    case 48: launch_tc<48, 2>(p, nsm, one, jobs, njobs, queue, err, s); break;
-    case 64: launch_tc<64, 2>(p, nsm, one, jobs, njobs, queue, err, s); break;
-    case 96: launch_tc<96, 3>(p, nsm, one, jobs, njobs, queue, err, s); break;
-    case 112: launch_tc<112, 4>(p, nsm, one, jobs, njobs, queue, err, s); break;
-    case 128: launch_tc<128, 4>(p, nsm, one, jobs, njobs, queue, err, s); break;
-    default: throw Error{FMM_EINVAL, "tensor-core M2L: unsupported p"};
+#define FMM_TC_CALL(NPV) launch_tc<NPV>(p, grid, one, jobs, njobs, queue, err, s)
+    FMM_TC_SWITCH(tc_np(p), FMM_TC_CALL)
+#undef FMM_TC_CALL
+}
+
+// words of the M2L workspace: per-level maxima, then one counter per tile
+constexpr int TCW_CNT = 32;
+
+// How many ranges the vectors of every tile are cut into. A CTA's time is
+// about (its vectors + 10) units, one unit a vector's copies, plus one per
+// range for the last CTA's sum of them; the launch takes the waves of
+// ntiles x nsplit CTAs over the SMs. One range wins as soon as the tiles fill
+// a few waves.
+void m2l_plan(fmm_ctx *h)
+{
+    h->m2l_nsplit = 1;
+    if (h->precision != FMM_MIXED || h->engine_used != FMM_M2L_TENSOR || h->ntiles_max < 1) return;
+    const int pool_max = h->m2l_pool >= 0 ? h->m2l_pool : 4 * TcCfg<64>::M;
+    int nv = 1;
+    for (int l = 2; l <= h->depth; l++) {
+        const int cells = h->lvl_start[(size_t)l + 1] - h->lvl_start[(size_t)l];
+        for (int o = cells <= pool_max ? 8 : 0; o < (cells <= pool_max ? 9 : 8); o++)
+            nv = std::max(nv, h->st_cnt[(size_t)o * (FMM_MAXLEVEL + 1) + l]);
+    }
+    double best = 1e300;
+    for (int s = 1; s <= 32; s++) {
+        const double waves = (double)(((int64_t)h->ntiles_max * s + h->nsm - 1) / h->nsm);
+        const double t = waves * ((double)nv / s + 10.0) + (s > 1 ? s : 0);
+        if (t < best) {
+            best = t;
+            h->m2l_nsplit = s;
+        }
     }
 }
 
-M2LJob m2l_tensor_job(fmm_ctx *h, float *L, const float *M, cudaStream_t s)
+M2LJob m2l_tensor_job(fmm_ctx *h, float *L)
 {
     tensor_tables_update(h);
-    const TcShape sh = tc_shape(h->p);
-    const int c0 = h->depth >= 2 ? h->lvl_start[2] : h->ncells;
-    const int nc = h->ncells, PP = h->p * h->p, KP = sh.KB * 32;
-    const float *mrow = M;
-    if (PP != KP) {  // zero-padded rows of KB * 32 coefficients
-        h->msplit.ensure(sizeof(float) * (size_t)nc * KP);
-        if (nc > c0) {
-            mpad_k<<<nblk((int64_t)(nc - c0) * KP, 256), 256, 0, s>>>(M, PP, KP, c0, nc, h->msplit.as<float>());
-            count_launch(h);
-        }
-        mrow = h->msplit.as<float>();
-    }
+    const int nc = h->ncells;
+    h->msplit.ensure(tc_row_bytes(h->p) * (size_t)nc);
+    h->m2l_ws.ensure(sizeof(unsigned) * (TCW_CNT + (size_t)h->ntiles_max));
+    if (h->m2l_nsplit > 1)
+        h->m2l_part.ensure(sizeof(float2) * (size_t)h->ntiles_max * h->m2l_nsplit * h->p * h->p * TcCfg<64>::M);
     M2LJob j;
     j.tiles = h->m2l_tiles.as<M2LTile>();
     j.ntiles = reinterpret_cast<const int *>(h->m2l_misc.as<unsigned>() + 24 * (FMM_MAXLEVEL + 1));
@@ -859,9 +900,15 @@ M2LJob m2l_tensor_job(fmm_ctx *h, float *L, const float *M, cudaStream_t s)
     j.map_pool = h->map_pool.as<int>();
     j.st = h->st_dev.as<int4>();
     j.st_off = stencil_offsets(h);
-    j.mrow = mrow;
-    j.ttab = h->ttab.as<unsigned char>();
+    j.mrow = h->msplit.as<unsigned char>();
+    j.ttab = h->ttab->buf.as<unsigned char>();
     j.L = L;
+    j.lmax = h->m2l_ws.as<unsigned>();
+    j.tcnt = h->m2l_ws.as<unsigned>() + TCW_CNT;
+    j.ws_words = TCW_CNT + h->ntiles_max;
+    j.part = h->m2l_part.as<float2>();
+    j.nsplit = h->m2l_nsplit;
+    j.rowexp = reinterpret_cast<const int *>(j.ttab + (size_t)h->nV * tc_op_bytes(h->p));
     j.lat_maps = nullptr;  // gathers on every level (the single-system launch sets the lattice levels)
     j.lat_levels = 0;
     j.item0 = 0;
@@ -891,19 +938,20 @@ static EncodeTiledFn encode_tiled()
 
 // The complete levels whose tiles are lattice blocks (at least 8^4 cells,
 // more than the pooling threshold, so every tile is 128 cells of one octant)
-// read their sources by TMA from a lattice copy of M~: one 5-D tensor map per
-// level over [octant bits][z/2][y/2][x/2][KP coefficients] (FP32), box
-// 32 coefficients x 8 x 4 x 1 x 1 = one warp's 32 rows, 128-byte swizzle
-// (the layout of the gathered stages). Levels beyond 9 keep the gathers.
+// read their sources by TMA from the lattice copy of their rows: one 5-D
+// tensor map per level over [octant bits][z/2][y/2][x/2][row] (FP16), box 64
+// halves x 8 x 4 x 4 x 1 = one half (hi or lo) of the tile's 128 rows,
+// 128-byte swizzle (the layout of the gathered stages). Levels beyond 9 keep
+// the gathers.
 void lattice_prepare(fmm_ctx *h, cudaStream_t s)
 {
     h->lat_levels = 0;
     if (!h->lattice_req || h->precision != FMM_MIXED || h->engine_used != FMM_M2L_TENSOR || !tensor_m2l_supported(h) ||
-        m2l_tile_size(h) != TcCfg<64, 2>::M)
+        m2l_tile_size(h) != TcCfg<64>::M)
         return;
     const EncodeTiledFn enc = encode_tiled();
     if (!enc) return;
-    const int KP = tc_shape(h->p).KB * 32;
+    const cuuint64_t row = tc_row_bytes(h->p);
     const int pool_max = h->m2l_pool >= 0 ? h->m2l_pool : 4 * m2l_tile_size(h);
     unsigned levels = 0;
     long long total = 0;
@@ -912,10 +960,10 @@ void lattice_prepare(fmm_ctx *h, cudaStream_t s)
         if (cells != (1ll << (3 * l)) || cells <= pool_max) continue;
         levels |= 1u << l;
         h->lat_off[l] = total;
-        total += cells * KP;
+        total += cells;
     }
     if (!levels) return;
-    h->mlat.ensure(sizeof(float) * (size_t)total);
+    h->mlat.ensure((size_t)row * (size_t)total);
     const size_t mbytes = sizeof(CUtensorMap) * (FMM_MAXLEVEL + 1);
     h->lat_maps.ensure(mbytes);
     h->lat_host.ensure(mbytes);
@@ -923,11 +971,11 @@ void lattice_prepare(fmm_ctx *h, cudaStream_t s)
     std::memset(mp, 0, mbytes);
     for (int l = 4; l <= 9; l++) {
         if (!((levels >> l) & 1u)) continue;
-        const cuuint64_t H = 1ull << (l - 1), row = sizeof(float) * (cuuint64_t)KP;
-        const cuuint64_t dims[5] = {(cuuint64_t)KP, H, H, H, 8};
+        const cuuint64_t H = 1ull << (l - 1);
+        const cuuint64_t dims[5] = {row / 2, H, H, H, 8};
         const cuuint64_t strides[4] = {row, row * H, row * H * H, row * H * H * H};
-        const cuuint32_t box[5] = {32, 8, 4, 1, 1}, estride[5] = {1, 1, 1, 1, 1};
-        const CUresult r = enc(&mp[l], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, h->mlat.as<float>() + h->lat_off[l], dims,
+        const cuuint32_t box[5] = {64, 8, 4, 4, 1}, estride[5] = {1, 1, 1, 1, 1};
+        const CUresult r = enc(&mp[l], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5, h->mlat.as<unsigned char>() + row * h->lat_off[l], dims,
                                strides, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) throw Error{FMM_ECUDA, "tensor-core M2L: encoding a lattice tensor map failed"};
@@ -936,23 +984,27 @@ void lattice_prepare(fmm_ctx *h, cudaStream_t s)
     h->lat_levels = levels;
 }
 
-__global__ void batch_mpad_k(int PP, int KP, const BatchSys *__restrict__ sys)
+template <int NP>
+__global__ void __launch_bounds__(256) batch_split_k(int PP, const BatchSys *__restrict__ sys)
 {
+    using C = TcCfg<NP>;
+    constexpr int NCH = NP / 8;
     const BatchSys &S = sys[blockIdx.y];
-    if (!S.mpad || S.c0 >= S.ncells) return;
-    const int64_t cnt = (int64_t)(S.ncells - S.c0) * KP;
+    if (!S.rows || S.c0 >= S.ncells) return;
+    const int64_t cnt = (int64_t)(S.ncells - S.c0) * NCH;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = S.c0 + (int)(i / KP), k = (int)(i % KP);
-        S.mpad[(size_t)c * KP + k] = k < PP ? S.M[(size_t)c * PP + k] : 0.f;
+        const int c = S.c0 + (int)(i / NCH), ch = (int)(i % NCH);
+        m2l_split_chunk<NP>(S.M + (size_t)c * PP, PP, ch, m2l_exponent(S.m2l_ws[S.xyz[c].w]),
+                            S.rows + (size_t)c * (C::KB * C::ROWB));
     }
 }
 
-void batch_mpad(int p, const BatchSys *sys, int nsys, cudaStream_t s)
+void batch_split(int p, const BatchSys *sys, int nsys, cudaStream_t s)
 {
-    const int PP = p * p, KP = tc_shape(p).KB * 32;
-    if (PP == KP) return;
-    batch_mpad_k<<<dim3(16, (unsigned)nsys), 256, 0, s>>>(PP, KP, sys);
-    check_launch("batch pad");
+#define FMM_TC_CALL(NPV) batch_split_k<NPV><<<dim3(16, (unsigned)nsys), 256, 0, s>>>(p *p, sys)
+    FMM_TC_SWITCH(tc_np(p), FMM_TC_CALL)
+#undef FMM_TC_CALL
+    check_launch("batch split");
 }
 
 void m2l_tensor_jobs(int p, int nsm, const M2LJob *jobs_dev, int njobs, int *queue, int *err, cudaStream_t s)
@@ -965,23 +1017,38 @@ void m2l_tensor_jobs(int p, int nsm, const M2LJob *jobs_dev, int njobs, int *que
 void m2l_tensor(fmm_ctx *h, float *L, const float *M)
 {
     cudaStream_t s = h->work;
-    M2LJob j = m2l_tensor_job(h, L, M, s);
-    if (h->lat_levels) {
-        const int PP = h->p * h->p, KP = tc_shape(h->p).KB * 32;
-        for (int l = 0; l <= FMM_MAXLEVEL; l++) {
-            if (!((h->lat_levels >> l) & 1u)) continue;
-            const int c0 = h->lvl_start[(size_t)l], c1 = h->lvl_start[(size_t)l + 1];
-            lattice_fill_k<<<nblk((int64_t)(c1 - c0) * KP, 256), 256, 0, s>>>(M, PP, KP, h->c_xyz.as<int4>(), c0, c1, l,
-                                                                            h->mlat.as<float>() + h->lat_off[l]);
-            count_launch(h);
-        }
-        j.lat_maps = h->lat_maps.as<unsigned char>();
-        j.lat_levels = h->lat_levels;
-    }
+    M2LJob j = m2l_tensor_job(h, L);
+    const int PP = h->p * h->p, nc = h->ncells, c0 = h->lvl_start[2];
     int *misc = reinterpret_cast<int *>(h->m2l_misc.as<unsigned>() + 24 * (FMM_MAXLEVEL + 1));
     int *err = misc + 4, *queue = misc + 6;
     FMM_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), s));
-    launch_tc_p(h->p, h->ntiles_max, j, nullptr, 1, queue, err, s);
+    if (nc <= c0) return;
+    FMM_CUDA_TRY(cudaMemsetAsync(h->m2l_ws.p, 0, sizeof(unsigned) * (size_t)j.ws_words, s));
+    M2LLevels lv;
+    int most = 0;
+    for (int l = 0; l <= FMM_MAXLEVEL + 1; l++) {
+        lv.start[l] = l < (int)h->lvl_start.size() ? h->lvl_start[(size_t)l] : nc;
+        if (l) most = std::max(most, lv.start[l] - lv.start[l - 1]);
+    }
+    // a block walks 64 cells or more; 4 blocks per SM at most
+    const unsigned gx = (unsigned)std::min((most + 63) / 64, 4 * h->nsm);
+    m2l_lmax_k<<<dim3(gx, (unsigned)h->depth - 1), 256, 0, s>>>(M, PP, lv, h->m2l_ws.as<unsigned>());
+    count_launch(h);
+    M2LLattice lat;
+    lat.levels = h->lat_levels;
+    for (int l = 0; l <= FMM_MAXLEVEL; l++) lat.off[l] = h->lat_off[l];
+#define FMM_TC_CALL(NPV)                                                                                           \
+    m2l_split_k<NPV><<<nblk((int64_t)(nc - c0) * (NPV / 8), 256), 256, 0, s>>>(                                     \
+        M, PP, h->c_xyz.as<int4>(), c0, nc, h->m2l_ws.as<unsigned>(), lat, h->msplit.as<unsigned char>(),           \
+        h->mlat.as<unsigned char>())
+    FMM_TC_SWITCH(tc_np(h->p), FMM_TC_CALL)
+#undef FMM_TC_CALL
+    count_launch(h);
+    if (h->lat_levels) {
+        j.lat_maps = h->lat_maps.as<unsigned char>();
+        j.lat_levels = h->lat_levels;
+    }
+    launch_tc_p(h->p, h->ntiles_max * j.nsplit, j, nullptr, 1, queue, err, s);
     count_launch(h);
     check_launch("m2l tensor");
 }

@@ -1025,6 +1025,8 @@ __global__ void batch_zero_k(int PP, const BatchSys *__restrict__ sys)
         S.cnt_up[threadIdx.x] = 0u;
         S.cnt_dn[threadIdx.x] = threadIdx.x == 0 ? 1u : 0u;
     }
+    if (blockIdx.x == 1)
+        for (int i = threadIdx.x; i < S.ws_words; i += blockDim.x) S.m2l_ws[i] = 0u;
 }
 
 void batch_zero(int p, const BatchSys *sys, int nsys, cudaStream_t s)

@@ -1,6 +1,6 @@
 // Inline-PTX wrappers for the Blackwell (sm_100 family) asynchronous
 // machinery the tensor-core kernels use: mbarriers, cp.async and bulk copies,
-// tcgen05 MMA issue, commit, tensor-memory loads and stores, TF32 rounding.
+// tcgen05 MMA issue, commit, tensor-memory loads.
 // Every wait here is bounded and reports a timeout to its caller.
 #pragma once
 
@@ -41,30 +41,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity)
         if (ok) return true;
     }
     return false;
-}
-
-// bounded wait for two (barrier, parity) pairs at once (bit k of `mask`
-// selects pair k); their tests overlap instead of running back to back, and a
-// waiting thread may be suspended instead of spinning on the issue slots
-__device__ __forceinline__ bool mbar_wait2(uint32_t mask, uint64_t *b0, uint32_t p0, uint64_t *b1, uint32_t p1)
-{
-    const uint32_t a0 = smem_u32(b0), a1 = smem_u32(b1);
-    for (int it = 0; it < (1 << 20) && mask; it++) {
-        uint32_t ok0 = 1, ok1 = 1;
-        if (mask & 1u)
-            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                         : "=r"(ok0)
-                         : "r"(a0), "r"(p0)
-                         : "memory");
-        if (mask & 2u)
-            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                         : "=r"(ok1)
-                         : "r"(a1), "r"(p1)
-                         : "memory");
-        if (ok0) mask &= ~1u;
-        if (ok1) mask &= ~2u;
-    }
-    return mask == 0;
 }
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32_t src_bytes)
@@ -132,28 +108,21 @@ __device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t a, uint64_t b, 
         : "memory");
 }
 
-// the same with A in tensor memory (atmem: lane 0 and the first of its K columns)
-__device__ __forceinline__ void mma_tf32_ta(uint32_t tmem, uint32_t atmem, uint64_t b, uint32_t idesc, uint32_t acc)
+// instruction descriptor: D f32, A and B f16, both K-major, M x N
+__host__ __device__ constexpr uint32_t idesc_f16(int M, int N)
+{
+    return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// one k-step (16 halves) of A and B in shared memory
+__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc)
 {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem),
-        "r"(atmem), "l"(b), "r"(idesc), "r"(acc)
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc)
         : "memory");
 }
-
-// 16 consecutive TMEM columns of this warp's 32 lanes (one row per thread)
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float *v)
-{
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(taddr),
-        "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
-        "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])),
-        "r"(__float_as_uint(v[8])), "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])), "r"(__float_as_uint(v[11])),
-        "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])), "r"(__float_as_uint(v[15]))
-        : "memory");
-}
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ void mma_commit(uint64_t *bar)
 {
@@ -185,13 +154,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float *v)
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 8; i++) v[i] = __uint_as_float(r[i]);
-}
-
-__device__ __forceinline__ float tf32_rn(float a)
-{
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(a));
-    return __uint_as_float(r);
 }
 
 __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float b)

@@ -1473,9 +1473,20 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
         const int tile = m2l_tile_size(h);
         const int c0 = depth >= 2 ? h->lvl_start[2] : ncells;
         const int nt = ncells - c0;
-        h->ntiles_max = nt / tile + 8 * (FMM_MAXLEVEL + 1) + 1;
+        const int pool_max = h->m2l_pool >= 0 ? h->m2l_pool : 4 * tile;
+        // pooled levels: one run of tiles; complete levels: equal octant
+        // groups; others: up to one partial tile per octant more
+        int pooled = 0;
+        h->ntiles_max = 0;
+        for (int l = 2; l <= depth; l++) {
+            const int cells = h->lvl_start[(size_t)l + 1] - h->lvl_start[(size_t)l];
+            if (cells <= pool_max) pooled += cells;
+            else if (l <= 10 && cells == (1 << (3 * l))) h->ntiles_max += 8 * ((cells / 8 + tile - 1) / tile);
+            else h->ntiles_max += cells / tile + 8;
+        }
+        h->ntiles_max += (pooled + tile - 1) / tile;
         h->m2l_tgt.ensure(sizeof(int) * (size_t)std::max(nt, 1));
-        h->m2l_tiles.ensure(sizeof(M2LTile) * (size_t)h->ntiles_max);
+        h->m2l_tiles.ensure(sizeof(M2LTile) * (size_t)std::max(h->ntiles_max, 1));
         h->m2l_misc.ensure(sizeof(unsigned) * 3 * 8 * (FMM_MAXLEVEL + 1) + 64);
         unsigned *grp = h->m2l_misc.as<unsigned>();
         unsigned *goff = grp + 8 * (FMM_MAXLEVEL + 1);
@@ -1486,7 +1497,6 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
             oct_count_k<<<nblocks(nt, TB), TB, 0, s>>>(c0, ncells, h->c_level.as<int>(), h->c_anchor.as<uint64_t>(), grp);
             count_launch(h);
         }
-        const int pool_max = h->m2l_pool >= 0 ? h->m2l_pool : 4 * tile;
         tiles_k<<<1, 1, 0, s>>>(depth, tile, pool_max, grp, goff, h->m2l_tiles.as<M2LTile>(), ntiles);
         count_launch(h);
         if (nt > 0) {
@@ -1496,6 +1506,7 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
         }
         check_launch("m2l tiles");
         lattice_prepare(h, s);
+        m2l_plan(h);
     }
 }
 
