@@ -24,29 +24,36 @@
 //   - a level's rows are multiplied by 2^e so that the largest coefficient of
 //     the level lies in [2^14, 2^15) (e from a maximum taken each evaluation).
 // FP16's subnormals end 2^-39 below that maximum, 15 bits below the rounding
-// of the FP32 sums. Every GV vectors the accumulator is drained into
-// per-thread FP32 (hi, lo) TwoSum registers; two TMEM buffers alternate so
-// the drain overlaps the next MMAs.
+// of the FP32 sums. Every GV vectors an accumulator is drained into
+// per-thread FP32 (hi, lo) TwoSum registers.
 //
-// Per CTA (320 threads: two groups of 4 worker warps, an MMA warp and a
-// producer warp) a ring of NS stages, one unit (vector v, k-block of 64
+// Per CTA (two groups of 4 worker warps, NM MMA warps and NM producer warps) a
+// ring of NS stages, one unit (vector v, k-block of 64
 // coefficients) each: 128 rows of A_hi and A_lo and the operator block
 // [T_hi ; T_lo], all 128B-swizzled in shared memory, where the MMAs read both
 // operands.
-//   - the producer brings the operator block with one bulk copy and, on
-//     complete levels (lattice tiles), A_hi and A_lo with one TMA tile load
-//     each; the workers then only drain.
+//   - a producer brings the unit's operator block with one bulk copy and, on
+//     complete levels (lattice tiles), A_hi and A_lo with one TMA tile load each;
+//     the workers then only drain.
 //   - on other levels the worker group u % 2 gathers the unit's rows with
 //     cp.async straight into the stage (sources found by lattice lookups
 //     fetched ahead into a ring; zero fill where a cell is absent). The
 //     copies' completion arrives on the stage's mbarrier; the MMA thread
 //     orders them before its asynchronous reads with a proxy fence.
-//   - the MMA warp issues the tcgen05.mma of a unit and commits it to the
-//     stage's "empty" barrier.
+//   - an MMA warp issues the tcgen05.mma of a vector's units into its
+//     accumulators and commits each unit to its stage's "empty" barrier. With
+//     one warp and NP <= 64 the tensor pipe idles while that warp waits for the
+//     next stage and commits (about 750 of 1,260 cycles per vector at p = 8):
+//     there two MMA warps and two producers take every other vector each, in
+//     stages of their own parity.
 // The rows are split into FP16 once per evaluation (m2l_split_k) and not once
 // per vector, so nothing but copies and MMAs is left per vector.
-// Bound: the copies into shared memory (48 KB per vector and tile at p = 8,
-// MEASURED_BOUND).
+// Bound (N = 1e7, p = 8, 7.1 ms; 19.8 with TF32 pairs split per vector in
+// worker warps, 12.2 with one MMA warp): the copies, 48 KB per vector and tile
+// from L2 at 69 bytes per clock and SM; without the MMAs the launch takes 6.75
+// ms.
+// p = 9 .. 11 (60 KB stages, three of them, one MMA warp): the waits and
+// commits between the units, 3.0 ms at N = 1e6, p = 10 (6.6 with TF32).
 //
 // A tree with few tiles (5 at N = 16,384) would leave most SMs idle: the
 // vectors of every tile are then cut into nsplit ranges, one CTA each
@@ -85,15 +92,16 @@ __device__ int g_no_cell = -1;
 // of 64 coefficients, each 128 bytes of hi and 128 bytes of lo; with NP <= 32
 // both halves fit one 128-byte row (PACK: hi in the first 64 bytes, lo in the
 // last), and so do T_hi and T_lo.
-// Tensor memory: two accumulator buffers of 2 NP columns (main | correction).
+// Tensor memory: two accumulator buffers of 2 NP columns (main | correction)
+// for each of the NM MMA warps. Warp m takes the vectors w = NM i + m, GV of
+// them to an accumulator: group (i + OFF m) / GV, so that the drains of two
+// warps alternate.
 // Thread (r, g) drains output columns [g HN, (g + 1) HN) of row r.
 template <int NP>
 struct TcCfg {
     static constexpr int M = 128;                  // target rows per tile
     static constexpr int NW = 8;                   // worker warps
     static constexpr int NG = 2;                   // worker groups
-    static constexpr int MMA_WARP = NW, P_WARP = NW + 1;
-    static constexpr int NT = NW * 32 + 64;        // threads (workers, MMA warp, producer warp)
     static constexpr bool PACK = NP <= 32;
     static constexpr int KB = (NP + 63) / 64;      // k-blocks per vector
     static constexpr int ROWB = PACK ? 128 : 256;  // bytes of a row's k-block (hi and lo)
@@ -105,16 +113,26 @@ struct TcCfg {
     static constexpr int RING = NG * RINGU * M * 4;
     static constexpr int BAR = 768;                // mbarriers (first 512 bytes), then the CTA's job
     static constexpr int NS_FIT = (226 * 1024 - RING - BAR - 1024) / STAGE;
-    static constexpr int NS = NS_FIT > 6 ? 6 : NS_FIT;
+    // MMA warps (and producers). Two only where a vector is one unit and the
+    // stages number an even count: unit u, stage u % NS, then always meets the
+    // same warps, and no wait on a stage's barrier can be two phases ahead
+    // (which its parity would not tell from a completed one).
+    static constexpr int NM = KB == 1 ? 2 : 1;
+    static constexpr int MMA_WARP = NW, P_WARP = NW + NM;
+    static constexpr int NT = 32 * (NW + 2 * NM);  // threads
+    static constexpr int NS = NS_FIT > 6 ? 6 : NM == 2 ? NS_FIT & ~1 : NS_FIT;
     static constexpr int SMEM = NS * STAGE + RING + BAR + 1024;
     static constexpr int TCOLS = 512;
+    static constexpr int AC = 2;                   // accumulator buffers per MMA warp
     static constexpr int GV = 8;                   // vectors per accumulator drain
+    static constexpr int OFF = GV / 2;
     static constexpr int HN = NP / 2;              // output coefficients per thread
-    // vectors into group gg + 1 at which a gathering worker drains group gg:
-    // its units have then been consumed (the ring is NS units deep)
-    static constexpr int DRAIN_AT = (NS + KB - 1) / KB;
-    static_assert(NP % 16 == 0 && STAGE % 1024 == 0 && NS >= 3 && DRAIN_AT < GV && 4 * NP <= TCOLS &&
-                      SMEM <= 227 * 1024 && 2 * QU >= NS,
+    // a gathering worker drains a group once it has to wait for a vector more
+    // than LATE past the group's last one: the group is then finished or about
+    // to be, and the next group of the same buffer has not begun
+    static constexpr int LATE = (NS + KB - 1) / KB;
+    static_assert(NP % 16 == 0 && STAGE % 1024 == 0 && NS >= 3 && 2 * NM * AC * NP <= TCOLS && SMEM <= 227 * 1024 &&
+                      LATE < GV && 2 * QU >= NS && (NM == 1 || (KB == 1 && NS % 2 == 0)),
                   "stage budget");
 };
 
@@ -221,7 +239,7 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     // CTA b computes item b of the single job `one`, read from the parameter
     // space, which measured faster for one system than the persistent loop.
     using C = TcCfg<NP>;
-    constexpr int NS = C::NS, QU = C::QU, RINGU = C::RINGU, KB = C::KB;
+    constexpr int NS = C::NS, NM = C::NM, QU = C::QU, RINGU = C::RINGU, KB = C::KB;
     constexpr bool PACK = C::PACK;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -230,15 +248,15 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     uint64_t *full = bar;                     // NS: bytes of the producer's copies
     uint64_t *gfull = full + NS;              // NS: cp.async arrivals of a group's 128 threads (gathered tiles)
     uint64_t *empty = gfull + NS;             // NS: MMA commits
-    uint64_t *acc_full = empty + NS;          // 2: MMA commits at the end of a group of vectors
-    uint64_t *acc_empty = acc_full + 2;       // 2: one arrival per worker warp after a drain
-    uint64_t *fin = acc_empty + 2;            // 1
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(fin + 1);
+    uint64_t *acc_full = empty + NS;          // 2 AC: MMA commits at the end of a group of vectors
+    uint64_t *acc_empty = acc_full + 2 * C::AC;  // 2 AC: one arrival per worker warp after a drain
+    uint64_t *fin = acc_empty + 2 * C::AC;    // 2: last commit of each MMA warp
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(fin + 2);
     int *abort_flag = reinterpret_cast<int *>(tmem_slot + 1);
     int *s_item = abort_flag + 1;                 // this CTA's current item (-1: none left)
     int *s_last = s_item + 1;                     // this CTA finished its tile last
     M2LJob *s_job = reinterpret_cast<M2LJob *>(reinterpret_cast<unsigned char *>(bar) + 512);  // its job
-    static_assert(sizeof(uint64_t) * (3 * NS + 5) + 16 <= 512 && 512 + sizeof(M2LJob) <= C::BAR, "barrier area");
+    static_assert(sizeof(uint64_t) * (3 * NS + 4 * C::AC + 2) + 16 <= 512 && 512 + sizeof(M2LJob) <= C::BAR, "barrier area");
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (!PERSIST && (int)blockIdx.x >= *one.ntiles * one.nsplit) return;
@@ -275,11 +293,12 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
             mbar_init(&gfull[s], 128);
             mbar_init(&empty[s], 1);
         }
-        for (int b = 0; b < 2; b++) {
+        for (int b = 0; b < 2 * C::AC; b++) {
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], C::NW);
         }
-        mbar_init(fin, 1);
+        mbar_init(&fin[0], 1);
+        mbar_init(&fin[1], 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -298,7 +317,6 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     const int w0 = (int)((long long)nvt * split / nsplit), w1 = (int)((long long)nvt * (split + 1) / nsplit);
     const int e0 = J.st_off[td.octant] + w0, nv = w1 - w0;
     const int nunits = nv * KB;
-    const int ngroups = (nv + C::GV - 1) / C::GV;
     // Lattice tile (a complete level with a lattice copy of M~): the tile is
     // an 8 x 4 x 4 block of its octant's sub-lattice with rows in x, y, z
     // order, and for every vector the sources form the same block shifted, in
@@ -307,81 +325,94 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     // (persistent launches serve the batch engine, which gathers everywhere)
     const bool lat = !PERSIST && J.lat_maps != nullptr && td.octant < 8 && ((J.lat_levels >> l) & 1u);
 
-    if (warp == C::MMA_WARP) {
-        // ------------------------------------------------------------ MMA warp
-        // one iteration per unit; the whole warp runs the loop, lane 0 issues
-        const uint32_t id_full = idesc_f16(128, 2 * NP), id_half = idesc_f16(128, NP);
-        for (int u = 0; u < nunits; u++) {
-            const int s = u % NS, vi = u / KB, kb = u % KB, g = vi / C::GV, b = g & 1;
-            const uint32_t ph = (uint32_t)((u / NS) & 1);
-            bool ok = mbar_wait(&full[s], ph);
-            if (!lat) ok = ok && mbar_wait(&gfull[s], ph);
-            if (ok && kb == 0 && vi % C::GV == 0 && g >= 2) ok = mbar_wait(&acc_empty[b], (uint32_t)(((g - 2) >> 1) & 1));
-            ok = __all_sync(0xffffffffu, ok) && !*(volatile int *)abort_flag;
-            if (!ok) {
-                if (lane == 0) atomicExch(abort_flag, 1);
-                break;
-            }
-            if (!lat) fence_proxy_async();  // the gathered rows (generic proxy) before the MMA's reads
-            tc_fence_after();
-            if (lane == 0) {
+    if (warp >= C::MMA_WARP && warp < C::P_WARP) {
+        // ----------------------------------------------------------- MMA warps
+        // (the waits and commits, a few hundred cycles per unit, of one warp
+        // overlap the other's MMAs). The whole warp runs the loop and one
+        // elected lane issues: the branch on elect.sync lets the compiler keep
+        // the descriptors in uniform registers (7.25 against 7.75 ms at
+        // N = 1e7, p = 8, with one lane running the loop).
+        const int m = warp - C::MMA_WARP;
+        {
+            const uint32_t id_full = idesc_f16(128, 2 * NP), id_half = idesc_f16(128, NP);
+            const uint64_t a0 = sdesc(smem_u32(base));
+            constexpr uint64_t LO = PACK ? 64 / 16 : 16384 / 16, B0 = C::A_BYTES / 16;  // descriptor units of 16 bytes
+            bool ok = true;
+            for (int w = m, i = 0; ok && w < nv; w += NM, i++) {
+                const int gi = i + C::OFF * m, g = gi / C::GV, b = m * C::AC + g % C::AC;
+                const bool start = gi % C::GV == 0 || i == 0;
+                if (start && g >= C::AC) ok = mbar_wait_or(&acc_empty[b], (uint32_t)((g / C::AC - 1) & 1), abort_flag);
                 const uint32_t dmain = tmem + (uint32_t)(b * 2 * NP), dcorr = dmain + NP;
-                const uint32_t first = (vi % C::GV == 0 && kb == 0) ? 0u : 1u;
-                const uint32_t ahi = smem_u32(base + s * C::STAGE), alo = ahi + (PACK ? 64u : 16384u);
-                const uint32_t bb = ahi + C::A_BYTES;
-                // k-steps of 16 coefficients holding any of the p^2 real ones
-                constexpr int KS = PACK ? NP / 16 : 4;
-                const int ks = min(KS, (PP - kb * 64 + 15) >> 4);
 #pragma unroll
-                for (int k = 0; k < KS; k++) {
-                    if (k >= ks) break;
-                    const uint32_t acc = k == 0 ? first : 1u;
-                    // A_hi [T_hi ; T_lo] -> main | correction, then A_lo T_hi -> correction
-                    if (PACK) {
-                        mma_f16(dmain, sdesc(ahi + 32 * k), sdesc(bb + 32 * k), id_half, acc);
-                        mma_f16(dcorr, sdesc(ahi + 32 * k), sdesc(bb + 64 + 32 * k), id_half, acc);
-                    } else {
-                        mma_f16(dmain, sdesc(ahi + 32 * k), sdesc(bb + 32 * k), id_full, acc);
+                for (int kb = 0; kb < KB; kb++) {
+                    const int u = w * KB + kb, s = u % NS;
+                    const uint32_t ph = (uint32_t)((u / NS) & 1);
+                    ok = ok && mbar_wait_or(&full[s], ph, abort_flag);
+                    if (!lat) {
+                        ok = ok && mbar_wait_or(&gfull[s], ph, abort_flag);
+                        fence_proxy_async();  // the gathered rows (generic proxy) before the MMA's reads
                     }
-                    mma_f16(dcorr, sdesc(alo + 32 * k), sdesc(bb + 32 * k), id_half, 1u);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        const uint64_t ad = a0 + (uint64_t)((uint32_t)s * (C::STAGE / 16)), bd = ad + B0;
+                        const uint32_t first = (start && kb == 0) ? 0u : 1u;
+                        // k-steps of 16 coefficients holding any of the p^2 real ones
+                        constexpr int KS = PACK ? NP / 16 : 4;
+                        const int ks = min(KS, (PP - kb * 64 + 15) >> 4);
+#pragma unroll
+                        for (int k = 0; k < KS; k++) {
+                            if (k >= ks) break;
+                            const uint32_t acc = k == 0 ? first : 1u;
+                            // A_hi [T_hi ; T_lo] -> main | correction, then A_lo T_hi -> correction
+                            if (PACK) {
+                                mma_f16(dmain, ad + 2 * k, bd + 2 * k, id_half, acc);
+                                mma_f16(dcorr, ad + 2 * k, bd + LO + 2 * k, id_half, acc);
+                            } else {
+                                mma_f16(dmain, ad + 2 * k, bd + 2 * k, id_full, acc);
+                            }
+                            mma_f16(dcorr, ad + LO + 2 * k, bd + 2 * k, id_half, 1u);
+                        }
+                        mma_commit(&empty[s]);
+                    }
+                    __syncwarp();
                 }
-                mma_commit(&empty[s]);
-                if (kb == KB - 1 && ((vi % C::GV == C::GV - 1) || vi == nv - 1)) mma_commit(&acc_full[b]);
+                if (ok && (gi % C::GV == C::GV - 1 || w + NM >= nv) && elect_one()) mma_commit(&acc_full[b]);
+                __syncwarp();
             }
-            __syncwarp();
-        }
-        if (lane == 0) {
+            if (!ok) atomicExch(abort_flag, 1);
             // every commit has arrived before the shared memory goes away
-            mma_commit(fin);
-            mbar_wait(fin, 0);
+            if (elect_one()) mma_commit(&fin[m]);
+            mbar_wait(&fin[m], 0);
         }
         __syncwarp();
-    } else if (warp == C::P_WARP) {
-        // ------------------------------------------------------- producer warp
-        if (lane == 0 && nunits > 0) {
+    } else if (warp >= C::P_WARP) {
+        // ------------------------------------------------------ producer warps
+        const int pw = warp - C::P_WARP;
+        if (lane == 0 && nunits > pw) {
             int ox = 0, oy = 0, oz = 0;  // tile origin in halved coordinates
             const int obx = td.octant & 1, oby = (td.octant >> 1) & 1, obz = (td.octant >> 2) & 1;
-            const void *lmap = nullptr;
+            const unsigned char *lmap = nullptr;
             if (lat) {
                 const int4 a = J.xyz[J.tgt[td.start]];
                 const int sh = FMM_MAXLEVEL - l + 1;
                 ox = a.x >> sh;
                 oy = a.y >> sh;
                 oz = a.z >> sh;
-                lmap = (const void *)(J.lat_maps + 128 * l);
+                lmap = J.lat_maps + 128 * l;
             }
             const unsigned char *ttab = J.ttab;
-            int issued = 0;
-            int4 vn = st[e0];
-            for (int u = 0; u < nunits; u++) {
-                const int s = u % NS, kb = u % KB, w = u / KB;
-                if (*(volatile int *)abort_flag) break;
-                if (u >= NS && !mbar_wait(&empty[s], (uint32_t)((u / NS - 1) & 1))) {
+            int issued = pw;  // first unit of this producer not issued
+            int4 vn = st[e0 + pw / KB];
+            for (int u = pw; u < nunits; u += NM) {
+                const int s = u % NS, kb = u % KB;
+                const int4 v = vn;
+                if (u + NM < nunits) vn = st[e0 + (u + NM) / KB];
+                if (u >= NS && !mbar_wait_or(&empty[s], (uint32_t)((u / NS - 1) & 1), abort_flag)) {
                     atomicExch(abort_flag, 1);
                     break;
                 }
-                const int4 v = vn;
-                if (kb == KB - 1 && w + 1 < nv) vn = st[e0 + w + 1];
                 const uint32_t sa = smem_u32(base + s * C::STAGE);
                 mbar_arrive_tx(&full[s], C::B_BYTES + (lat ? C::A_BYTES : 0));
                 if (lat) {
@@ -394,13 +425,15 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
                     if (!PACK) tma_load_5d(sa + 16384, lmap, kb * (C::ROWB / 2) + 64, x, y, z, ps, &full[s]);
                 }
                 bulk_g2s(sa + C::A_BYTES, ttab + ((size_t)(v.w & 0xffff) * KB + kb) * C::B_BYTES, C::B_BYTES, &full[s]);
-                issued = u + 1;
+                issued = u + NM;
             }
             // copies still in flight when the pipeline stopped early land
             // before the shared memory goes away (bounded waits)
             if (*(volatile int *)abort_flag)
-                for (int u = max(0, issued - NS); u < issued; u++) mbar_wait(&full[u % NS], (uint32_t)((u / NS) & 1));
+                for (int u = pw; u < issued; u += NM)
+                    if (u + NS >= issued) mbar_wait(&full[u % NS], (uint32_t)((u / NS) & 1));
         }
+        __syncwarp();
     } else {
         // ---------------------------------------------------------- worker warps
         constexpr int HN = C::HN;
@@ -423,29 +456,37 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
             ro = (px & 1) | ((py & 1) << 1) | ((pz & 1) << 2);
         }
 
-        auto drain = [&](int gg) {
-            const int b = gg & 1;
+        // Groups are drained in the order of their last vectors: (warp 1, 0),
+        // (0, 0), (1, 1), (0, 1), ...; a group past its warp's last is skipped.
+        const int nd = NM * ((nv + NM * C::GV - 1) / (NM * C::GV) + 1);  // bound of the sequence
+        auto warp_of = [&](int d) { return NM - 1 - d % NM; };
+        auto last_vector = [&](int d) { return NM * ((d / NM + 1) * C::GV - C::OFF * warp_of(d) - 1) + warp_of(d); };
+        auto drain = [&](int d) {
+            const int m = warp_of(d), gg = d / NM, b = m * C::AC + gg % C::AC;
+            const int nm = (nv - m + NM - 1) / NM;  // vectors of warp m
+            if (nm <= 0 || gg >= (nm + C::OFF * m + C::GV - 1) / C::GV) return;
             __syncwarp();
-            const bool ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (uint32_t)((gg >> 1) & 1)));
+            const bool ok = __all_sync(0xffffffffu, mbar_wait_or(&acc_full[b], (uint32_t)((gg / C::AC) & 1), abort_flag));
             if (!ok) {
                 atomicExch(abort_flag, 1);
                 return;
             }
             tc_fence_after();
             const uint32_t taddr = tmem + tlane + (uint32_t)(b * 2 * NP + g * HN);
-            float mv[16], cv[16];
+            // columns per read: 8 where the sums alone take most registers
+            constexpr int CH = HN % 16 == 0 && HN <= 32 ? 16 : 8;
+            float mv[CH], cv[CH];
 #pragma unroll
-            for (int k0 = 0; k0 < HN; k0 += 16) {
-                if (k0 + 16 <= HN) {
+            for (int k0 = 0; k0 < HN; k0 += CH) {
+                if constexpr (CH == 16) {
                     tmem_ld16(taddr + k0, mv);
                     tmem_ld16(taddr + NP + k0, cv);
-                } else {  // 8 remaining columns
+                } else {
                     tmem_ld8(taddr + k0, mv);
                     tmem_ld8(taddr + NP + k0, cv);
                 }
 #pragma unroll
-                for (int k = 0; k < 16; k++)
-                    if (k0 + k < HN) two_sum_acc(acc_hi[k0 + k], acc_lo[k0 + k], mv[k] + cv[k]);
+                for (int k = 0; k < CH; k++) two_sum_acc(acc_hi[k0 + k], acc_lo[k0 + k], mv[k] + cv[k]);
             }
             tc_fence_before();
             __syncwarp();
@@ -501,8 +542,13 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
             cp_async_wait_all();
             for (int j = 0; j < nown; j++) {
                 if (*(volatile int *)abort_flag) break;
-                const int u = 2 * j + g, s = u % NS, kb = u % KB, vi = u / KB;
-                const bool ok = u < NS || mbar_wait(&empty[s], (uint32_t)((u / NS - 1) & 1));
+                const int u = 2 * j + g, s = u % NS, kb = u % KB;
+                // the groups before the vector this unit's stage waits for
+                while (u >= NS && last_vector(drained) + C::LATE < (u - NS) / KB && !*(volatile int *)abort_flag) {
+                    drain(drained);
+                    drained++;
+                }
+                const bool ok = u < NS || mbar_wait_or(&empty[s], (uint32_t)((u / NS - 1) & 1), abort_flag);
                 if (!__all_sync(0xffffffffu, ok)) {
                     atomicExch(abort_flag, 1);
                     break;
@@ -530,16 +576,11 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
                 fetch(j + QU);
                 cp_async_arrive_noinc(&gfull[s]);
                 cp_async_commit();
-                // drain group gg once group gg + 1 is well under way
-                if (vi >= C::DRAIN_AT && (vi - C::DRAIN_AT) / C::GV > drained) {
-                    drain(drained);
-                    drained++;
-                }
             }
             cp_async_wait_all();
             __syncwarp();
         }
-        while (drained < ngroups && !*(volatile int *)abort_flag) {
+        while (drained < nd && !*(volatile int *)abort_flag) {
             drain(drained);
             drained++;
         }
@@ -547,8 +588,18 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
         // failed, or the last drain saw the last MMA and nothing is waiting
         named_barrier_sync(1, C::NW * 32);
         if (!*(volatile int *)abort_flag) {
-            bool write = true;
-            if (nsplit > 1) {
+            const int e = cell >= 0 ? m2l_exponent(J.lmax[rl]) : 0;
+            float *Lc = J.L + (size_t)(cell >= 0 ? cell : 0) * PP;
+            // back from the operands' powers of two
+            auto put = [&](int k, float x) {
+                const int t = J.rowexp[k] - e;
+                if (cell >= 0) Lc[k] += (x * m2l_pow2(t >> 1)) * m2l_pow2(t - (t >> 1));
+            };
+            if (nsplit == 1) {
+#pragma unroll
+                for (int k = 0; k < HN; k++)
+                    if (g * HN + k < PP) put(g * HN + k, acc_hi[k] + acc_lo[k]);
+            } else {
                 // the range's sums, [item][coefficient][row]; the tile's last
                 // range to finish adds them all in order
                 const size_t rng = (size_t)PP * C::M;
@@ -565,34 +616,30 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
                     __threadfence();
                 }
                 named_barrier_sync(1, C::NW * 32);
-                write = *(volatile int *)s_last != 0;
-                if (write) {
-                    pt = J.part + (size_t)tile * nsplit * rng + row;
+                if (*(volatile int *)s_last) {
+                    constexpr int CH = HN % 16 == 0 && HN <= 32 ? 16 : 8;  // coefficients in flight per range
+                    const float2 *p0 = J.part + (size_t)tile * nsplit * rng + row;
+                    for (int k0 = g * HN; k0 < (g + 1) * HN && k0 < PP; k0 += CH) {
+                        float hi[CH], lo[CH];
 #pragma unroll
-                    for (int k = 0; k < HN; k++) acc_hi[k] = acc_lo[k] = 0.f;
-                    for (int r = 0; r < nsplit; r++, pt += rng) {
-                        float2 v[HN];
+                        for (int k = 0; k < CH; k++) hi[k] = lo[k] = 0.f;
+#pragma unroll 2
+                        for (int r = 0; r < nsplit; r++) {
+                            float2 v[CH];
 #pragma unroll
-                        for (int k = 0; k < HN; k++)
-                            v[k] = g * HN + k < PP ? __ldcg(&pt[(size_t)(g * HN + k) * C::M]) : make_float2(0.f, 0.f);
+                            for (int k = 0; k < CH; k++)
+                                v[k] = k0 + k < PP ? __ldcg(&p0[(size_t)r * rng + (size_t)(k0 + k) * C::M]) : make_float2(0.f, 0.f);
 #pragma unroll
-                        for (int k = 0; k < HN; k++) {
-                            two_sum_acc(acc_hi[k], acc_lo[k], v[k].x);
-                            acc_lo[k] += v[k].y;
+                            for (int k = 0; k < CH; k++) {
+                                two_sum_acc(hi[k], lo[k], v[k].x);
+                                lo[k] += v[k].y;
+                            }
                         }
+#pragma unroll
+                        for (int k = 0; k < CH; k++)
+                            if (k0 + k < PP) put(k0 + k, hi[k] + lo[k]);
                     }
                 }
-            }
-            if (write && cell >= 0) {
-                // back from the operands' powers of two
-                const int e = m2l_exponent(J.lmax[rl]);
-                float *Lc = J.L + (size_t)cell * PP + g * HN;
-#pragma unroll
-                for (int k = 0; k < HN; k++)
-                    if (g * HN + k < PP) {
-                        const int t = J.rowexp[g * HN + k] - e;
-                        Lc[k] += ((acc_hi[k] + acc_lo[k]) * m2l_pow2(t >> 1)) * m2l_pow2(t - (t >> 1));
-                    }
             }
         }
     }
@@ -975,8 +1022,8 @@ void lattice_prepare(fmm_ctx *h, cudaStream_t s)
         const cuuint64_t dims[5] = {row / 2, H, H, H, 8};
         const cuuint64_t strides[4] = {row, row * H, row * H * H, row * H * H * H};
         const cuuint32_t box[5] = {64, 8, 4, 4, 1}, estride[5] = {1, 1, 1, 1, 1};
-        const CUresult r = enc(&mp[l], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5, h->mlat.as<unsigned char>() + row * h->lat_off[l], dims,
-                               strides, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+        const CUresult r = enc(&mp[l], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 5, h->mlat.as<unsigned char>() + row * h->lat_off[l],
+                               dims, strides, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) throw Error{FMM_ECUDA, "tensor-core M2L: encoding a lattice tensor map failed"};
     }

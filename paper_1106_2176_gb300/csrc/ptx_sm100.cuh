@@ -10,6 +10,14 @@ namespace fmm {
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// true in one lane of the (converged) warp, the same lane every time
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void mbar_init(uint64_t *b, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count));
@@ -39,6 +47,24 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity)
             : "r"(a), "r"(parity)
             : "memory");
         if (ok) return true;
+    }
+    return false;
+}
+
+// the same, giving up as well once *abort is set (looked at only while the
+// phase is not complete, so a wait that finds it complete reads nothing else)
+__device__ __forceinline__ bool mbar_wait_or(uint64_t *b, uint32_t parity, const int *abort)
+{
+    const uint32_t a = smem_u32(b);
+    for (int it = 0; it < (1 << 20); it++) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(a), "r"(parity)
+            : "memory");
+        if (ok) return true;
+        if (*(volatile const int *)abort) return false;
     }
     return false;
 }
