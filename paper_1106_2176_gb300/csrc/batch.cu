@@ -136,7 +136,7 @@ int fmm_batch_create(const fmm_handle *handles, int nsys, void *const *phi, void
             S.flag = h->pr_flag.as<unsigned>();
             S.p2p_ptr = h->p2p_ptr.as<int>();
             S.nrun = h->p2p_nrun.as<int>();
-            S.runs_pr = h->p2p_runs_pr.as<int2>();
+            S.runs_pr = h->p2p_runs.as<int2>();
             S.phi = static_cast<float *>(phi[i]);
             S.grad = static_cast<float *>(grad[i]);
             S.cnt_up = b->cnt.as<unsigned>() + (size_t)i * 2 * (FMM_MAXLEVEL + 1);

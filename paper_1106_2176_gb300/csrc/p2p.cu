@@ -709,21 +709,6 @@ __global__ void pr_fill_k(int64_t n, const float4 *__restrict__ xs, const unsign
     }
 }
 
-// runs of particles [b, e) (whole leaves) -> runs of records
-// [(b + pad[b]) / 2, (e + pad[e - 1] + flag[e - 1]) / 2)
-__global__ void pr_runs_k(int nleaves, const int *__restrict__ leaves, const int *__restrict__ ptr,
-                          const int *__restrict__ nrun, const int2 *__restrict__ runs, const unsigned *__restrict__ pad,
-                          const unsigned *__restrict__ flag, int2 *__restrict__ runs_pr)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nleaves) return;
-    const int A = leaves[i];
-    for (int k = ptr[A]; k < ptr[A] + nrun[A]; k++) {
-        const int2 r = runs[k];
-        runs_pr[k] = make_int2((int)((r.x + pad[r.x]) >> 1), (int)((r.y + pad[r.y - 1] + flag[r.y - 1]) >> 1));
-    }
-}
-
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *b, uint32_t tx)
 {
     asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(tx) : "memory");
@@ -1087,16 +1072,11 @@ void p2p_prepare(fmm_ctx *h, cudaStream_t s)
     h->pr_pad.ensure(sizeof(unsigned) * (size_t)n);
     // at most one padding record half per leaf
     h->pr_pairs.ensure(sizeof(float) * 8 * (size_t)((n + h->nleaves + 1) / 2 + 1));
-    h->p2p_runs_pr.ensure(sizeof(int2) * (size_t)std::max<int64_t>(h->n_p2p, 1));
     pr_flag_k<<<nblk(n, 256), 256, 0, s>>>(n, h->pcell.as<int>(), h->c_begin.as<int>(), h->c_end.as<int>(),
                                            h->pr_flag.as<unsigned>());
     count_launch(h);
     scan_exclusive_u32(h, h->pr_flag.as<unsigned>(), h->pr_pad.as<unsigned>(), n, nullptr, s);
-    pr_runs_k<<<nblk(h->nleaves, 128), 128, 0, s>>>(h->nleaves, h->leaves.as<int>(), h->p2p_ptr.as<int>(),
-                                                   h->p2p_nrun.as<int>(), h->p2p_runs.as<int2>(), h->pr_pad.as<unsigned>(),
-                                                   h->pr_flag.as<unsigned>(), h->p2p_runs_pr.as<int2>());
-    count_launch(h);
-    check_launch("p2p pair runs");
+    check_launch("p2p pair records");
     h->pr_ready = true;
     p2p_pairs_fill(h, s);
 }
@@ -1119,7 +1099,7 @@ void near_field(fmm_ctx *h, cudaStream_t s)
         FMM_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), s));
         p2p_pr_k<FMM_P2P_TPT><<<h->nleaves, P2P_T, 0, s>>>(h->xs32.as<float4>(), h->pr_pairs.as<float>(),
                                                           h->pr_pad.as<unsigned>(), h->pr_flag.as<unsigned>(), lv, cb, ce,
-                                                          pp, h->p2p_runs_pr.as<int2>(), nr, out, err);
+                                                          pp, ru, nr, out, err);
     } else
         p2p_k<float, false, FMM_P2P_TPT><<<h->nleaves, P2P_T, 0, s>>>(h->xs32.as<float4>(), nullptr, lv, cb, ce, pp, ru, nr, out);
     count_launch(h);

@@ -45,9 +45,12 @@ __device__ __forceinline__ double ord_dec(unsigned long long e)
 }
 
 // ---------------------------------------------------------------------------
-// exclusive scan of uint32 (three kernels; any length up to 2^31)
+// exclusive scan of uint32 (any length up to 2^31): one block for up to
+// SCAN_SMALL entries, three kernels beyond
 // ---------------------------------------------------------------------------
 constexpr int SCAN_T = 1024, SCAN_I = 4, SCAN_TILE = SCAN_T * SCAN_I;
+// one block walks 4 tiles in about the time of the two further launches
+constexpr int SCAN_SMALL = 4 * SCAN_TILE;
 
 __device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned *sw, unsigned *total)
 {
@@ -124,11 +127,41 @@ __global__ void scan_apply_k(const unsigned *__restrict__ in, unsigned *__restri
     }
 }
 
+__global__ void __launch_bounds__(SCAN_T) scan_small_k(const unsigned *__restrict__ in, unsigned *__restrict__ out, int n,
+                                                       unsigned *total)
+{
+    __shared__ unsigned sw[32];
+    unsigned carry = 0;
+    for (int b0 = 0; b0 < n; b0 += SCAN_TILE) {
+        const int base = b0 + (int)threadIdx.x * SCAN_I;
+        unsigned v[SCAN_I], s = 0, tot;
+#pragma unroll
+        for (int k = 0; k < SCAN_I; k++) {
+            v[k] = base + k < n ? in[base + k] : 0u;
+            s += v[k];
+        }
+        unsigned ex = carry + block_excl_scan(s, sw, &tot);
+#pragma unroll
+        for (int k = 0; k < SCAN_I; k++) {
+            if (base + k < n) out[base + k] = ex;
+            ex += v[k];
+        }
+        carry += tot;
+    }
+    if (threadIdx.x == 0 && total) *total = carry;
+}
+
 void scan_exclusive_u32(fmm_ctx *h, const unsigned *in, unsigned *out, int64_t count, unsigned *total_dev,
                         cudaStream_t s)
 {
     if (count <= 0) {
         if (total_dev) FMM_CUDA_TRY(cudaMemsetAsync(total_dev, 0, sizeof(unsigned), s));
+        return;
+    }
+    if (count <= SCAN_SMALL) {
+        scan_small_k<<<1, SCAN_T, 0, s>>>(in, out, (int)count, total_dev);
+        count_launch(h);
+        check_launch("scan");
         return;
     }
     int nb = (int)nblocks(count, SCAN_TILE);
@@ -476,33 +509,39 @@ __global__ void root_k(int n, int *level, uint64_t *anchor, int *begin, int *end
     xyz[0] = make_int4(0, 0, 0, 0);
 }
 
+// Eight lanes per cell, lane o searching the first key of octant o on its own:
+// the searches of a cell are dependent loads of about 0.4 us each, so one
+// thread doing the seven in turn takes 7 log2(range) of them (30 us a level for
+// a handful of cells).
 __global__ void split_count_k(int ls, int le, int l, int ncrit, const uint64_t *__restrict__ keys,
                               const int *__restrict__ begin, const int *__restrict__ end, unsigned *__restrict__ cnt,
                               int *__restrict__ bnd)
 {
-    int c = ls + blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= le) return;
-    int b = begin[c], e = end[c];
-    unsigned nc = 0;
-    int *bb = bnd + (size_t)(c - ls) * 9;
-    if (l < FMM_MAXLEVEL && e - b > ncrit) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = ls + (t >> 3), o = t & 7;
+    const bool in = c < le;
+    const int b = in ? begin[c] : 0, e = in ? end[c] : 0;
+    const bool split = in && l < FMM_MAXLEVEL && e - b > ncrit;
+    int L = b;
+    if (split && o > 0) {
         const int shift = 3 * (FMM_MAXLEVEL - 1 - l);
-        bb[0] = b;
-        int lo = b;
-        for (int o = 1; o < 8; o++) {
-            int L = lo, H = e;  // first index with digit >= o
-            while (L < H) {
-                int mid = (L + H) >> 1;
-                if ((int)((keys[mid] >> shift) & 7u) < o) L = mid + 1;
-                else H = mid;
-            }
-            bb[o] = L;
-            lo = L;
+        int H = e;  // first index with digit >= o
+        while (L < H) {
+            const int mid = L + ((H - L) >> 1);
+            if ((int)((keys[mid] >> shift) & 7u) < o) L = mid + 1;
+            else H = mid;
         }
-        bb[8] = e;
-        for (int o = 0; o < 8; o++) nc += bb[o + 1] > bb[o];
     }
-    cnt[c - ls] = nc;
+    int next = __shfl_down_sync(0xffffffffu, L, 1, 8);
+    if (o == 7) next = e;
+    const unsigned full = __ballot_sync(0xffffffffu, split && next > L);
+    if (!in) return;
+    if (split) {
+        int *bb = bnd + (size_t)(c - ls) * 9;
+        bb[o] = L;
+        if (o == 7) bb[8] = e;
+    }
+    if (o == 0) cnt[c - ls] = __popc((full >> (threadIdx.x & 24)) & 0xffu);
 }
 
 __global__ void split_write_k(int ls, int le, int l, const unsigned *__restrict__ cnt, const unsigned *__restrict__ off,
@@ -686,44 +725,59 @@ __global__ void pair_rows_k(const uint64_t *__restrict__ keys, int64_t np, int b
     if ((int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(&rowcnt[row], (unsigned)__popc(same));
 }
 
-__global__ void interactions_k(const int *__restrict__ ptr, const int *__restrict__ src, const int *__restrict__ begin,
-                               const int *__restrict__ end, int nc, unsigned long long *out)
-{
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned long long s = 0;
-    if (c < nc) {
-        long long na = end[c] - begin[c];
-        for (int k = ptr[c]; k < ptr[c + 1]; k++) {
-            int b = src[k];
-            s += (unsigned long long)(na * (long long)(end[b] - begin[b]));
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0 && s) atomicAdd(out, s);
-}
-
 // P2P source leaves of a target leaf that are adjacent in the sorted particle
 // order are merged into runs [begin, end); runs of leaf A are stored at
 // [ptr[A], ptr[A] + nrun[A]) of the run array (never more runs than leaves).
-__global__ void p2p_runs_k(int nleaves, const int *__restrict__ leaves, const int *__restrict__ ptr,
-                           const int *__restrict__ src, const int *__restrict__ begin, const int *__restrict__ end,
-                           int2 *__restrict__ runs, int *__restrict__ nrun)
+// With pad and flag (packed P2P) the runs are in records: particles [b, e) are
+// records [(b + pad[b]) / 2, (e + pad[e - 1] + flag[e - 1]) / 2). One warp per
+// leaf: an entry opens a run when it does not begin where its predecessor
+// ends, and closes it when its successor does not begin where it ends; ballots
+// number the runs. (One thread per leaf, its loads in turn, took 0.38 ms for
+// 4,096 leaves of 250 sources and 0.74 ms for 53,000 of 178.) The entries'
+// particle counts add up to the number of interactions.
+constexpr int RUN_WARPS = 8;
+__global__ void __launch_bounds__(32 * RUN_WARPS) p2p_runs_k(int nleaves, const int *__restrict__ leaves,
+                                                             const int *__restrict__ ptr, const int *__restrict__ src,
+                                                             const int *__restrict__ begin, const int *__restrict__ end,
+                                                             const unsigned *__restrict__ pad,
+                                                             const unsigned *__restrict__ flag, int2 *__restrict__ runs,
+                                                             int *__restrict__ nrun, unsigned long long *inter)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nleaves) return;
-    const int A = leaves[i];
-    int k = ptr[A], o = ptr[A];
-    const int k1 = ptr[A + 1];
-    while (k < k1) {
-        int b = begin[src[k]], e = end[src[k]];
-        k++;
-        while (k < k1 && begin[src[k]] == e) {
-            e = end[src[k]];
-            k++;
+    __shared__ unsigned long long ssum[RUN_WARPS];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.x * RUN_WARPS + w;
+    unsigned long long sum = 0;
+    if (i < nleaves) {
+        const int A = leaves[i], k0 = ptr[A], k1 = ptr[A + 1];
+        int o = k0;
+        for (int kb = k0; kb < k1; kb += 32) {
+            const int k = kb + lane;
+            bool open = false, close = false;
+            int b = 0, e = 0;
+            if (k < k1) {
+                const int s = src[k];
+                b = begin[s];
+                e = end[s];
+                open = k == k0 || end[src[k - 1]] != b;
+                close = k + 1 == k1 || begin[src[k + 1]] != e;
+                sum += (unsigned long long)(e - b);
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, open);
+            const int pos = o + __popc(m & (0xffffffffu >> (31 - lane))) - 1;  // run of this entry
+            if (open) runs[pos].x = pad ? (int)((b + pad[b]) >> 1) : b;
+            if (close) runs[pos].y = pad ? (int)((e + pad[e - 1] + flag[e - 1]) >> 1) : e;
+            o += __popc(m);
         }
-        runs[o++] = make_int2(b, e);
+        if (lane == 0) nrun[A] = o - k0;
+        for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+        sum *= (unsigned long long)(end[A] - begin[A]);
     }
-    nrun[A] = o - ptr[A];
+    if (lane == 0) ssum[w] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < RUN_WARPS; k++) sum += ssum[k];
+        if (sum) atomicAdd(inter, sum);
+    }
 }
 
 // (target, source) pairs -> CSR rows without a global sort: rows are counted
@@ -765,28 +819,29 @@ __global__ void row_max_k(int nc, const unsigned *__restrict__ cnt, unsigned *__
 
 constexpr int ROW_SORT_WARPS = 8, ROW_SORT_CAP = 1024;
 
-// Ascending bitonic sort of 256 keys held by one warp, lane l holding keys
-// 8 l .. 8 l + 7: partners 8 or more apart are exchanged with shuffles, the
+// Ascending bitonic sort of 32 R keys held by one warp, lane l holding keys
+// R l .. R l + R - 1: partners R or more apart are exchanged with shuffles, the
 // others inside the lane's registers.
-__device__ __forceinline__ void warp_bitonic256(int (&v)[8], int lane)
+template <int R>
+__device__ __forceinline__ void warp_bitonic(int (&v)[R], int lane)
 {
 #pragma unroll
-    for (int k = 2; k <= 256; k <<= 1) {
+    for (int k = 2; k <= 32 * R; k <<= 1) {
 #pragma unroll
         for (int j = k >> 1; j > 0; j >>= 1) {
-            if (j >= 8) {
+            if (j >= R) {
 #pragma unroll
-                for (int r = 0; r < 8; r++) {
-                    const int i = lane * 8 + r;
-                    const int y = __shfl_xor_sync(0xffffffffu, v[r], j >> 3);
+                for (int r = 0; r < R; r++) {
+                    const int i = lane * R + r;
+                    const int y = __shfl_xor_sync(0xffffffffu, v[r], j / R);
                     const bool up = (i & k) == 0, low = (i & j) == 0;
                     v[r] = low == up ? min(v[r], y) : max(v[r], y);
                 }
             } else {
 #pragma unroll
-                for (int r = 0; r < 8; r++) {
+                for (int r = 0; r < R; r++) {
                     if (r & j) continue;
-                    const bool up = ((lane * 8 + r) & k) == 0;
+                    const bool up = ((lane * R + r) & k) == 0;
                     const int a = v[r], b = v[r | j];
                     v[r] = up ? min(a, b) : max(a, b);
                     v[r | j] = up ? max(a, b) : min(a, b);
@@ -796,36 +851,30 @@ __device__ __forceinline__ void warp_bitonic256(int (&v)[8], int lane)
     }
 }
 
-// Each CSR row in ascending order, one warp per row: rows of up to 256
-// entries by a bitonic sort in registers, longer ones (up to ROW_SORT_CAP)
-// by exact ranks in shared memory.
+template <int R>
+__device__ __forceinline__ void row_sort_warp(int *src, int len, int lane)
+{
+    int v[R];
+#pragma unroll
+    for (int k = 0; k < R; k++) v[k] = lane * R + k < len ? src[lane * R + k] : INT_MAX;
+    warp_bitonic<R>(v, lane);
+#pragma unroll
+    for (int k = 0; k < R; k++)
+        if (lane * R + k < len) src[lane * R + k] = v[k];
+}
+
+// Each CSR row of up to ROW_SORT_CAP entries in ascending order, one warp per
+// row, by a bitonic sort in registers of the next of 256, 512 and 1024 entries.
 __global__ void __launch_bounds__(32 * ROW_SORT_WARPS) row_sort_k(int nc, const int *__restrict__ ptr, int *__restrict__ src)
 {
-    __shared__ int sh[ROW_SORT_WARPS][ROW_SORT_CAP];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int r = blockIdx.x * ROW_SORT_WARPS + w;
     if (r >= nc) return;
     const int b = ptr[r], len = ptr[r + 1] - b;
     if (len <= 1 || len > ROW_SORT_CAP) return;
-    if (len <= 256) {
-        int v[8];
-#pragma unroll
-        for (int k = 0; k < 8; k++) v[k] = lane * 8 + k < len ? src[b + lane * 8 + k] : INT_MAX;
-        warp_bitonic256(v, lane);
-#pragma unroll
-        for (int k = 0; k < 8; k++)
-            if (lane * 8 + k < len) src[b + lane * 8 + k] = v[k];
-        return;
-    }
-    int *row = sh[w];
-    for (int k = lane; k < len; k += 32) row[k] = src[b + k];
-    __syncwarp();
-    for (int k = lane; k < len; k += 32) {
-        const int e = row[k];
-        int rank = 0;
-        for (int t = 0; t < len; t++) rank += row[t] < e;
-        src[b + rank] = e;
-    }
+    if (len <= 256) row_sort_warp<8>(src + b, len, lane);
+    else if (len <= 512) row_sort_warp<16>(src + b, len, lane);
+    else row_sort_warp<32>(src + b, len, lane);
 }
 
 // ---------------------------------------------------------------------------
@@ -838,25 +887,54 @@ __global__ void __launch_bounds__(32 * ROW_SORT_WARPS) row_sort_k(int nc, const 
 // parent offset with |u_d| <= (|v_d| + 1) / 2, so
 // |u|^2 <= (|v|^2 + 2 sqrt(3) |v| + 3) / 4 < K0.
 // ---------------------------------------------------------------------------
-// write = false: row counts into cnt[c]; write = true: the rows at ptr[c]
-__global__ void near_rows_k(int ls, int le, int L, const int4 *__restrict__ xyz, const int4 *__restrict__ near,
-                            int nnear, unsigned *__restrict__ cnt, const int *__restrict__ ptr,
-                            int *__restrict__ src, bool write)
+// One warp per cell, its lanes over the stencil. Row counts into cnt[c] ...
+__global__ void __launch_bounds__(256) near_count_k(int ls, int le, int L, const int4 *__restrict__ xyz,
+                                                    const int4 *__restrict__ near, int nnear, unsigned *__restrict__ cnt)
 {
-    const int c = ls + blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31, c = ls + (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (c >= le) return;
-    const int sh = FMM_MAXLEVEL - L, side = 1 << L;
+    const int sh = FMM_MAXLEVEL - L;
+    const unsigned side = 1u << L;
     const int4 a = xyz[c];
     const int px = a.x >> sh, py = a.y >> sh, pz = a.z >> sh;
-    int k = 0, base = write ? ptr[c] : 0;
-    for (int e = 0; e < nnear; e++) {
+    int k = 0;
+    for (int e = lane; e < nnear; e += 32) {
         const int4 v = near[e];
-        const int qx = px + v.x, qy = py + v.y, qz = pz + v.z;
-        if (qx < 0 || qy < 0 || qz < 0 || qx >= side || qy >= side || qz >= side) continue;
-        if (write) src[base + k] = ls + (int)morton3((uint32_t)qx, (uint32_t)qy, (uint32_t)qz);
-        k++;
+        k += (unsigned)(px + v.x) < side && (unsigned)(py + v.y) < side && (unsigned)(pz + v.z) < side;
     }
-    if (!write) cnt[c] = (unsigned)k;
+    k = __reduce_add_sync(0xffffffffu, k);
+    if (lane == 0) cnt[c] = (unsigned)k;
+}
+
+// ... and the rows at ptr[c], sorted in registers before they are written
+// (32 R >= nnear; positions outside the lattice sort to the end)
+template <int R>
+__global__ void __launch_bounds__(256) near_rows_k(int ls, int le, int L, const int4 *__restrict__ xyz,
+                                                   const int4 *__restrict__ near, int nnear, const int *__restrict__ ptr,
+                                                   int *__restrict__ src)
+{
+    const int lane = threadIdx.x & 31, c = ls + (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (c >= le) return;
+    const int sh = FMM_MAXLEVEL - L;
+    const unsigned side = 1u << L;
+    const int4 a = xyz[c];
+    const int px = a.x >> sh, py = a.y >> sh, pz = a.z >> sh;
+    int v[R];
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+        const int e = 32 * r + lane;
+        v[r] = INT_MAX;
+        if (e < nnear) {
+            const int4 d = near[e];
+            const unsigned qx = (unsigned)(px + d.x), qy = (unsigned)(py + d.y), qz = (unsigned)(pz + d.z);
+            if (qx < side && qy < side && qz < side) v[r] = ls + (int)morton3(qx, qy, qz);
+        }
+    }
+    warp_bitonic<R>(v, lane);
+    const int b = ptr[c], len = ptr[c + 1] - b;
+#pragma unroll
+    for (int r = 0; r < R; r++)
+        if (lane * R + r < len) src[b + lane * R + r] = v[r];
 }
 
 static int bits_for(int64_t v)
@@ -1106,8 +1184,8 @@ static bool uniform_lists(fmm_ctx *h, long long K0, cudaStream_t s)
     h->p2p_ptr.ensure(sizeof(int) * (size_t)(nc + 1));
     h->row_cnt.ensure(sizeof(unsigned) * (size_t)(nc + 1));
     FMM_CUDA_TRY(cudaMemsetAsync(h->row_cnt.p, 0, sizeof(unsigned) * (size_t)(nc + 1), s));
-    near_rows_k<<<nblocks(le - ls, 128), 128, 0, s>>>(ls, le, L, h->c_xyz.as<int4>(), h->near_dev.as<int4>(), nn,
-                                                      h->row_cnt.as<unsigned>(), nullptr, nullptr, false);
+    const unsigned nb = nblocks((int64_t)(le - ls) * 32, 256);
+    near_count_k<<<nb, 256, 0, s>>>(ls, le, L, h->c_xyz.as<int4>(), h->near_dev.as<int4>(), nn, h->row_cnt.as<unsigned>());
     count_launch(h);
     scan_exclusive_u32(h, h->row_cnt.as<unsigned>(), reinterpret_cast<unsigned *>(h->p2p_ptr.as<int>()), nc + 1, nullptr, s);
     unsigned *hp = h->hpin.as<unsigned>();
@@ -1115,10 +1193,9 @@ static bool uniform_lists(fmm_ctx *h, long long K0, cudaStream_t s)
     FMM_CUDA_TRY(cudaStreamSynchronize(s));
     h->n_p2p = (int64_t)*hp;
     h->p2p_src.ensure(sizeof(int) * (size_t)std::max<int64_t>(h->n_p2p, 1));
-    near_rows_k<<<nblocks(le - ls, 128), 128, 0, s>>>(ls, le, L, h->c_xyz.as<int4>(), h->near_dev.as<int4>(), nn,
-                                                      nullptr, h->p2p_ptr.as<int>(), h->p2p_src.as<int>(), true);
-    count_launch(h);
-    row_sort_k<<<nblocks(nc, ROW_SORT_WARPS), 32 * ROW_SORT_WARPS, 0, s>>>(nc, h->p2p_ptr.as<int>(), h->p2p_src.as<int>());
+    auto *rows = nn <= 256 ? near_rows_k<8> : nn <= 512 ? near_rows_k<16> : near_rows_k<32>;
+    rows<<<nb, 256, 0, s>>>(ls, le, L, h->c_xyz.as<int4>(), h->near_dev.as<int4>(), nn, h->p2p_ptr.as<int>(),
+                            h->p2p_src.as<int>());
     count_launch(h);
     check_launch("uniform lists");
     int64_t m2l = 0;
@@ -1230,7 +1307,7 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
         h->split_cnt.ensure(sizeof(unsigned) * (m + 1));
         h->split_off.ensure(sizeof(unsigned) * (m + 1));
         h->split_bnd.ensure(sizeof(int) * 9 * (size_t)m);
-        split_count_k<<<nblocks(m, TB), TB, 0, s>>>(ls, le, l, h->ncrit, h->keys.as<uint64_t>(), h->c_begin.as<int>(),
+        split_count_k<<<nblocks((int64_t)m * 8, TB), TB, 0, s>>>(ls, le, l, h->ncrit, h->keys.as<uint64_t>(), h->c_begin.as<int>(),
                                                     h->c_end.as<int>(), h->split_cnt.as<unsigned>(), h->split_bnd.as<int>());
         count_launch(h);
         unsigned *tot = reinterpret_cast<unsigned *>(h->counters.as<char>() + sizeof(TravCounters));
@@ -1392,20 +1469,18 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
     pairs_to_csr(h, h->m2lx_pairs.as<int2>(), h->n_m2lx, h->m2lx_ptr, h->m2lx_src, s);
     h->p2p_runs.ensure(sizeof(int2) * (size_t)std::max<int64_t>(h->n_p2p, 1));
     h->p2p_nrun.ensure(sizeof(int) * (size_t)ncells);
-    if (h->nleaves > 0) {
-        p2p_runs_k<<<nblocks(h->nleaves, 128), 128, 0, s>>>(h->nleaves, h->leaves.as<int>(), h->p2p_ptr.as<int>(),
-                                                            h->p2p_src.as<int>(), h->c_begin.as<int>(), h->c_end.as<int>(),
-                                                            h->p2p_runs.as<int2>(), h->p2p_nrun.as<int>());
-        count_launch(h);
-        check_launch("p2p runs");
-    }
     p2p_prepare(h, s);
     {
         unsigned long long *acc = reinterpret_cast<unsigned long long *>(h->counters.as<char>() + sizeof(TravCounters) + 8);
         FMM_CUDA_TRY(cudaMemsetAsync(acc, 0, 8, s));
-        interactions_k<<<nblocks(ncells, 256), 256, 0, s>>>(h->p2p_ptr.as<int>(), h->p2p_src.as<int>(), h->c_begin.as<int>(),
-                                                            h->c_end.as<int>(), ncells, acc);
-        count_launch(h);
+        if (h->nleaves > 0) {
+            p2p_runs_k<<<nblocks(h->nleaves, RUN_WARPS), 32 * RUN_WARPS, 0, s>>>(
+                h->nleaves, h->leaves.as<int>(), h->p2p_ptr.as<int>(), h->p2p_src.as<int>(), h->c_begin.as<int>(),
+                h->c_end.as<int>(), h->pr_ready ? h->pr_pad.as<unsigned>() : nullptr, h->pr_flag.as<unsigned>(),
+                h->p2p_runs.as<int2>(), h->p2p_nrun.as<int>(), acc);
+            count_launch(h);
+            check_launch("p2p runs");
+        }
         unsigned long long *hp = h->hpin.as<unsigned long long>();
         FMM_CUDA_TRY(cudaMemcpyAsync(hp, acc, 8, cudaMemcpyDeviceToHost, s));
         FMM_CUDA_TRY(cudaStreamSynchronize(s));
