@@ -361,7 +361,7 @@ FMM_API int fmm_batch_destroy(fmm_batch b);
  *   fmm_build computes and fmm_export_tree returns;
  *   stream: cudaStream_t (NULL = legacy default stream).
  * No allocation: temporaries live in one fixed array that the library
- * reserves on every GPU that loads it (about 12.3 MB, held until the process
+ * reserves on every GPU that loads it (about 12.6 MiB, held until the process
  * exits); n above 1048576 is rejected with FMM_EINVAL. The first call on a
  * device looks up the array's device address with that device current; make
  * that first call before any stream capture. All calls share the array: calls

@@ -77,13 +77,13 @@ struct PinnedBuf {
 
 // root cube, computed on the device
 struct Box {
-    unsigned long long enc_lo[3], enc_hi[3];  // order-preserving encodings of min / max
+    unsigned long long enc[6];  // order-preserving encodings: complements of the minima, maxima
     double origin[3];
     double R0;     // half width of the root cube
     double s;      // 2^21 / (2 R0)
     double h;      // 2 R0 / 2^21 (grid spacing)
     int nonfinite; // set when a coordinate is NaN or infinite
-    int pad;
+    unsigned ticket; // blocks of the bounding-box kernel that are done
 };
 
 // open-addressed table slot: Morton index of a cell at its level plus one
@@ -271,7 +271,7 @@ struct fmm_ctx {
     fmm::DevBuf pcell;                  // leaf cell of each sorted particle
     fmm::DevBuf cgeo;                   // per cell: geometric centre and 1 / width (double4)
     fmm::DevBuf energy_buf;             // block sums of the weighted energy
-    fmm::DevBuf hist, scan_tmp;
+    fmm::DevBuf sort_ws, scan_tmp;
     fmm::DevBuf xs64, xs32, xs32lo;
     fmm::DevBuf c_level, c_anchor, c_begin, c_end, c_child, c_nchild, c_parent, c_xyz;
     fmm::DevBuf split_cnt, split_off, split_bnd;
@@ -315,8 +315,9 @@ void tree_export(fmm_ctx *h, uint64_t *keys, int32_t *perm, int32_t *level, uint
                  int32_t *begin, int32_t *end, int32_t *child, int32_t *nchild, int32_t *parent,
                  int64_t *p2p_ptr, int32_t *p2p_idx, int64_t *m2l_ptr, int32_t *m2l_idx, double *box);
 int64_t tree_m2l_total(fmm_ctx *h);
-void morton_sort_into(const void *x, int64_t n, int dt, uint64_t *keys, int *perm, uint64_t *keys_tmp, int *perm_tmp,
-                      unsigned *hist, unsigned *bsum, Box *box, int nsm, cudaStream_t s);
+size_t sort_ws_bytes(int64_t n);
+int morton_sort_into(const void *x, int64_t n, int dt, uint64_t *keys, int *perm, uint64_t *keys_tmp, int *perm_tmp,
+                     void *ws, Box *box, int nsm, cudaStream_t s);
 int m2l_tile_size(fmm_ctx *h);
 void scan_exclusive_u32(fmm_ctx *h, const unsigned *in, unsigned *out, int64_t count, unsigned *total_dev,
                         cudaStream_t s);

@@ -11,7 +11,7 @@
 // the octree build without the library allocating anything.
 //
 // The scratch is a file-scope __device__ array, so every GPU that loads the
-// library holds it (NOALLOC_MAX_N * 12 bytes plus histograms, about 12.3 MB)
+// library holds it (NOALLOC_MAX_N * 12 bytes plus 0.6 MB, about 12.6 MiB)
 // until the process exits. Host code cannot use the array's name as a device
 // address; its address is read with cudaGetSymbolAddress once per device, on
 // the first call made with that device current.
@@ -22,12 +22,10 @@
 namespace fmm {
 
 constexpr int64_t NOALLOC_MAX_N = 1 << 20;                       // largest n a call accepts
-constexpr int64_t NOALLOC_TILES = NOALLOC_MAX_N / 4096;          // radix-sort tiles at that size
 constexpr size_t NOALLOC_KEYS = sizeof(uint64_t) * NOALLOC_MAX_N; // ping-pong keys
 constexpr size_t NOALLOC_PERM = sizeof(int) * NOALLOC_MAX_N;      // ping-pong indices
-constexpr size_t NOALLOC_HIST = sizeof(unsigned) * 256 * NOALLOC_TILES;
-constexpr size_t NOALLOC_BSUM = sizeof(unsigned) * 1024;
-constexpr size_t NOALLOC_BYTES = NOALLOC_KEYS + NOALLOC_PERM + NOALLOC_HIST + NOALLOC_BSUM + 256;
+constexpr size_t NOALLOC_WS = 640 * 1024;                         // sort workspace: most for 2^19 keys, in 512 tiles
+constexpr size_t NOALLOC_BYTES = NOALLOC_KEYS + NOALLOC_PERM + NOALLOC_WS + 256;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
 
@@ -78,11 +76,11 @@ extern "C" FMM_API int fmm_morton_sort_noalloc(const void *x, int64_t n, int dty
         }
         uint64_t *ktmp = reinterpret_cast<uint64_t *>(base);
         int *ptmp = reinterpret_cast<int *>(base + NOALLOC_KEYS);
-        unsigned *hist = reinterpret_cast<unsigned *>(base + NOALLOC_KEYS + NOALLOC_PERM);
-        unsigned *bsum = reinterpret_cast<unsigned *>(base + NOALLOC_KEYS + NOALLOC_PERM + NOALLOC_HIST);
-        Box *box = reinterpret_cast<Box *>(base + NOALLOC_KEYS + NOALLOC_PERM + NOALLOC_HIST + NOALLOC_BSUM);
+        unsigned char *ws = base + NOALLOC_KEYS + NOALLOC_PERM;
+        Box *box = reinterpret_cast<Box *>(ws + NOALLOC_WS);
+        if (sort_ws_bytes(n) > NOALLOC_WS) throw Error{FMM_EINVAL, "fmm_morton_sort_noalloc: workspace too small"};
         static_assert(sizeof(Box) <= 256, "root-cube scratch");
-        morton_sort_into(x, n, dtype, keys, perm, ktmp, ptmp, hist, bsum, box, nsm, (cudaStream_t)stream);
+        morton_sort_into(x, n, dtype, keys, perm, ktmp, ptmp, ws, box, nsm, (cudaStream_t)stream);
         return FMM_OK;
     } catch (const Error &e) {
         set_error(e.msg);
