@@ -135,7 +135,7 @@ struct M2LJob {
     // copy of M~ (bit l: level l); lat_maps holds a 128-byte tensor map per level
     const unsigned char *lat_maps;
     unsigned lat_levels;
-    int nsplit;                 // ranges the vectors of a tile are cut into, one CTA each
+    int nsplit, chunk;          // ranges of `chunk` vectors a tile's list is cut into, one CTA each
     int ws_words;               // words of the workspace at lmax (maxima, counters) to zero per evaluation
     int item0;
     int count;
@@ -253,7 +253,7 @@ struct fmm_ctx {
     int rot_nv = -1, rot_kind = 0;  // vectors and precision (1 FP32, 2 FP64) of rot_tab
     fmm::DevBuf msplit;         // M~ split into FP16 (hi, lo) rows for the tensor-core M2L
     fmm::DevBuf m2l_ws, m2l_part;  // its level maxima and tile counters; sums of the ranges of split tiles
-    int m2l_nsplit = 1;         // ranges per tile (m2l_plan)
+    int m2l_nsplit = 1, m2l_chunk = 0;  // ranges per tile and their length (m2l_plan)
     // tensor-core M2L on complete levels: the rows of each such level in lattice
     // order (octant bits, then z, y, x of the halved position), one TMA tensor
     // map per level (device copy and its pinned staging)
@@ -362,6 +362,7 @@ void m2l_tensor(fmm_ctx *h, float *L, const float *M);
 // the same-level M2L of several systems (same p; rows already split) in one persistent launch
 void m2l_tensor_jobs(int p, int nsm, const M2LJob *jobs_dev, int njobs, int *queue, int *err, cudaStream_t s);
 M2LJob m2l_tensor_job(fmm_ctx *h, float *L);  // the handle's arrays; allocates its workspaces
+int m2l_longest_list(fmm_ctx *h);              // vectors of the longest list a tile walks
 void m2l_plan(fmm_ctx *h);                     // (build) ranges per tile
 // (build) which complete levels the tensor-core M2L reads through TMA tile
 // loads: their lattice buffer and tensor maps

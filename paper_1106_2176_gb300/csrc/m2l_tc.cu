@@ -58,12 +58,16 @@
 // A tree with few tiles (5 at N = 16,384) would leave most SMs idle: the
 // vectors of every tile are then cut into nsplit ranges, one CTA each
 // (m2l_plan). Each CTA writes its (hi, lo) sums and the last one of a tile to
-// finish adds the ranges in order, so results do not depend on scheduling.
+// finish adds the ranges in order, so results do not depend on scheduling. The
+// ranges start at multiples of one chunk of whole drain groups, whatever the
+// length of the tile's own list: a cell's sums do not depend on the tile that
+// it falls into either (cells of incomplete levels are placed in arrival order).
 //
 // Every wait is bounded; on a timeout the kernel records an error code and
 // leaves after its copies have landed and its TMEM is released.
 #include <algorithm>
 #include <array>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -314,7 +318,7 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     // the set's entries are sorted by reach: only a prefix can hit a cell;
     // this CTA's range of it
     const int nvt = J.st_off[10 + td.octant * (FMM_MAXLEVEL + 1) + l];
-    const int w0 = (int)((long long)nvt * split / nsplit), w1 = (int)((long long)nvt * (split + 1) / nsplit);
+    const int w0 = (int)min((long long)nvt, (long long)split * J.chunk), w1 = (int)min((long long)nvt, (long long)w0 + J.chunk);
     const int e0 = J.st_off[td.octant] + w0, nv = w1 - w0;
     const int nunits = nv * KB;
     // Lattice tile (a complete level with a lattice copy of M~): the tile is
@@ -902,29 +906,40 @@ static void launch_tc_p(int p, int grid, const M2LJob &one, const M2LJob *jobs, 
 // words of the M2L workspace: per-level maxima, then one counter per tile
 constexpr int TCW_CNT = 32;
 
+// the longest list of vectors that a tile of the tree walks
+int m2l_longest_list(fmm_ctx *h)
+{
+    const int pool_max = h->m2l_pool >= 0 ? h->m2l_pool : 4 * m2l_tile_size(h);
+    int nv = 1;
+    for (int l = 2; l <= h->depth; l++) {
+        const bool pooled = h->lvl_start[(size_t)l + 1] - h->lvl_start[(size_t)l] <= pool_max;
+        for (int o = pooled ? 8 : 0; o < (pooled ? 9 : 8); o++)
+            nv = std::max(nv, h->st_cnt[(size_t)o * (FMM_MAXLEVEL + 1) + l]);
+    }
+    return nv;
+}
+
 // How many ranges the vectors of every tile are cut into. A CTA's time is
-// about (its vectors + 10) units, one unit a vector's copies, plus one per
-// range for the last CTA's sum of them; the launch takes the waves of
+// about (its vectors + 10) units, one unit a vector's copies (+ 13 with its
+// sums' way through memory), plus one per range for the last CTA's sum of them; the launch takes the waves of
 // ntiles x nsplit CTAs over the SMs. One range wins as soon as the tiles fill
-// a few waves.
+// a few waves. Ranges are whole drain groups of both MMA warps.
 void m2l_plan(fmm_ctx *h)
 {
     h->m2l_nsplit = 1;
+    h->m2l_chunk = INT_MAX;
     if (h->precision != FMM_MIXED || h->engine_used != FMM_M2L_TENSOR || h->ntiles_max < 1) return;
-    const int pool_max = h->m2l_pool >= 0 ? h->m2l_pool : 4 * TcCfg<64>::M;
-    int nv = 1;
-    for (int l = 2; l <= h->depth; l++) {
-        const int cells = h->lvl_start[(size_t)l + 1] - h->lvl_start[(size_t)l];
-        for (int o = cells <= pool_max ? 8 : 0; o < (cells <= pool_max ? 9 : 8); o++)
-            nv = std::max(nv, h->st_cnt[(size_t)o * (FMM_MAXLEVEL + 1) + l]);
-    }
+    const int nv = m2l_longest_list(h);
     double best = 1e300;
-    for (int s = 1; s <= 32; s++) {
+    for (int want = 1; want <= 32; want++) {
+        constexpr int G = 2 * TcCfg<64>::GV;
+        const int chunk = (nv + want * G - 1) / (want * G) * G, s = (nv + chunk - 1) / chunk;
         const double waves = (double)(((int64_t)h->ntiles_max * s + h->nsm - 1) / h->nsm);
-        const double t = waves * ((double)nv / s + 10.0) + (s > 1 ? s : 0);
+        const double t = waves * ((double)std::min(chunk, nv) + (s > 1 ? 13.0 : 10.0)) + (s > 1 ? s : 0);
         if (t < best) {
             best = t;
             h->m2l_nsplit = s;
+            h->m2l_chunk = chunk;
         }
     }
 }
@@ -955,6 +970,7 @@ M2LJob m2l_tensor_job(fmm_ctx *h, float *L)
     j.ws_words = TCW_CNT + h->ntiles_max;
     j.part = h->m2l_part.as<float2>();
     j.nsplit = h->m2l_nsplit;
+    j.chunk = h->m2l_chunk;
     j.rowexp = reinterpret_cast<const int *>(j.ttab + (size_t)h->nV * tc_op_bytes(h->p));
     j.lat_maps = nullptr;  // gathers on every level (the single-system launch sets the lattice levels)
     j.lat_levels = 0;
