@@ -249,7 +249,10 @@ struct fmm_ctx {
     std::shared_ptr<fmm::TcImage> ttab;  // tensor-core M2L operators (split FP16 images), per vector
     int ttab_nv = -1;           // stencil vectors the operator images were made for
     std::vector<int> st_cnt;    // per set (octants, union) and level: entries that can reach a cell
-    fmm::DevBuf rot_tab;        // rotation M2L maps per vector ([A | B], FP32 or FP64)
+    fmm::DevBuf rot_tab;        // rotation M2L: maps per polar angle, data per vector, c_nm (FP32 or FP64)
+    fmm::DevBuf rot_angle;      // polar angle of every vector
+    fmm::DevBuf rot_m;          // multipoles times c_nm
+    size_t rot_vec_off = 0, rot_c_off = 0;  // entries before the vectors' data and the c_nm in rot_tab
     int rot_nv = -1, rot_kind = 0;  // vectors and precision (1 FP32, 2 FP64) of rot_tab
     fmm::DevBuf msplit;         // M~ split into FP16 (hi, lo) rows for the tensor-core M2L
     fmm::DevBuf m2l_ws, m2l_part;  // its level maxima and tile counters; sums of the ranges of split tiles
@@ -325,7 +328,7 @@ void scan_exclusive_u32(fmm_ctx *h, const unsigned *in, unsigned *out, int64_t c
 // expansions.cu
 void operators_init(fmm_ctx *h);  // R tables of M2M / L2L
 void stencil_update(fmm_ctx *h);  // same-level M2L stencil for the current tree depth
-// rotation-based M2L: per-degree maps into / out of the frame whose z axis is u
+// rotation-based M2L: per-degree maps into / out of the frame whose z axis is u (host reference)
 int rot_deg_off(int n);
 int rot_map_size(int p);
 void rotation_maps(int p, const double u[3], double *A, double *B);
@@ -333,7 +336,7 @@ void m2l_rotation_ref(int p, const double u[3], const double *M, double *L);
 template <class T>
 void m2l_rotation(fmm_ctx *h, T *L, const T *M);  // same-level M2L of all tiles by rotation
 bool rotation_m2l_supported(fmm_ctx *h);           // p <= 16 (the maps of a vector fit shared memory)
-int rotation_tile_rows(fmm_ctx *h);  // target cells per tile (two per warp)
+int rotation_tile_rows(fmm_ctx *h);  // target cells per tile
 // per (octant, level): how many of the octant's entries (shortest first) can
 // reach a cell of that level in the current tree; written after the offsets
 void stencil_levels(fmm_ctx *h, cudaStream_t s);

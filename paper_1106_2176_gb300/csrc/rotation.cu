@@ -29,6 +29,7 @@
 #include <algorithm>
 #include <array>
 #include <cmath>
+#include <cstring>
 #include <complex>
 #include <exception>
 #include <map>
@@ -39,6 +40,7 @@
 #include <vector>
 
 #include "fmm_internal.cuh"
+#include "ptx_sm100.cuh"
 
 namespace fmm {
 
@@ -225,68 +227,130 @@ void m2l_rotation_ref(int p, const double u[3], const double *M, double *L)
 
 // ---------------------------------------------------------------------------
 // device engine
+//
+// On the device the azimuth and the polar angle are applied apart. With the
+// coefficients multiplied by c_nm, X^m = c_m M^m e^{ima} (a phase per order),
+// and, because V is real and X^{-m} = (-1)^m conj(X^m), the polar rotation acts
+// on real and imaginary parts separately:
+//   Re M'^m' = sum_m T_mm' Re X^m / c_m',  T = V_mm' + (-1)^m V_{-m m'}  (X^0 halved)
+//   Im M'^m' = sum_m Q_mm' Im X^m / c_m',  Q = V_mm' - (-1)^m V_{-m m'}
+// two maps of (n+1)^2 and n^2 entries instead of one of (2n+1)^2. The way back
+// takes the same two: L^m = c_m e^{ima} (sum_m' T_mm' Re L'^m' + i sum_m' Q_mm'
+// Im L'^m') / c_m' (L'^0 halved), because (-1)^m' V_{m,-m'} = (-1)^m V_{-m,m'}.
+// The maps T_mm' / c_m' and Q_mm' / c_m' depend on the polar angle alone: about
+// 400 of them serve the 1,740 vectors of theta = 0.5.
+//
+// One CTA per tile of 32 target cells and range of the tile's vectors; lane i
+// of every warp is target i, and the warps share the coefficients. Per vector:
+//   gather   c M~ of the 32 sources (zero where absent), whole rows by cp.async,
+//            transposed to [coefficient][target] in shared memory
+//   forward  warps take (degree, part): e^{ima}, then a map row against the 32
+//            targets at once, the map read by broadcast
+//   along z  warps take (order, part): sums over the degrees of equal order
+//   back     as forward
+//   phases   e^{ima}, added to the warp's coefficients of L~ in registers
+//            (FP32: TwoSum pairs)
+// The (degree, part) jobs, K^2 multiply-adds each (K = n + 1 or n), are dealt
+// to the warps by size. The next vector's rows and maps arrive while the
+// current one is translated.
+//
+// Bound: FP32 by instruction issue (a map's 16 bytes are one load and two packed
+// multiply-adds), FP64 by GB300's FP64 pipe. N = 60,001, p = 16, FP32: 8.3 ms;
+// N = 50,000, p = 8, FP64: 18.4 ms. One warp per two targets with lanes over a
+// map's outputs (32 rows apart in shared memory: bank conflicts) took 39.7 and
+// 34.3 ms.
 // ---------------------------------------------------------------------------
 namespace fmm {
 
-// Device layout of one vector's data (padded so that rows and degree blocks
-// start on 16 bytes): A then B, degree n a block of K = 2n+1 rows of
-// K4 = K rounded up to 4 entries (zeros past K), then the factors
-// g_l = l! / |u|^(l+1), l < 2p - 1, rounded up to 4 entries.
-static int k4(int n) { return (2 * n + 1 + 3) & ~3; }
-static int rot_blocks(int p)  // entries of A (or B), padded
-{
-    int s = 0;
-    for (int n = 0; n < p; n++) s += (2 * n + 1) * k4(n);
-    return s;
-}
-static int rot_vec_stride(int p) { return 2 * rot_blocks(p) + ((2 * p - 1 + 3) & ~3); }
+constexpr int ROT_MAXP = 16, ROT_ROWS = 32;
+constexpr int ROT_LD = ROT_ROWS + 1;  // row pitch of [coefficient][target]: transposed writes without bank conflicts
+constexpr int ROT_G = 40;  // factors per vector: g_l = l!/|u|^(l+1), l <= 2 p - 2, zeros after
 
-// one host image per process for each (p, MAC constant, stencil bound)
-static std::mutex g_rot_mu;
-static std::map<std::tuple<int, double, int>, std::shared_ptr<const std::vector<double>>> g_rot_cache;
+// the jobs of every warp and where each map starts in a polar angle's table
+struct RotPlan {
+    int off[2][ROT_MAXP + 1];     // [part][K]: part 0 real (K = n + 1), 1 imaginary (K = n)
+    int ds;                       // entries of one table
+    unsigned char njob[8];
+    unsigned char job[8][32];     // K | part << 7
+    unsigned char nm[ROT_MAXP * (ROT_MAXP + 1) / 2][2];  // coefficient pair -> degree, order
+};
 
-static std::shared_ptr<const std::vector<double>> rot_image(fmm_ctx *h)
+// Entries per vector: the phases e^{ima} as the pairs that make the real part
+// of a product, (cos, -sin), and the imaginary part, (sin, cos); then the
+// factors from g_0, g_1, g_2 and g_3 on, so that a window of them starting
+// anywhere is aligned in one of the copies.
+constexpr int ROT_PH = 2 * ROT_MAXP, ROT_VS = 2 * ROT_PH + 4 * ROT_G;
+
+// Inside the kernel the coefficients of a degree are in the order Re (n, 0) ..
+// Re (n, n), Im (n, 1) .. Im (n, n): entry i of a (degree, part) job.
+__host__ __device__ constexpr int rot_idx(int n, int part, int i) { return n * n + part * (n + 1) + i; }
+
+template <class T>
+struct RotVec;
+template <>
+struct RotVec<float> {
+    using type = float4;
+    static constexpr int n = 4;
+};
+template <>
+struct RotVec<double> {
+    using type = double2;
+    static constexpr int n = 2;
+};
+
+// K rounded up to whole 16-byte vectors: the length of a map's rows
+template <class T>
+static int rot_pad(int K) { return (K + RotVec<T>::n - 1) / RotVec<T>::n * RotVec<T>::n; }
+
+template <class T>
+static RotPlan rot_plan(int p, int W)
 {
-    const auto key = std::make_tuple(h->p, h->cmac, h->st_R);
-    {
-        std::lock_guard<std::mutex> lk(g_rot_mu);
-        auto it = g_rot_cache.find(key);
-        if (it != g_rot_cache.end()) return it->second;
-    }
-    const int p = h->p, RS = rot_map_size(p), nv = h->nV, VS = rot_vec_stride(p), SA = rot_blocks(p);
-    std::vector<std::array<int, 3>> vec((size_t)nv);
-    const int ne = h->st_off[8];
-    for (int e = 0; e < ne; e++) {
-        const int *v = &h->st_host[4 * (size_t)e];
-        vec[(size_t)(v[3] & 0xffff)] = {v[0], v[1], v[2]};
-    }
-    auto img = std::make_shared<std::vector<double>>((size_t)nv * VS, 0.0);
-    // vectors in parallel on the host cores; u = c_L - c_M = -(source - target)
-    const unsigned nt = std::max(1u, std::min(32u, std::thread::hardware_concurrency()));
-    // stride t of the vectors: i = t, t + nt, ...
-    auto stride = [&](unsigned t) {
-        std::vector<double> A(RS), B(RS);
-        for (int i = (int)t; i < nv; i += (int)nt) {
-            const double u[3] = {-(double)vec[i][0], -(double)vec[i][1], -(double)vec[i][2]};
-            rotation_maps(p, u, A.data(), B.data());
-            double *o = img->data() + (size_t)i * VS;
-            int off = 0;
-            for (int n = 0; n < p; n++) {
-                const int K = 2 * n + 1, K4 = k4(n);
-                for (int r = 0; r < K; r++)
-                    for (int c = 0; c < K; c++) {
-                        o[off + r * K4 + c] = A[rot_deg_off(n) + r * K + c];
-                        o[SA + off + r * K4 + c] = B[rot_deg_off(n) + r * K + c];
-                    }
-                off += K * K4;
-            }
-            const double d = std::sqrt(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-            double g = 1.0 / d;
-            for (int l = 0; l < 2 * p - 1; l++) {
-                if (l) g *= (double)l / d;
-                o[2 * SA + l] = g;
-            }
+    RotPlan P;
+    std::memset(&P, 0, sizeof(P));
+    std::vector<std::pair<int, int>> jobs;  // (K, part), largest first
+    for (int part = 0; part < 2; part++)
+        for (int K = 1; K <= p - part; K++) {
+            P.off[part][K] = P.ds;
+            P.ds += K * rot_pad<T>(K);
+            jobs.push_back({K, part});
         }
+    std::sort(jobs.begin(), jobs.end(), [](auto &x, auto &y) { return x.first != y.first ? x.first > y.first : x.second < y.second; });
+    int load[8] = {};
+    for (auto &j : jobs) {
+        int w = 0;
+        for (int k = 1; k < W; k++)
+            if (load[k] < load[w]) w = k;
+        load[w] += j.first * rot_pad<T>(j.first) + 8;
+        P.job[w][P.njob[w]++] = (unsigned char)(j.first | j.second << 7);
+    }
+    int q = 0;
+    for (int n = 0; n < p; n++)
+        for (int m = 0; m <= n; m++, q++) {
+            P.nm[q][0] = (unsigned char)n;
+            P.nm[q][1] = (unsigned char)m;
+        }
+    return P;
+}
+
+// Host image, FP64: per distinct polar angle the maps (rows unpadded, parts and
+// sizes in order), per vector its angle, phases and factors. One per process
+// for each (p, MAC constant, stencil bound).
+struct RotImage {
+    int na = 0;
+    std::vector<double> maps;   // na x sum K^2
+    std::vector<int> angle;     // per vector
+    std::vector<double> vec;    // per vector ROT_VS
+};
+static std::mutex g_rot_mu;
+static std::map<std::tuple<int, double, int>, std::shared_ptr<const RotImage>> g_rot_cache;
+
+// run f(0 .. count - 1) on the host cores; the first exception is rethrown
+template <class F>
+static void host_parallel(int count, F f)
+{
+    const unsigned nt = std::max(1u, std::min(32u, std::thread::hardware_concurrency()));
+    auto stride = [&](unsigned t) {
+        for (int i = (int)t; i < count; i += (int)nt) f(i);
     };
     std::vector<std::thread> pool;
     std::vector<std::exception_ptr> fault(nt);  // an exception stays in its thread until the join
@@ -312,256 +376,654 @@ static std::shared_ptr<const std::vector<double>> rot_image(fmm_ctx *h)
         }
     }
     for (auto &th : pool) th.join();
-    for (auto &f : fault)
-        if (f) std::rethrow_exception(f);
+    for (auto &e : fault)
+        if (e) std::rethrow_exception(e);
+}
+
+static std::shared_ptr<const RotImage> rot_image(fmm_ctx *h)
+{
+    const auto key = std::make_tuple(h->p, h->cmac, h->st_R);
+    {
+        std::lock_guard<std::mutex> lk(g_rot_mu);
+        auto it = g_rot_cache.find(key);
+        if (it != g_rot_cache.end()) return it->second;
+    }
+    const int p = h->p, nv = h->nV;
+    auto img = std::make_shared<RotImage>();
+    img->angle.assign((size_t)nv, 0);
+    img->vec.assign((size_t)nv * ROT_VS, 0.0);
+    std::map<std::pair<int, int>, int> angles;  // (u_z, u_x^2 + u_y^2)
+    std::vector<double> beta;
+    const int ne = h->st_off[8];
+    for (int e = 0; e < ne; e++) {
+        const int *v = &h->st_host[4 * (size_t)e];
+        const int id = v[3] & 0xffff;
+        // u = c_L - c_M = -(source - target)
+        const double u[3] = {-(double)v[0], -(double)v[1], -(double)v[2]};
+        const double rxy = std::hypot(u[0], u[1]), a = rxy > 0 ? std::atan2(u[1], u[0]) : 0.0;
+        auto it = angles.emplace(std::make_pair(-v[2], v[0] * v[0] + v[1] * v[1]), (int)beta.size());
+        if (it.second) beta.push_back(std::atan2(rxy, u[2]));
+        img->angle[(size_t)id] = it.first->second;
+        double *o = img->vec.data() + (size_t)id * ROT_VS;
+        for (int m = 0; m < p; m++) {
+            const double co = std::cos(m * a), si = std::sin(m * a);
+            o[2 * m] = co;
+            o[2 * m + 1] = -si;
+            o[ROT_PH + 2 * m] = si;
+            o[ROT_PH + 2 * m + 1] = co;
+        }
+        const double d = std::sqrt(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+        double g = 1.0 / d;
+        for (int l = 0; l < 2 * p - 1; l++) {
+            if (l) g *= (double)l / d;
+            for (int k = 0; k <= std::min(l, 3); k++) o[2 * ROT_PH + k * ROT_G + l - k] = g;
+        }
+    }
+    img->na = (int)beta.size();
+    size_t per = 0;
+    for (int K = 1; K <= p; K++) per += (size_t)K * K + (K < p ? (size_t)K * K : 0);
+    img->maps.assign((size_t)img->na * per, 0.0);
+    host_parallel(img->na, [&](int i) {
+        const auto V = vmaps(p, beta[(size_t)i]);
+        double *o = img->maps.data() + (size_t)i * per;
+        for (int part = 0; part < 2; part++)
+            for (int K = 1; K <= p - part; K++) {
+                const int n = part ? K : K - 1, S = 2 * n + 1;
+                for (int m = part; m <= n; m++)
+                    for (int mp = part; mp <= n; mp++) {
+                        const double s = ((m & 1) ? -1.0 : 1.0) * V[n][(size_t)(n - m) * S + n + mp];
+                        const double t = V[n][(size_t)(n + m) * S + n + mp];
+                        *o++ = (part ? t - s : t + s) / std::sqrt(fact(n + mp) * fact(n - mp));
+                    }
+            }
+    });
     std::lock_guard<std::mutex> lk(g_rot_mu);
     g_rot_cache[key] = img;
     return img;
 }
 
-void rotation_tables_update(fmm_ctx *h, bool fp64)
+// device copy: maps (padded rows), vectors, c per coefficient pair and (halved
+// for order 0) per coefficient, angle indices
+template <class T>
+static void rotation_tables_update(fmm_ctx *h, const RotPlan &P)
 {
-    const int want = fp64 ? 2 : 1;
+    const int want = sizeof(T) == 8 ? 2 : 1;
     if (h->rot_nv == h->nV && h->rot_kind == want && h->rot_tab.p) return;
     auto img = rot_image(h);
-    if (fp64) {
-        h->rot_tab.ensure(sizeof(double) * img->size());
-        FMM_CUDA_TRY(cudaMemcpy(h->rot_tab.p, img->data(), sizeof(double) * img->size(), cudaMemcpyHostToDevice));
-    } else {
-        std::vector<float> f(img->size());
-        for (size_t i = 0; i < f.size(); i++) f[i] = (float)(*img)[i];
-        h->rot_tab.ensure(sizeof(float) * f.size());
-        FMM_CUDA_TRY(cudaMemcpy(h->rot_tab.p, f.data(), sizeof(float) * f.size(), cudaMemcpyHostToDevice));
-    }
+    const int p = h->p;
+    std::vector<T> buf((size_t)img->na * P.ds + (size_t)h->nV * ROT_VS + ROT_MAXP * (ROT_MAXP + 1) / 2 + ROT_MAXP * ROT_MAXP, T(0));
+    const double *in = img->maps.data();
+    for (int i = 0; i < img->na; i++)
+        for (int part = 0; part < 2; part++)
+            for (int K = 1; K <= p - part; K++) {
+                T *o = buf.data() + (size_t)i * P.ds + P.off[part][K];
+                for (int r = 0; r < K; r++)
+                    for (int c = 0; c < K; c++) o[r * rot_pad<T>(K) + c] = (T)*in++;
+            }
+    h->rot_vec_off = (size_t)img->na * P.ds;
+    for (size_t i = 0; i < img->vec.size(); i++) buf[h->rot_vec_off + i] = (T)img->vec[i];
+    h->rot_c_off = h->rot_vec_off + img->vec.size();
+    for (int n = 0, q = 0; n < p; n++)
+        for (int m = 0; m <= n; m++, q++) {
+            const T c = (T)std::sqrt(fact(n + m) * fact(n - m));
+            buf[h->rot_c_off + q] = c;
+            T *ck = buf.data() + h->rot_c_off + ROT_MAXP * (ROT_MAXP + 1) / 2;
+            ck[rot_idx(n, 0, m)] = m ? c : T(0.5) * c;
+            if (m) ck[rot_idx(n, 1, m - 1)] = c;
+        }
+    h->rot_tab.ensure(sizeof(T) * buf.size());
+    FMM_CUDA_TRY(cudaMemcpy(h->rot_tab.p, buf.data(), sizeof(T) * buf.size(), cudaMemcpyHostToDevice));
+    h->rot_angle.ensure(sizeof(int) * img->angle.size());
+    FMM_CUDA_TRY(cudaMemcpy(h->rot_angle.p, img->angle.data(), sizeof(int) * img->angle.size(), cudaMemcpyHostToDevice));
     h->rot_nv = h->nV;
     h->rot_kind = want;
 }
 
-// 16-byte vectors of T and their dot product
+// sum of one coefficient over the vectors: FP64, or an FP32 TwoSum pair
 template <class T>
-struct V16;
+struct RotSum;
 template <>
-struct V16<float> {
-    using type = float4;
-    static constexpr int n = 4;
-    static __device__ __forceinline__ float dot(float4 a, float4 b, float s)
+struct RotSum<double> {
+    double s;
+    __device__ __forceinline__ void zero() { s = 0.0; }
+    __device__ __forceinline__ void add(double v) { s += v; }
+    __device__ __forceinline__ double get() const { return s; }
+    using part = double;
+    __device__ __forceinline__ double pack() const { return s; }
+    __device__ __forceinline__ void merge(double v) { s += v; }
+};
+template <>
+struct RotSum<float> {
+    float hi, lo;
+    __device__ __forceinline__ void zero() { hi = lo = 0.f; }
+    __device__ __forceinline__ void add(float v)
     {
-        return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, s))));
+        const float s = hi + v, b = s - hi;
+        lo += (hi - (s - b)) + (v - b);
+        hi = s;
+    }
+    __device__ __forceinline__ float get() const { return hi + lo; }
+    using part = float2;
+    __device__ __forceinline__ float2 pack() const { return make_float2(hi, lo); }
+    __device__ __forceinline__ void merge(float2 v)
+    {
+        add(v.x);
+        lo += v.y;
     }
 };
+
+// Runs of 16 bytes of T against scalars and runs: FP32 as packed pairs (one
+// instruction for two multiply-adds, and half the issue slots).
+template <class T>
+struct RotPk;
 template <>
-struct V16<double> {
-    using type = double2;
-    static constexpr int n = 2;
-    static __device__ __forceinline__ double dot(double2 a, double2 b, double s) { return fma(a.y, b.y, fma(a.x, b.x, s)); }
+struct RotPk<float> {
+    using type = unsigned long long;
+    static constexpr int n = 2;  // values per register pair
+    static __device__ __forceinline__ type dup(float a)
+    {
+        type d;
+        asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(a));
+        return d;
+    }
+    static __device__ __forceinline__ type make(float a, float b)
+    {
+        type d;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+        return d;
+    }
+    static __device__ __forceinline__ void get(type v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+    static __device__ __forceinline__ void mad(type &acc, type a, type b)
+    {
+        asm("fma.rn.ftz.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+    }
 };
 
-template <class T>
-struct RotCfg {
-    static constexpr int W = 8;  // warps per CTA, two target cells each
-    static constexpr int MINB = sizeof(T) == 4 ? 2 : 1;  // CTAs per SM the registers are sized for
-    static constexpr int NK = 8;                       // packed outputs per lane: p^2 <= 256
-    static constexpr int NL = 10;                      // padded entries per lane: sum K4 <= 320
-};
-
-// One CTA per tile of up to 2W target cells, two per warp. For each stencil
-// vector of the tile's set (the prefix that can reach the level), the CTA
-// stages the vector's maps and z factors in shared memory; each warp loads
-// the M~ of its two cells' sources at that offset (zero where there is none),
-// rotates them (lane i: packed output i, 16-byte dot products over its
-// degree's padded row, one map entry for both cells), translates along z
-// (sums over j of equal order), rotates back and adds into FP64 registers.
-// The cells' L~ is written once at the end.
-template <class T>
-__global__ void __launch_bounds__(32 * RotCfg<T>::W, RotCfg<T>::MINB) m2l_rot_k(int p, const M2LTile *__restrict__ tiles,
-                                                             const int *__restrict__ ntiles, const int *__restrict__ tgt,
-                                                             const int4 *__restrict__ xyz, const uint64_t *__restrict__ anchor,
-                                                             const LevelDesc *__restrict__ ld, const int *__restrict__ map_pool,
-                                                             const int4 *__restrict__ st, const int *__restrict__ st_off,
-                                                             const T *__restrict__ rot, int VS, int SA, int PP4,
-                                                             const T *__restrict__ M, T *__restrict__ L)
+// forward: outputs in registers, one input (with its phase) and one map row at
+// a time; from the gathered rows r to x
+template <class T, int NC>
+__device__ __forceinline__ void rot_forward(const T *r, T *x, const T *ph, const T *map, int K, int n, int part)
 {
-    using C = RotCfg<T>;
-    using VT = typename V16<T>::type;
-    constexpr int VN = V16<T>::n;
-    if ((int)blockIdx.x >= *ntiles) return;
-    const M2LTile td = tiles[blockIdx.x];
-    const int PP = p * p;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *sTab = reinterpret_cast<T *>(smem_raw);
-    const T *sA = sTab, *sB = sTab + SA, *sg = sTab + 2 * SA;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    T *sM[2], *sP[2];
-    sM[0] = sTab + VS + (size_t)warp * 4 * PP4;
-    sM[1] = sM[0] + PP4;
-    sP[0] = sM[0] + 2 * PP4;
-    sP[1] = sM[0] + 3 * PP4;
-    // the warp's two cells
-    int cell[2], rl[2], px[2], py[2], pz[2], ro[2];
+    const T *re = r + (n * n + part) * ROT_LD, *im = r + rot_idx(n, 1, part - 1) * ROT_LD;
+    // order 0 has no imaginary part: its sine is 0, and the value read in its
+    // place is the degree's last real one
+    const T *pp = ph + part * (ROT_PH + 2);
+    T *out = x + rot_idx(n, part, 0) * ROT_LD;
+    if constexpr (sizeof(T) == 4) {
+        using P = RotPk<float>;
+        unsigned long long o[2 * NC];
 #pragma unroll
-    for (int r = 0; r < 2; r++) {
-        cell[r] = -1;
-        rl[r] = td.level;
-        px[r] = py[r] = pz[r] = ro[r] = 0;
-        if (2 * warp + r < td.count) {
-            cell[r] = tgt[td.start + 2 * warp + r];
-            const int4 a = xyz[cell[r]];
-            rl[r] = a.w;
-            const int sh = FMM_MAXLEVEL - a.w;
-            px[r] = a.x >> sh;
-            py[r] = a.y >> sh;
-            pz[r] = a.z >> sh;
-            ro[r] = (px[r] & 1) | ((py[r] & 1) << 1) | ((pz[r] & 1) << 2);
-        }
-    }
-    // this lane's packed outputs i = lane + 32 k: degree n, index a in the
-    // degree, position of the entry in the padded layout and of its map rows
-    int on[C::NK], oa[C::NK], opos[C::NK], orow[C::NK];
+        for (int j = 0; j < 2 * NC; j++) o[j] = 0ull;
+        const ulonglong2 *row = reinterpret_cast<const ulonglong2 *>(map);
+#pragma unroll 2
+        for (int i = 0; i < K; i++, row += NC, re += ROT_LD, im += ROT_LD, pp += 2) {
+            const float2 w = *reinterpret_cast<const float2 *>(pp);
+            const unsigned long long a = P::dup(*re * w.x + *im * w.y);
 #pragma unroll
-    for (int k = 0; k < C::NK; k++) {
-        const int i = lane + 32 * k;
-        int n = 0, pos = 0, row = 0;
-        while ((n + 1) * (n + 1) <= i) {
-            const int K4 = (2 * n + 1 + 3) & ~3;
-            pos += K4;
-            row += (2 * n + 1) * K4;
-            n++;
-        }
-        on[k] = i < PP ? n : -1;
-        oa[k] = i - n * n;
-        opos[k] = pos + oa[k];
-        orow[k] = row + oa[k] * ((2 * n + 1 + 3) & ~3);
-    }
-    // this lane's padded entries j = lane + 32 t: source index in the packed M~ (-1: padding)
-    int lsrc[C::NL];
-#pragma unroll
-    for (int t = 0; t < C::NL; t++) {
-        const int j = lane + 32 * t;
-        int n = 0, pos = 0;
-        while (n < p && pos + ((2 * n + 1 + 3) & ~3) <= j) {
-            pos += (2 * n + 1 + 3) & ~3;
-            n++;
-        }
-        lsrc[t] = (j < PP4 && j - pos < 2 * n + 1) ? n * n + (j - pos) : -1;
-    }
-    for (int j = lane; j < PP4; j += 32) sP[0][j] = sP[1][j] = T(0);
-    double acc[2][C::NK];
-#pragma unroll
-    for (int k = 0; k < C::NK; k++) acc[0][k] = acc[1][k] = 0.0;
-
-    const int e0 = st_off[td.octant], nvec = st_off[10 + td.octant * (FMM_MAXLEVEL + 1) + td.level];
-    for (int e = e0; e < e0 + nvec; e++) {
-        const int4 v = st[e];
-        __syncthreads();
-        {
-            const VT *src = reinterpret_cast<const VT *>(rot + (size_t)(v.w & 0xffff) * VS);
-            VT *dst = reinterpret_cast<VT *>(sTab);
-            for (int i = threadIdx.x; i < VS / VN; i += blockDim.x) dst[i] = src[i];
-        }
-        __syncthreads();
-        int b[2];
-#pragma unroll
-        for (int r = 0; r < 2; r++) {
-            b[r] = -1;
-            if (cell[r] >= 0 && ((v.w >> (16 + ro[r])) & 1))
-                b[r] = level_lookup(ld[rl[r]], map_pool, anchor, rl[r], px[r] + v.x, py[r] + v.y, pz[r] + v.z);
-        }
-        if (b[0] < 0 && b[1] < 0) continue;  // warp-uniform
-#pragma unroll
-        for (int r = 0; r < 2; r++)
-#pragma unroll
-            for (int t = 0; t < C::NL; t++) {
-                const int j = lane + 32 * t;
-                if (j < PP4) sM[r][j] = (b[r] >= 0 && lsrc[t] >= 0) ? M[(size_t)b[r] * PP + lsrc[t]] : T(0);
+            for (int c = 0; c < NC; c++) {
+                const ulonglong2 d = row[c];
+                P::mad(o[2 * c], d.x, a);
+                P::mad(o[2 * c + 1], d.y, a);
             }
-        __syncwarp();
-        // multipoles into the rotated frame
-#pragma unroll
-        for (int k = 0; k < C::NK; k++) {
-            if (on[k] < 0) continue;
-            const int n = on[k], K4 = (2 * n + 1 + 3) & ~3, base = opos[k] - oa[k];
-            const VT *ar = reinterpret_cast<const VT *>(sA + orow[k]);
-            const VT *m0 = reinterpret_cast<const VT *>(sM[0] + base), *m1 = reinterpret_cast<const VT *>(sM[1] + base);
-            T s0 = 0, s1 = 0;
-            for (int c = 0; c < K4 / VN; c++) {
-                const VT w = ar[c];
-                s0 = V16<T>::dot(w, m0[c], s0);
-                s1 = V16<T>::dot(w, m1[c], s1);
-            }
-            sP[0][opos[k]] = s0;
-            sP[1][opos[k]] = s1;
         }
-        __syncwarp();
-        // translation along z: only equal orders couple
 #pragma unroll
-        for (int k = 0; k < C::NK; k++) {
-            if (on[k] < 0) continue;
-            const int n = on[k], a = oa[k], m = (a + 1) >> 1;
-            int pj = 0;
-            for (int j = 0; j < m; j++) pj += (2 * j + 1 + 3) & ~3;
-            T s0 = 0, s1 = 0;
-            for (int j = m; j < p; j++) {
-                const T g = sg[j + n];
-                s0 += sP[0][pj + a] * g;
-                s1 += sP[1][pj + a] * g;
-                pj += (2 * j + 1 + 3) & ~3;
-            }
-            const bool neg = (((n + m) & 1) != 0) != (a > 0 && !(a & 1));
-            sM[0][opos[k]] = neg ? -s0 : s0;
-            sM[1][opos[k]] = neg ? -s1 : s1;
+        for (int c = 0; c < 2 * NC; c++) {
+            float a, b;
+            P::get(o[c], a, b);
+            if (2 * c < 4 * NC - 3 || 2 * c < K) out[2 * c * ROT_LD] = a;
+            if (2 * c + 1 < 4 * NC - 3 || 2 * c + 1 < K) out[(2 * c + 1) * ROT_LD] = b;
         }
-        __syncwarp();
-        // locals back to the original frame
+    } else {
+        T o[2 * NC];
 #pragma unroll
-        for (int k = 0; k < C::NK; k++) {
-            if (on[k] < 0) continue;
-            const int n = on[k], K4 = (2 * n + 1 + 3) & ~3, base = opos[k] - oa[k];
-            const VT *br = reinterpret_cast<const VT *>(sB + orow[k]);
-            const VT *l0 = reinterpret_cast<const VT *>(sM[0] + base), *l1 = reinterpret_cast<const VT *>(sM[1] + base);
-            T s0 = 0, s1 = 0;
-            for (int c = 0; c < K4 / VN; c++) {
-                const VT w = br[c];
-                s0 = V16<T>::dot(w, l0[c], s0);
-                s1 = V16<T>::dot(w, l1[c], s1);
+        for (int j = 0; j < 2 * NC; j++) o[j] = T(0);
+        const double2 *row = reinterpret_cast<const double2 *>(map);
+#pragma unroll 2
+        for (int i = 0; i < K; i++, row += NC, re += ROT_LD, im += ROT_LD, pp += 2) {
+            const double2 w = *reinterpret_cast<const double2 *>(pp);
+            const T a = *re * w.x + *im * w.y;
+#pragma unroll
+            for (int c = 0; c < NC; c++) {
+                const double2 d = row[c];
+                o[2 * c] += d.x * a;
+                if (c < NC - 1 || 2 * NC == K) o[2 * c + 1] += d.y * a;
             }
-            acc[0][k] += s0;
-            acc[1][k] += s1;
         }
-        __syncwarp();
-    }
 #pragma unroll
-    for (int r = 0; r < 2; r++) {
-        if (cell[r] < 0) continue;
-#pragma unroll
-        for (int k = 0; k < C::NK; k++)
-            if (on[k] >= 0) L[(size_t)cell[r] * PP + lane + 32 * k] += (T)acc[r][k];
+        for (int j = 0; j < 2 * NC; j++)
+            if (j < 2 * NC - 1 || j < K) out[j * ROT_LD] = o[j];
     }
 }
 
+// back: inputs in registers, one output at a time
+template <class T, int NC>
+__device__ __forceinline__ void rot_back(T *x, const T *map, int K, int n, int part)
+{
+    T *v = x + rot_idx(n, part, 0) * ROT_LD;
+    if constexpr (sizeof(T) == 4) {
+        using P = RotPk<float>;
+        unsigned long long r[2 * NC];
+#pragma unroll
+        for (int c = 0; c < 2 * NC; c++)
+            r[c] = P::make(2 * c < 4 * NC - 3 || 2 * c < K ? v[2 * c * ROT_LD] : 0.f,
+                           2 * c + 1 < 4 * NC - 3 || 2 * c + 1 < K ? v[(2 * c + 1) * ROT_LD] : 0.f);
+        const ulonglong2 *row = reinterpret_cast<const ulonglong2 *>(map);
+#pragma unroll 2
+        for (int i = 0; i < K; i++, row += NC, v += ROT_LD) {
+            unsigned long long s0 = 0ull, s1 = 0ull;
+#pragma unroll
+            for (int c = 0; c < NC; c++) {
+                const ulonglong2 d = row[c];
+                P::mad(s0, d.x, r[2 * c]);
+                P::mad(s1, d.y, r[2 * c + 1]);
+            }
+            float a, b, c, d;
+            P::get(s0, a, b);
+            P::get(s1, c, d);
+            *v = (a + b) + (c + d);
+        }
+    } else {
+        T r[2 * NC];
+#pragma unroll
+        for (int j = 0; j < 2 * NC; j++) r[j] = j < 2 * NC - 1 || j < K ? v[j * ROT_LD] : T(0);
+        const double2 *row = reinterpret_cast<const double2 *>(map);
+#pragma unroll 2
+        for (int i = 0; i < K; i++, row += NC, v += ROT_LD) {
+            T s0 = 0, s1 = 0;
+#pragma unroll
+            for (int c = 0; c < NC; c++) {
+                const double2 d = row[c];
+                s0 += d.x * r[2 * c];
+                if (c < NC - 1 || 2 * NC == K) s1 += d.y * r[2 * c + 1];
+            }
+            *v = s0 + s1;
+        }
+    }
+}
+
+// along z: order m = p - K, out_n = +-sum_j g_{j+n} in_j over the degrees m .. p-1
+// (order m of degree n is entry m - part of its part)
+template <class T, int NC>
+__device__ __forceinline__ void rot_along(T *x, const T *g, int K, int m, int part)
+{
+    constexpr int VN = RotVec<T>::n;
+    // rot_idx(n, part, m - part): steps of 2 n + 1 + part from degree to degree
+    T *const x0 = x + rot_idx(m, part, m - part) * ROT_LD;
+    const int d0 = (2 * m + 1 + part) * ROT_LD;
+    const T sg = (part ? T(-1) : T(1)) * (m == 0 ? T(0.5) : T(1));  // and alternating with the degree
+    T r[NC * VN];
+    {
+        const T *v = x0;
+        int d = d0;
+#pragma unroll
+        for (int j = 0; j < NC * VN; j++) {
+            r[j] = j < (NC - 1) * VN + 1 || j < K ? *v : T(0);
+            if (j + 1 < (NC - 1) * VN + 1 || j + 1 < K) v += d;
+            d += 2 * ROT_LD;
+        }
+    }
+    T *v = x0;
+    int d = d0;
+    if constexpr (sizeof(T) == 4) {
+        using P = RotPk<float>;
+        unsigned long long rp[2 * NC];
+#pragma unroll
+        for (int c = 0; c < 2 * NC; c++) rp[c] = P::make(r[2 * c], r[2 * c + 1]);
+        // windows of factors for outputs nn .. nn + 3: from g_{2m + nn}, and from
+        // the next one for the odd outputs
+        const int sh = 2 * (m & 1);
+        const ulonglong2 *wa = reinterpret_cast<const ulonglong2 *>(g + sh * ROT_G + 2 * m - sh);
+        const ulonglong2 *wb = reinterpret_cast<const ulonglong2 *>(g + (sh + 1) * ROT_G + 2 * m - sh);
+        for (int nn = 0; nn < K; nn += 4, wa++, wb++) {
+            unsigned long long a[2 * NC + 2], b[2 * NC + 2];
+#pragma unroll
+            for (int c = 0; c <= NC; c++) {
+                const ulonglong2 u = wa[c], w = wb[c];
+                a[2 * c] = u.x;
+                a[2 * c + 1] = u.y;
+                b[2 * c] = w.x;
+                b[2 * c + 1] = w.y;
+            }
+            unsigned long long s[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+            for (int c = 0; c < 2 * NC; c++) {
+                P::mad(s[0], a[c], rp[c]);
+                P::mad(s[1], b[c], rp[c]);
+                P::mad(s[2], a[c + 1], rp[c]);
+                P::mad(s[3], b[c + 1], rp[c]);
+            }
+#pragma unroll
+            for (int o = 0; o < 4; o++) {
+                float lo, hi;
+                P::get(s[o], lo, hi);
+                if (nn + o < K) *v = (lo + hi) * (o & 1 ? -sg : sg);
+                v += d;
+                d += 2 * ROT_LD;
+            }
+        }
+    } else {
+        const double2 *w = reinterpret_cast<const double2 *>(g + 2 * m);
+        for (int nn = 0; nn < K; nn += 2, w++) {
+            T gw[2 * NC + 2];
+#pragma unroll
+            for (int c = 0; c <= NC; c++) {
+                const double2 u = w[c];
+                gw[2 * c] = u.x;
+                gw[2 * c + 1] = u.y;
+            }
+            T s[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int c = 0; c < NC; c++) {
+                s[0] += gw[2 * c] * r[2 * c];
+                s[1] += gw[2 * c + 1] * r[2 * c];
+                if (c < NC - 1 || 2 * NC == K) {
+                    s[2] += gw[2 * c + 1] * r[2 * c + 1];
+                    s[3] += gw[2 * c + 2] * r[2 * c + 1];
+                }
+            }
+#pragma unroll
+            for (int o = 0; o < 2; o++) {
+                if (nn + o < K) *v = (s[o] + s[o + 2]) * (o ? -sg : sg);
+                v += d;
+                d += 2 * ROT_LD;
+            }
+        }
+    }
+}
+
+#define ROT_CASES(NCV, CALL)          \
+    switch (NCV) {                    \
+    case 1: CALL(1); break;           \
+    case 2: CALL(2); break;           \
+    case 3: CALL(3); break;           \
+    case 4: CALL(4); break;           \
+    default:                          \
+        if constexpr (NCMAX > 4) {    \
+            switch (NCV) {            \
+            case 5: CALL(5); break;   \
+            case 6: CALL(6); break;   \
+            case 7: CALL(7); break;   \
+            default: CALL(8); break;  \
+            }                         \
+        }                             \
+    }
+
+struct RotJob {
+    const M2LTile *tiles;
+    const int *ntiles, *tgt;
+    const int4 *xyz;
+    const uint64_t *anchor;
+    const LevelDesc *ld;
+    const int *map_pool;
+    const int4 *st;
+    const int *st_off;
+    const int *angle;
+    unsigned *tcnt;
+    void *part;
+    int nsplit, chunk;
+};
+
+// c M~ of the cells from level 2 on (halved for order 0, as the forward maps
+// take it), in the kernel's coefficient order
+template <class T>
+__global__ void __launch_bounds__(256) rot_scale_k(const T *__restrict__ M, int PP, int c0, int nc, const T *__restrict__ ck,
+                                                   T *__restrict__ CM)
+{
+    const int64_t i = (int64_t)c0 * PP + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)nc * PP) return;
+    const int k = (int)(i % PP);
+    int n = 0;
+    while ((n + 1) * (n + 1) <= k) n++;
+    const int j = k - n * n;  // Re 0, then Re and Im of 1 .. n
+    const int o = rot_idx(n, j && !(j & 1), j & 1 ? (j + 1) / 2 : j ? j / 2 - 1 : 0);
+    CM[i - k + o] = M[i] * ck[o];
+}
+
+// W warps, NQ >= p (p + 1) / 2 / W coefficient pairs per warp
+template <class T, int W, int NQ>
+__global__ void __launch_bounds__(32 * W, W == 8 ? 2 : NQ > 9 ? 3 : 4)
+    m2l_rot_k(int p, const __grid_constant__ RotJob J, const __grid_constant__ RotPlan P, const T *__restrict__ maps,
+              const T *__restrict__ vecs, const T *__restrict__ cfac, const T *__restrict__ CM, T *__restrict__ L)
+{
+    using S = RotSum<T>;
+    using V = typename RotVec<T>::type;
+    constexpr int VN = RotVec<T>::n, NCMAX = ROT_MAXP / VN;
+    if ((int)blockIdx.x >= *J.ntiles * J.nsplit) return;
+    const int tile = (int)blockIdx.x / J.nsplit, split = (int)blockIdx.x - tile * J.nsplit;
+    const M2LTile td = J.tiles[tile];
+    const int PP = p * p, npair = p * (p + 1) / 2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    // two buffers of a vector's phases and factors and its maps, then the
+    // gathered rows and the coefficients in work
+    T *const sv = reinterpret_cast<T *>(smem_raw);
+    const int vstep = ROT_VS + P.ds;
+    T *const sr = sv + 2 * vstep, *const sx = sr + (size_t)PP * ROT_LD;
+    __shared__ int s_last;
+    __shared__ int4 s_pair[W * NQ];  // coefficient pair -> rows of its parts, 2 m
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    T *x = sx + lane;
+    int cell = -1, rl = td.level, px = 0, py = 0, pz = 0, ro = 0;
+    if (lane < td.count) {
+        cell = J.tgt[td.start + lane];
+        const int4 a = J.xyz[cell];
+        rl = a.w;
+        const int sh = FMM_MAXLEVEL - rl;
+        px = a.x >> sh;
+        py = a.y >> sh;
+        pz = a.z >> sh;
+        ro = (px & 1) | ((py & 1) << 1) | ((pz & 1) << 2);
+    }
+    for (int q = threadIdx.x; q < npair; q += 32 * W) {
+        const int n = P.nm[q][0], m = P.nm[q][1];
+        s_pair[q] = make_int4(rot_idx(n, 0, m) * ROT_LD, rot_idx(n, m ? 1 : 0, m ? m - 1 : 0) * ROT_LD, 2 * m, 0);
+    }
+    const LevelDesc LD = J.ld[rl];
+    const bool whole = rl <= 10 && LD.end - LD.start == (1 << (3 * rl));  // every lattice cell present
+    S acc[2 * NQ];
+#pragma unroll
+    for (int k = 0; k < 2 * NQ; k++) acc[k].zero();
+    // the set's entries are sorted by reach: only a prefix can hit a cell;
+    // this CTA's range of it
+    const int nvt = J.st_off[10 + td.octant * (FMM_MAXLEVEL + 1) + td.level];
+    // (ranges of a fixed length: a cell's sums do not depend on its tile's list)
+    int e = J.st_off[td.octant] + min(nvt, split * J.chunk);
+    const int e1 = J.st_off[td.octant] + min(nvt, (split + 1) * J.chunk);
+
+    // next entry from e on that hits a cell of some lane (every warp finds the
+    // same), with this lane's source cell
+    auto advance = [&](int &id, int &src) {
+        for (; e < e1; e++) {
+            const int4 v = J.st[e];
+            int b = -1;
+            if (cell >= 0 && ((v.w >> (16 + ro)) & 1)) {
+                const int qx = px + v.x, qy = py + v.y, qz = pz + v.z;
+                const unsigned side = 1u << rl;
+                if ((unsigned)qx < side && (unsigned)qy < side && (unsigned)qz < side)
+                    b = whole ? LD.start + (int)morton3_10((uint32_t)qx, (uint32_t)qy, (uint32_t)qz)
+                              : level_lookup(LD, J.map_pool, J.anchor, rl, qx, qy, qz);
+            }
+            if (__any_sync(0xffffffffu, b >= 0)) {
+                id = v.w & 0xffff;
+                src = b;
+                e++;
+                return true;
+            }
+        }
+        return false;
+    };
+    auto fetch = [&](int id, int buf) {
+        const V *gv = reinterpret_cast<const V *>(vecs + (size_t)id * ROT_VS);
+        const V *gm = reinterpret_cast<const V *>(maps + (size_t)J.angle[id] * P.ds);
+        for (int i = threadIdx.x; i < ROT_VS / VN; i += 32 * W) cp_async16(smem_u32(sv + buf * vstep + i * VN), gv + i, 16);
+        for (int i = threadIdx.x; i < P.ds / VN; i += 32 * W) cp_async16(smem_u32(sv + buf * vstep + ROT_VS + i * VN), gm + i, 16);
+    };
+    auto gather = [&](int src) {
+#pragma unroll 2
+        for (int r = warp; r < ROT_ROWS; r += W) {
+            const int b = __shfl_sync(0xffffffffu, src, r);
+            const T *row = CM + (size_t)(b >= 0 ? b : 0) * PP;
+            for (int j = lane; j < PP; j += 32) cp_async_n<sizeof(T)>(smem_u32(sr + j * ROT_LD + r), row + j, b >= 0);
+        }
+    };
+
+    int id = 0, src = -1, buf = 0;
+    bool have = advance(id, src);
+    if (have) {
+        fetch(id, 0);
+        gather(src);
+    }
+    while (have) {
+        have = advance(id, src);
+        cp_async_wait_all();
+        __syncthreads();  // the vector's data is here, and no warp reads the other buffer any more
+        const T *ph = sv + buf * vstep, *g = ph + 2 * ROT_PH, *mp = ph + ROT_VS;
+        for (int j = 0; j < P.njob[warp]; j++) {
+            const int K = P.job[warp][j] & 127, part = P.job[warp][j] >> 7, n = part ? K : K - 1;
+#define ROT_CALL(NC) rot_forward<T, NC>(sr + lane, x, ph, mp + P.off[part][K], K, n, part)
+            ROT_CASES((K + VN - 1) / VN, ROT_CALL)
+#undef ROT_CALL
+        }
+        __syncthreads();
+        if (have) {  // the gathered rows are used up
+            fetch(id, buf ^ 1);
+            gather(src);
+        }
+        for (int j = 0; j < P.njob[warp]; j++) {
+            const int K = P.job[warp][j] & 127, part = P.job[warp][j] >> 7;
+#define ROT_CALL(NC) rot_along<T, NC>(x, g, K, p - K, part)
+            ROT_CASES((K + VN - 1) / VN, ROT_CALL)
+#undef ROT_CALL
+        }
+        __syncthreads();
+        for (int j = 0; j < P.njob[warp]; j++) {
+            const int K = P.job[warp][j] & 127, part = P.job[warp][j] >> 7, n = part ? K : K - 1;
+#define ROT_CALL(NC) rot_back<T, NC>(x, mp + P.off[part][K], K, n, part)
+            ROT_CASES((K + VN - 1) / VN, ROT_CALL)
+#undef ROT_CALL
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < NQ; k++) {
+            const int q = min(warp + W * k, npair - 1);  // (a clamped pair's sums are not used)
+            const int4 s = s_pair[q];
+            const T yr = x[s.x], yi = x[s.y], si = ph[ROT_PH + s.z], co = ph[ROT_PH + s.z + 1];
+            acc[2 * k].add(yr * co - yi * si);
+            acc[2 * k + 1].add(yr * si + yi * co);  // m = 0: not used
+        }
+        buf ^= 1;
+    }
+    auto put = [&](int q, const S &re, const S &im) {
+        if (cell < 0) return;
+        const int n = P.nm[q][0], m = P.nm[q][1];
+        T *Lc = L + (size_t)cell * PP;
+        Lc[re_idx(n, m)] += re.get() * cfac[q];
+        if (m) Lc[im_idx(n, m)] += im.get() * cfac[q];
+    };
+    if (J.nsplit == 1) {
+#pragma unroll
+        for (int k = 0; k < NQ; k++)
+            if (warp + W * k < npair) put(warp + W * k, acc[2 * k], acc[2 * k + 1]);
+        return;
+    }
+    // the range's sums, [item][pair][re, im][lane]; the tile's last range to
+    // finish adds them all in order
+    using Pt = typename S::part;
+    Pt *part = static_cast<Pt *>(J.part);
+    const size_t rng = (size_t)npair * 2 * ROT_ROWS;
+    Pt *mine = part + (size_t)blockIdx.x * rng + lane;
+#pragma unroll
+    for (int k = 0; k < NQ; k++) {
+        const int q = warp + W * k;
+        if (q >= npair) break;
+        __stcg(&mine[(size_t)(2 * q) * ROT_ROWS], acc[2 * k].pack());
+        __stcg(&mine[(size_t)(2 * q + 1) * ROT_ROWS], acc[2 * k + 1].pack());
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_last = atomicAdd(&J.tcnt[tile], 1u) == (unsigned)(J.nsplit - 1);
+        if (s_last) J.tcnt[tile] = 0u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
+    const Pt *first = part + (size_t)tile * J.nsplit * rng + lane;
+    for (int q = warp; q < npair; q += W) {
+        S re, im;
+        re.zero();
+        im.zero();
+#pragma unroll 4
+        for (int r = 0; r < J.nsplit; r++) {
+            re.merge(__ldcg(&first[(size_t)r * rng + (size_t)(2 * q) * ROT_ROWS]));
+            im.merge(__ldcg(&first[(size_t)r * rng + (size_t)(2 * q + 1) * ROT_ROWS]));
+        }
+        put(q, re, im);
+    }
+}
+
+// Ranges per tile: about 8 CTAs per SM, so that the tiles at the boundary of
+// the domain, which have fewer sources, even out, of 24 vectors or more.
+static int rot_nsplit(fmm_ctx *h, int nv)
+{
+    const int want = (8 * h->nsm + h->ntiles_max - 1) / std::max(h->ntiles_max, 1);
+    return std::max(1, std::min(want, std::min(nv / 24, 32)));
+}
+
+template <class T, int W, int NQ>
+static void launch_rot(fmm_ctx *h, T *L, const T *M)
+{
+    const int p = h->p;
+    const RotPlan P = rot_plan<T>(p, W);
+    rotation_tables_update<T>(h, P);
+    const int nv = m2l_longest_list(h);
+    RotJob j;
+    const int want = rot_nsplit(h, nv);
+    j.chunk = (nv + want - 1) / want;
+    j.nsplit = (nv + j.chunk - 1) / j.chunk;
+    h->m2l_ws.ensure(sizeof(unsigned) * (size_t)h->ntiles_max);
+    if (j.nsplit > 1) h->m2l_part.ensure(sizeof(double) * (size_t)h->ntiles_max * j.nsplit * p * (p + 1) * ROT_ROWS);
+    FMM_CUDA_TRY(cudaMemsetAsync(h->m2l_ws.p, 0, sizeof(unsigned) * (size_t)h->ntiles_max, h->work));
+    j.tiles = h->m2l_tiles.as<M2LTile>();
+    j.ntiles = reinterpret_cast<const int *>(h->m2l_misc.as<unsigned>() + 24 * (FMM_MAXLEVEL + 1));
+    j.tgt = h->m2l_tgt.as<int>();
+    j.xyz = h->c_xyz.as<int4>();
+    j.anchor = h->c_anchor.as<uint64_t>();
+    j.ld = h->lvl_desc.as<LevelDesc>();
+    j.map_pool = h->map_pool.as<int>();
+    j.st = h->st_dev.as<int4>();
+    j.st_off = stencil_offsets(h);
+    j.angle = h->rot_angle.as<int>();
+    j.tcnt = h->m2l_ws.as<unsigned>();
+    j.part = h->m2l_part.p;
+    const size_t smem = sizeof(T) * (2 * (size_t)p * p * ROT_LD + 2 * ((size_t)ROT_VS + P.ds));
+    ensure_smem((const void *)m2l_rot_k<T, W, NQ>, smem);
+    const T *tab = h->rot_tab.as<T>();
+    const int c0 = h->lvl_start[2], nc = h->ncells, PP = p * p;
+    h->rot_m.ensure(sizeof(T) * (size_t)nc * PP);
+    if (nc <= c0) return;
+    rot_scale_k<T><<<(unsigned)(((int64_t)(nc - c0) * PP + 255) / 256), 256, 0, h->work>>>(
+        M, PP, c0, nc, tab + h->rot_c_off + ROT_MAXP * (ROT_MAXP + 1) / 2, h->rot_m.as<T>());
+    count_launch(h);
+    m2l_rot_k<T, W, NQ><<<(unsigned)h->ntiles_max * j.nsplit, 32 * W, smem, h->work>>>(
+        p, j, P, tab, tab + h->rot_vec_off, tab + h->rot_c_off, h->rot_m.as<T>(), L);
+    count_launch(h);
+    check_launch("m2l rotation");
+}
+
+// Eight warps share the 136 coefficient pairs of p = 16; up to p = 10 four do
+// (the largest of the jobs is then no more than a warp's share of them).
 template <class T>
 void m2l_rotation(fmm_ctx *h, T *L, const T *M)
 {
-    using C = RotCfg<T>;
-    rotation_tables_update(h, sizeof(T) == 8);
-    const int p = h->p, VS = rot_vec_stride(p), SA = rot_blocks(p);
-    int PP4 = 0;
-    for (int n = 0; n < p; n++) PP4 += k4(n);
-    if (PP4 > 32 * C::NL) throw Error{FMM_EINVAL, "rotation M2L: p too large"};
-    const size_t smem = sizeof(T) * ((size_t)VS + (size_t)C::W * 4 * PP4);
-    ensure_smem((const void *)m2l_rot_k<T>, smem);
-    const int *ntiles = reinterpret_cast<const int *>(h->m2l_misc.as<unsigned>() + 24 * (FMM_MAXLEVEL + 1));
-    m2l_rot_k<T><<<h->ntiles_max, 32 * C::W, smem, h->work>>>(
-        p, h->m2l_tiles.as<M2LTile>(), ntiles, h->m2l_tgt.as<int>(), h->c_xyz.as<int4>(), h->c_anchor.as<uint64_t>(),
-        h->lvl_desc.as<LevelDesc>(), h->map_pool.as<int>(), h->st_dev.as<int4>(), stencil_offsets(h),
-        h->rot_tab.as<T>(), VS, SA, PP4, M, L);
-    count_launch(h);
-    check_launch("m2l rotation");
+    if (h->p <= 8) launch_rot<T, 4, 9>(h, L, M);
+    else if (h->p <= 10) launch_rot<T, 4, 14>(h, L, M);
+    else launch_rot<T, 8, 17>(h, L, M);
 }
 
 template void m2l_rotation<float>(fmm_ctx *, float *, const float *);
 template void m2l_rotation<double>(fmm_ctx *, double *, const double *);
 
-bool rotation_m2l_supported(fmm_ctx *h) { return h->p >= 1 && h->p <= 16; }
-int rotation_tile_rows(fmm_ctx *h) { return 2 * (h->precision == FMM_FP64 ? RotCfg<double>::W : RotCfg<float>::W); }
+bool rotation_m2l_supported(fmm_ctx *h) { return h->p >= 1 && h->p <= ROT_MAXP; }
+int rotation_tile_rows(fmm_ctx *) { return ROT_ROWS; }
 
 }  // namespace fmm
