@@ -212,6 +212,7 @@ __device__ __forceinline__ void bbox_block(const T *__restrict__ x, int64_t n, i
     if constexpr (sizeof(T) == 4) {
         // (no finite value encodes to 0xffffffff or to 0: the initial values mark "none seen")
         unsigned elo[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, ehi[3] = {0u, 0u, 0u};
+#pragma unroll 4
         for (int64_t i = i0; i < n; i += stride) {
 #pragma unroll
             for (int k = 0; k < 3; k++) {
@@ -410,8 +411,21 @@ __global__ void __launch_bounds__(256) rs_count_k(const uint64_t *__restrict__ k
         if (cnt[i]) atomicAdd(&ws->count[0][0] + i, cnt[i]);
 }
 
-// Each warp ranks its 32 R consecutive keys in R rounds of 32 (match_any on
-// the digit), so the rank of a key among equal digits follows input order;
+// the lanes whose 8-bit digit equals this lane's, by eight ballots (match_any
+// takes longer: 291 against 269 us for a sort of 10^6 keys)
+__device__ __forceinline__ unsigned digit_peers(unsigned d)
+{
+    unsigned m = 0xffffffffu;
+#pragma unroll
+    for (int b = 0; b < 8; b++) {
+        const unsigned v = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+        m &= ((d >> b) & 1u) ? v : ~v;
+    }
+    return m;
+}
+
+// Each warp ranks its 32 R consecutive keys in R rounds of 32 (the lanes of
+// equal digit by ballots), so the rank of a key among equal digits follows input order;
 // the tile is staged in shared memory in digit order and written out in runs.
 // Tiles are numbered in the order in which their blocks start, so a tile only
 // waits for tiles that are already running; every wait is bounded (ws->err).
@@ -451,7 +465,7 @@ __global__ void __launch_bounds__(RS_T) rs_pass_k(const uint64_t *__restrict__ k
 #pragma unroll
     for (int r = 0; r < R; r++) {
         const unsigned d = (unsigned)(k[r] >> shift) & 255u;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const unsigned peers = digit_peers(d);
         const unsigned c = wcnt[w * 256 + d];
         rank[r] = c + __popc(peers & lt);
         __syncwarp();
@@ -608,7 +622,7 @@ __global__ void __launch_bounds__(SMALL_T) sort_small_k(const T *__restrict__ x,
         for (int r = 0; r < SMALL_R; r++) {
             if (r >= R) break;
             const unsigned d = (unsigned)(k[r] >> shift) & 255u;
-            const unsigned peers = __match_any_sync(0xffffffffu, d);
+            const unsigned peers = digit_peers(d);
             const unsigned c = wcnt[w * 256 + d];
             rank[r] = c + __popc(peers & lt);
             __syncwarp();
@@ -675,7 +689,7 @@ int morton_sort_into(const void *x, int64_t n, int dt, uint64_t *keys, int *perm
     SortWs *w = static_cast<SortWs *>(ws);
     // blocks: enough loads in flight for the box, 4096 keys or more per block
     // for the counts (2,048 atomics per block)
-    const unsigned gb = (unsigned)std::min<int64_t>(nblocks(n, 256), (int64_t)nsm * 8);
+    const unsigned gb = (unsigned)std::min<int64_t>(nblocks(n, 1024), (int64_t)nsm * 8);
     const unsigned gk = (unsigned)std::min<int64_t>(nblocks(n, 2048), (int64_t)nsm * 6);
     if (f64) {
         bbox_k<double><<<gb, 256, 0, s>>>((const double *)x, n, box);
