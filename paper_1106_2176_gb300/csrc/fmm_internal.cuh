@@ -278,7 +278,7 @@ struct fmm_ctx {
     fmm::DevBuf xs64, xs32, xs32lo;
     fmm::DevBuf c_level, c_anchor, c_begin, c_end, c_child, c_nchild, c_parent, c_xyz;
     fmm::DevBuf split_cnt, split_off, split_bnd;
-    fmm::DevBuf leaves;
+    fmm::DevBuf leaves, small_tree;
     fmm::DevBuf frontA, frontB;
     fmm::DevBuf p2p_pairs, m2lx_pairs;
     fmm::DevBuf near_dev;       // near-field stencil of the uniform fast path (int4)
