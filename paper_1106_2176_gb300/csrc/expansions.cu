@@ -381,15 +381,68 @@ __global__ void l2l_k(int p, int ls, int le, const int *__restrict__ parent, con
     if (l) Lc[im_idx(k, l)] += sc * si;
 }
 
-// M2M and L2L of the mixed path as dense maps: one warp per cell, lane i
-// owns output rows i, i + 32, ... (NR of them); the input expansion is staged
-// in shared memory and every lane reads the map column by column (coalesced).
+// M2M and L2L of the mixed path as dense maps: lane i owns output rows i, i +
+// 32, ... (NR of them) and reads the map column by column (coalesced); the
+// input expansions are staged in shared memory. Bound: the maps (16 KB at p =
+// 8) come from L2 for every cell. A warp therefore applies a map to MC cells of one
+// octant at once on levels with cells enough (M2M at N = 1e7, p = 8: 0.435 ->
+// 0.23 ms; L2L 0.285 -> 0.26 ms), and L2L reads eight columns ahead (N = 1e5, p =
+// 10: 0.132 -> 0.102 ms, N = 6e4, p = 16: 0.53 -> 0.37 ms; M2M gained nothing by that).
 constexpr int MV_WARPS = 8;
+constexpr int MV_MC = 4;
+
+// acc[k][r] += sum_j T[j][lane + 32 r] x_k[j], j ascending; x_k at sx + k PP
+template <int NR, int MC, int U>
+__device__ __forceinline__ void mv_accum(const float *__restrict__ T, int PP, int lane, const float *sx, float (&acc)[MC][NR])
+{
+#pragma unroll U
+    for (int j = 0; j < PP; j++) {
+        const float *col = T + (size_t)j * PP;
+        float t[NR];
+#pragma unroll
+        for (int r = 0; r < NR; r++) t[r] = lane + 32 * r < PP ? col[lane + 32 * r] : 0.f;
+#pragma unroll
+        for (int k = 0; k < MC; k++) {
+            const float xj = sx[k * PP + j];
+#pragma unroll
+            for (int r = 0; r < NR; r++) acc[k][r] = fmaf(t[r], xj, acc[k][r]);
+        }
+    }
+}
+
+// the maps of MC cells (octants o[k], -1: no cell) into acc: shared reads where
+// the octants agree
+template <int NR, int MC, int U>
+__device__ __forceinline__ void mv_cells(const int (&o)[MC], const float *__restrict__ mat, int PP, int lane, const float *sx,
+                                         float (&acc)[MC][NR])
+{
+    bool same = true;
+#pragma unroll
+    for (int k = 0; k < MC; k++) {
+        same = same && o[k] == o[0];
+#pragma unroll
+        for (int r = 0; r < NR; r++) acc[k][r] = 0.f;
+    }
+    if (same && o[0] >= 0) {
+        mv_accum<NR, MC, U>(mat + (size_t)o[0] * PP * PP, PP, lane, sx, acc);
+        return;
+    }
+#pragma unroll
+    for (int k = 0; k < MC; k++) {
+        if (o[k] < 0) continue;
+        float one[1][NR];
+#pragma unroll
+        for (int r = 0; r < NR; r++) one[0][r] = 0.f;
+        mv_accum<NR, 1, U>(mat + (size_t)o[k] * PP * PP, PP, lane, sx + k * PP, one);
+#pragma unroll
+        for (int r = 0; r < NR; r++) acc[k][r] = one[0][r];
+    }
+}
 
 // M2M: one block per parent, warp w maps child w; the partial expansions are
 // added in child order, so the result does not depend on scheduling
 template <int NR>
-__global__ void __launch_bounds__(32 * MV_WARPS) m2m_mv_k(int PP, int ls, int le, const int *__restrict__ child,
+__global__ void __launch_bounds__(32 * MV_WARPS) m2m_one_k(int PP, int ls, int le, const int *__restrict__ child,
                                                          const int *__restrict__ nchild, const int4 *__restrict__ xyz,
                                                          const float *__restrict__ mat, float *__restrict__ M)
 {
@@ -433,46 +486,93 @@ __global__ void __launch_bounds__(32 * MV_WARPS) m2m_mv_k(int PP, int ls, int le
     }
 }
 
-// L2L into child c by one warp, sx: PP floats of the warp's shared memory
+// The same for MC parents per block, warp w mapping child w of each (in a full
+// tree all of octant w)
+template <int NR, int MC>
+__global__ void __launch_bounds__(32 * MV_WARPS) m2m_mv_k(int PP, int ls, int le, const int *__restrict__ child,
+                                                         const int *__restrict__ nchild, const int4 *__restrict__ xyz,
+                                                         const float *__restrict__ mat, float *__restrict__ M)
+{
+    extern __shared__ float sm_mv[];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int c0 = ls + blockIdx.x * MC;
+    float *sx = sm_mv + w * MC * PP;                // the warp's child expansions
+    float *part = sm_mv + MV_WARPS * MC * PP;       // [parent][child][PP] partial results
+    int o[MC];
+#pragma unroll
+    for (int k = 0; k < MC; k++) {
+        o[k] = -1;
+        if (c0 + k >= le || w >= nchild[c0 + k]) continue;  // (a leaf keeps its P2M expansion)
+        const int ch = child[c0 + k] + w;
+        o[k] = child_octant(xyz[ch]);
+        const float *Mc = M + (size_t)ch * PP;
+        for (int j = lane; j < PP; j += 32) sx[k * PP + j] = Mc[j];
+    }
+    __syncwarp();
+    float acc[MC][NR];
+    mv_cells<NR, MC, 4>(o, mat, PP, lane, sx, acc);
+#pragma unroll
+    for (int k = 0; k < MC; k++)
+#pragma unroll
+        for (int r = 0; r < NR; r++)
+            if (o[k] >= 0 && lane + 32 * r < PP) part[(k * MV_WARPS + w) * PP + lane + 32 * r] = acc[k][r];
+    __syncthreads();
+    for (int i = threadIdx.x; i < MC * PP; i += 32 * MV_WARPS) {
+        const int k = i / PP, e = i - k * PP;
+        const int nc = c0 + k < le ? nchild[c0 + k] : 0;
+        if (nc == 0) continue;
+        float sum = 0.f;
+        for (int ch = 0; ch < nc; ch++) sum += part[(k * MV_WARPS + ch) * PP + e];
+        M[(size_t)(c0 + k) * PP + e] = sum;
+    }
+}
+
+// L2L into cells c, c + 8, ... (MC of them below le; in a full tree all of one
+// octant) by one warp; sx: MC PP floats of the warp's shared memory
+template <int NR, int MC>
+__device__ __forceinline__ void l2l_children_warp(int c, int le, int lane, int PP, const int *__restrict__ parent,
+                                                  const int4 *__restrict__ xyz, const float *__restrict__ mat,
+                                                  float *__restrict__ L, float *sx)
+{
+    int o[MC];
+#pragma unroll
+    for (int k = 0; k < MC; k++) {
+        const int ck = c + k * MV_WARPS;
+        o[k] = -1;
+        if (ck >= le) continue;
+        o[k] = child_octant(xyz[ck]);
+        const float *Lp = L + (size_t)parent[ck] * PP;
+        for (int j = lane; j < PP; j += 32) sx[k * PP + j] = __ldcg(Lp + j);
+    }
+    __syncwarp();
+    float acc[MC][NR];
+    mv_cells<NR, MC, 8>(o, mat, PP, lane, sx, acc);
+#pragma unroll
+    for (int k = 0; k < MC; k++) {
+        if (o[k] < 0) continue;
+        float *Lc = L + (size_t)(c + k * MV_WARPS) * PP;
+#pragma unroll
+        for (int r = 0; r < NR; r++)
+            if (lane + 32 * r < PP) Lc[lane + 32 * r] = __ldcg(Lc + lane + 32 * r) + acc[k][r];
+    }
+}
+
 template <int NR>
 __device__ __forceinline__ void l2l_child_warp(int c, int lane, int PP, const int *__restrict__ parent,
                                                const int4 *__restrict__ xyz, const float *__restrict__ mat,
                                                float *__restrict__ L, float *sx)
 {
-    const float *T = mat + (size_t)child_octant(xyz[c]) * PP * PP;
-    const float *Lp = L + (size_t)parent[c] * PP;
-    for (int j = lane; j < PP; j += 32) sx[j] = __ldcg(Lp + j);
-    __syncwarp();
-    float acc[NR];
-#pragma unroll
-    for (int r = 0; r < NR; r++) acc[r] = 0.f;
-    for (int j = 0; j < PP; j++) {
-        const float xj = sx[j];
-        const float *col = T + (size_t)j * PP;
-#pragma unroll
-        for (int r = 0; r < NR; r++) {
-            const int i = lane + 32 * r;
-            if (i < PP) acc[r] = fmaf(col[i], xj, acc[r]);
-        }
-    }
-    float *Lc = L + (size_t)c * PP;
-#pragma unroll
-    for (int r = 0; r < NR; r++) {
-        const int i = lane + 32 * r;
-        if (i < PP) Lc[i] = __ldcg(Lc + i) + acc[r];
-    }
+    l2l_children_warp<NR, 1>(c, c + 1, lane, PP, parent, xyz, mat, L, sx);
 }
 
-template <int NR>
+template <int NR, int MC>
 __global__ void __launch_bounds__(32 * MV_WARPS) l2l_mv_k(int PP, int ls, int le, const int *__restrict__ parent,
                                                          const int4 *__restrict__ xyz, const float *__restrict__ mat,
                                                          float *__restrict__ L)
 {
     extern __shared__ float sm_mv[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int c = ls + blockIdx.x * MV_WARPS + w;
-    if (c >= le) return;
-    l2l_child_warp<NR>(c, lane, PP, parent, xyz, mat, L, sm_mv + w * PP);
+    l2l_children_warp<NR, MC>(ls + blockIdx.x * MV_WARPS * MC + w, le, lane, PP, parent, xyz, mat, L, sm_mv + w * MC * PP);
 }
 
 // M2M of parent c by one warp, with the arithmetic of m2m_mv_k (each child's
@@ -518,14 +618,23 @@ __device__ __forceinline__ void m2m_parent_warp(int c, int lane, int PP, const i
     }
 }
 
+// several cells per warp from MV_FEW on (below, more warps count for more), if
+// the staging fits 48 KB
+constexpr int MV_FEW = 2048;
+
 static void m2m_mv(int PP, int ls, int le, const int *child, const int *nchild, const int4 *xyz, const float *mat,
                    float *M, cudaStream_t s)
 {
-    const unsigned g = (unsigned)(le - ls);
-    const size_t sm = sizeof(float) * 2 * MV_WARPS * PP;
+    const bool many = le - ls >= MV_FEW && sizeof(float) * 2 * MV_WARPS * MV_MC * PP <= 48 * 1024;
+    const int mc = many ? MV_MC : 1;
+    const unsigned g = nblk(le - ls, mc);
+    const size_t sm = sizeof(float) * 2 * MV_WARPS * mc * PP;
     switch ((PP + 31) / 32) {
-#define FMM_MV_CASE(R) \
-    case R: m2m_mv_k<R><<<g, 32 * MV_WARPS, sm, s>>>(PP, ls, le, child, nchild, xyz, mat, M); break;
+#define FMM_MV_CASE(R)                                                                                                 \
+    case R:                                                                                                            \
+        if (many) m2m_mv_k<R, MV_MC><<<g, 32 * MV_WARPS, sm, s>>>(PP, ls, le, child, nchild, xyz, mat, M);             \
+        else m2m_one_k<R><<<g, 32 * MV_WARPS, sm, s>>>(PP, ls, le, child, nchild, xyz, mat, M);                        \
+        break;
         FMM_MV_CASE(1) FMM_MV_CASE(2) FMM_MV_CASE(3) FMM_MV_CASE(4) FMM_MV_CASE(5) FMM_MV_CASE(6) FMM_MV_CASE(7)
         FMM_MV_CASE(8) FMM_MV_CASE(9) FMM_MV_CASE(10) FMM_MV_CASE(11) FMM_MV_CASE(12) FMM_MV_CASE(13)
 #undef FMM_MV_CASE
@@ -535,11 +644,16 @@ static void m2m_mv(int PP, int ls, int le, const int *child, const int *nchild, 
 
 static void l2l_mv(int PP, int ls, int le, const int *parent, const int4 *xyz, const float *mat, float *L, cudaStream_t s)
 {
-    const unsigned g = nblk(le - ls, MV_WARPS);
-    const size_t sm = sizeof(float) * MV_WARPS * PP;
+    const bool many = le - ls >= MV_FEW && sizeof(float) * MV_WARPS * MV_MC * PP <= 48 * 1024;
+    const int mc = many ? MV_MC : 1;
+    const unsigned g = nblk(le - ls, MV_WARPS * mc);
+    const size_t sm = sizeof(float) * MV_WARPS * mc * PP;
     switch ((PP + 31) / 32) {
-#define FMM_MV_CASE(R) \
-    case R: l2l_mv_k<R><<<g, 32 * MV_WARPS, sm, s>>>(PP, ls, le, parent, xyz, mat, L); break;
+#define FMM_MV_CASE(R)                                                                                  \
+    case R:                                                                                             \
+        if (many) l2l_mv_k<R, MV_MC><<<g, 32 * MV_WARPS, sm, s>>>(PP, ls, le, parent, xyz, mat, L);     \
+        else l2l_mv_k<R, 1><<<g, 32 * MV_WARPS, sm, s>>>(PP, ls, le, parent, xyz, mat, L);              \
+        break;
         FMM_MV_CASE(1) FMM_MV_CASE(2) FMM_MV_CASE(3) FMM_MV_CASE(4) FMM_MV_CASE(5) FMM_MV_CASE(6) FMM_MV_CASE(7)
         FMM_MV_CASE(8) FMM_MV_CASE(9) FMM_MV_CASE(10) FMM_MV_CASE(11) FMM_MV_CASE(12) FMM_MV_CASE(13)
 #undef FMM_MV_CASE
