@@ -67,9 +67,9 @@ enum { FMM_F32 = 0, FMM_F64 = 1, FMM_HOST_MEM = 0x100 };
 enum {
     FMM_FP64 = 0,  /* every stage in FP64 (the on-device reference path) */
     FMM_MIXED = 1  /* FP32 P2P and expansions, M2L on the tensor cores in
-                      split TF32 with FP32 accumulation (p <= 11; FP32
-                      rotation M2L above), FP64 tree, FP64 offsets and final
-                      sums */
+                      split FP16 (two halves of 11 bits, scaled by powers of
+                      two) with FP32 accumulation (p <= 11; FP32 rotation M2L
+                      above), FP64 tree, FP64 offsets and final sums */
 };
 
 /* M2L engine of the same-level pairs (fmm_set_m2l_engine) */
@@ -125,7 +125,7 @@ FMM_API int fmm_set_precision(fmm_handle h, int mode);
 
 /* Select the M2L engine; takes effect at the next build. FMM_M2L_AUTO: the
  * tensor cores for FMM_MIXED with p <= 11, otherwise rotation for p <= 16
- * (FP64 included), otherwise the CUDA-core dense contraction. FMM_M2L_TENSOR: split-TF32 tcgen05 contraction (FMM_MIXED,
+ * (FP64 included), otherwise the CUDA-core dense contraction. FMM_M2L_TENSOR: split-FP16 tcgen05 contraction (FMM_MIXED,
  * p <= 11). FMM_M2L_CUDACORE: dense O(p^4) contraction on the CUDA cores.
  * FMM_M2L_ROTATION: rotate each translation onto the z axis, translate along
  * z and rotate back, O(p^3) per pair (either precision, p <= 16). The
@@ -175,9 +175,11 @@ FMM_API int fmm_set_m2l_pool(fmm_handle h, int max_cells);
  * order (octant bits, then z, y, x of the halved position), and the kernel
  * brings a tile's sources for one translation as TMA tile loads of a shifted
  * block, positions outside the level as zeros; no per-row lookups or row
- * gathers. on = 0: per-row lookups and gathers on every level. The results
- * are bitwise the same. Takes effect at the next build; fmm_stats
- * .lattice_levels says which levels the last build set up (bit l: level l).
+ * gathers. Such levels with at least three quarters of their cells are read
+ * the same way, the missing cells as zeros. on = 0: per-row lookups and
+ * gathers on every level. The results are bitwise the same. Takes effect at
+ * the next build; fmm_stats.lattice_levels says which complete levels the
+ * last build set up (bit l: level l).
  * Returns FMM_EINVAL for a NULL handle or on not 0/1.
  */
 FMM_API int fmm_set_m2l_lattice(fmm_handle h, int on);

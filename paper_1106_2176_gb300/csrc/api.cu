@@ -502,7 +502,7 @@ int fmm_get_stats(fmm_handle h, fmm_stats *out)
     }
     out->kernel_launches = h->launches;
     out->uniform_path = h->uniform_used ? 1 : 0;
-    out->lattice_levels = (int32_t)h->lat_levels;
+    out->lattice_levels = (int32_t)h->lat_complete;
     phase_means(h, 1, out);
     return FMM_OK;
     API_END

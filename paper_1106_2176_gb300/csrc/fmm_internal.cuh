@@ -109,6 +109,7 @@ struct M2LTile {
     int count;
     int level;
     int octant;
+    int block;   // lattice levels: block of the octant's sub-lattice (Morton order), otherwise -1
 };
 
 // One system's share of a persistent tensor-core M2L launch: its tile list
@@ -131,10 +132,9 @@ struct M2LJob {
     const unsigned *lmax;       // per level: the bits of its largest coefficient (sets the rows' scale)
     unsigned *tcnt;             // per tile: ranges finished (nsplit > 1)
     float2 *part;               // per (tile, range): its (hi, lo) sums (nsplit > 1)
-    // complete levels whose sources come by TMA tile loads from the lattice
-    // copy of M~ (bit l: level l); lat_maps holds a 128-byte tensor map per level
+    // 128-byte tensor map per level of the lattice copy of the rows, from which
+    // lattice tiles read their sources by TMA tile loads (null: gather)
     const unsigned char *lat_maps;
-    unsigned lat_levels;
     int nsplit, chunk;          // ranges of `chunk` vectors a tile's list is cut into, one CTA each
     int ws_words;               // words of the workspace at lmax (maxima, counters) to zero per evaluation
     int item0;
@@ -257,12 +257,15 @@ struct fmm_ctx {
     fmm::DevBuf msplit;         // M~ split into FP16 (hi, lo) rows for the tensor-core M2L
     fmm::DevBuf m2l_ws, m2l_part;  // its level maxima and tile counters; sums of the ranges of split tiles
     int m2l_nsplit = 1, m2l_chunk = 0;  // ranges per tile and their length (m2l_plan)
-    // tensor-core M2L on complete levels: the rows of each such level in lattice
+    // tensor-core M2L on lattice levels: the rows of each such level in lattice
     // order (octant bits, then z, y, x of the halved position), one TMA tensor
     // map per level (device copy and its pinned staging)
     bool lattice_req = true;    // fmm_set_m2l_lattice
     unsigned lat_levels = 0;    // bit l: level l reads its sources from the lattice copy
+    unsigned lat_complete = 0;  // those of them that hold every cell
     long long lat_off[FMM_MAXLEVEL + 1] = {};  // first row of level l in mlat
+    long long lat_rows = 0;     // rows of mlat
+    int m2l_plan_tiles = 0;     // tiles the ranges of the vectors are planned for
     fmm::DevBuf mlat, lat_maps;
     fmm::PinnedBuf lat_host;
 
@@ -367,8 +370,9 @@ void m2l_tensor_jobs(int p, int nsm, const M2LJob *jobs_dev, int njobs, int *que
 M2LJob m2l_tensor_job(fmm_ctx *h, float *L);  // the handle's arrays; allocates its workspaces
 int m2l_longest_list(fmm_ctx *h);              // vectors of the longest list a tile walks
 void m2l_plan(fmm_ctx *h);                     // (build) ranges per tile
-// (build) which complete levels the tensor-core M2L reads through TMA tile
-// loads: their lattice buffer and tensor maps
+// (build) which levels the tensor-core M2L reads through TMA tile loads; their
+// lattice buffer and tensor maps
+void lattice_select(fmm_ctx *h, int pool_max);
 void lattice_prepare(fmm_ctx *h, cudaStream_t s);
 void batch_split(int p, const BatchSys *sys, int nsys, cudaStream_t s);  // every system's FP16 rows
 

@@ -33,8 +33,8 @@
 // [T_hi ; T_lo], all 128B-swizzled in shared memory, where the MMAs read both
 // operands.
 //   - a producer brings the unit's operator block with one bulk copy and, on
-//     complete levels (lattice tiles), A_hi and A_lo with one TMA tile load each;
-//     the workers then only drain.
+//     complete and nearly complete levels (lattice tiles), A_hi and A_lo with
+//     one TMA tile load each; the workers then only drain.
 //   - on other levels the worker group u % 2 gathers the unit's rows with
 //     cp.async straight into the stage (sources found by lattice lookups
 //     fetched ahead into a ring; zero fill where a cell is absent). The
@@ -233,6 +233,17 @@ __global__ void __launch_bounds__(256) m2l_split_k(const float *__restrict__ M, 
     m2l_split_chunk<NP>(M + (size_t)c * PP, PP, ch, m2l_exponent(lmax[l]), row);
 }
 
+// bits 0, 3, 6, ... of a Morton code below 2^30
+__device__ __forceinline__ uint32_t every_third(uint32_t v)
+{
+    v &= 0x09249249u;
+    v = (v | (v >> 2)) & 0x030c30c3u;
+    v = (v | (v >> 4)) & 0x0300f00fu;
+    v = (v | (v >> 8)) & 0x030000ffu;
+    v = (v | (v >> 16)) & 0x3ffu;
+    return v;
+}
+
 template <int NP, bool PERSIST>
 __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     m2l_tc_k(int p, const __grid_constant__ M2LJob one, const M2LJob *__restrict__ jobs, int njobs,
@@ -321,13 +332,13 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     const int w0 = (int)min((long long)nvt, (long long)split * J.chunk), w1 = (int)min((long long)nvt, (long long)w0 + J.chunk);
     const int e0 = J.st_off[td.octant] + w0, nv = w1 - w0;
     const int nunits = nv * KB;
-    // Lattice tile (a complete level with a lattice copy of M~): the tile is
-    // an 8 x 4 x 4 block of its octant's sub-lattice with rows in x, y, z
+    // Lattice tile (a level with a lattice copy of its rows): the tile is an
+    // 8 x 4 x 4 block of its octant's sub-lattice with rows in x, y, z
     // order, and for every vector the sources form the same block shifted, in
-    // the sub-lattice of the source octant; positions outside the level
-    // arrive as zeros, as absent cells do.
+    // the sub-lattice of the source octant; positions outside the level or
+    // without a cell arrive as zeros, as absent cells do.
     // (persistent launches serve the batch engine, which gathers everywhere)
-    const bool lat = !PERSIST && J.lat_maps != nullptr && td.octant < 8 && ((J.lat_levels >> l) & 1u);
+    const bool lat = !PERSIST && J.lat_maps != nullptr && td.block >= 0;
 
     if (warp >= C::MMA_WARP && warp < C::P_WARP) {
         // ----------------------------------------------------------- MMA warps
@@ -399,11 +410,11 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
             const int obx = td.octant & 1, oby = (td.octant >> 1) & 1, obz = (td.octant >> 2) & 1;
             const unsigned char *lmap = nullptr;
             if (lat) {
-                const int4 a = J.xyz[J.tgt[td.start]];
-                const int sh = FMM_MAXLEVEL - l + 1;
-                ox = a.x >> sh;
-                oy = a.y >> sh;
-                oz = a.z >> sh;
+                // its first position, 128 td.block in Morton order
+                const unsigned k = (unsigned)td.block * C::M;
+                ox = (int)every_third(k);
+                oy = (int)every_third(k >> 1);
+                oz = (int)every_third(k >> 2);
                 lmap = J.lat_maps + 128 * l;
             }
             const unsigned char *ttab = J.ttab;
@@ -449,8 +460,8 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
         // this row's cell, its level, lattice position and octant (a pooled
         // tile mixes levels and octants)
         int px = 0, py = 0, pz = 0, cell = -1, rl = l, ro = 0;
-        if (row < td.count) {
-            cell = J.tgt[td.start + row];
+        if (row < td.count) cell = J.tgt[td.start + row];  // (-1: a lattice position without a cell)
+        if (cell >= 0) {
             const int4 a = J.xyz[cell];
             rl = a.w;
             const int sh = FMM_MAXLEVEL - rl;
@@ -934,7 +945,7 @@ void m2l_plan(fmm_ctx *h)
     for (int want = 1; want <= 32; want++) {
         constexpr int G = 2 * TcCfg<64>::GV;
         const int chunk = (nv + want * G - 1) / (want * G) * G, s = (nv + chunk - 1) / chunk;
-        const double waves = (double)(((int64_t)h->ntiles_max * s + h->nsm - 1) / h->nsm);
+        const double waves = (double)(((int64_t)h->m2l_plan_tiles * s + h->nsm - 1) / h->nsm);
         const double t = waves * ((double)std::min(chunk, nv) + (s > 1 ? 13.0 : 10.0)) + (s > 1 ? s : 0);
         if (t < best) {
             best = t;
@@ -972,8 +983,7 @@ M2LJob m2l_tensor_job(fmm_ctx *h, float *L)
     j.nsplit = h->m2l_nsplit;
     j.chunk = h->m2l_chunk;
     j.rowexp = reinterpret_cast<const int *>(j.ttab + (size_t)h->nV * tc_op_bytes(h->p));
-    j.lat_maps = nullptr;  // gathers on every level (the single-system launch sets the lattice levels)
-    j.lat_levels = 0;
+    j.lat_maps = nullptr;  // gathers on every level (the single-system launch sets the lattice maps)
     j.item0 = 0;
     j.count = -1;
     return j;
@@ -999,34 +1009,77 @@ static EncodeTiledFn encode_tiled()
     return fn;
 }
 
-// The complete levels whose tiles are lattice blocks (at least 8^4 cells,
-// more than the pooling threshold, so every tile is 128 cells of one octant)
-// read their sources by TMA from the lattice copy of their rows: one 5-D
-// tensor map per level over [octant bits][z/2][y/2][x/2][row] (FP16), box 64
-// halves x 8 x 4 x 4 x 1 = one half (hi or lo) of the tile's 128 rows,
-// 128-byte swizzle (the layout of the gathered stages). Levels beyond 9 keep
-// the gathers.
-void lattice_prepare(fmm_ctx *h, cudaStream_t s)
+// Lattice levels: at least three quarters of the positions hold a cell, at
+// least 8^4 positions, more cells than the pooling threshold, level 9 at most.
+// Their tiles are blocks of 128 positions of one octant, with or without a
+// cell, and read their sources by TMA from the lattice copy of the level's
+// rows, zeros where there is no cell. A tile by TMA takes about 0.45 of the
+// time of one with gathered rows (N = 1e6 Plummer against uniform trees), so
+// the rows without a cell cost less than the gathers from half full on; the
+// batch engine, which gathers on every level, pays for them. M2L at N = 3e5
+// uniform, p = 8, whose level 5 is 85 % full: 2.66 -> 2.14 ms.
+static unsigned dense_levels(fmm_ctx *h, int pool_max)
 {
-    h->lat_levels = 0;
-    if (!h->lattice_req || h->precision != FMM_MIXED || h->engine_used != FMM_M2L_TENSOR || !tensor_m2l_supported(h) ||
-        m2l_tile_size(h) != TcCfg<64>::M)
-        return;
-    const EncodeTiledFn enc = encode_tiled();
-    if (!enc) return;
-    const cuuint64_t row = tc_row_bytes(h->p);
-    const int pool_max = h->m2l_pool >= 0 ? h->m2l_pool : 4 * m2l_tile_size(h);
-    unsigned levels = 0;
-    long long total = 0;
+    unsigned m = 0;
     for (int l = 4; l <= std::min(h->depth, 9); l++) {
         const long long cells = (long long)h->lvl_start[(size_t)l + 1] - h->lvl_start[(size_t)l];
-        if (cells != (1ll << (3 * l)) || cells <= pool_max) continue;
-        levels |= 1u << l;
-        h->lat_off[l] = total;
-        total += cells;
+        if (4 * cells >= 3ll << (3 * l) && cells > pool_max) m |= 1u << l;
     }
+    return m;
+}
+
+// tiles of the tree with every such level in lattice tiles
+static int plan_tiles(fmm_ctx *h)
+{
+    constexpr int M = TcCfg<64>::M;
+    const int pool_max = h->m2l_pool >= 0 ? h->m2l_pool : 4 * M;
+    const unsigned dense = dense_levels(h, pool_max);
+    int64_t pooled = 0, nt = 0;
+    for (int l = 2; l <= h->depth; l++) {
+        const int cells = h->lvl_start[(size_t)l + 1] - h->lvl_start[(size_t)l];
+        if (cells <= pool_max) pooled += cells;
+        else nt += (dense >> l) & 1u ? (1ll << (3 * l)) / M : cells / M + 8;
+    }
+    return (int)(nt + (pooled + M - 1) / M);
+}
+
+void lattice_select(fmm_ctx *h, int pool_max)
+{
+    h->lat_levels = h->lat_complete = 0;
+    // the ranges of the vectors are planned for these tiles with or without the
+    // lattice loads, whose results are then the same bit for bit
+    const unsigned dense = dense_levels(h, pool_max);
+    h->m2l_plan_tiles = plan_tiles(h);
+    if (!h->lattice_req || h->precision != FMM_MIXED || h->engine_used != FMM_M2L_TENSOR || !tensor_m2l_supported(h) ||
+        m2l_tile_size(h) != TcCfg<64>::M || !encode_tiled())
+        return;
+    long long total = 0;
+    for (int l = 4; l <= std::min(h->depth, 9); l++) {
+        const long long cells = (long long)h->lvl_start[(size_t)l + 1] - h->lvl_start[(size_t)l], all = 1ll << (3 * l);
+        if (!((dense >> l) & 1u)) continue;
+        h->lat_levels |= 1u << l;
+        if (cells == all) h->lat_complete |= 1u << l;
+        h->lat_off[l] = total;
+        total += all;
+    }
+    h->lat_rows = total;
+}
+
+// One 5-D tensor map per lattice level over [octant bits][z/2][y/2][x/2][row]
+// (FP16), box 64 halves x 8 x 4 x 4 x 1 = one half (hi or lo) of the tile's 128
+// rows, 128-byte swizzle (the layout of the gathered stages).
+void lattice_prepare(fmm_ctx *h, cudaStream_t s)
+{
+    const unsigned levels = h->lat_levels;
     if (!levels) return;
+    const EncodeTiledFn enc = encode_tiled();
+    const cuuint64_t row = tc_row_bytes(h->p);
+    const long long total = h->lat_rows;
     h->mlat.ensure((size_t)row * (size_t)total);
+    // rows of positions without a cell, which no evaluation writes
+    for (int l = 4; l <= 9; l++)
+        if (((levels & ~h->lat_complete) >> l) & 1u)
+            FMM_CUDA_TRY(cudaMemsetAsync(h->mlat.as<unsigned char>() + row * h->lat_off[l], 0, (size_t)row << (3 * l), s));
     const size_t mbytes = sizeof(CUtensorMap) * (FMM_MAXLEVEL + 1);
     h->lat_maps.ensure(mbytes);
     h->lat_host.ensure(mbytes);
@@ -1044,7 +1097,6 @@ void lattice_prepare(fmm_ctx *h, cudaStream_t s)
         if (r != CUDA_SUCCESS) throw Error{FMM_ECUDA, "tensor-core M2L: encoding a lattice tensor map failed"};
     }
     FMM_CUDA_TRY(cudaMemcpyAsync(h->lat_maps.p, mp, mbytes, cudaMemcpyHostToDevice, s));
-    h->lat_levels = levels;
 }
 
 template <int NP>
@@ -1109,7 +1161,6 @@ void m2l_tensor(fmm_ctx *h, float *L, const float *M)
     count_launch(h);
     if (h->lat_levels) {
         j.lat_maps = h->lat_maps.as<unsigned char>();
-        j.lat_levels = h->lat_levels;
     }
     launch_tc_p(h->p, h->ntiles_max * j.nsplit, j, nullptr, 1, queue, err, s);
     count_launch(h);

@@ -1410,7 +1410,9 @@ __global__ void oct_count_k(int c0, int nc, const int *__restrict__ level, const
 // tiles of the 8 octant groups are interleaved (tile k of octant 0, tile k of
 // octant 1, ...), so that tiles running at the same time cover one compact
 // region and share sources in L2.
-__global__ void tiles_k(int depth, int tile, int pool_max, const unsigned *__restrict__ grp,
+// Lattice levels (bit l of lat) take every position of the level, cells or not,
+// so that each tile is one block of its octant's sub-lattice.
+__global__ void tiles_k(int depth, int tile, int pool_max, unsigned lat, const unsigned *__restrict__ grp,
                         unsigned *__restrict__ goff, M2LTile *__restrict__ tiles, int *__restrict__ ntiles)
 {
     unsigned run = 0;
@@ -1442,26 +1444,28 @@ __global__ void tiles_k(int depth, int tile, int pool_max, const unsigned *__res
         d.count = (int)cnt;
         d.level = lv;
         d.octant = 8;
+        d.block = -1;
         tiles[nt++] = d;
     }
     for (int l = 2; l <= depth; l++) {
         if (level_cells(l) <= (unsigned)pool_max) continue;
         unsigned kmax = 0;
         for (int o = 0; o < 8; o++) {
-            const unsigned c = grp[l * 8 + o];
+            const unsigned c = (lat >> l) & 1u ? 1u << (3 * (l - 1)) : grp[l * 8 + o];
             goff[l * 8 + o] = run;
             run += c;
             kmax = max(kmax, (c + tile - 1) / tile);
         }
         for (unsigned k = 0; k < kmax; k++)
             for (int o = 0; o < 8; o++) {
-                const unsigned c = grp[l * 8 + o], t = k * tile;
+                const unsigned c = (lat >> l) & 1u ? 1u << (3 * (l - 1)) : grp[l * 8 + o], t = k * tile;
                 if (t >= c) continue;
                 M2LTile d;
                 d.start = (int)(goff[l * 8 + o] + t);
                 d.count = (int)min((unsigned)tile, c - t);
                 d.level = l;
                 d.octant = o;
+                d.block = (lat >> l) & 1u ? (int)k : -1;
                 tiles[nt++] = d;
             }
     }
@@ -1477,14 +1481,14 @@ __global__ void tiles_k(int depth, int tile, int pool_max, const unsigned *__res
 // loads a shifted block of sources by TMA. Other groups in arrival order.
 __global__ void oct_scatter_k(int c0, int nc, const int *__restrict__ level, const uint64_t *__restrict__ anchor,
                               const unsigned *__restrict__ grp, const unsigned *__restrict__ goff,
-                              unsigned *__restrict__ fill, int raster, int *__restrict__ tgt)
+                              unsigned *__restrict__ fill, int raster, unsigned lat, int *__restrict__ tgt)
 {
     int c = c0 + blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= nc) return;
     int l = level[c];
     const uint64_t code = anchor[c] >> (3 * (FMM_MAXLEVEL - l));
     int o = (int)(code & 7u);
-    const bool complete = l <= 10 && grp[l * 8 + o] == (1u << (3 * (l - 1)));
+    const bool complete = ((lat >> l) & 1u) || (l <= 10 && grp[l * 8 + o] == (1u << (3 * (l - 1))));
     unsigned hm = (unsigned)(code >> 3);
     if (complete && raster && l >= 4) {
         const unsigned m = hm & 127u;
@@ -1949,18 +1953,26 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
         const int c0 = depth >= 2 ? h->lvl_start[2] : ncells;
         const int nt = ncells - c0;
         const int pool_max = h->m2l_pool >= 0 ? h->m2l_pool : 4 * tile;
-        // pooled levels: one run of tiles; complete levels: equal octant
-        // groups; others: up to one partial tile per octant more
+        lattice_select(h, pool_max);
+        // pooled levels: one run of tiles; lattice levels: all positions;
+        // complete levels: equal octant groups; others: up to one partial
+        // tile per octant more
         int pooled = 0;
+        int64_t ntgt = 0;
         h->ntiles_max = 0;
         for (int l = 2; l <= depth; l++) {
             const int cells = h->lvl_start[(size_t)l + 1] - h->lvl_start[(size_t)l];
+            const bool lat = (h->lat_levels >> l) & 1u;
+            ntgt += lat ? 1LL << (3 * l) : cells;
             if (cells <= pool_max) pooled += cells;
+            else if (lat) h->ntiles_max += (1 << (3 * l)) / tile;
             else if (l <= 10 && cells == (1 << (3 * l))) h->ntiles_max += 8 * ((cells / 8 + tile - 1) / tile);
             else h->ntiles_max += cells / tile + 8;
         }
         h->ntiles_max += (pooled + tile - 1) / tile;
-        h->m2l_tgt.ensure(sizeof(int) * (size_t)std::max(nt, 1));
+        h->m2l_tgt.ensure(sizeof(int) * (size_t)std::max<int64_t>(ntgt, 1));
+        // positions of lattice levels without a cell
+        if (ntgt > nt) FMM_CUDA_TRY(cudaMemsetAsync(h->m2l_tgt.p, 0xff, sizeof(int) * (size_t)ntgt, s));
         h->m2l_tiles.ensure(sizeof(M2LTile) * (size_t)std::max(h->ntiles_max, 1));
         h->m2l_misc.ensure(sizeof(unsigned) * 3 * 8 * (FMM_MAXLEVEL + 1) + 64);
         unsigned *grp = h->m2l_misc.as<unsigned>();
@@ -1972,11 +1984,11 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
             oct_count_k<<<nblocks(nt, TB), TB, 0, s>>>(c0, ncells, h->c_level.as<int>(), h->c_anchor.as<uint64_t>(), grp);
             count_launch(h);
         }
-        tiles_k<<<1, 1, 0, s>>>(depth, tile, pool_max, grp, goff, h->m2l_tiles.as<M2LTile>(), ntiles);
+        tiles_k<<<1, 1, 0, s>>>(depth, tile, pool_max, h->lat_levels, grp, goff, h->m2l_tiles.as<M2LTile>(), ntiles);
         count_launch(h);
         if (nt > 0) {
             oct_scatter_k<<<nblocks(nt, TB), TB, 0, s>>>(c0, ncells, h->c_level.as<int>(), h->c_anchor.as<uint64_t>(),
-                                                         grp, goff, fill, tile == 128 ? 1 : 0, h->m2l_tgt.as<int>());
+                                                         grp, goff, fill, tile == 128 ? 1 : 0, h->lat_levels, h->m2l_tgt.as<int>());
             count_launch(h);
         }
         check_launch("m2l tiles");

@@ -126,3 +126,67 @@ def test_batch_of_lattice_systems_matches_their_own_evaluations():
         assert bool((p == pr).all()) and bool((g == gr).all())
     assert b.status()[0] == 0
     b.close()
+
+
+def _corner_out(n, seed):
+    # a cube without the particles of one of 64 sub-cubes: every third-level
+    # block of that corner is missing, the rest of level 4 is there
+    x, q = inputs.uniform_cube(n, seed)
+    keep = ~np.all(x < x.min() + 0.25 * (x.max() - x.min()), axis=1)
+    return x[keep], q[keep]
+
+
+# levels with at least three quarters of their cells (uniform: level 5 where some
+# cells of level 4 stay leaves; corner: a block of both levels is missing), read
+# like complete ones, and one with fewer (n = 250000), gathered
+@pytest.mark.parametrize("P,gen,n,full", [(1, "uniform", 300000, True), (5, "uniform", 300000, True), (8, "uniform", 300001, True),
+                                          (11, "uniform", 300000, True), (8, "corner", 500000, True),
+                                          (6, "uniform", 250000, False)])
+def test_nearly_complete_levels_give_the_gathered_results_bitwise(P, gen, n, full):
+    x, q = inputs.uniform_cube(n, 90 + P) if gen == "uniform" else _corner_out(n, 90 + P)
+    x, q = x.astype(np.float32), q.astype(np.float32)
+    p1, g1, f1 = run_fmm(x, q, P, 0.5, 64, precision="mixed", dtype=np.float32, m2l_lattice=True)
+    p0, g0, f0 = run_fmm(x, q, P, 0.5, 64, precision="mixed", dtype=np.float32, m2l_lattice=False)
+    n5 = int(np.sum(f1.export_tree()["level"] == 5))
+    assert (4 * n5 >= 3 * 8**5) == full and 0 < n5 < 8**5
+    assert f1.stats()["async_error"] == 0 and f0.stats()["async_error"] == 0
+    assert np.array_equal(p1, p0) and np.array_equal(g1, g0)
+    _, L1 = f1.export_expansions()
+    _, L0 = f0.export_expansions()
+    assert np.array_equal(L1, L0)
+    # again on another tree of the same handle: rows of positions that no longer
+    # hold a cell are zero
+    torch = torch_cuda()
+    xb, qb = _corner_out(n, 190 + P)
+    xb, qb = xb[:len(x)], qb[:len(x)]
+    xb, qb = torch.tensor(xb, dtype=torch.float32, device="cuda"), torch.tensor(qb, dtype=torch.float32, device="cuda")
+    out = []
+    for f in (f1, f0):
+        f.build(xb, qb)
+        out.append([t.clone() for t in f.evaluate()])
+        torch.cuda.synchronize()
+        assert f.stats()["async_error"] == 0
+    assert all(bool((a == b).all()) for a, b in zip(*out))
+    f1.close()
+    f0.close()
+
+
+def test_batch_of_nearly_complete_systems_matches_their_own_evaluations():
+    torch = torch_cuda()
+    ensure_built()
+    from paper_1106_2176_gb300.batch import FMMBatch
+    systems = []
+    for k, n in enumerate((300000, 5000, 290000)):
+        x, q = inputs.uniform_cube(n, 95 + k, dtype=np.float32)
+        systems.append((torch.tensor(x, device="cuda"), torch.tensor(q, device="cuda")))
+    b = FMMBatch(systems, p=8, theta=0.5, ncrit=64, precision="mixed")
+    ref = [(p.clone(), g.clone()) for p, g in b.evaluate_each()]
+    for p, g in b.out:
+        p.fill_(float("nan"))
+        g.fill_(float("nan"))
+    b.evaluate()
+    torch.cuda.synchronize()
+    for (p, g), (pr, gr) in zip(b.out, ref):
+        assert bool((p == pr).all()) and bool((g == gr).all())
+    assert b.status()[0] == 0
+    b.close()
