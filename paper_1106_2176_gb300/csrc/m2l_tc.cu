@@ -123,7 +123,7 @@ struct TcCfg {
     // (which its parity would not tell from a completed one).
     static constexpr int NM = KB == 1 ? 2 : 1;
     static constexpr int MMA_WARP = NW, P_WARP = NW + NM;
-    static constexpr int NT = 32 * (NW + 2 * NM);  // threads
+    static constexpr int NT = 32 * (NW + 4);       // threads (with NM = 1 two warps idle)
     static constexpr int NS = NS_FIT > 6 ? 6 : NM == 2 ? NS_FIT & ~1 : NS_FIT;
     static constexpr int SMEM = NS * STAGE + RING + BAR + 1024;
     static constexpr int TCOLS = 512;
@@ -131,6 +131,14 @@ struct TcCfg {
     static constexpr int GV = 8;                   // vectors per accumulator drain
     static constexpr int OFF = GV / 2;
     static constexpr int HN = NP / 2;              // output coefficients per thread
+    // Registers: 168 a thread at launch (384 threads). The workers hold 2 HN sums
+    // besides the gathers' state; from NP = 64 on they take REG_W and the other
+    // four warps keep REG_O, together 63,488 of the launch's 64,512 (launch_tc
+    // checks). Spills at NP = 112 (p = 10) 184 -> 8 bytes; M2L at N = 1e5, p = 10
+    // 1.20 -> 0.92 ms, at N = 1e6 3.09 -> 2.66 ms. Not in the persistent kernel,
+    // whose roles meet again at every item.
+    static constexpr int REG_W = 216, REG_O = 64;
+    static constexpr bool REGS = NP >= 64;
     // a gathering worker drains a group once it has to wait for a vector more
     // than LATE past the group's last one: the group is then finished or about
     // to be, and the next group of the same buffer has not begun
@@ -340,117 +348,121 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     // (persistent launches serve the batch engine, which gathers everywhere)
     const bool lat = !PERSIST && J.lat_maps != nullptr && td.block >= 0;
 
-    if (warp >= C::MMA_WARP && warp < C::P_WARP) {
-        // ----------------------------------------------------------- MMA warps
-        // (the waits and commits, a few hundred cycles per unit, of one warp
-        // overlap the other's MMAs). The whole warp runs the loop and one
-        // elected lane issues: the branch on elect.sync lets the compiler keep
-        // the descriptors in uniform registers (7.25 against 7.75 ms at
-        // N = 1e7, p = 8, with one lane running the loop).
-        const int m = warp - C::MMA_WARP;
-        {
-            const uint32_t id_full = idesc_f16(128, 2 * NP), id_half = idesc_f16(128, NP);
-            const uint64_t a0 = sdesc(smem_u32(base));
-            constexpr uint64_t LO = PACK ? 64 / 16 : 16384 / 16, B0 = C::A_BYTES / 16;  // descriptor units of 16 bytes
-            bool ok = true;
-            for (int w = m, i = 0; ok && w < nv; w += NM, i++) {
-                const int gi = i + C::OFF * m, g = gi / C::GV, b = m * C::AC + g % C::AC;
-                const bool start = gi % C::GV == 0 || i == 0;
-                if (start && g >= C::AC) ok = mbar_wait_or(&acc_empty[b], (uint32_t)((g / C::AC - 1) & 1), abort_flag);
-                const uint32_t dmain = tmem + (uint32_t)(b * 2 * NP), dcorr = dmain + NP;
+    if (warp >= C::NW) {
+        if constexpr (!PERSIST && C::REGS) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::REG_O));
+        if (warp < C::P_WARP) {
+            // ----------------------------------------------------------- MMA warps
+            // (the waits and commits, a few hundred cycles per unit, of one warp
+            // overlap the other's MMAs). The whole warp runs the loop and one
+            // elected lane issues: the branch on elect.sync lets the compiler keep
+            // the descriptors in uniform registers (7.25 against 7.75 ms at
+            // N = 1e7, p = 8, with one lane running the loop).
+            const int m = warp - C::MMA_WARP;
+            {
+                const uint32_t id_full = idesc_f16(128, 2 * NP), id_half = idesc_f16(128, NP);
+                const uint64_t a0 = sdesc(smem_u32(base));
+                constexpr uint64_t LO = PACK ? 64 / 16 : 16384 / 16, B0 = C::A_BYTES / 16;  // descriptor units of 16 bytes
+                bool ok = true;
+                for (int w = m, i = 0; ok && w < nv; w += NM, i++) {
+                    const int gi = i + C::OFF * m, g = gi / C::GV, b = m * C::AC + g % C::AC;
+                    const bool start = gi % C::GV == 0 || i == 0;
+                    if (start && g >= C::AC) ok = mbar_wait_or(&acc_empty[b], (uint32_t)((g / C::AC - 1) & 1), abort_flag);
+                    const uint32_t dmain = tmem + (uint32_t)(b * 2 * NP), dcorr = dmain + NP;
 #pragma unroll
-                for (int kb = 0; kb < KB; kb++) {
-                    const int u = w * KB + kb, s = u % NS;
-                    const uint32_t ph = (uint32_t)((u / NS) & 1);
-                    ok = ok && mbar_wait_or(&full[s], ph, abort_flag);
-                    if (!lat) {
-                        ok = ok && mbar_wait_or(&gfull[s], ph, abort_flag);
-                        fence_proxy_async();  // the gathered rows (generic proxy) before the MMA's reads
-                    }
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) break;
-                    tc_fence_after();
-                    if (elect_one()) {
-                        const uint64_t ad = a0 + (uint64_t)((uint32_t)s * (C::STAGE / 16)), bd = ad + B0;
-                        const uint32_t first = (start && kb == 0) ? 0u : 1u;
-                        // k-steps of 16 coefficients holding any of the p^2 real ones
-                        constexpr int KS = PACK ? NP / 16 : 4;
-                        const int ks = min(KS, (PP - kb * 64 + 15) >> 4);
-#pragma unroll
-                        for (int k = 0; k < KS; k++) {
-                            if (k >= ks) break;
-                            const uint32_t acc = k == 0 ? first : 1u;
-                            // A_hi [T_hi ; T_lo] -> main | correction, then A_lo T_hi -> correction
-                            if (PACK) {
-                                mma_f16(dmain, ad + 2 * k, bd + 2 * k, id_half, acc);
-                                mma_f16(dcorr, ad + 2 * k, bd + LO + 2 * k, id_half, acc);
-                            } else {
-                                mma_f16(dmain, ad + 2 * k, bd + 2 * k, id_full, acc);
-                            }
-                            mma_f16(dcorr, ad + LO + 2 * k, bd + 2 * k, id_half, 1u);
+                    for (int kb = 0; kb < KB; kb++) {
+                        const int u = w * KB + kb, s = u % NS;
+                        const uint32_t ph = (uint32_t)((u / NS) & 1);
+                        ok = ok && mbar_wait_or(&full[s], ph, abort_flag);
+                        if (!lat) {
+                            ok = ok && mbar_wait_or(&gfull[s], ph, abort_flag);
+                            fence_proxy_async();  // the gathered rows (generic proxy) before the MMA's reads
                         }
-                        mma_commit(&empty[s]);
+                        ok = __all_sync(0xffffffffu, ok);
+                        if (!ok) break;
+                        tc_fence_after();
+                        if (elect_one()) {
+                            const uint64_t ad = a0 + (uint64_t)((uint32_t)s * (C::STAGE / 16)), bd = ad + B0;
+                            const uint32_t first = (start && kb == 0) ? 0u : 1u;
+                            // k-steps of 16 coefficients holding any of the p^2 real ones
+                            constexpr int KS = PACK ? NP / 16 : 4;
+                            const int ks = min(KS, (PP - kb * 64 + 15) >> 4);
+#pragma unroll
+                            for (int k = 0; k < KS; k++) {
+                                if (k >= ks) break;
+                                const uint32_t acc = k == 0 ? first : 1u;
+                                // A_hi [T_hi ; T_lo] -> main | correction, then A_lo T_hi -> correction
+                                if (PACK) {
+                                    mma_f16(dmain, ad + 2 * k, bd + 2 * k, id_half, acc);
+                                    mma_f16(dcorr, ad + 2 * k, bd + LO + 2 * k, id_half, acc);
+                                } else {
+                                    mma_f16(dmain, ad + 2 * k, bd + 2 * k, id_full, acc);
+                                }
+                                mma_f16(dcorr, ad + LO + 2 * k, bd + 2 * k, id_half, 1u);
+                            }
+                            mma_commit(&empty[s]);
+                        }
+                        __syncwarp();
                     }
+                    if (ok && (gi % C::GV == C::GV - 1 || w + NM >= nv) && elect_one()) mma_commit(&acc_full[b]);
                     __syncwarp();
                 }
-                if (ok && (gi % C::GV == C::GV - 1 || w + NM >= nv) && elect_one()) mma_commit(&acc_full[b]);
-                __syncwarp();
+                if (!ok) atomicExch(abort_flag, 1);
+                // every commit has arrived before the shared memory goes away
+                if (elect_one()) mma_commit(&fin[m]);
+                mbar_wait(&fin[m], 0);
             }
-            if (!ok) atomicExch(abort_flag, 1);
-            // every commit has arrived before the shared memory goes away
-            if (elect_one()) mma_commit(&fin[m]);
-            mbar_wait(&fin[m], 0);
-        }
-        __syncwarp();
-    } else if (warp >= C::P_WARP) {
-        // ------------------------------------------------------ producer warps
-        const int pw = warp - C::P_WARP;
-        if (lane == 0 && nunits > pw) {
-            int ox = 0, oy = 0, oz = 0;  // tile origin in halved coordinates
-            const int obx = td.octant & 1, oby = (td.octant >> 1) & 1, obz = (td.octant >> 2) & 1;
-            const unsigned char *lmap = nullptr;
-            if (lat) {
-                // its first position, 128 td.block in Morton order
-                const unsigned k = (unsigned)td.block * C::M;
-                ox = (int)every_third(k);
-                oy = (int)every_third(k >> 1);
-                oz = (int)every_third(k >> 2);
-                lmap = J.lat_maps + 128 * l;
-            }
-            const unsigned char *ttab = J.ttab;
-            int issued = pw;  // first unit of this producer not issued
-            int4 vn = st[e0 + pw / KB];
-            for (int u = pw; u < nunits; u += NM) {
-                const int s = u % NS, kb = u % KB;
-                const int4 v = vn;
-                if (u + NM < nunits) vn = st[e0 + (u + NM) / KB];
-                if (u >= NS && !mbar_wait_or(&empty[s], (uint32_t)((u / NS - 1) & 1), abort_flag)) {
-                    atomicExch(abort_flag, 1);
-                    break;
-                }
-                const uint32_t sa = smem_u32(base + s * C::STAGE);
-                mbar_arrive_tx(&full[s], C::B_BYTES + (lat ? C::A_BYTES : 0));
+            __syncwarp();
+        } else {
+            // ------------------------------------------------------ producer warps
+            const int pw = warp - C::P_WARP;
+            if (lane == 0 && pw < NM && nunits > pw) {
+                int ox = 0, oy = 0, oz = 0;  // tile origin in halved coordinates
+                const int obx = td.octant & 1, oby = (td.octant >> 1) & 1, obz = (td.octant >> 2) & 1;
+                const unsigned char *lmap = nullptr;
                 if (lat) {
-                    // source octant bits and the block's shift in halved
-                    // coordinates (arithmetic shifts: floor division by 2)
-                    const int sx = obx + v.x, sy = oby + v.y, sz = obz + v.z;
-                    const int ps = (sx & 1) | ((sy & 1) << 1) | ((sz & 1) << 2);
-                    const int x = ox + (sx >> 1), y = oy + (sy >> 1), z = oz + (sz >> 1);
-                    tma_load_5d(sa, lmap, kb * (C::ROWB / 2), x, y, z, ps, &full[s]);
-                    if (!PACK) tma_load_5d(sa + 16384, lmap, kb * (C::ROWB / 2) + 64, x, y, z, ps, &full[s]);
+                    // its first position, 128 td.block in Morton order
+                    const unsigned k = (unsigned)td.block * C::M;
+                    ox = (int)every_third(k);
+                    oy = (int)every_third(k >> 1);
+                    oz = (int)every_third(k >> 2);
+                    lmap = J.lat_maps + 128 * l;
                 }
-                bulk_g2s(sa + C::A_BYTES, ttab + ((size_t)(v.w & 0xffff) * KB + kb) * C::B_BYTES, C::B_BYTES, &full[s]);
-                issued = u + NM;
+                const unsigned char *ttab = J.ttab;
+                int issued = pw;  // first unit of this producer not issued
+                int4 vn = st[e0 + pw / KB];
+                for (int u = pw; u < nunits; u += NM) {
+                    const int s = u % NS, kb = u % KB;
+                    const int4 v = vn;
+                    if (u + NM < nunits) vn = st[e0 + (u + NM) / KB];
+                    if (u >= NS && !mbar_wait_or(&empty[s], (uint32_t)((u / NS - 1) & 1), abort_flag)) {
+                        atomicExch(abort_flag, 1);
+                        break;
+                    }
+                    const uint32_t sa = smem_u32(base + s * C::STAGE);
+                    mbar_arrive_tx(&full[s], C::B_BYTES + (lat ? C::A_BYTES : 0));
+                    if (lat) {
+                        // source octant bits and the block's shift in halved
+                        // coordinates (arithmetic shifts: floor division by 2)
+                        const int sx = obx + v.x, sy = oby + v.y, sz = obz + v.z;
+                        const int ps = (sx & 1) | ((sy & 1) << 1) | ((sz & 1) << 2);
+                        const int x = ox + (sx >> 1), y = oy + (sy >> 1), z = oz + (sz >> 1);
+                        tma_load_5d(sa, lmap, kb * (C::ROWB / 2), x, y, z, ps, &full[s]);
+                        if (!PACK) tma_load_5d(sa + 16384, lmap, kb * (C::ROWB / 2) + 64, x, y, z, ps, &full[s]);
+                    }
+                    bulk_g2s(sa + C::A_BYTES, ttab + ((size_t)(v.w & 0xffff) * KB + kb) * C::B_BYTES, C::B_BYTES, &full[s]);
+                    issued = u + NM;
+                }
+                // copies still in flight when the pipeline stopped early land
+                // before the shared memory goes away (bounded waits)
+                if (*(volatile int *)abort_flag)
+                    for (int u = pw; u < issued; u += NM)
+                        if (u + NS >= issued) mbar_wait(&full[u % NS], (uint32_t)((u / NS) & 1));
             }
-            // copies still in flight when the pipeline stopped early land
-            // before the shared memory goes away (bounded waits)
-            if (*(volatile int *)abort_flag)
-                for (int u = pw; u < issued; u += NM)
-                    if (u + NS >= issued) mbar_wait(&full[u % NS], (uint32_t)((u / NS) & 1));
+            __syncwarp();
         }
-        __syncwarp();
     } else {
         // ---------------------------------------------------------- worker warps
+        if constexpr (!PERSIST && C::REGS) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::REG_W));
         constexpr int HN = C::HN;
         const int row = tid & 127, g = (tid >> 7) & 1;  // target row and group
         float acc_hi[HN], acc_lo[HN];
@@ -890,6 +902,13 @@ static void launch_tc(int p, int grid, const M2LJob &one, const M2LJob *jobs, in
         m2l_tc_k<NP, true><<<grid, C::NT, C::SMEM, s>>>(p, one, jobs, njobs, queue, err);
     } else {
         ensure_smem((const void *)m2l_tc_k<NP, false>, C::SMEM);
+        // the workers' registers come out of the launch's: with fewer they would wait for ever
+        static const bool fits = [] {
+            cudaFuncAttributes a;
+            return cudaFuncGetAttributes(&a, (const void *)m2l_tc_k<NP, false>) == cudaSuccess &&
+                   a.numRegs * C::NT >= 32 * (C::NW * C::REG_W + 4 * C::REG_O);
+        }();
+        if (C::REGS && !fits) throw Error{FMM_ECUDA, "tensor-core M2L: too few registers at launch"};
         m2l_tc_k<NP, false><<<grid, C::NT, C::SMEM, s>>>(p, one, jobs, njobs, queue, err);
     }
 }
