@@ -96,10 +96,14 @@ struct HashSlot {
 // per-level lookup from lattice position to cell index (M2L stencil)
 struct LevelDesc {
     int start, end;         // cell index range of the level
-    long long map_off;      // offset of a dense map (8^l int32) in the map pool, or -1
-    const HashSlot *hash;   // levels without a dense map: a table of at least twice their cells, or null
+    long long map_off;      // offset of a dense map (8^l int32) or of the level's bricks in the map pool, or -1
+    const HashSlot *hash;   // levels without either: a table of at least twice their cells, or null
     unsigned hash_mask;     // table size - 1 (a power of two)
-    int pad;
+    // up > 0: the map is made of bricks, one of 8^up positions for every cell
+    // of the level `up` above (its cells from top_start on, its dense map at top_off)
+    int up;
+    long long top_off;
+    int top_start, pad;
 };
 
 // M2L tile: up to TILE target cells of one level and one octant, or (octant
@@ -441,7 +445,12 @@ __device__ inline int level_lookup(const LevelDesc &L, const int *__restrict__ m
     const int side = 1 << l;
     if (x < 0 || y < 0 || z < 0 || x >= side || y >= side || z >= side) return -1;
     const uint64_t k = morton3((uint32_t)x, (uint32_t)y, (uint32_t)z);
-    if (L.map_off >= 0) return map_pool[L.map_off + (long long)k];
+    if (L.map_off >= 0) {
+        if (L.up == 0) return map_pool[L.map_off + (long long)k];
+        const int a = map_pool[L.top_off + (long long)(k >> (3 * L.up))];
+        const uint64_t low = k & ((1ull << (3 * L.up)) - 1ull);
+        return a < 0 ? -1 : map_pool[L.map_off + ((long long)(a - L.top_start) << (3 * L.up)) + (long long)low];
+    }
     if (L.hash) {
         // linear probing from the key's hash; the table is at most half full
         const unsigned long long key = k + 1;

@@ -86,9 +86,6 @@ namespace fmm {
 
 static inline unsigned nblk(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
-// source index of an absent cell, copied like a lattice-map entry
-__device__ int g_no_cell = -1;
-
 // ---------------------------------------------------------------------------
 // tile geometry
 // ---------------------------------------------------------------------------
@@ -112,8 +109,8 @@ struct TcCfg {
     static constexpr int A_BYTES = M * ROWB;
     static constexpr int B_BYTES = (PACK ? 1 : 2) * NP * 128;
     static constexpr int STAGE = A_BYTES + B_BYTES;
-    static constexpr int QU = 8;                   // lookahead of the source lookups (units of the group)
-    static constexpr int RINGU = 2 * QU;
+    static constexpr int QU = 7;                   // lookahead of either read of a source lookup (units of the group)
+    static constexpr int RINGU = 16;               // slots, more than 2 QU
     static constexpr int RING = NG * RINGU * M * 4;
     static constexpr int BAR = 768;                // mbarriers (first 512 bytes), then the CTA's job
     static constexpr int NS_FIT = (226 * 1024 - RING - BAR - 1024) / STAGE;
@@ -527,15 +524,35 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
             const unsigned char *__restrict__ mrow = J.mrow;
             const int nown = nunits > g ? (nunits - g + 1) / 2 : 0;  // units u = g, g + 2, ... of this group
             int *myring = ring + g * RINGU * C::M;
-            const bool dense = LD.map_off >= 0;  // the level has a lattice map: lookups arrive by cp.async
+            const bool dense = LD.map_off >= 0;  // the level has a map: lookups arrive by cp.async
             const bool whole = rl <= 10 && LD.end - LD.start == (1 << (3 * rl));  // every lattice cell present
+            const bool bricks = dense && !whole && LD.up > 0;  // a map in bricks: the ancestor's cell first, then the brick's entry
+            const bool two = __any_sync(0xffffffffu, bricks);
             // source cell of this row for the group's unit j, looked up QU units
             // ahead into ring slot j % RINGU (cp.async of the lattice-map entry,
-            // or a search of the level's keys); only this thread reads the slot
-            // stencil entry of the group's unit j; the next call's entry is
-            // loaded one call ahead (calls come in order), so its latency is hidden
-            int4 st_next = make_int4(0, 0, 0, 0);
-            int st_next_j = -1;
+            // or a search of the level's keys); only this thread reads the slot.
+            // Of a map in bricks `first` brings the ancestor's cell 2 QU units ahead.
+            // The stencil entry of the next call is loaded one call ahead (calls
+            // come in order), so its latency is hidden
+            int4 st_next = make_int4(0, 0, 0, 0), st_first = make_int4(0, 0, 0, 0);
+            int st_next_j = -1, st_first_j = -1;
+            const unsigned side = 1u << rl;
+            auto first = [&](int j) {
+                if (!two || j >= nown) return;
+                const int4 v = st_first_j == j ? st_first : st[e0 + (2 * j + g) / KB];
+                if (j + 1 < nown) {
+                    st_first = st[e0 + (2 * (j + 1) + g) / KB];
+                    st_first_j = j + 1;
+                }
+                if (!bricks || cell < 0) return;
+                int *const slot = myring + (j % RINGU) * C::M + row;
+                const int x = px + v.x, y = py + v.y, z = pz + v.z;
+                if (((v.w >> (16 + ro)) & 1) && (unsigned)x < side && (unsigned)y < side && (unsigned)z < side)
+                    cp_async4(smem_u32(slot), map_pool + LD.top_off +
+                                                  morton3_10((uint32_t)(x >> LD.up), (uint32_t)(y >> LD.up), (uint32_t)(z >> LD.up)));
+                else
+                    *slot = -1;
+            };
             auto fetch = [&](int j) {
                 if (j >= nown) return;
                 const int4 v = st_next_j == j ? st_next : st[e0 + (2 * j + g) / KB];
@@ -546,24 +563,35 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
                 int *const slot = myring + (j % RINGU) * C::M + row;
                 int r = -1;
                 if (cell >= 0) {
-                    const int x = px + v.x, y = py + v.y, z = pz + v.z, side = 1 << rl;
-                    if (((v.w >> (16 + ro)) & 1) && x >= 0 && y >= 0 && z >= 0 && x < side && y < side && z < side) {
+                    const int x = px + v.x, y = py + v.y, z = pz + v.z;
+                    if (bricks) {
+                        const int a = *slot;
+                        const uint32_t m = (1u << LD.up) - 1u;
+                        if (a >= 0)
+                            cp_async4(smem_u32(slot), map_pool + LD.map_off + ((long long)(a - LD.top_start) << (3 * LD.up)) +
+                                                          morton3_10((uint32_t)x & m, (uint32_t)y & m, (uint32_t)z & m));
+                        return;
+                    }
+                    if (((v.w >> (16 + ro)) & 1) && (unsigned)x < side && (unsigned)y < side && (unsigned)z < side) {
                         // a complete level holds every lattice cell in Morton order:
                         // the index follows from the position
+                        const uint32_t k = morton3_10((uint32_t)x, (uint32_t)y, (uint32_t)z);
                         if (whole) {
-                            *slot = LD.start + (int)morton3_10((uint32_t)x, (uint32_t)y, (uint32_t)z);
+                            *slot = LD.start + (int)k;
                             return;
                         }
                         if (dense) {
-                            cp_async4(smem_u32(slot), map_pool + LD.map_off + (long long)morton3((uint32_t)x, (uint32_t)y, (uint32_t)z));
+                            cp_async4(smem_u32(slot), map_pool + LD.map_off + k);
                             return;
                         }
                         r = level_lookup(LD, map_pool, J.anchor, rl, x, y, z);
                     }
                 }
-                if (dense && !whole) cp_async4(smem_u32(slot), &g_no_cell);
-                else *slot = r;
+                *slot = r;
             };
+            for (int j = 0; j < 2 * QU; j++) first(j);
+            cp_async_commit();
+            cp_async_wait_all();
             for (int j = 0; j < QU; j++) fetch(j);
             cp_async_commit();
             cp_async_wait_all();
@@ -601,6 +629,7 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
                                colp + (size_t)(sc >= 0 ? sc : 0) * (KB * C::ROWB), sc >= 0 ? 16u : 0u);
                 }
                 fetch(j + QU);
+                first(j + 2 * QU);
                 cp_async_arrive_noinc(&gfull[s]);
                 cp_async_commit();
             }

@@ -1374,7 +1374,19 @@ __global__ void map_fill_k(int ls, int le, int l, const uint64_t *__restrict__ a
     map[anchor[c] >> (3 * (FMM_MAXLEVEL - l))] = c;
 }
 
-// the cells of a level without a dense map into its open-addressed table
+// the cells of a level into the bricks of their ancestors `up` levels above,
+// whose dense map is `top`
+__global__ void brick_fill_k(int ls, int le, int l, int up, int top_start, const uint64_t *__restrict__ anchor,
+                             const int *__restrict__ top, int *__restrict__ bricks)
+{
+    int c = ls + blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= le) return;
+    const uint64_t k = anchor[c] >> (3 * (FMM_MAXLEVEL - l));
+    const int a = top[k >> (3 * up)];
+    bricks[((long long)(a - top_start) << (3 * up)) + (long long)(k & ((1ull << (3 * up)) - 1ull))] = c;
+}
+
+// the cells of a level without a map into its open-addressed table
 // (linear probing; at most half full, so every insertion finds a slot)
 __global__ void hash_fill_k(int ls, int le, int l, const uint64_t *__restrict__ anchor, HashSlot *__restrict__ tab,
                             unsigned mask)
@@ -1899,10 +1911,28 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
             ld[l].start = l <= depth ? h->lvl_start[l] : ncells;
             ld[l].end = l <= depth ? h->lvl_start[l + 1] : ncells;
             ld[l].map_off = -1;
+            ld[l].up = 0;
             if (l >= 2 && l <= depth && l <= FMM_DENSE_MAP_MAXLEVEL) {
                 ld[l].map_off = pool;
                 pool += 1LL << (3 * l);
             }
+        }
+        // deeper levels: bricks below the cells of the last dense level, while
+        // all of them together are no larger than its map (64 MB). A lookup is two
+        // reads of known addresses, which the tensor-core M2L has in flight ahead
+        // of use; a search of a table stalls its thread until it ends. N = 1e6
+        // Plummer, whose levels 9 and 10 hold half of the cells: M2L 8.2 -> 7.6 ms.
+        const int top = FMM_DENSE_MAP_MAXLEVEL;
+        const long long dense_end = pool;
+        for (int l = top + 1; l <= depth; l++) {
+            if (l - top > top) break;  // (8^top positions a brick, the limit)
+            const long long words = (long long)(ld[top].end - ld[top].start) << (3 * (l - top));
+            if (pool - dense_end + words > 1LL << (3 * top)) break;
+            ld[l].map_off = pool;
+            ld[l].up = l - top;
+            ld[l].top_off = ld[top].map_off;
+            ld[l].top_start = ld[top].start;
+            pool += words;
         }
         h->map_pool.ensure(sizeof(int) * (size_t)std::max<long long>(pool, 1));
         if (pool > 0) FMM_CUDA_TRY(cudaMemsetAsync(h->map_pool.p, 0xff, sizeof(int) * (size_t)pool, s));
@@ -1913,14 +1943,22 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
                                                      h->map_pool.as<int>() + ld[l].map_off);
             count_launch(h);
         }
-        // deeper levels: hash tables of at least twice their cells
+        for (int l = top + 1; l <= depth && ld[l].map_off >= 0; l++) {
+            const int m = ld[l].end - ld[l].start;
+            if (m == 0) continue;
+            brick_fill_k<<<nblocks(m, TB), TB, 0, s>>>(ld[l].start, ld[l].end, l, ld[l].up, ld[l].top_start,
+                                                       h->c_anchor.as<uint64_t>(), h->map_pool.as<int>() + ld[l].top_off,
+                                                       h->map_pool.as<int>() + ld[l].map_off);
+            count_launch(h);
+        }
+        // the levels left: hash tables of at least twice their cells
         std::vector<long long> hoff(FMM_MAXLEVEL + 1, -1);
         long long hpool = 0;
         for (int l = FMM_DENSE_MAP_MAXLEVEL + 1; l <= depth; l++) {
             const long long m = ld[l].end - ld[l].start;
             ld[l].hash = nullptr;
             ld[l].hash_mask = 0;
-            if (m == 0) continue;
+            if (m == 0 || ld[l].map_off >= 0) continue;
             long long t = 64;
             while (t < 2 * m) t <<= 1;
             hoff[l] = hpool;
