@@ -53,7 +53,7 @@
 // from L2 at 69 bytes per clock and SM; without the MMAs the launch takes 6.75
 // ms.
 // p = 9 .. 11 (60 KB stages, three of them, one MMA warp): the waits and
-// commits between the units, 3.0 ms at N = 1e6, p = 10 (6.6 with TF32).
+// commits between the units, 2.66 ms at N = 1e6, p = 10 (6.6 with TF32).
 //
 // A tree with few tiles (5 at N = 16,384) would leave most SMs idle: the
 // vectors of every tile are then cut into nsplit ranges, one CTA each

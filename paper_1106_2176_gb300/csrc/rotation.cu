@@ -255,8 +255,8 @@ void m2l_rotation_ref(int p, const double u[3], const double *M, double *L)
 // current one is translated.
 //
 // Bound: FP32 by instruction issue (a map's 16 bytes are one load and two packed
-// multiply-adds), FP64 by GB300's FP64 pipe. N = 60,001, p = 16, FP32: 8.3 ms;
-// N = 50,000, p = 8, FP64: 18.4 ms. One warp per two targets with lanes over a
+// multiply-adds), FP64 by GB300's FP64 pipe. N = 60,001, p = 16, FP32: 7.9 ms;
+// N = 50,000, p = 8, FP64: 18.2 ms. One warp per two targets with lanes over a
 // map's outputs (32 rows apart in shared memory: bank conflicts) took 39.7 and
 // 34.3 ms.
 // ---------------------------------------------------------------------------
@@ -779,6 +779,14 @@ __global__ void __launch_bounds__(256) rot_scale_k(const T *__restrict__ M, int 
     CM[i - k + o] = M[i] * ck[o];
 }
 
+// Lookups on levels without a dense map, kept out of the kernel's registers: N
+// = 60,001, p = 16 takes 7.9 ms, with them in line 8.5.
+static __device__ __noinline__ int rot_lookup(const LevelDesc *L, const int *map_pool, const uint64_t *anchor, int l, int x, int y,
+                                              int z)
+{
+    return level_lookup(*L, map_pool, anchor, l, x, y, z);
+}
+
 // W warps, NQ >= p (p + 1) / 2 / W coefficient pairs per warp
 template <class T, int W, int NQ>
 __global__ void __launch_bounds__(32 * W, W == 8 ? 2 : NQ > 9 ? 3 : 4)
@@ -817,8 +825,12 @@ __global__ void __launch_bounds__(32 * W, W == 8 ? 2 : NQ > 9 ? 3 : 4)
         const int n = P.nm[q][0], m = P.nm[q][1];
         s_pair[q] = make_int4(rot_idx(n, 0, m) * ROT_LD, rot_idx(n, m ? 1 : 0, m ? m - 1 : 0) * ROT_LD, 2 * m, 0);
     }
-    const LevelDesc LD = J.ld[rl];
-    const bool whole = rl <= 10 && LD.end - LD.start == (1 << (3 * rl));  // every lattice cell present
+    // source lookups: the first cell of a level with every lattice cell, the
+    // level's dense map, or neither (-1)
+    const LevelDesc *ld = J.ld + rl;
+    const bool whole = rl <= 10 && ld->end - ld->start == (1 << (3 * rl));
+    const int start = ld->start;
+    const int *const map = ld->map_off >= 0 && ld->up == 0 ? J.map_pool + ld->map_off : nullptr;
     S acc[2 * NQ];
 #pragma unroll
     for (int k = 0; k < 2 * NQ; k++) acc[k].zero();
@@ -839,8 +851,9 @@ __global__ void __launch_bounds__(32 * W, W == 8 ? 2 : NQ > 9 ? 3 : 4)
                 const int qx = px + v.x, qy = py + v.y, qz = pz + v.z;
                 const unsigned side = 1u << rl;
                 if ((unsigned)qx < side && (unsigned)qy < side && (unsigned)qz < side)
-                    b = whole ? LD.start + (int)morton3_10((uint32_t)qx, (uint32_t)qy, (uint32_t)qz)
-                              : level_lookup(LD, J.map_pool, J.anchor, rl, qx, qy, qz);
+                    b = whole ? start + (int)morton3_10((uint32_t)qx, (uint32_t)qy, (uint32_t)qz)
+                        : map ? map[morton3_10((uint32_t)qx, (uint32_t)qy, (uint32_t)qz)]
+                              : rot_lookup(ld, J.map_pool, J.anchor, rl, qx, qy, qz);
             }
             if (__any_sync(0xffffffffu, b >= 0)) {
                 id = v.w & 0xffff;
