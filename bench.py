@@ -219,13 +219,13 @@ def p2p_traffic(interactions, n):
         return None
 
 
-def phase_rooflines(phase, st, N, p, peaks, fp32_peak, tf32_peak):
+def phase_rooflines(phase, st, N, p, peaks, fp32_peak):
     """Achieved rates of the phases other than P2P, from algorithmic bytes or
     flops per phase (the minimal work each phase must do, FP32 storage). The
     tree, M2M, L2L and the combine move data: HBM-bound, against the measured
     copy bandwidth. P2M and L2P run the regular-harmonic recurrences per
     particle: ALU-bound, against the measured FP32 FMA peak. M2L against the
-    measured TF32 tensor-core peak."""
+    measured rate of a 16-bit tensor-core GEMM."""
     pp4 = 4 * p * p  # bytes of one expansion
     ntri = p * (p + 1) // 2  # (n, m >= 0) terms
     nc, nl = st["ncells"], st["nleaves"]
@@ -262,10 +262,11 @@ def phase_rooflines(phase, st, N, p, peaks, fp32_peak, tf32_peak):
     flops = 2.0 * p ** 4 * st["n_m2l_pairs"]
     if phase["ms_m2l"] > 0:
         tf = flops / (phase["ms_m2l"] / 1000.0) / 1e12
-        out["m2l"] = {"bound": "tensor", "flops": flops, "ms": phase["ms_m2l"], "achieved": tf, "peak": tf32_peak,
-                      "unit": "TFLOP/s", "frac": tf / tf32_peak,
-                      "note": "useful 2 p^4 flop per pair against the measured TF32 MMA peak; the split-TF32 "
-                              "scheme issues 3 MMA passes of it"}
+        fp16 = float(peaks.get("bf16_tflops", 1895.0))
+        out["m2l"] = {"bound": "tensor", "flops": flops, "ms": phase["ms_m2l"], "achieved": tf, "peak": fp16,
+                      "unit": "TFLOP/s", "frac": tf / fp16,
+                      "note": "useful 2 p^4 flop per pair against the measured 16-bit GEMM rate (bf16, burst); the "
+                              "split-FP16 scheme issues 3 products of it"}
     return out
 
 
@@ -461,7 +462,7 @@ def run_diff(a, dev):
 def run_m2l_engines(a, dev):
     """M2L launch time of each engine at p = 8, 10, 16 on one uniform cube
     (theta = 0.5, ncrit = 64, FP32 inputs, mixed precision, far and near field
-    in turn so the M2L events time the phase alone): the split-TF32 tensor-core
+    in turn so the M2L events time the phase alone): the split-FP16 tensor-core
     contraction (p <= 11), the dense CUDA-core contraction and the rotation
     engine. Error: relative L2 of phi on 512 sampled targets against the
     library's FP64 direct sum."""
@@ -540,13 +541,12 @@ def main():
         f.evaluate(phi, grad)
     torch.cuda.synchronize()
 
-    # measured peaks of the FP32 FMA pipe (scalar and packed pairs) and of
-    # the TF32 tensor-core MMA: the denominators of the roofline fractions
+    # measured peaks of the FP32 FMA pipe (scalar and packed pairs), the
+    # denominator of the P2P's roofline fraction, and of the TF32 MMA
     from paper_1106_2176_gb300.fmm import measure_peak
     pk = {"fp32_fma": measure_peak("fp32"), "fp32x2_fma": measure_peak("fp32x2"),
           "tf32_mma_n128": measure_peak("tf32", 128), "tf32_mma_n256": measure_peak("tf32", 256)}
     fp32_peak = max(pk["fp32_fma"], pk["fp32x2_fma"])
-    tf32_peak = max(pk["tf32_mma_n128"], pk["tf32_mma_n256"])
     torch.cuda.synchronize()
 
     stream = torch.cuda.current_stream()
@@ -656,7 +656,7 @@ def main():
                 "peak_nominal": peak_nominal, "frac_nominal": achieved / peak_nominal,
                 "peak_nominal_note": "%d SMs x 128 lanes x 2 flop x %.0f MHz (max SM clock)" % (nsm, sm_max),
                 "peaks_measured_tflops": pk, "interactions": inter, "p2p_ms": p2p_avg}
-    phases_roof = phase_rooflines(phase, st1, N, a.p, peaks, fp32_peak, tf32_peak)
+    phases_roof = phase_rooflines(phase, st1, N, a.p, peaks, fp32_peak)
 
     cpu = None
     if rank == 0 and world == 1 and not a.no_cpu_baseline:
