@@ -260,7 +260,7 @@ struct fmm_ctx {
     int rot_nv = -1, rot_kind = 0;  // vectors and precision (1 FP32, 2 FP64) of rot_tab
     fmm::DevBuf msplit;         // M~ split into FP16 (hi, lo) rows for the tensor-core M2L
     fmm::DevBuf m2l_ws, m2l_part;  // its level maxima and tile counters; sums of the ranges of split tiles
-    int m2l_nsplit = 1, m2l_chunk = 0;  // ranges per tile and their length (m2l_plan)
+    int m2l_nsplit = 1, m2l_chunk = 0;  // ranges per tile and their length (m2l_plan, rotation_plan)
     // tensor-core M2L on lattice levels: the rows of each such level in lattice
     // order (octant bits, then z, y, x of the halved position), one TMA tensor
     // map per level (device copy and its pinned staging)
@@ -344,6 +344,7 @@ template <class T>
 void m2l_rotation(fmm_ctx *h, T *L, const T *M);  // same-level M2L of all tiles by rotation
 bool rotation_m2l_supported(fmm_ctx *h);           // p <= 16 (the maps of a vector fit shared memory)
 int rotation_tile_rows(fmm_ctx *h);  // target cells per tile
+void rotation_plan(fmm_ctx *h);      // (build) ranges per tile
 // per (octant, level): how many of the octant's entries (shortest first) can
 // reach a cell of that level in the current tree; written after the offsets
 void stencil_levels(fmm_ctx *h, cudaStream_t s);

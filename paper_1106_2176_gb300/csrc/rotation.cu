@@ -839,7 +839,7 @@ __global__ void __launch_bounds__(32 * W, W == 8 ? 2 : NQ > 9 ? 3 : 4)
     const int nvt = J.st_off[10 + td.octant * (FMM_MAXLEVEL + 1) + td.level];
     // (ranges of a fixed length: a cell's sums do not depend on its tile's list)
     int e = J.st_off[td.octant] + min(nvt, split * J.chunk);
-    const int e1 = J.st_off[td.octant] + min(nvt, (split + 1) * J.chunk);
+    const int e1 = J.st_off[td.octant] + (split + 1 < J.nsplit ? min(nvt, (split + 1) * J.chunk) : nvt);
 
     // next entry from e on that hits a cell of some lane (every warp finds the
     // same), with this lane's source cell
@@ -975,11 +975,17 @@ __global__ void __launch_bounds__(32 * W, W == 8 ? 2 : NQ > 9 ? 3 : 4)
 }
 
 // Ranges per tile: about 8 CTAs per SM, so that the tiles at the boundary of
-// the domain, which have fewer sources, even out, of 24 vectors or more.
-static int rot_nsplit(fmm_ctx *h, int nv)
+// the domain, which have fewer sources, even out, of 24 vectors or more. Part of
+// the build, which fixes the tiles (the pooling threshold may be set anew before
+// the next evaluation): the ranges cover the longest list of these tiles.
+void rotation_plan(fmm_ctx *h)
 {
-    const int want = (8 * h->nsm + h->ntiles_max - 1) / std::max(h->ntiles_max, 1);
-    return std::max(1, std::min(want, std::min(nv / 24, 32)));
+    if (h->engine_used != FMM_M2L_ROTATION) return;
+    const int nv = m2l_longest_list(h);
+    const int fill = (8 * h->nsm + h->ntiles_max - 1) / std::max(h->ntiles_max, 1);
+    const int want = std::max(1, std::min(fill, std::min(nv / 24, 32)));
+    h->m2l_chunk = (nv + want - 1) / want;
+    h->m2l_nsplit = (nv + h->m2l_chunk - 1) / h->m2l_chunk;
 }
 
 template <class T, int W, int NQ>
@@ -988,11 +994,9 @@ static void launch_rot(fmm_ctx *h, T *L, const T *M)
     const int p = h->p;
     const RotPlan P = rot_plan<T>(p, W);
     rotation_tables_update<T>(h, P);
-    const int nv = m2l_longest_list(h);
     RotJob j;
-    const int want = rot_nsplit(h, nv);
-    j.chunk = (nv + want - 1) / want;
-    j.nsplit = (nv + j.chunk - 1) / j.chunk;
+    j.chunk = h->m2l_chunk;
+    j.nsplit = h->m2l_nsplit;
     h->m2l_ws.ensure(sizeof(unsigned) * (size_t)h->ntiles_max);
     if (j.nsplit > 1) h->m2l_part.ensure(sizeof(double) * (size_t)h->ntiles_max * j.nsplit * p * (p + 1) * ROT_ROWS);
     FMM_CUDA_TRY(cudaMemsetAsync(h->m2l_ws.p, 0, sizeof(unsigned) * (size_t)h->ntiles_max, h->work));

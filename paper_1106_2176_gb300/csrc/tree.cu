@@ -2044,6 +2044,7 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
         check_launch("m2l tiles");
         lattice_prepare(h, s);
         m2l_plan(h);
+        rotation_plan(h);
     }
 }
 
