@@ -41,8 +41,9 @@ struct fmm_batch_s {
 namespace fmm {
 
 // misc: [0] up queue, [1] down queue, [2] M2L queue, [3] P2P queue,
-// [4] dependency waits (bit 0), [5] tensor-core M2L, [6] P2P
-enum { BQ_UP = 0, BQ_DN = 1, BQ_M2L = 2, BQ_P2P = 3, BE_DEP = 4, BE_M2L = 5, BE_P2P = 6, BMISC = 8 };
+// [4] dependency waits (bit 0), [5] tensor-core M2L, [6] P2P, [7] a system has
+// wide levels (m2l_norm.cuh)
+enum { BQ_UP = 0, BQ_DN = 1, BQ_M2L = 2, BQ_P2P = 3, BE_DEP = 4, BE_M2L = 5, BE_P2P = 6, B_WIDE = 7, BMISC = 8 };
 
 template <class T>
 static void upload(DevBuf &b, const std::vector<T> &v)
@@ -153,7 +154,8 @@ int fmm_batch_create(const fmm_handle *handles, int nsys, void *const *phi, void
             if (h->depth >= 2) {
                 M2LJob j = m2l_tensor_job(h, S.L);
                 S.rows = const_cast<unsigned char *>(j.mrow);
-                S.m2l_ws = const_cast<unsigned *>(j.lmax);
+                S.m2l_ws = const_cast<unsigned *>(j.ws);
+                S.m2l_cmax = const_cast<unsigned *>(j.cmax);
                 S.ws_words = j.ws_words;
                 int nt = 0;
                 FMM_CUDA_TRY(cudaMemcpy(&nt, j.ntiles, sizeof(int), cudaMemcpyDeviceToHost));
@@ -244,7 +246,7 @@ int fmm_batch_evaluate(fmm_batch b, void *stream)
         const BatchSys *sys = b->sys.as<BatchSys>();
         int *misc = b->misc.as<int>();
         fmm_ctx *h0 = b->hs[0];
-        FMM_CUDA_TRY(cudaMemsetAsync(misc + BE_DEP, 0, sizeof(int) * 3, s));
+        FMM_CUDA_TRY(cudaMemsetAsync(misc + BE_DEP, 0, sizeof(int) * 4, s));
         // the near field has no dependency on the far field: second stream
         FMM_CUDA_TRY(cudaEventRecord(b->fork, s));
         FMM_CUDA_TRY(cudaStreamWaitEvent(b->side, b->fork, 0));
@@ -252,9 +254,10 @@ int fmm_batch_evaluate(fmm_batch b, void *stream)
         FMM_CUDA_TRY(cudaEventRecord(b->join, b->side));
         batch_zero(b->p, sys, b->nsys, s);
         batch_up(b->p, b->nsm, sys, b->up.as<int4>(), b->n_up, misc + BQ_UP, h0->m2m_mat.as<float>(), misc + BE_DEP, s);
-        batch_split(b->p, sys, b->nsys, s);
+        unsigned *wide = reinterpret_cast<unsigned *>(misc + B_WIDE);
+        batch_split(b->p, sys, b->nsys, wide, s);
         if (b->n_jobs > 0)
-            m2l_tensor_jobs(b->p, b->nsm, b->jobs.as<M2LJob>(), b->n_jobs, misc + BQ_M2L, misc + BE_M2L, s);
+            m2l_tensor_jobs(b->p, b->nsm, b->jobs.as<M2LJob>(), b->n_jobs, misc + BQ_M2L, wide, misc + BE_M2L, s);
         batch_m2lx(b->p, sys, b->mx.as<int2>(), b->n_mx, s);
         batch_down(b->p, b->nsm, sys, b->dn.as<int4>(), b->n_dn, misc + BQ_DN, h0->l2l_mat.as<float>(), misc + BE_DEP, s);
         FMM_CUDA_TRY(cudaStreamWaitEvent(s, b->join, 0));

@@ -1838,7 +1838,7 @@ __global__ void __launch_bounds__(32 * MV_WARPS) batch_up_k(const BatchSys *__re
             m2m_parent_warp<NR>(item.z, lane, P * P, S.child, S.nchild, S.xyz, mat, S.M, sx[w]);
         }
         __syncwarp();
-        if (S.m2l_ws) m2l_row_max(S.M + (size_t)item.z * P * P, P * P, lane, S.m2l_ws + item.w);
+        if (S.m2l_ws) m2l_row_max(S.M + (size_t)item.z * P * P, P * P, lane, S.m2l_cmax + item.z, S.m2l_ws + item.w);
         if (lane == 0) batch_done(S.cnt_up + item.w);
     }
 }

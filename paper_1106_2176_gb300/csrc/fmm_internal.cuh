@@ -133,14 +133,16 @@ struct M2LJob {
     const unsigned char *ttab;  // operator image
     const int *rowexp;          // its power of two per output coefficient: L~ = 2^(rowexp - e) sums
     float *L;
-    const unsigned *lmax;       // per level: the bits of its largest coefficient (sets the rows' scale)
+    const float *M;             // M~ (the wide tiles' rows)
+    const unsigned *cmax;       // per cell: the bits of its largest coefficient
+    const unsigned *ws;         // workspace (m2l_norm.cuh): the levels' largest coefficients, which set the rows' scale, ...
     unsigned *tcnt;             // per tile: ranges finished (nsplit > 1)
     float2 *part;               // per (tile, range): its (hi, lo) sums (nsplit > 1)
     // 128-byte tensor map per level of the lattice copy of the rows, from which
     // lattice tiles read their sources by TMA tile loads (null: gather)
     const unsigned char *lat_maps;
     int nsplit, chunk;          // ranges of `chunk` vectors a tile's list is cut into, one CTA each
-    int ws_words;               // words of the workspace at lmax (maxima, counters) to zero per evaluation
+    int ws_words;               // its words, to zero per evaluation
     int item0;
     int count;
 };
@@ -177,7 +179,7 @@ struct BatchSys {
     float *phi, *grad;              // caller's order
     unsigned *cnt_up, *cnt_dn;      // per level: cells whose M (up) / L (down) is final
     unsigned char *rows;            // FP16 (hi, lo) rows of the tensor-core M2L, or null (no same-level M2L)
-    unsigned *m2l_ws;               // its per-level maxima, then tile counters: ws_words words
+    unsigned *m2l_ws, *m2l_cmax;    // its workspace of ws_words words, and the cells' largest coefficients
     int ws_words;
     int n, ncells, nleaves, depth, c0;  // c0: first cell of level 2
     int lvl_start[FMM_MAXLEVEL + 2];
@@ -259,7 +261,7 @@ struct fmm_ctx {
     size_t rot_vec_off = 0, rot_c_off = 0;  // entries before the vectors' data and the c_nm in rot_tab
     int rot_nv = -1, rot_kind = 0;  // vectors and precision (1 FP32, 2 FP64) of rot_tab
     fmm::DevBuf msplit;         // M~ split into FP16 (hi, lo) rows for the tensor-core M2L
-    fmm::DevBuf m2l_ws, m2l_part;  // its level maxima and tile counters; sums of the ranges of split tiles
+    fmm::DevBuf m2l_ws, m2l_cmax, m2l_part;  // its workspace, largest coefficient per cell, sums of the ranges of split tiles
     int m2l_nsplit = 1, m2l_chunk = 0;  // ranges per tile and their length (m2l_plan, rotation_plan)
     // tensor-core M2L on lattice levels: the rows of each such level in lattice
     // order (octant bits, then z, y, x of the halved position), one TMA tensor
@@ -371,7 +373,8 @@ void tensor_tables_init(fmm_ctx *h);
 bool tensor_m2l_supported(fmm_ctx *h);
 void m2l_tensor(fmm_ctx *h, float *L, const float *M);
 // the same-level M2L of several systems (same p; rows already split) in one persistent launch
-void m2l_tensor_jobs(int p, int nsm, const M2LJob *jobs_dev, int njobs, int *queue, int *err, cudaStream_t s);
+void m2l_tensor_jobs(int p, int nsm, const M2LJob *jobs_dev, int njobs, int *queue, const unsigned *any, int *err,
+                     cudaStream_t s);
 M2LJob m2l_tensor_job(fmm_ctx *h, float *L);  // the handle's arrays; allocates its workspaces
 int m2l_longest_list(fmm_ctx *h);              // vectors of the longest list a tile walks
 void m2l_plan(fmm_ctx *h);                     // (build) ranges per tile
@@ -379,7 +382,7 @@ void m2l_plan(fmm_ctx *h);                     // (build) ranges per tile
 // lattice buffer and tensor maps
 void lattice_select(fmm_ctx *h, int pool_max);
 void lattice_prepare(fmm_ctx *h, cudaStream_t s);
-void batch_split(int p, const BatchSys *sys, int nsys, cudaStream_t s);  // every system's FP16 rows
+void batch_split(int p, const BatchSys *sys, int nsys, unsigned *any, cudaStream_t s);  // every system's FP16 rows
 
 // p2p.cu
 void near_field(fmm_ctx *h, cudaStream_t s);  // P2P into h->near

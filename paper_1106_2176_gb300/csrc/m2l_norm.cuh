@@ -74,14 +74,50 @@ __device__ __forceinline__ int m2l_exponent(unsigned mag)
 // 2^e, -126 <= e <= 127
 __device__ __forceinline__ float m2l_pow2(int e) { return __uint_as_float((unsigned)(e + 127) << 23); }
 
-// the row maximum of one cell (by one warp, after its row is written) into its
-// level's: a plain read first, so that almost no cell needs the atomic
-__device__ __forceinline__ void m2l_row_max(const float *Mc, int PP, int lane, unsigned *lmax)
+// the row maximum of one cell (by one warp, after its row is written) to *cmax
+// and into its level's: a plain read first, so that almost no cell needs the atomic
+__device__ __forceinline__ void m2l_row_max(const float *Mc, int PP, int lane, unsigned *cmax, unsigned *lmax)
 {
     unsigned best = 0;
     for (int k = lane; k < PP; k += 32) best = max(best, m2l_mag(__ldcg(Mc + k) * m2l_norm(k)));
     best = __reduce_max_sync(0xffffffffu, best);
-    if (lane == 0 && best > *(volatile unsigned *)lmax) atomicMax(lmax, best);
+    if (lane != 0) return;
+    *cmax = best;
+    if (best > *(volatile unsigned *)lmax) atomicMax(lmax, best);
+}
+
+// Workspace of one evaluation, zero before it: the level maxima (word l), which
+// levels are wide (bit l), and the tiles' counters.
+constexpr int M2LW_WIDE = 24, M2LW_CNT = 32;
+
+// FP16 rounds a row scaled with its level to 2^-40 of the level's largest
+// coefficient: a cell within 2^-16 of it keeps 2^-24 of its own largest
+// coefficient, FP32's rounding, a lower one fewer bits.
+constexpr int M2L_SPAN = 16;
+
+// Whether the lost bits may show at a target cell c of level l: an expansion whose
+// largest coefficient is a is a potential of about a / w one cell width w away, so
+// the potential at c is about the largest a / w of c and its ancestors (the root's:
+// the whole system as seen from afar) or more, and FP32 leaves 2^-24 of that open
+// anyway. Exposed: 2^-16 of the level's largest a / w and less. (N = 10^6 Plummer:
+// 43 of 60,000 cells lie 2^-16 and more below their level's largest; none is exposed.)
+__device__ inline bool m2l_exposed(int c, int l, unsigned lmax, const unsigned *cmax, const int *parent)
+{
+    const int need = (int)(lmax >> 23) - M2L_SPAN + l;
+    if ((int)(cmax[c] >> 23) + l > need || (int)(cmax[0] >> 23) > need) return false;
+    for (int a = parent[c], la = l - 1; a > 0; a = parent[a], la--)
+        if ((int)(cmax[a] >> 23) + la > need) return false;
+    return true;
+}
+
+// marks cell c's level l in the workspace (and *any) if it is exposed
+__device__ inline void m2l_mark(int c, int l, const unsigned *cmax, const int *parent, unsigned *ws, unsigned *any)
+{
+    const unsigned lm = ws[l];
+    if ((int)(lm >> 23) - (int)(cmax[c] >> 23) < M2L_SPAN || ((*(volatile unsigned *)(ws + M2LW_WIDE) >> l) & 1u)) return;
+    if (!m2l_exposed(c, l, lm, cmax, parent)) return;
+    atomicOr(ws + M2LW_WIDE, 1u << l);
+    if (any) atomicOr(any, 1u);
 }
 
 }  // namespace fmm

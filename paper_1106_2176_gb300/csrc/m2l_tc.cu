@@ -23,8 +23,11 @@
 //     entries of every degree's rows lie in [2^13, 2^14);
 //   - a level's rows are multiplied by 2^e so that the largest coefficient of
 //     the level lies in [2^14, 2^15) (e from a maximum taken each evaluation).
-// FP16's subnormals end 2^-39 below that maximum, 15 bits below the rounding
-// of the FP32 sums. Every GV vectors an accumulator is drained into
+// FP16's subnormals end 2^-39 below that maximum: a cell far below its level's
+// largest keeps fewer bits than FP32. Where that may show, at targets all of
+// whose surroundings are 2^-16 below (weak charges far from strong ones that
+// cancel: m2l_exposed), the level is "wide" and its tiles are summed in FP32 on
+// the CUDA cores (m2l_wide_tile). Every GV vectors an accumulator is drained into
 // per-thread FP32 (hi, lo) TwoSum registers.
 //
 // Per CTA (two groups of 4 worker warps, NM MMA warps and NM producer warps) a
@@ -148,25 +151,39 @@ struct TcCfg {
 // ---------------------------------------------------------------------------
 // operand rows
 // ---------------------------------------------------------------------------
-// Largest |M~ a| (a: m2l_norm) of every level from 2 on, as FP32 bits (the order of
+// Largest |M~ a| (a: m2l_norm) of every cell and level, as FP32 bits (the order of
 // non-negative floats), over the finite coefficients; lmax starts at zero.
 // grid.y: levels; a warp walks cells, lane i holds coefficients i, i + 32, ...
 __global__ void __launch_bounds__(256) m2l_lmax_k(const float *__restrict__ M, int PP, const __grid_constant__ M2LLevels lv,
-                                                  unsigned *__restrict__ lmax)
+                                                  unsigned *__restrict__ cmax, unsigned *__restrict__ lmax)
 {
-    const int l = 2 + blockIdx.y, lane = threadIdx.x & 31;
+    const int l = blockIdx.y, lane = threadIdx.x & 31;
     const int c1 = lv.start[l + 1];
     float a[4];
 #pragma unroll
     for (int r = 0; r < 4; r++) a[r] = m2l_norm(lane + 32 * r);
     unsigned best = 0;
-    for (int c = lv.start[l] + (int)(blockIdx.x * 8 + (threadIdx.x >> 5)); c < c1; c += (int)gridDim.x * 8) {
-        const float *Mc = M + (size_t)c * PP;
+    constexpr int U = 4;  // cells in flight
+    const int step = (int)gridDim.x * 8;
+    for (int c0 = lv.start[l] + (int)(blockIdx.x * 8 + (threadIdx.x >> 5)); c0 < c1; c0 += U * step) {
+        unsigned b[U];
 #pragma unroll
-        for (int r = 0; r < 4; r++)
-            if (lane + 32 * r < PP) best = max(best, m2l_mag(Mc[lane + 32 * r] * a[r]));
+        for (int u = 0; u < U; u++) {
+            b[u] = 0;
+            if (c0 + u * step >= c1) continue;
+            const float *Mc = M + (size_t)(c0 + u * step) * PP;
+#pragma unroll
+            for (int r = 0; r < 4; r++)
+                if (lane + 32 * r < PP) b[u] = max(b[u], m2l_mag(Mc[lane + 32 * r] * a[r]));
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (c0 + u * step >= c1) break;
+            b[u] = __reduce_max_sync(0xffffffffu, b[u]);
+            if (lane == 0) cmax[c0 + u * step] = b[u];
+            best = max(best, b[u]);
+        }
     }
-    best = __reduce_max_sync(0xffffffffu, best);
     __shared__ unsigned sb[8];
     if (lane == 0) sb[threadIdx.x >> 5] = best;
     __syncthreads();
@@ -208,7 +225,7 @@ __device__ __forceinline__ void m2l_split_chunk(const float *__restrict__ Mc, in
     *reinterpret_cast<uint4 *>(row + off + (C::PACK ? 64 : 128)) = *reinterpret_cast<const uint4 *>(w);
 }
 
-// FP16 rows of the cells from level 2 on. A cell of a lattice level (bit l of
+// FP16 rows of the cells from level 2 on, and the marks of wide levels. A cell of a lattice level (bit l of
 // lat.levels) goes to the lattice copy of its level: the row of position (x, y,
 // z) at ((b H + z/2) H + y/2) H + x/2, b = (x & 1) | (y & 1) << 1 | (z & 1) << 2
 // its octant bits and H = 2^(l-1), so that the cells of one octant form an H^3
@@ -216,7 +233,8 @@ __device__ __forceinline__ void m2l_split_chunk(const float *__restrict__ Mc, in
 // translation are a shifted block. Other cells go to row c of `rows`.
 template <int NP>
 __global__ void __launch_bounds__(256) m2l_split_k(const float *__restrict__ M, int PP, const int4 *__restrict__ xyz, int c0,
-                                                   int nc, const unsigned *__restrict__ lmax,
+                                                   int nc, const int *__restrict__ parent,
+                                                   const unsigned *__restrict__ cmax, unsigned *ws,
                                                    const __grid_constant__ M2LLattice lat, unsigned char *__restrict__ rows,
                                                    unsigned char *__restrict__ mlat)
 {
@@ -235,7 +253,8 @@ __global__ void __launch_bounds__(256) m2l_split_k(const float *__restrict__ M, 
         const int b = (x & 1) | ((y & 1) << 1) | ((z & 1) << 2);
         row = mlat + (lat.off[l] + ((b * H + (z >> 1)) * H + (y >> 1)) * H + (x >> 1)) * RB;
     }
-    m2l_split_chunk<NP>(M + (size_t)c * PP, PP, ch, m2l_exponent(lmax[l]), row);
+    m2l_split_chunk<NP>(M + (size_t)c * PP, PP, ch, m2l_exponent(ws[l]), row);
+    if (ch == 0) m2l_mark(c, l, cmax, parent, ws, nullptr);
 }
 
 // bits 0, 3, 6, ... of a Morton code below 2^30
@@ -249,15 +268,149 @@ __device__ __forceinline__ uint32_t every_third(uint32_t v)
     return v;
 }
 
+// tiles of a wide level, and pooled tiles once any level is wide
+__device__ __forceinline__ bool m2l_is_wide(unsigned wide, const M2LTile &t)
+{
+    return wide && (t.octant == 8 || ((wide >> t.level) & 1u));
+}
+
+// One tile in FP32 on the CUDA cores, by the first 256 threads of a block (all of
+// them take part in the barriers). Per vector C[row][r] += sum_c A[row][c] T[r][c]:
+// A the sources' M~ a, T = (hi + lo) 2^-14 of the operator image, both staged in
+// shared memory 32 coefficients at a time; thread (ty, tx) holds rows 8 ty .. 8 ty
+// + 7 and columns tx, tx + 16, .... Sums run over 8 vectors in FP32, as in tensor
+// memory, then into (hi, lo) pairs. Slow (milliseconds a tile) and rare.
+constexpr int WD_T = 256, WD_KC = 32, WD_LD = 132, WD_V = 8;
+template <int NP>
+struct WideShared {
+    float A[WD_KC][WD_LD];
+    float T[WD_KC][NP];
+    int src[WD_V][128];
+    int any[WD_V];
+};
+
+template <int NP>
+__device__ __noinline__ void m2l_wide_tile(const M2LJob &J, int p, int tile, WideShared<NP> &sh)
+{
+    using C = TcCfg<NP>;
+    constexpr int NC = NP / 16;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, PP = p * p;
+    const int tx = tid & 15, ty = (tid >> 4) & 15;
+    const bool on = tid < WD_T;
+    const M2LTile td = J.tiles[tile];
+    const int nv = J.st_off[10 + td.octant * (FMM_MAXLEVEL + 1) + td.level], e0 = J.st_off[td.octant];
+    // thread t looks up sources of row t % 128
+    int cell = -1, rl = td.level, px = 0, py = 0, pz = 0, ro = 0;
+    if (on && (tid & 127) < td.count) cell = J.tgt[td.start + (tid & 127)];  // (-1: a lattice position without a cell)
+    if (cell >= 0) {
+        const int4 a = J.xyz[cell];
+        rl = a.w;
+        const int s = FMM_MAXLEVEL - rl;
+        px = a.x >> s;
+        py = a.y >> s;
+        pz = a.z >> s;
+        ro = (px & 1) | ((py & 1) << 1) | ((pz & 1) << 2);
+    }
+    float acc[8][NC], hi[8][NC], lo[8][NC];
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+#pragma unroll
+        for (int j = 0; j < NC; j++) hi[i][j] = lo[i][j] = 0.f;
+    for (int v0 = 0; v0 < nv; v0 += WD_V) {
+        __syncthreads();  // the last group's sources are used up
+        if (tid < WD_V) sh.any[tid] = 0;
+        __syncthreads();
+        if (on)
+            for (int k = tid >> 7; k < WD_V; k += WD_T / 128) {
+                int b = -1;
+                if (v0 + k < nv && cell >= 0) {
+                    const int4 v = J.st[e0 + v0 + k];
+                    if ((v.w >> (16 + ro)) & 1) b = level_lookup(J.ld[rl], J.map_pool, J.anchor, rl, px + v.x, py + v.y, pz + v.z);
+                }
+                sh.src[k][tid & 127] = b;
+                if (b >= 0) sh.any[k] = 1;
+            }
+#pragma unroll
+        for (int i = 0; i < 8; i++)
+#pragma unroll
+            for (int j = 0; j < NC; j++) acc[i][j] = 0.f;
+        __syncthreads();
+        for (int k = 0; k < WD_V && v0 + k < nv; k++) {
+            if (!sh.any[k]) continue;  // (the same in every thread)
+            const unsigned char *op = J.ttab + (size_t)(J.st[e0 + v0 + k].w & 0xffff) * C::KB * C::B_BYTES;
+            for (int c0 = 0; c0 < PP; c0 += WD_KC) {
+                __syncthreads();  // the staged coefficients are used up
+                if (on) {
+                    const float a = c0 + lane < PP ? m2l_norm(c0 + lane) : 0.f;
+                    for (int r = warp; r < 128; r += WD_T / 32) {
+                        const int b = sh.src[k][r];
+                        sh.A[lane][r] = b >= 0 && c0 + lane < PP ? J.M[(size_t)b * PP + c0 + lane] * a : 0.f;
+                    }
+                    // 8 coefficients of one output a thread
+                    for (int i = tid; i < NP * (WD_KC / 8); i += WD_T) {
+                        const int r = i % NP, q = i / NP;
+                        const int ch = ((c0 & 63) >> 3) + q;  // its 16-byte chunk in the k-block's row
+                        const unsigned char *blk = op + (size_t)(c0 >> 6) * C::B_BYTES;
+                        const unsigned char *ph = blk + r * 128 + ((ch ^ (r & 7)) << 4);
+                        const unsigned char *pl = C::PACK ? blk + r * 128 + (((ch + 4) ^ (r & 7)) << 4)
+                                                          : blk + (NP + r) * 128 + ((ch ^ ((NP + r) & 7)) << 4);
+                        const uint4 h4 = *reinterpret_cast<const uint4 *>(ph), l4 = *reinterpret_cast<const uint4 *>(pl);
+                        const unsigned hw[4] = {h4.x, h4.y, h4.z, h4.w}, lw[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+                        for (int m = 0; m < 8; m++) {
+                            const unsigned short hb = (unsigned short)(hw[m / 2] >> (16 * (m & 1)));
+                            const unsigned short lb = (unsigned short)(lw[m / 2] >> (16 * (m & 1)));
+                            sh.T[8 * q + m][r] = (__half2float(__ushort_as_half(hb)) + __half2float(__ushort_as_half(lb))) * 0x1p-14f;
+                        }
+                    }
+                }
+                __syncthreads();
+                if (on) {
+                    const int kc = min(WD_KC, PP - c0);
+                    for (int c = 0; c < kc; c++) {
+                        float a[8], t[NC];
+#pragma unroll
+                        for (int i = 0; i < 8; i++) a[i] = sh.A[c][8 * ty + i];
+#pragma unroll
+                        for (int j = 0; j < NC; j++) t[j] = sh.T[c][tx + 16 * j];
+#pragma unroll
+                        for (int i = 0; i < 8; i++)
+#pragma unroll
+                            for (int j = 0; j < NC; j++) acc[i][j] = fmaf(a[i], t[j], acc[i][j]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 8; i++)
+#pragma unroll
+            for (int j = 0; j < NC; j++) two_sum_acc(hi[i][j], lo[i][j], acc[i][j]);
+    }
+    if (on)
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            const int row = 8 * ty + i, c = row < td.count ? J.tgt[td.start + row] : -1;
+#pragma unroll
+            for (int j = 0; j < NC; j++) {
+                const int r = tx + 16 * j;
+                if (c < 0 || r >= PP) continue;
+                const int t = J.rowexp[r] + 14;
+                J.L[(size_t)c * PP + r] += ((hi[i][j] + lo[i][j]) * m2l_pow2(t >> 1)) * m2l_pow2(t - (t >> 1));
+            }
+        }
+}
+
 template <int NP, bool PERSIST>
 __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     m2l_tc_k(int p, const __grid_constant__ M2LJob one, const M2LJob *__restrict__ jobs, int njobs,
-             int *__restrict__ queue, int *__restrict__ err)
+             int *__restrict__ queue, const unsigned *__restrict__ any, int *__restrict__ err)
 {
     // PERSIST (many systems: jobs[], njobs entries sorted by item0): each CTA
     // takes (tile, range) items from the queue until it is empty. Otherwise
     // CTA b computes item b of the single job `one`, read from the parameter
     // space, which measured faster for one system than the persistent loop.
+    // *any: zero if no level is wide. The item of a wide tile's first range is the
+    // whole tile, its other items are empty.
     using C = TcCfg<NP>;
     constexpr int NS = C::NS, NM = C::NM, QU = C::QU, RINGU = C::RINGU, KB = C::KB;
     constexpr bool PACK = C::PACK;
@@ -275,11 +428,20 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     int *abort_flag = reinterpret_cast<int *>(tmem_slot + 1);
     int *s_item = abort_flag + 1;                 // this CTA's current item (-1: none left)
     int *s_last = s_item + 1;                     // this CTA finished its tile last
+    int *s_wide = s_last + 1;                     // the item's tile is wide
     M2LJob *s_job = reinterpret_cast<M2LJob *>(reinterpret_cast<unsigned char *>(bar) + 512);  // its job
-    static_assert(sizeof(uint64_t) * (3 * NS + 4 * C::AC + 2) + 16 <= 512 && 512 + sizeof(M2LJob) <= C::BAR, "barrier area");
+    static_assert(sizeof(uint64_t) * (3 * NS + 4 * C::AC + 2) + 20 <= 512 && 512 + sizeof(M2LJob) <= C::BAR, "barrier area");
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (!PERSIST && (int)blockIdx.x >= *one.ntiles * one.nsplit) return;
+    if (!PERSIST) {
+        const unsigned wide = *any;
+        if ((int)blockIdx.x >= *one.ntiles * one.nsplit) return;
+        if (wide && m2l_is_wide(wide, one.tiles[(int)blockIdx.x / one.nsplit])) {
+            if ((int)blockIdx.x % one.nsplit == 0)
+                m2l_wide_tile<NP>(one, p, (int)blockIdx.x / one.nsplit, *reinterpret_cast<WideShared<NP> *>(base));
+            return;
+        }
+    }
     if (warp == C::MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(C::TCOLS));
@@ -303,6 +465,7 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
             *s_job = jobs[lo];
             const int t = it - s_job->item0;
             *s_item = (t >= 0 && t < s_job->count) ? t : -1;
+            *s_wide = *any != 0u && *s_item >= 0 && m2l_is_wide(s_job->ws[M2LW_WIDE], s_job->tiles[t / s_job->nsplit]);
         } else {
             *s_item = (int)blockIdx.x;
         }
@@ -326,6 +489,16 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     const int item = *s_item;
     if (item < 0) break;
     const M2LJob &J = PERSIST ? *s_job : one;
+    if constexpr (PERSIST) {
+        static_assert(sizeof(WideShared<NP>) <= NS * C::STAGE, "shared memory of a wide tile");
+        if (*s_wide) {
+            if (item % J.nsplit == 0) m2l_wide_tile<NP>(J, p, item / J.nsplit, *reinterpret_cast<WideShared<NP> *>(base));
+            // plain writes to the stages before the asynchronous copies of the next item
+            fence_proxy_async();
+            __syncthreads();
+            continue;
+        }
+    }
     const int nsplit = J.nsplit, tile = item / nsplit, split = item - tile * nsplit;
     const M2LTile td = J.tiles[tile];
     const int PP = p * p;
@@ -644,7 +817,7 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
         // failed, or the last drain saw the last MMA and nothing is waiting
         named_barrier_sync(1, C::NW * 32);
         if (!*(volatile int *)abort_flag) {
-            const int e = cell >= 0 ? m2l_exponent(J.lmax[rl]) : 0;
+            const int e = cell >= 0 ? m2l_exponent(J.ws[rl]) : 0;
             float *Lc = J.L + (size_t)(cell >= 0 ? cell : 0) * PP;
             // back from the operands' powers of two
             auto put = [&](int k, float x) {
@@ -920,15 +1093,15 @@ void tensor_tables_update(fmm_ctx *h)
 }
 
 template <int NP>
-static void launch_tc(int p, int grid, const M2LJob &one, const M2LJob *jobs, int njobs, int *queue, int *err,
-                      cudaStream_t s)
+static void launch_tc(int p, int grid, const M2LJob &one, const M2LJob *jobs, int njobs, int *queue, const unsigned *any,
+                      int *err, cudaStream_t s)
 {
     using C = TcCfg<NP>;
     // grid: one CTA per SM with a job list (persistent), else one per item
     if (jobs) {
         ensure_smem((const void *)m2l_tc_k<NP, true>, C::SMEM);
         FMM_CUDA_TRY(cudaMemsetAsync(queue, 0, sizeof(int), s));
-        m2l_tc_k<NP, true><<<grid, C::NT, C::SMEM, s>>>(p, one, jobs, njobs, queue, err);
+        m2l_tc_k<NP, true><<<grid, C::NT, C::SMEM, s>>>(p, one, jobs, njobs, queue, any, err);
     } else {
         ensure_smem((const void *)m2l_tc_k<NP, false>, C::SMEM);
         // the workers' registers come out of the launch's: with fewer they would wait for ever
@@ -938,7 +1111,7 @@ static void launch_tc(int p, int grid, const M2LJob &one, const M2LJob *jobs, in
                    a.numRegs * C::NT >= 32 * (C::NW * C::REG_W + 4 * C::REG_O);
         }();
         if (C::REGS && !fits) throw Error{FMM_ECUDA, "tensor-core M2L: too few registers at launch"};
-        m2l_tc_k<NP, false><<<grid, C::NT, C::SMEM, s>>>(p, one, jobs, njobs, queue, err);
+        m2l_tc_k<NP, false><<<grid, C::NT, C::SMEM, s>>>(p, one, jobs, njobs, queue, any, err);
     }
 }
 
@@ -954,16 +1127,13 @@ static void launch_tc(int p, int grid, const M2LJob &one, const M2LJob *jobs, in
     default: throw Error{FMM_EINVAL, "tensor-core M2L: unsupported p"};    \
     }
 
-static void launch_tc_p(int p, int grid, const M2LJob &one, const M2LJob *jobs, int njobs, int *queue, int *err,
-                        cudaStream_t s)
+static void launch_tc_p(int p, int grid, const M2LJob &one, const M2LJob *jobs, int njobs, int *queue, const unsigned *any,
+                        int *err, cudaStream_t s)
 {
-#define FMM_TC_CALL(NPV) launch_tc<NPV>(p, grid, one, jobs, njobs, queue, err, s)
+#define FMM_TC_CALL(NPV) launch_tc<NPV>(p, grid, one, jobs, njobs, queue, any, err, s)
     FMM_TC_SWITCH(tc_np(p), FMM_TC_CALL)
 #undef FMM_TC_CALL
 }
-
-// words of the M2L workspace: per-level maxima, then one counter per tile
-constexpr int TCW_CNT = 32;
 
 // the longest list of vectors that a tile of the tree walks
 int m2l_longest_list(fmm_ctx *h)
@@ -1008,7 +1178,8 @@ M2LJob m2l_tensor_job(fmm_ctx *h, float *L)
     tensor_tables_update(h);
     const int nc = h->ncells;
     h->msplit.ensure(tc_row_bytes(h->p) * (size_t)nc);
-    h->m2l_ws.ensure(sizeof(unsigned) * (TCW_CNT + (size_t)h->ntiles_max));
+    h->m2l_ws.ensure(sizeof(unsigned) * (M2LW_CNT + (size_t)h->ntiles_max));
+    h->m2l_cmax.ensure(sizeof(unsigned) * (size_t)nc);
     if (h->m2l_nsplit > 1)
         h->m2l_part.ensure(sizeof(float2) * (size_t)h->ntiles_max * h->m2l_nsplit * h->p * h->p * TcCfg<64>::M);
     M2LJob j;
@@ -1024,9 +1195,11 @@ M2LJob m2l_tensor_job(fmm_ctx *h, float *L)
     j.mrow = h->msplit.as<unsigned char>();
     j.ttab = h->ttab->buf.as<unsigned char>();
     j.L = L;
-    j.lmax = h->m2l_ws.as<unsigned>();
-    j.tcnt = h->m2l_ws.as<unsigned>() + TCW_CNT;
-    j.ws_words = TCW_CNT + h->ntiles_max;
+    j.M = h->Mexp.as<float>();
+    j.cmax = h->m2l_cmax.as<unsigned>();
+    j.ws = h->m2l_ws.as<unsigned>();
+    j.tcnt = h->m2l_ws.as<unsigned>() + M2LW_CNT;
+    j.ws_words = M2LW_CNT + h->ntiles_max;
     j.part = h->m2l_part.as<float2>();
     j.nsplit = h->m2l_nsplit;
     j.chunk = h->m2l_chunk;
@@ -1148,7 +1321,7 @@ void lattice_prepare(fmm_ctx *h, cudaStream_t s)
 }
 
 template <int NP>
-__global__ void __launch_bounds__(256) batch_split_k(int PP, const BatchSys *__restrict__ sys)
+__global__ void __launch_bounds__(256) batch_split_k(int PP, const BatchSys *__restrict__ sys, unsigned *any)
 {
     using C = TcCfg<NP>;
     constexpr int NCH = NP / 8;
@@ -1156,25 +1329,26 @@ __global__ void __launch_bounds__(256) batch_split_k(int PP, const BatchSys *__r
     if (!S.rows || S.c0 >= S.ncells) return;
     const int64_t cnt = (int64_t)(S.ncells - S.c0) * NCH;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = S.c0 + (int)(i / NCH), ch = (int)(i % NCH);
-        m2l_split_chunk<NP>(S.M + (size_t)c * PP, PP, ch, m2l_exponent(S.m2l_ws[S.xyz[c].w]),
-                            S.rows + (size_t)c * (C::KB * C::ROWB));
+        const int c = S.c0 + (int)(i / NCH), ch = (int)(i % NCH), l = S.xyz[c].w;
+        m2l_split_chunk<NP>(S.M + (size_t)c * PP, PP, ch, m2l_exponent(S.m2l_ws[l]), S.rows + (size_t)c * (C::KB * C::ROWB));
+        if (ch == 0) m2l_mark(c, l, S.m2l_cmax, S.parent, S.m2l_ws, any);
     }
 }
 
-void batch_split(int p, const BatchSys *sys, int nsys, cudaStream_t s)
+void batch_split(int p, const BatchSys *sys, int nsys, unsigned *any, cudaStream_t s)
 {
-#define FMM_TC_CALL(NPV) batch_split_k<NPV><<<dim3(16, (unsigned)nsys), 256, 0, s>>>(p *p, sys)
+#define FMM_TC_CALL(NPV) batch_split_k<NPV><<<dim3(16, (unsigned)nsys), 256, 0, s>>>(p *p, sys, any)
     FMM_TC_SWITCH(tc_np(p), FMM_TC_CALL)
 #undef FMM_TC_CALL
     check_launch("batch split");
 }
 
-void m2l_tensor_jobs(int p, int nsm, const M2LJob *jobs_dev, int njobs, int *queue, int *err, cudaStream_t s)
+void m2l_tensor_jobs(int p, int nsm, const M2LJob *jobs_dev, int njobs, int *queue, const unsigned *any, int *err,
+                     cudaStream_t s)
 {
     M2LJob none;
     std::memset(&none, 0, sizeof(none));
-    launch_tc_p(p, nsm, none, jobs_dev, njobs, queue, err, s);
+    launch_tc_p(p, nsm, none, jobs_dev, njobs, queue, any, err, s);
 }
 
 void m2l_tensor(fmm_ctx *h, float *L, const float *M)
@@ -1195,22 +1369,22 @@ void m2l_tensor(fmm_ctx *h, float *L, const float *M)
     }
     // a block walks 64 cells or more; 4 blocks per SM at most
     const unsigned gx = (unsigned)std::min((most + 63) / 64, 4 * h->nsm);
-    m2l_lmax_k<<<dim3(gx, (unsigned)h->depth - 1), 256, 0, s>>>(M, PP, lv, h->m2l_ws.as<unsigned>());
+    m2l_lmax_k<<<dim3(gx, (unsigned)h->depth + 1), 256, 0, s>>>(M, PP, lv, h->m2l_cmax.as<unsigned>(), h->m2l_ws.as<unsigned>());
     count_launch(h);
     M2LLattice lat;
     lat.levels = h->lat_levels;
     for (int l = 0; l <= FMM_MAXLEVEL; l++) lat.off[l] = h->lat_off[l];
 #define FMM_TC_CALL(NPV)                                                                                           \
     m2l_split_k<NPV><<<nblk((int64_t)(nc - c0) * (NPV / 8), 256), 256, 0, s>>>(                                     \
-        M, PP, h->c_xyz.as<int4>(), c0, nc, h->m2l_ws.as<unsigned>(), lat, h->msplit.as<unsigned char>(),           \
-        h->mlat.as<unsigned char>())
+        M, PP, h->c_xyz.as<int4>(), c0, nc, h->c_parent.as<int>(), h->m2l_cmax.as<unsigned>(),                       \
+        h->m2l_ws.as<unsigned>(), lat, h->msplit.as<unsigned char>(), h->mlat.as<unsigned char>())
     FMM_TC_SWITCH(tc_np(h->p), FMM_TC_CALL)
 #undef FMM_TC_CALL
     count_launch(h);
     if (h->lat_levels) {
         j.lat_maps = h->lat_maps.as<unsigned char>();
     }
-    launch_tc_p(h->p, h->ntiles_max * j.nsplit, j, nullptr, 1, queue, err, s);
+    launch_tc_p(h->p, h->ntiles_max * j.nsplit, j, nullptr, 1, queue, j.ws + M2LW_WIDE, err, s);
     count_launch(h);
     check_launch("m2l tensor");
 }
