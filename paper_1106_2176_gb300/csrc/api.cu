@@ -317,6 +317,14 @@ int fmm_set_m2l_lattice(fmm_handle h, int on)
     return FMM_OK;
 }
 
+int fmm_set_sort_polls(fmm_handle h, int polls)
+{
+    if (!h) return fail(FMM_EINVAL, "fmm_set_sort_polls: NULL handle");
+    if (polls < 0) return fail(FMM_EINVAL, "fmm_set_sort_polls: polls must be >= 0");
+    h->sort_polls = polls;
+    return FMM_OK;
+}
+
 int fmm_set_stream(fmm_handle h, void *stream)
 {
     if (!h) return fail(FMM_EINVAL, "fmm_set_stream: NULL handle");

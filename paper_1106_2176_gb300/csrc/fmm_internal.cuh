@@ -31,6 +31,7 @@
 
 #define FMM_MAXP 20
 #define FMM_MAXLEVEL 21
+#define FMM_SORT_POLLS (1 << 20)  // fruitless looks before a block of the sort counts for itself
 #define FMM_DENSE_MAP_MAXLEVEL 8  // levels with 8^l <= 2^24 get a dense lattice map
 
 namespace fmm {
@@ -284,6 +285,7 @@ struct fmm_ctx {
     fmm::DevBuf cgeo;                   // per cell: geometric centre and 1 / width (double4)
     fmm::DevBuf energy_buf;             // block sums of the weighted energy
     fmm::DevBuf sort_ws, scan_tmp;
+    int sort_polls = FMM_SORT_POLLS;    // fmm_set_sort_polls
     fmm::DevBuf xs64, xs32, xs32lo;
     fmm::DevBuf c_level, c_anchor, c_begin, c_end, c_child, c_nchild, c_parent, c_xyz;
     fmm::DevBuf split_cnt, split_off, split_bnd;
@@ -329,7 +331,7 @@ void tree_export(fmm_ctx *h, uint64_t *keys, int32_t *perm, int32_t *level, uint
 int64_t tree_m2l_total(fmm_ctx *h);
 size_t sort_ws_bytes(int64_t n);
 int morton_sort_into(const void *x, int64_t n, int dt, uint64_t *keys, int *perm, uint64_t *keys_tmp, int *perm_tmp,
-                     void *ws, Box *box, int nsm, cudaStream_t s);
+                     void *ws, Box *box, int nsm, int polls, cudaStream_t s);
 int m2l_tile_size(fmm_ctx *h);
 void scan_exclusive_u32(fmm_ctx *h, const unsigned *in, unsigned *out, int64_t count, unsigned *total_dev,
                         cudaStream_t s);

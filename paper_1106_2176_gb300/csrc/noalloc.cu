@@ -80,7 +80,7 @@ extern "C" FMM_API int fmm_morton_sort_noalloc(const void *x, int64_t n, int dty
         Box *box = reinterpret_cast<Box *>(ws + NOALLOC_WS);
         if (sort_ws_bytes(n) > NOALLOC_WS) throw Error{FMM_EINVAL, "fmm_morton_sort_noalloc: workspace too small"};
         static_assert(sizeof(Box) <= 256, "root-cube scratch");
-        morton_sort_into(x, n, dtype, keys, perm, ktmp, ptmp, ws, box, nsm, (cudaStream_t)stream);
+        morton_sort_into(x, n, dtype, keys, perm, ktmp, ptmp, ws, box, nsm, FMM_SORT_POLLS, (cudaStream_t)stream);
         return FMM_OK;
     } catch (const Error &e) {
         set_error(e.msg);

@@ -361,8 +361,6 @@ constexpr int64_t RS_FEW = 1 << 19;
 struct SortWs {
     unsigned count[RS_PASSES][256];
     unsigned ticket[RS_PASSES];
-    int err;
-    int pad[7];
 };
 static int rs_tile(int64_t n) { return RS_T * (n <= RS_FEW ? RS_R_MIN : RS_R_MAX); }
 // status: pass + 1 in the top 4 bits (a word left by another pass counts as not
@@ -428,11 +426,13 @@ __device__ __forceinline__ unsigned digit_peers(unsigned d)
 // equal digit by ballots), so the rank of a key among equal digits follows input order;
 // the tile is staged in shared memory in digit order and written out in runs.
 // Tiles are numbered in the order in which their blocks start, so a tile only
-// waits for tiles that are already running; every wait is bounded (ws->err).
+// waits for tiles that are already running. A tile that has looked `polls` times
+// in vain for the one before counts the keys before its own itself: no wait is
+// longer, and the sort does not depend on one.
 template <bool VALS, int R, class W>
 __global__ void __launch_bounds__(RS_T) rs_pass_k(const uint64_t *__restrict__ kin, const int *__restrict__ vin,
                                                   uint64_t *__restrict__ kout, int *__restrict__ vout, int n, int pass,
-                                                  SortWs *__restrict__ ws, W *status)
+                                                  SortWs *__restrict__ ws, W *status, int polls)
 {
     constexpr int TILE = RS_T * R, CB = 8 * sizeof(W) - 6;  // bits of a count
     extern __shared__ unsigned char smem_raw[];
@@ -491,10 +491,11 @@ __global__ void __launch_bounds__(RS_T) rs_pass_k(const uint64_t *__restrict__ k
     const unsigned gbase = block_excl_scan(ws->count[pass][d0], sw, nullptr);
     // the counts of the tiles before, eight words in flight
     unsigned before = 0;
+    bool known = tile == 0;
     if (tile > 0) {
         constexpr int LB = 8;
-        int t = tile - 1, polls = 0;
-        for (bool done = false; !done;) {
+        int t = tile - 1;
+        for (int n0 = 0; !known && n0 < polls;) {
             W x[LB];
 #pragma unroll
             for (int j = 0; j < LB; j++) x[j] = t - j >= 0 ? st[(size_t)(t - j) * 256 + d0] : 0;
@@ -506,20 +507,27 @@ __global__ void __launch_bounds__(RS_T) rs_pass_k(const uint64_t *__restrict__ k
                 if (go) {
                     before += (unsigned)(x[j] & (((W)1 << CB) - 1));
                     taken++;
-                    done = ((x[j] >> CB) & 3) == 2;
-                    go = !done;
+                    known = ((x[j] >> CB) & 3) == 2;
+                    go = !known;
                 }
             }
             t -= taken;
-            if (!done && taken == 0 && ++polls > (1 << 20)) {
-                atomicOr(&ws->err, 1);
-                break;
-            }
+            n0 += taken == 0;
         }
-        st[(size_t)tile * 256 + d0] = tag | ((W)2 << CB) | (W)(before + own);
+        if (known) st[(size_t)tile * 256 + d0] = tag | ((W)2 << CB) | (W)(before + own);
     }
     goff[d0] = gbase + before;
-    __syncthreads();
+    if (__syncthreads_or(!known)) {
+        unsigned *const cnt = reinterpret_cast<unsigned *>(skey);  // (not in use yet)
+        cnt[d0] = 0;
+        __syncthreads();
+        for (int64_t i = d0; i < base; i += RS_T) atomicAdd(&cnt[(unsigned)(kin[i] >> shift) & 255u], 1u);
+        __syncthreads();
+        before = cnt[d0];
+        if (!known) st[(size_t)tile * 256 + d0] = tag | ((W)2 << CB) | (W)(before + own);
+        goff[d0] = gbase + before;
+        __syncthreads();
+    }
 #pragma unroll
     for (int r = 0; r < R; r++) {
         const unsigned d = (unsigned)(k[r] >> shift) & 255u;
@@ -533,10 +541,8 @@ __global__ void __launch_bounds__(RS_T) rs_pass_k(const uint64_t *__restrict__ k
         const uint64_t kk = skey[j];
         const unsigned d = (unsigned)(kk >> shift) & 255u;
         const unsigned g = goff[d] + (unsigned)j - dstart[d];
-        if (g < (unsigned)n) {  // (not so only after a wait gave up)
-            kout[g] = kk;
-            if (VALS) vout[g] = sval[j];
-        }
+        kout[g] = kk;
+        if (VALS) vout[g] = sval[j];
     }
 }
 
@@ -546,13 +552,13 @@ static size_t rs_smem() { return (size_t)RS_T * R * 12 + (size_t)(RS_W * 256 + 2
 // Sorts by the low `bits` bits of the keys; ws holds their digit counts, zeros
 // elsewhere. Returns true when the result sits in (kt, vt) rather than (k, v).
 template <bool VALS, int R, class W>
-static bool radix_passes(uint64_t *k, int *v, uint64_t *kt, int *vt, int n, int bits, SortWs *ws, cudaStream_t s)
+static bool radix_passes(uint64_t *k, int *v, uint64_t *kt, int *vt, int n, int bits, SortWs *ws, int polls, cudaStream_t s)
 {
     const int ntiles = (int)nblocks(n, RS_T * R);
     ensure_smem((const void *)rs_pass_k<VALS, R, W>, rs_smem<R>());
     bool swapped = false;
     for (int pass = 0; 8 * pass < bits; pass++) {
-        rs_pass_k<VALS, R, W><<<ntiles, RS_T, rs_smem<R>(), s>>>(k, v, kt, vt, n, pass, ws, reinterpret_cast<W *>(ws + 1));
+        rs_pass_k<VALS, R, W><<<ntiles, RS_T, rs_smem<R>(), s>>>(k, v, kt, vt, n, pass, ws, reinterpret_cast<W *>(ws + 1), polls);
         check_launch("radix sort");
         std::swap(k, kt);
         std::swap(v, vt);
@@ -562,12 +568,12 @@ static bool radix_passes(uint64_t *k, int *v, uint64_t *kt, int *vt, int n, int 
 }
 
 template <bool VALS>
-static bool radix_sort(uint64_t *k, int *v, uint64_t *kt, int *vt, int64_t n, int bits, SortWs *ws, cudaStream_t s)
+static bool radix_sort(uint64_t *k, int *v, uint64_t *kt, int *vt, int64_t n, int bits, SortWs *ws, int polls, cudaStream_t s)
 {
     if (n > 0x7fffffffLL) throw Error{FMM_EINVAL, "radix sort: too many keys"};
-    if (rs_wide(n)) return radix_passes<VALS, RS_R_MAX, unsigned long long>(k, v, kt, vt, (int)n, bits, ws, s);
-    if (n <= RS_FEW) return radix_passes<VALS, RS_R_MIN, unsigned>(k, v, kt, vt, (int)n, bits, ws, s);
-    return radix_passes<VALS, RS_R_MAX, unsigned>(k, v, kt, vt, (int)n, bits, ws, s);
+    if (rs_wide(n)) return radix_passes<VALS, RS_R_MAX, unsigned long long>(k, v, kt, vt, (int)n, bits, ws, polls, s);
+    if (n <= RS_FEW) return radix_passes<VALS, RS_R_MIN, unsigned>(k, v, kt, vt, (int)n, bits, ws, polls, s);
+    return radix_passes<VALS, RS_R_MAX, unsigned>(k, v, kt, vt, (int)n, bits, ws, polls, s);
 }
 
 // Up to SMALL_N points: cube, keys and all passes in one block (a launch per
@@ -672,9 +678,10 @@ __global__ void __launch_bounds__(SMALL_T) sort_small_k(const T *__restrict__ x,
 // buffers (no allocation; both the tree build and the allocation-free entry
 // point): keys[n], perm[n] the sorted keys and the input index of each,
 // keys_tmp, perm_tmp ping-pong buffers, ws sort_ws_bytes(n) of workspace. The
-// result is in keys and perm (an even number of passes). Returns the launches.
+// result is in keys and perm (an even number of passes). polls: as in rs_pass_k.
+// Returns the launches.
 int morton_sort_into(const void *x, int64_t n, int dt, uint64_t *keys, int *perm, uint64_t *keys_tmp, int *perm_tmp,
-                     void *ws, Box *box, int nsm, cudaStream_t s)
+                     void *ws, Box *box, int nsm, int polls, cudaStream_t s)
 {
     const bool f64 = dt == FMM_F64;
     if (n <= SMALL_N) {
@@ -699,7 +706,7 @@ int morton_sort_into(const void *x, int64_t n, int dt, uint64_t *keys, int *perm
         keys_k<float><<<gk, 256, 0, s>>>((const float *)x, n, box, keys, perm, w);
     }
     check_launch("keys");
-    radix_sort<true>(keys, perm, keys_tmp, perm_tmp, n, 63, w, s);
+    radix_sort<true>(keys, perm, keys_tmp, perm_tmp, n, 63, w, polls, s);
     return 2 + RS_PASSES;
 }
 
@@ -817,7 +824,7 @@ __global__ void split_write_k(int ls, int le, int l, const unsigned *__restrict_
 // 0.37 ms. Numbering and fields
 // are those of the kernels above.
 struct SmallTree {
-    int nonfinite, sort_err, overflow;
+    int nonfinite, overflow;
     int ncells, depth, nleaves;
     int lvl_start[FMM_MAXLEVEL + 2];
     int ext[6 * (FMM_MAXLEVEL + 1)];  // per level x y z: minima, then maxima
@@ -827,7 +834,7 @@ constexpr int64_t TREE_SMALL_CELLS = 65536;  // ... cells that could arise (8 pe
 constexpr int TS_T = 1024;
 
 __global__ void __launch_bounds__(TS_T) tree_small_k(int n, int ncrit, int cap, const uint64_t *__restrict__ keys,
-                                                     const Box *__restrict__ box, const int *__restrict__ sort_err,
+                                                     const Box *__restrict__ box,
                                                      int *level, uint64_t *anchor, int *begin, int *end, int *child,
                                                      int *nchild, int *parent, int4 *xyz, int *leaves, int *pcell,
                                                      SmallTree *out)
@@ -839,7 +846,6 @@ __global__ void __launch_bounds__(TS_T) tree_small_k(int n, int ncrit, int cap, 
     for (int i = tid; i < 2 * NE; i += TS_T) s_ext[i] = i < NE ? INT_MAX : -1;
     if (tid == 0) {
         out->nonfinite = box->nonfinite;
-        out->sort_err = sort_err ? *sort_err : 0;
         out->overflow = 0;
         level[0] = 0;
         anchor[0] = 0;
@@ -1363,11 +1369,8 @@ static void pairs_to_csr(fmm_ctx *h, const int2 *pairs, int64_t np, DevBuf &ptr,
         FMM_CUDA_TRY(cudaMemsetAsync(ws, 0, sort_ws_bytes(np), s));
         rs_count_k<<<std::min(nblocks(np, 2048), (unsigned)h->nsm * 6), 256, 0, s>>>(k1, np, (2 * bs + 7) / 8, ws);
         count_launch(h);
-        const bool sw = radix_sort<false>(k1, nullptr, k2, nullptr, np, 2 * bs, ws, s);
+        const bool sw = radix_sort<false>(k1, nullptr, k2, nullptr, np, 2 * bs, ws, h->sort_polls, s);
         h->launches += (2 * bs + 7) / 8;
-        FMM_CUDA_TRY(cudaMemcpyAsync(hp, &ws->err, sizeof(int), cudaMemcpyDeviceToHost, s));
-        FMM_CUDA_TRY(cudaStreamSynchronize(s));
-        if (*hp) throw Error{FMM_ECUDA, "pair sort: a device-side wait timed out"};
         const uint64_t *ks = sw ? k2 : k1;
         pair_rows_k<<<nblocks(np, 256), 256, 0, s>>>(ks, np, bs, h->row_cnt.as<unsigned>(), src.as<int>());
         count_launch(h);
@@ -1629,7 +1632,7 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
     h->idx2.ensure(sizeof(int) * n);
     h->sort_ws.ensure(sort_ws_bytes(n));
     h->launches += morton_sort_into(x, n, dt, h->keys.as<uint64_t>(), h->idx.as<int>(), h->keys2.as<uint64_t>(),
-                                    h->idx2.as<int>(), h->sort_ws.p, box, h->nsm, s);
+                                    h->idx2.as<int>(), h->sort_ws.p, box, h->nsm, h->sort_polls, s);
 
     // 3. sorted particles
     const bool mixed = h->precision == FMM_MIXED;
@@ -1653,9 +1656,8 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
     count_launch(h);
     check_launch("gather");
 
-    auto check_input = [&](int nonfinite, int sort_err) {
+    auto check_input = [&](int nonfinite) {
         if (nonfinite) throw Error{FMM_ENONFINITE, "fmm_build: a position is NaN or infinite"};
-        if (sort_err) throw Error{FMM_ECUDA, "fmm_build: a device-side wait of the sort timed out"};
     };
     // 4. cells
     // all cell arrays grow together; c_level's capacity stands for all of them
@@ -1692,7 +1694,7 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
         h->pcell.ensure(sizeof(int) * (size_t)n);
         h->small_tree.ensure(sizeof(SmallTree));
         tree_small_k<<<1, TS_T, 0, s>>>((int)n, h->ncrit, (int)most, h->keys.as<uint64_t>(), box,
-                                       n > SMALL_N ? &h->sort_ws.as<SortWs>()->err : nullptr, h->c_level.as<int>(),
+                                       h->c_level.as<int>(),
                                        h->c_anchor.as<uint64_t>(), h->c_begin.as<int>(), h->c_end.as<int>(),
                                        h->c_child.as<int>(), h->c_nchild.as<int>(), h->c_parent.as<int>(),
                                        h->c_xyz.as<int4>(), h->leaves.as<int>(), h->pcell.as<int>(),
@@ -1702,7 +1704,7 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
         SmallTree *st = h->hpin.as<SmallTree>();
         FMM_CUDA_TRY(cudaMemcpyAsync(st, h->small_tree.p, sizeof(SmallTree), cudaMemcpyDeviceToHost, s));
         FMM_CUDA_TRY(cudaStreamSynchronize(s));
-        check_input(st->nonfinite, st->sort_err);
+        check_input(st->nonfinite);
         small = !st->overflow;
         if (small) {
             ncells = st->ncells;
@@ -1719,10 +1721,8 @@ void tree_build(fmm_ctx *h, const void *x, const void *q, int64_t n, int dt)
         {
             int *hp = h->hpin.as<int>();
             FMM_CUDA_TRY(cudaMemcpyAsync(hp, &box->nonfinite, sizeof(int), cudaMemcpyDeviceToHost, s));
-            if (n > SMALL_N)
-                FMM_CUDA_TRY(cudaMemcpyAsync(hp + 1, &h->sort_ws.as<SortWs>()->err, sizeof(int), cudaMemcpyDeviceToHost, s));
             FMM_CUDA_TRY(cudaStreamSynchronize(s));
-            check_input(hp[0], n > SMALL_N ? hp[1] : 0);
+            check_input(*hp);
         }
 
         const int cap = (int)std::min<int64_t>(std::max<int64_t>(1024, 2 * (n / std::max(1, h->ncrit)) + 64), 0x7fffffff);

@@ -80,6 +80,7 @@ def lib():
     L.fmm_set_overlap.argtypes = [_vp, i32]
     L.fmm_set_m2l_pool.argtypes = [_vp, i32]
     L.fmm_set_m2l_lattice.argtypes = [_vp, ctypes.c_int]
+    L.fmm_set_sort_polls.argtypes = [_vp, i32]
     L.fmm_set_stream.argtypes = [_vp, _vp]
     L.fmm_set_uniform_path.argtypes = [_vp, ctypes.c_int]
     L.fmm_m2l_rotation_host.argtypes = [ctypes.c_int, _vp, _vp, _vp]

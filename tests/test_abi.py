@@ -96,6 +96,11 @@ def test_m2l_lattice_setter_checks_arguments(L):
     assert b"fmm_set_m2l_lattice" in L.fmm_last_error(None)
 
 
+def test_sort_polls_setter_checks_arguments(L):
+    assert L.fmm_set_sort_polls(None, 0) == fmm.FMM_EINVAL
+    assert b"fmm_set_sort_polls" in L.fmm_last_error(None)
+
+
 def test_stats_layout_matches_the_header():
     # the ctypes mirror of fmm_stats lists the header's fields in order
     import re
