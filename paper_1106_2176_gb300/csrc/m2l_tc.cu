@@ -151,13 +151,13 @@ struct TcCfg {
 // ---------------------------------------------------------------------------
 // operand rows
 // ---------------------------------------------------------------------------
-// Largest |M~ a| (a: m2l_norm) of every cell and level, as FP32 bits (the order of
-// non-negative floats), over the finite coefficients; lmax starts at zero.
-// grid.y: levels; a warp walks cells, lane i holds coefficients i, i + 32, ...
+// Largest |M~ a| (a: m2l_norm) of every cell and of every level from 2 on, as FP32
+// bits (the order of non-negative floats), over the finite coefficients; lmax starts
+// at zero. grid.y: levels from 2 on (the few cells above go with 2); a warp walks cells, lane i holds coefficients i, i + 32, ...
 __global__ void __launch_bounds__(256) m2l_lmax_k(const float *__restrict__ M, int PP, const __grid_constant__ M2LLevels lv,
                                                   unsigned *__restrict__ cmax, unsigned *__restrict__ lmax)
 {
-    const int l = blockIdx.y, lane = threadIdx.x & 31;
+    const int l = 2 + blockIdx.y, lane = threadIdx.x & 31;
     const int c1 = lv.start[l + 1];
     float a[4];
 #pragma unroll
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(256) m2l_lmax_k(const float *__restrict__ M, i
     unsigned best = 0;
     constexpr int U = 4;  // cells in flight
     const int step = (int)gridDim.x * 8;
-    for (int c0 = lv.start[l] + (int)(blockIdx.x * 8 + (threadIdx.x >> 5)); c0 < c1; c0 += U * step) {
+    for (int c0 = (l > 2 ? lv.start[l] : 0) + (int)(blockIdx.x * 8 + (threadIdx.x >> 5)); c0 < c1; c0 += U * step) {
         unsigned b[U];
 #pragma unroll
         for (int u = 0; u < U; u++) {
@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(256) m2l_lmax_k(const float *__restrict__ M, i
             if (c0 + u * step >= c1) break;
             b[u] = __reduce_max_sync(0xffffffffu, b[u]);
             if (lane == 0) cmax[c0 + u * step] = b[u];
-            best = max(best, b[u]);
+            if (c0 + u * step >= lv.start[l]) best = max(best, b[u]);
         }
     }
     __shared__ unsigned sb[8];
@@ -1369,7 +1369,7 @@ void m2l_tensor(fmm_ctx *h, float *L, const float *M)
     }
     // a block walks 64 cells or more; 4 blocks per SM at most
     const unsigned gx = (unsigned)std::min((most + 63) / 64, 4 * h->nsm);
-    m2l_lmax_k<<<dim3(gx, (unsigned)h->depth + 1), 256, 0, s>>>(M, PP, lv, h->m2l_cmax.as<unsigned>(), h->m2l_ws.as<unsigned>());
+    m2l_lmax_k<<<dim3(gx, (unsigned)h->depth - 1), 256, 0, s>>>(M, PP, lv, h->m2l_cmax.as<unsigned>(), h->m2l_ws.as<unsigned>());
     count_launch(h);
     M2LLattice lat;
     lat.levels = h->lat_levels;
