@@ -186,8 +186,8 @@ FMM_API int fmm_set_m2l_lattice(fmm_handle h, int on);
 
 /* For tests: how often a block of the build's radix sort looks for the digit
  * counts of the block before it until it counts the keys before its own itself
- * (default 2^20, so that no wait is unbounded; 0: it does not wait at all). The
- * keys and their order are the same whatever the value. Takes effect at the next
+ * (default 2^20, so that every wait is bounded; 0: it counts after the first look
+ * in vain). The keys and their order are the same whatever the value. Takes effect at the next
  * build. Returns FMM_EINVAL for a NULL handle or polls < 0. */
 FMM_API int fmm_set_sort_polls(fmm_handle h, int polls);
 

@@ -422,13 +422,24 @@ __device__ __forceinline__ unsigned digit_peers(unsigned d)
     return m;
 }
 
+// how many of the first `base` keys have digit threadIdx.x (by the whole block; cnt:
+// 256 words of its shared memory)
+static __device__ __noinline__ unsigned rs_recount(const uint64_t *kin, int64_t base, int shift, unsigned *cnt)
+{
+    cnt[threadIdx.x] = 0;
+    __syncthreads();
+    for (int64_t i = threadIdx.x; i < base; i += RS_T) atomicAdd(&cnt[(unsigned)(kin[i] >> shift) & 255u], 1u);
+    __syncthreads();
+    return cnt[threadIdx.x];
+}
+
 // Each warp ranks its 32 R consecutive keys in R rounds of 32 (the lanes of
 // equal digit by ballots), so the rank of a key among equal digits follows input order;
 // the tile is staged in shared memory in digit order and written out in runs.
 // Tiles are numbered in the order in which their blocks start, so a tile only
-// waits for tiles that are already running. A tile that has looked `polls` times
-// in vain for the one before counts the keys before its own itself: no wait is
-// longer, and the sort does not depend on one.
+// waits for tiles that are already running. A tile that has looked more than `polls`
+// times in vain for the one before counts the keys before its own itself: every wait
+// is bounded, and the sort does not depend on one.
 template <bool VALS, int R, class W>
 __global__ void __launch_bounds__(RS_T) rs_pass_k(const uint64_t *__restrict__ kin, const int *__restrict__ vin,
                                                   uint64_t *__restrict__ kout, int *__restrict__ vout, int n, int pass,
@@ -443,9 +454,13 @@ __global__ void __launch_bounds__(RS_T) rs_pass_k(const uint64_t *__restrict__ k
     unsigned *goff = dstart + 256;                                         // 256
     unsigned *sw = goff + 256;                                             // 32
     __shared__ unsigned s_tile;
+    __shared__ int s_unknown;  // a thread gave up
 
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, d0 = threadIdx.x, shift = 8 * pass;
-    if (threadIdx.x == 0) s_tile = atomicAdd(&ws->ticket[pass], 1u);
+    if (threadIdx.x == 0) {
+        s_tile = atomicAdd(&ws->ticket[pass], 1u);
+        s_unknown = 0;
+    }
     for (int i = threadIdx.x; i < RS_W * 256; i += RS_T) wcnt[i] = 0;
     __syncthreads();
     const int tile = (int)s_tile;
@@ -491,11 +506,11 @@ __global__ void __launch_bounds__(RS_T) rs_pass_k(const uint64_t *__restrict__ k
     const unsigned gbase = block_excl_scan(ws->count[pass][d0], sw, nullptr);
     // the counts of the tiles before, eight words in flight
     unsigned before = 0;
-    bool known = tile == 0;
     if (tile > 0) {
         constexpr int LB = 8;
-        int t = tile - 1;
-        for (int n0 = 0; !known && n0 < polls;) {
+        int t = tile - 1, n0 = 0;
+        bool known = false;
+        while (!known) {
             W x[LB];
 #pragma unroll
             for (int j = 0; j < LB; j++) x[j] = t - j >= 0 ? st[(size_t)(t - j) * 256 + d0] : 0;
@@ -512,19 +527,16 @@ __global__ void __launch_bounds__(RS_T) rs_pass_k(const uint64_t *__restrict__ k
                 }
             }
             t -= taken;
-            n0 += taken == 0;
+            if (!known && taken == 0 && ++n0 > polls) break;
         }
-        if (known) st[(size_t)tile * 256 + d0] = tag | ((W)2 << CB) | (W)(before + own);
+        if (!known) s_unknown = 1;
+        else st[(size_t)tile * 256 + d0] = tag | ((W)2 << CB) | (W)(before + own);
     }
     goff[d0] = gbase + before;
-    if (__syncthreads_or(!known)) {
-        unsigned *const cnt = reinterpret_cast<unsigned *>(skey);  // (not in use yet)
-        cnt[d0] = 0;
-        __syncthreads();
-        for (int64_t i = d0; i < base; i += RS_T) atomicAdd(&cnt[(unsigned)(kin[i] >> shift) & 255u], 1u);
-        __syncthreads();
-        before = cnt[d0];
-        if (!known) st[(size_t)tile * 256 + d0] = tag | ((W)2 << CB) | (W)(before + own);
+    __syncthreads();
+    if (s_unknown) {
+        before = rs_recount(kin, base, shift, reinterpret_cast<unsigned *>(skey));  // (not in use yet)
+        st[(size_t)tile * 256 + d0] = tag | ((W)2 << CB) | (W)(before + own);
         goff[d0] = gbase + before;
         __syncthreads();
     }

@@ -40,9 +40,9 @@ def test_sorted_stably_at_tile_edges(n):
     assert np.array_equal(np.argsort(raw, kind="stable"), perm) and np.array_equal(np.sort(raw), keys)
 
 
-# blocks that give up waiting for the ones before (0: all of them at once; 1: those
-# that do not find the counts at the first look) count the keys themselves: the
-# same keys and order, with tiles of 1024 and of 4096 keys and the last one partly filled
+# blocks that give up waiting for the ones before (at the first or second look in
+# vain) count the keys themselves: the same keys and order, with tiles of 1024 and of
+# 4096 keys and the last one partly filled
 @pytest.mark.parametrize("polls", [0, 1])
 @pytest.mark.parametrize("n", [4097, 70001, (1 << 19) + 1])
 def test_sorted_stably_without_waiting_for_other_blocks(n, polls):
