@@ -199,7 +199,7 @@ __device__ __forceinline__ void m2l_split_chunk(const float *__restrict__ Mc, in
                                                 unsigned char *__restrict__ row)
 {
     using C = TcCfg<NP>;
-    float v[8];
+    __align__(16) float v[8];  // (written and read as 16-byte vectors, whether in registers or in memory)
 #pragma unroll
     for (int i = 0; i < 8; i++) v[i] = 0.f;
     const int k0 = 8 * ch;
@@ -213,7 +213,7 @@ __device__ __forceinline__ void m2l_split_chunk(const float *__restrict__ Mc, in
     }
     // 2^e in two factors: e may lie outside the exponent range of one float
     const float s1 = m2l_pow2(e >> 1), s2 = m2l_pow2(e - (e >> 1));
-    __half h[8], w[8];
+    __align__(16) __half h[8], w[8];
 #pragma unroll
     for (int i = 0; i < 8; i++) {
         const float x = (v[i] * m2l_norm(k0 + i)) * s1 * s2;
