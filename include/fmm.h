@@ -100,7 +100,8 @@ typedef struct {
     double ms_p2m, ms_m2m, ms_m2l, ms_l2l, ms_l2p, ms_p2p, ms_combine;
     int64_t kernel_launches; /* kernels this handle launched since creation */
     int32_t uniform_path;    /* 1 if the last build took the full-octree fast path */
-    int32_t lattice_levels;  /* bit l: level l's M2L sources come by TMA tile loads (fmm_set_m2l_lattice) */
+    int32_t lattice_levels;  /* bit l: level l is complete and its M2L sources come by TMA tile loads
+                                (fmm_set_m2l_lattice; fmm_get_lattice_levels lists incomplete ones too) */
 } fmm_stats;
 
 /* Sizes of the arrays fmm_export_tree writes. */
@@ -179,10 +180,15 @@ FMM_API int fmm_set_m2l_pool(fmm_handle h, int max_cells);
  * the same way, the missing cells as zeros. on = 0: per-row lookups and
  * gathers on every level. The results are bitwise the same. Takes effect at
  * the next build; fmm_stats.lattice_levels says which complete levels the
- * last build set up (bit l: level l).
- * Returns FMM_EINVAL for a NULL handle or on not 0/1.
+ * last build set up (bit l: level l), fmm_get_lattice_levels which levels,
+ * complete or not. Returns FMM_EINVAL for a NULL handle or on not 0/1.
  */
 FMM_API int fmm_set_m2l_lattice(fmm_handle h, int on);
+
+/* Bit l of *levels: the last build set level l, complete or not, up for TMA tile
+ * loads (fmm_set_m2l_lattice). Returns FMM_ESTATE before a build, FMM_EINVAL for
+ * a NULL argument. */
+FMM_API int fmm_get_lattice_levels(fmm_handle h, int32_t *levels);
 
 /* For tests: how often a block of the build's radix sort looks for the digit
  * counts of the block before it until it counts the keys before its own itself

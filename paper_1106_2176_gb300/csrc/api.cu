@@ -482,6 +482,14 @@ int fmm_energy_adjoint(fmm_handle h, double gE, const void *w, const void *q, co
     API_END
 }
 
+int fmm_get_lattice_levels(fmm_handle h, int32_t *levels)
+{
+    if (!h || !levels) return fail(FMM_EINVAL, "fmm_get_lattice_levels: NULL argument");
+    if (!h->built) return fail(FMM_ESTATE, "fmm_get_lattice_levels: no successful fmm_build");
+    *levels = (int32_t)h->lat_levels;
+    return FMM_OK;
+}
+
 int fmm_get_stats(fmm_handle h, fmm_stats *out)
 {
     if (!h || !out) return fail(FMM_EINVAL, "fmm_get_stats: NULL argument");

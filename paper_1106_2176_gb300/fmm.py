@@ -86,6 +86,7 @@ def lib():
     L.fmm_m2l_rotation_host.argtypes = [ctypes.c_int, _vp, _vp, _vp]
     L.fmm_build.argtypes = [_vp, _vp, _vp, i64, i32]
     L.fmm_evaluate.argtypes = [_vp, _vp, _vp]
+    L.fmm_get_lattice_levels.argtypes = [_vp, ctypes.POINTER(ctypes.c_int32)]
     L.fmm_get_stats.argtypes = [_vp, ctypes.POINTER(fmm_stats)]
     L.fmm_get_stats_mean.argtypes = [_vp, i32, ctypes.POINTER(fmm_stats)]
     L.fmm_get_tree_sizes.argtypes = [_vp, ctypes.POINTER(fmm_tree_sizes)]
@@ -173,8 +174,8 @@ class FMM:
         self.m2l_pool = int(max_cells)
 
     def set_m2l_lattice(self, on):
-        """True: the tensor-core M2L brings the sources of complete levels
-        (8^4 cells and more) by TMA tile loads from a lattice copy of M~;
+        """True: the tensor-core M2L brings the sources of complete and nearly
+        complete levels (8^4 cells and more) by TMA tile loads from a lattice copy of M~;
         False: per-row lookups and gathers everywhere. Same results. Next build."""
         _check(lib().fmm_set_m2l_lattice(self._h, 1 if on else 0), self._h)
         self.m2l_lattice = bool(on)
@@ -275,6 +276,12 @@ class FMM:
         else:
             _check(lib().fmm_get_stats_mean(self._h, int(mean_of), ctypes.byref(s)), self._h)
         return {k: getattr(s, k) for k, _ in fmm_stats._fields_}
+
+    def lattice_levels(self):
+        """Bit l: the last build set level l, complete or not, up for TMA tile loads (set_m2l_lattice)."""
+        v = ctypes.c_int32()
+        _check(lib().fmm_get_lattice_levels(self._h, ctypes.byref(v)), self._h)
+        return v.value
 
     def tree_sizes(self):
         s = fmm_tree_sizes()

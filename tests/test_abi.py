@@ -101,6 +101,12 @@ def test_sort_polls_setter_checks_arguments(L):
     assert b"fmm_set_sort_polls" in L.fmm_last_error(None)
 
 
+def test_lattice_levels_checks_arguments(L):
+    v = ctypes.c_int32()
+    assert L.fmm_get_lattice_levels(None, ctypes.byref(v)) == fmm.FMM_EINVAL
+    assert b"fmm_get_lattice_levels" in L.fmm_last_error(None)
+
+
 def test_stats_layout_matches_the_header():
     # the ctypes mirror of fmm_stats lists the header's fields in order
     import re

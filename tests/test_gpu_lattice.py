@@ -149,6 +149,9 @@ def test_nearly_complete_levels_give_the_gathered_results_bitwise(P, gen, n, ful
     p0, g0, f0 = run_fmm(x, q, P, 0.5, 64, precision="mixed", dtype=np.float32, m2l_lattice=False)
     n5 = int(np.sum(f1.export_tree()["level"] == 5))
     assert (4 * n5 >= 3 * 8**5) == full and 0 < n5 < 8**5
+    # P = 1 has no tensor-core M2L
+    assert f1.lattice_levels() & 1 << 5 == (1 << 5 if full and P > 1 else 0) and f0.lattice_levels() == 0
+    assert f1.stats()["lattice_levels"] & 1 << 5 == 0
     assert f1.stats()["async_error"] == 0 and f0.stats()["async_error"] == 0
     assert np.array_equal(p1, p0) and np.array_equal(g1, g0)
     _, L1 = f1.export_expansions()
