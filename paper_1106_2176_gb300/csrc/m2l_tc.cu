@@ -274,12 +274,13 @@ __device__ __forceinline__ bool m2l_is_wide(unsigned wide, const M2LTile &t)
     return wide && (t.octant == 8 || ((wide >> t.level) & 1u));
 }
 
-// One tile in FP32 on the CUDA cores, by the first 256 threads of a block (all of
-// them take part in the barriers). Per vector C[row][r] += sum_c A[row][c] T[r][c]:
+// One (tile, range) item in FP32 on the CUDA cores, by the first 256 threads of a
+// block (all of them take part in the barriers). Per vector C[row][r] += sum_c A[row][c] T[r][c]:
 // A the sources' M~ a, T = (hi + lo) 2^-14 of the operator image, both staged in
 // shared memory 32 coefficients at a time; thread (ty, tx) holds rows 8 ty .. 8 ty
 // + 7 and columns tx, tx + 16, .... Sums run over 8 vectors in FP32, as in tensor
-// memory, then into (hi, lo) pairs. Slow (milliseconds a tile) and rare.
+// memory, then into (hi, lo) pairs, and over the ranges of a tile as there. Slow
+// (4 us a vector at p = 8) and rare.
 constexpr int WD_T = 256, WD_KC = 32, WD_LD = 132, WD_V = 8;
 template <int NP>
 struct WideShared {
@@ -287,18 +288,22 @@ struct WideShared {
     float T[WD_KC][NP];
     int src[WD_V][128];
     int any[WD_V];
+    int last;
 };
 
 template <int NP>
-__device__ __noinline__ void m2l_wide_tile(const M2LJob &J, int p, int tile, WideShared<NP> &sh)
+__device__ __noinline__ void m2l_wide_tile(const M2LJob &J, int p, int item, WideShared<NP> &sh)
 {
     using C = TcCfg<NP>;
     constexpr int NC = NP / 16;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, PP = p * p;
     const int tx = tid & 15, ty = (tid >> 4) & 15;
     const bool on = tid < WD_T;
+    const int tile = item / J.nsplit, split = item - tile * J.nsplit;
     const M2LTile td = J.tiles[tile];
-    const int nv = J.st_off[10 + td.octant * (FMM_MAXLEVEL + 1) + td.level], e0 = J.st_off[td.octant];
+    const int nvt = J.st_off[10 + td.octant * (FMM_MAXLEVEL + 1) + td.level];
+    const int w0 = (int)min((long long)nvt, (long long)split * J.chunk), w1 = (int)min((long long)nvt, (long long)w0 + J.chunk);
+    const int e0 = J.st_off[td.octant] + w0, nv = w1 - w0;
     // thread t looks up sources of row t % 128
     int cell = -1, rl = td.level, px = 0, py = 0, pz = 0, ro = 0;
     if (on && (tid & 127) < td.count) cell = J.tgt[td.start + (tid & 127)];  // (-1: a lattice position without a cell)
@@ -386,18 +391,41 @@ __device__ __noinline__ void m2l_wide_tile(const M2LJob &J, int p, int tile, Wid
 #pragma unroll
             for (int j = 0; j < NC; j++) two_sum_acc(hi[i][j], lo[i][j], acc[i][j]);
     }
+    auto put = [&](int row, int r, float x) {
+        const int c = row < td.count ? J.tgt[td.start + row] : -1, t = J.rowexp[r] + 14;
+        if (c >= 0) J.L[(size_t)c * PP + r] += (x * m2l_pow2(t >> 1)) * m2l_pow2(t - (t >> 1));
+    };
+    const size_t rng = (size_t)PP * 128;
     if (on)
 #pragma unroll
-        for (int i = 0; i < 8; i++) {
-            const int row = 8 * ty + i, c = row < td.count ? J.tgt[td.start + row] : -1;
+        for (int i = 0; i < 8; i++)
 #pragma unroll
             for (int j = 0; j < NC; j++) {
-                const int r = tx + 16 * j;
-                if (c < 0 || r >= PP) continue;
-                const int t = J.rowexp[r] + 14;
-                J.L[(size_t)c * PP + r] += ((hi[i][j] + lo[i][j]) * m2l_pow2(t >> 1)) * m2l_pow2(t - (t >> 1));
+                const int row = 8 * ty + i, r = tx + 16 * j;
+                if (r >= PP) continue;
+                if (J.nsplit == 1) put(row, r, hi[i][j] + lo[i][j]);
+                else __stcg(&J.part[(size_t)item * rng + (size_t)r * 128 + row], make_float2(hi[i][j], lo[i][j]));
             }
+    if (J.nsplit == 1) return;
+    // the tile's last range to finish adds them all in order
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+        sh.last = atomicAdd(&J.tcnt[tile], 1u) == (unsigned)(J.nsplit - 1);
+        if (sh.last) J.tcnt[tile] = 0u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!sh.last || !on) return;
+    for (int i = tid; i < PP * 128; i += WD_T) {
+        float h = 0.f, w = 0.f;
+        for (int k = 0; k < J.nsplit; k++) {
+            const float2 v = __ldcg(&J.part[((size_t)tile * J.nsplit + k) * rng + i]);
+            two_sum_acc(h, w, v.x);
+            w += v.y;
         }
+        put(i & 127, i >> 7, h + w);
+    }
 }
 
 template <int NP, bool PERSIST>
@@ -409,8 +437,7 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     // takes (tile, range) items from the queue until it is empty. Otherwise
     // CTA b computes item b of the single job `one`, read from the parameter
     // space, which measured faster for one system than the persistent loop.
-    // *any: zero if no level is wide. The item of a wide tile's first range is the
-    // whole tile, its other items are empty.
+    // *any: zero if no level is wide.
     using C = TcCfg<NP>;
     constexpr int NS = C::NS, NM = C::NM, QU = C::QU, RINGU = C::RINGU, KB = C::KB;
     constexpr bool PACK = C::PACK;
@@ -437,8 +464,7 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
         const unsigned wide = *any;
         if ((int)blockIdx.x >= *one.ntiles * one.nsplit) return;
         if (wide && m2l_is_wide(wide, one.tiles[(int)blockIdx.x / one.nsplit])) {
-            if ((int)blockIdx.x % one.nsplit == 0)
-                m2l_wide_tile<NP>(one, p, (int)blockIdx.x / one.nsplit, *reinterpret_cast<WideShared<NP> *>(base));
+            m2l_wide_tile<NP>(one, p, (int)blockIdx.x, *reinterpret_cast<WideShared<NP> *>(base));
             return;
         }
     }
@@ -492,7 +518,7 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     if constexpr (PERSIST) {
         static_assert(sizeof(WideShared<NP>) <= NS * C::STAGE, "shared memory of a wide tile");
         if (*s_wide) {
-            if (item % J.nsplit == 0) m2l_wide_tile<NP>(J, p, item / J.nsplit, *reinterpret_cast<WideShared<NP> *>(base));
+            m2l_wide_tile<NP>(J, p, item, *reinterpret_cast<WideShared<NP> *>(base));
             // plain writes to the stages before the asynchronous copies of the next item
             fence_proxy_async();
             __syncthreads();
