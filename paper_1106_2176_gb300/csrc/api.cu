@@ -96,7 +96,7 @@ fmm_ctx::~fmm_ctx()
     fmm::DevBuf *bufs[] = {&st_dev, &rtab64, &rtab32, &m2m_mat, &l2l_mat, &box, &x_in, &q_in, &w_in, &keys, &keys2, &idx, &inv, &pcell, &cgeo, &energy_buf,
                            &idx2, &sort_ws, &scan_tmp, &xs64, &xs32, &xs32lo, &c_level, &c_anchor, &c_begin, &c_end, &c_child,
                            &c_nchild, &c_parent, &c_xyz, &split_cnt, &split_off, &split_bnd, &leaves, &small_tree, &frontA,
-                           &frontB, &p2p_pairs, &m2lx_pairs, &near_dev, &pair_keys, &pair_keys2, &pair_vals, &pair_vals2,
+                           &frontB, &p2p_pairs, &m2lx_pairs, &near_dev, &pair_keys, &pair_keys2,
                            &p2p_ptr, &p2p_src, &p2p_runs, &p2p_nrun, &pr_pad, &pr_flag, &pr_pairs, &m2lx_ptr, &m2lx_src, &row_cnt, &counters, &lvl_desc, &map_pool, &hash_pool,
                            &m2l_tgt, &m2l_tiles, &m2l_misc, &msplit, &Mexp, &Lexp, &far, &near, &out_phi, &out_grad,
                            &direct_part, &rot_tab, &rot_angle, &rot_m, &mlat, &lat_maps, &m2l_ws, &m2l_cmax, &m2l_part};
@@ -222,7 +222,6 @@ int fmm_create(int64_t N, int p, double theta, int ncrit, fmm_handle *out)
     for (auto &t : h->tms)
         for (auto &e : t.ev) FMM_CUDA_TRY(cudaEventCreate(&e));
     fmm::operators_init(h);
-    fmm::tensor_tables_init(h);
     FMM_CUDA_TRY(cudaDeviceSynchronize());
     *out = h;
     return FMM_OK;

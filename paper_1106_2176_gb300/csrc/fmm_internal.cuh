@@ -293,7 +293,7 @@ struct fmm_ctx {
     fmm::DevBuf frontA, frontB;
     fmm::DevBuf p2p_pairs, m2lx_pairs;
     fmm::DevBuf near_dev;       // near-field stencil of the uniform fast path (int4)
-    fmm::DevBuf pair_keys, pair_keys2, pair_vals, pair_vals2;
+    fmm::DevBuf pair_keys, pair_keys2;
     fmm::DevBuf p2p_ptr, p2p_src, m2lx_ptr, m2lx_src, row_cnt;
     fmm::DevBuf p2p_runs, p2p_nrun;     // P2P sources merged into particle runs per target leaf
     // packed P2P of FP32 inputs: sorted particles as pair records (x0 x1 y0 y1 | z0 z1 q0 q1), each leaf
@@ -371,7 +371,6 @@ void batch_combine(const BatchSys *sys, int nsys, const int *blk0, int nblocks, 
 void cell_geometry(fmm_ctx *h, cudaStream_t s);  // h->cgeo: centre and 1 / width of every cell
 
 // m2l_tc.cu
-void tensor_tables_init(fmm_ctx *h);
 bool tensor_m2l_supported(fmm_ctx *h);
 void m2l_tensor(fmm_ctx *h, float *L, const float *M);
 // the same-level M2L of several systems (same p; rows already split) in one persistent launch

@@ -930,8 +930,6 @@ static size_t tc_op_bytes(int p) { return (size_t)tc_kb(p) * (tc_np(p) <= 32 ? 1
 
 bool tensor_m2l_supported(fmm_ctx *h) { return h->p >= 2 && tc_np(h->p) > 0 && h->cc_major == 10; }
 
-void tensor_tables_init(fmm_ctx *) {}
-
 // I_n^m(x) in full storage (n*n + n + m), degrees < Q, from the Cartesian
 // recurrences of the irregular solid harmonics
 static void build_irregular_full(int Q, double x, double y, double z, std::vector<double> &re, std::vector<double> &im)
