@@ -69,7 +69,10 @@ enum {
     FMM_MIXED = 1  /* FP32 P2P and expansions, M2L on the tensor cores in
                       split FP16 (two halves of 11 bits, scaled by powers of
                       two) with FP32 accumulation (p <= 11; FP32 rotation M2L
-                      above), FP64 tree, FP64 offsets and final sums */
+                      above), FP64 tree, FP64 offsets and final sums. Levels
+                      that hold targets 2^-16 and more below the level's
+                      strongest cell, with all their surroundings, are summed
+                      in FP32 on the CUDA cores instead (slower) */
 };
 
 /* M2L engine of the same-level pairs (fmm_set_m2l_engine) */
@@ -389,9 +392,9 @@ FMM_API int fmm_morton_sort_noalloc(const void *x, int64_t n, int dtype, uint64_
 
 /*
  * Measured peak rate of one arithmetic pipe of the current device, in TFLOP/s
- * (2 flop per multiply-add). The paper has no counterpart: these are the
- * denominators of the roofline fractions the benchmark reports for P2P (FP32
- * FMA) and for the tensor-core M2L (TF32 MMA).
+ * (2 flop per multiply-add). The paper has no counterpart: the benchmark reports
+ * P2P as a fraction of the FP32 FMA rate, and the TF32 MMA rate beside it (the
+ * tensor-core M2L issues 16-bit MMAs).
  *   kind FMM_PEAK_FP32_FMA / FMM_PEAK_FP32X2_FMA: every thread of a full-
  *     occupancy grid runs 8 independent FMA chains (param ignored);
  *   kind FMM_PEAK_TF32_MMA: one CTA per SM, one thread issuing M = 128,

@@ -1260,8 +1260,9 @@ static EncodeTiledFn encode_tiled()
 // cell, and read their sources by TMA from the lattice copy of the level's
 // rows, zeros where there is no cell. A tile by TMA takes about 0.45 of the
 // time of one with gathered rows (N = 1e6 Plummer against uniform trees), so
-// the rows without a cell cost less than the gathers from half full on; the
-// batch engine, which gathers on every level, pays for them. M2L at N = 3e5
+// the rows without a cell should cost less than the gathers from half full on;
+// the line lies higher because the batch engine, which gathers on every level,
+// pays for them (a third more rows at most). M2L at N = 3e5
 // uniform, p = 8, whose level 5 is 85 % full: 2.66 -> 2.14 ms.
 static unsigned dense_levels(fmm_ctx *h, int pool_max)
 {

@@ -1,6 +1,7 @@
-// Measured arithmetic peaks of the current GPU: the denominators of the
-// roofline fractions of the P2P kernel (FP32 FMA on the CUDA cores) and of the
-// tensor-core M2L (tcgen05.mma kind::tf32). The paper has no counterpart;
+// Measured arithmetic peaks of the current GPU: FP32 FMA on the CUDA cores, the
+// denominator of the P2P kernel's roofline fraction, and the TF32 MMA rate
+// (tcgen05.mma kind::tf32), reported beside it. (The tensor-core M2L issues
+// kind::f16; its fraction is against a 16-bit GEMM.) The paper has no counterpart;
 // this is measurement infrastructure (fmm_measure_peak in include/fmm.h).
 //
 // FP32: every thread runs 8 independent FMA chains (scalar fma.rn.ftz.f32, or

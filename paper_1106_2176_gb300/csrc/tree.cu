@@ -350,7 +350,7 @@ __device__ __forceinline__ uint64_t morton_key(const T *__restrict__ x, int64_t 
 // scan with decoupled look-back, 2016; Adinets and Merrill, Onesweep, 2022).
 // Bound: one read and one write of 12 bytes per key and pass. The passes as
 // tile histograms, a scan of three kernels and a scatter took 376 us for
-// n = 10^6 and 1.3 ms for 10^7; this takes 216 us and 1.1 ms.
+// n = 10^6 and 1.3 ms for 10^7; this takes 213 us and 1.1 ms.
 // ---------------------------------------------------------------------------
 constexpr int RS_T = 256, RS_W = RS_T / 32, RS_PASSES = 8;
 constexpr int RS_R_MAX = 16;            // keys per thread: tiles of 4096 keys ...
@@ -409,8 +409,8 @@ __global__ void __launch_bounds__(256) rs_count_k(const uint64_t *__restrict__ k
         if (cnt[i]) atomicAdd(&ws->count[0][0] + i, cnt[i]);
 }
 
-// the lanes whose 8-bit digit equals this lane's, by eight ballots (match_any
-// takes longer: 291 against 269 us for a sort of 10^6 keys)
+// the lanes whose 8-bit digit equals this lane's, by eight ballots (with match_any a
+// sort of 10^6 keys takes 8 % longer)
 __device__ __forceinline__ unsigned digit_peers(unsigned d)
 {
     unsigned m = 0xffffffffu;

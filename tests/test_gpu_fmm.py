@@ -193,7 +193,7 @@ def test_rebuild_same_handle_is_deterministic():
 
 @pytest.mark.parametrize("P", [4, 6, 8])
 def test_tensor_core_m2l_matches_fp64_expansions(P):
-    # the local expansions of the mixed path (tcgen05 M2L in split TF32) against
+    # the local expansions of the mixed path (tcgen05 M2L in split FP16) against
     # the FP64 path's, cell by cell, relative to each cell's largest coefficient
     x, q = inputs.uniform_cube(60000, 21)
     _, _, f64 = run_fmm(x, q, P, 0.5, 32, precision="fp64")
