@@ -98,23 +98,27 @@ def test_wide_levels_are_the_same_with_and_without_lattice_loads(P):
     f0.close()
 
 
-def test_batch_with_wide_systems_matches_their_own_evaluations():
+# a few systems, and enough of them that every block takes wide and other items in turn
+@pytest.mark.parametrize("P,copies", [(6, 1), (4, 12), (8, 12), (10, 6)])
+def test_batch_with_wide_systems_matches_their_own_evaluations(P, copies):
     torch = torch_cuda()
     ensure_built()
     from paper_1106_2176_gb300.batch import FMMBatch
-    systems = [two_groups(4000, 2.0**28, 2.0**-12, 5), inputs.uniform_cube(5000, 6, dtype=np.float32),
-               inputs.plummer(20000, 7, dtype=np.float32), two_groups(1000, 2.0**40, 2.0**-9, 8)]
-    b = FMMBatch([(torch.tensor(x, device="cuda"), torch.tensor(q, device="cuda")) for x, q in systems], p=6, theta=0.5,
+    systems = []
+    for k in range(copies):
+        systems += [two_groups(4000, 2.0**28, 2.0**-12, 5 + k), inputs.uniform_cube(5000, 6 + k, dtype=np.float32),
+                    inputs.plummer(20000, 7 + k, dtype=np.float32), two_groups(1000, 2.0**40, 2.0**-9, 8 + k)]
+    b = FMMBatch([(torch.tensor(x, device="cuda"), torch.tensor(q, device="cuda")) for x, q in systems], p=P, theta=0.5,
                  ncrit=32, precision="mixed")
-    assert [bool(exposed_levels(f, 6)) for f in b.handles] == [True, False, False, True]
+    assert [bool(exposed_levels(f, P)) for f in b.handles[:4]] == [True, False, False, True]
     ref = [(p.clone(), g.clone()) for p, g in b.evaluate_each()]
-    for k in range(2):  # the second one on the first one's workspaces
+    for k in range(3):  # the later ones on the earlier ones' workspaces
         for p, g in b.out:
             p.fill_(float("nan"))
             g.fill_(float("nan"))
-        b.evaluate() if k == 0 else b.replay()
+        b.evaluate() if k < 2 else b.replay()
         torch.cuda.synchronize()
+        assert b.status()[0] == 0
         for (p, g), (pr, gr) in zip(b.out, ref):
             assert bool((p == pr).all()) and bool((g == gr).all())
-    assert b.status()[0] == 0
     b.close()
