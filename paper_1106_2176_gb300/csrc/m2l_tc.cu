@@ -346,26 +346,39 @@ __device__ __noinline__ void m2l_wide_tile(const M2LJob &J, int p, int item, Wid
             for (int c0 = 0; c0 < PP; c0 += WD_KC) {
                 __syncthreads();  // the staged coefficients are used up
                 if (on) {
+                    // all loads in flight before the first store: 16 rows a warp, one
+                    // coefficient a lane, and 8 coefficients of one output a thread
+                    constexpr int RW = 128 / (WD_T / 32), TI = (NP * (WD_KC / 8) + WD_T - 1) / WD_T;
                     const float a = c0 + lane < PP ? m2l_norm(c0 + lane) : 0.f;
-                    for (int r = warp; r < 128; r += WD_T / 32) {
-                        const int b = sh.src[k][r];
-                        sh.A[lane][r] = b >= 0 && c0 + lane < PP ? J.M[(size_t)b * PP + c0 + lane] * a : 0.f;
-                    }
-                    // 8 coefficients of one output a thread
-                    for (int i = tid; i < NP * (WD_KC / 8); i += WD_T) {
-                        const int r = i % NP, q = i / NP;
-                        const int ch = ((c0 & 63) >> 3) + q;  // its 16-byte chunk in the k-block's row
-                        const unsigned char *blk = op + (size_t)(c0 >> 6) * C::B_BYTES;
-                        const unsigned char *ph = blk + r * 128 + ((ch ^ (r & 7)) << 4);
-                        const unsigned char *pl = C::PACK ? blk + r * 128 + (((ch + 4) ^ (r & 7)) << 4)
-                                                          : blk + (NP + r) * 128 + ((ch ^ ((NP + r) & 7)) << 4);
-                        const uint4 h4 = *reinterpret_cast<const uint4 *>(ph), l4 = *reinterpret_cast<const uint4 *>(pl);
-                        const unsigned hw[4] = {h4.x, h4.y, h4.z, h4.w}, lw[4] = {l4.x, l4.y, l4.z, l4.w};
+                    float m[RW];
+                    uint4 th[TI], tl[TI];
 #pragma unroll
-                        for (int m = 0; m < 8; m++) {
-                            const unsigned short hb = (unsigned short)(hw[m / 2] >> (16 * (m & 1)));
-                            const unsigned short lb = (unsigned short)(lw[m / 2] >> (16 * (m & 1)));
-                            sh.T[8 * q + m][r] = (__half2float(__ushort_as_half(hb)) + __half2float(__ushort_as_half(lb))) * 0x1p-14f;
+                    for (int i = 0; i < RW; i++) {
+                        const int b = sh.src[k][warp + i * (WD_T / 32)];
+                        m[i] = b >= 0 && c0 + lane < PP ? J.M[(size_t)b * PP + c0 + lane] * a : 0.f;
+                    }
+                    const unsigned char *blk = op + (size_t)(c0 >> 6) * C::B_BYTES;
+#pragma unroll
+                    for (int t = 0; t < TI; t++) {
+                        const int i = tid + t * WD_T, r = i % NP;
+                        const int ch = ((c0 & 63) >> 3) + i / NP;  // its 16-byte chunk in the k-block's row
+                        if (i >= NP * (WD_KC / 8)) break;
+                        th[t] = *reinterpret_cast<const uint4 *>(blk + r * 128 + ((ch ^ (r & 7)) << 4));
+                        tl[t] = *reinterpret_cast<const uint4 *>(C::PACK ? blk + r * 128 + (((ch + 4) ^ (r & 7)) << 4)
+                                                                         : blk + (NP + r) * 128 + ((ch ^ ((NP + r) & 7)) << 4));
+                    }
+#pragma unroll
+                    for (int i = 0; i < RW; i++) sh.A[lane][warp + i * (WD_T / 32)] = m[i];
+#pragma unroll
+                    for (int t = 0; t < TI; t++) {
+                        const int i = tid + t * WD_T, r = i % NP, q = i / NP;
+                        if (i >= NP * (WD_KC / 8)) break;
+                        const unsigned hw[4] = {th[t].x, th[t].y, th[t].z, th[t].w}, lw[4] = {tl[t].x, tl[t].y, tl[t].z, tl[t].w};
+#pragma unroll
+                        for (int n = 0; n < 8; n++) {
+                            const unsigned short hb = (unsigned short)(hw[n / 2] >> (16 * (n & 1)));
+                            const unsigned short lb = (unsigned short)(lw[n / 2] >> (16 * (n & 1)));
+                            sh.T[8 * q + n][r] = (__half2float(__ushort_as_half(hb)) + __half2float(__ushort_as_half(lb))) * 0x1p-14f;
                         }
                     }
                 }
