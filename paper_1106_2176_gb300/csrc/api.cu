@@ -99,7 +99,7 @@ fmm_ctx::~fmm_ctx()
                            &frontB, &p2p_pairs, &m2lx_pairs, &near_dev, &pair_keys, &pair_keys2,
                            &p2p_ptr, &p2p_src, &p2p_runs, &p2p_nrun, &pr_pad, &pr_flag, &pr_pairs, &m2lx_ptr, &m2lx_src, &row_cnt, &counters, &lvl_desc, &map_pool, &hash_pool,
                            &m2l_tgt, &m2l_tiles, &m2l_misc, &msplit, &Mexp, &Lexp, &far, &near, &out_phi, &out_grad,
-                           &direct_part, &rot_tab, &rot_angle, &rot_m, &mlat, &lat_maps, &m2l_ws, &m2l_cmax, &m2l_part};
+                           &direct_part, &rot_tab, &rot_angle, &rot_m, &mlat, &lat_maps, &m2l_ws, &m2l_part};
     for (auto *b : bufs) b->release();
     hpin.release();
     lat_host.release();

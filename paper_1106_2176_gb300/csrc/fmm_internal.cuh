@@ -262,7 +262,7 @@ struct fmm_ctx {
     size_t rot_vec_off = 0, rot_c_off = 0;  // entries before the vectors' data and the c_nm in rot_tab
     int rot_nv = -1, rot_kind = 0;  // vectors and precision (1 FP32, 2 FP64) of rot_tab
     fmm::DevBuf msplit;         // M~ split into FP16 (hi, lo) rows for the tensor-core M2L
-    fmm::DevBuf m2l_ws, m2l_cmax, m2l_part;  // its workspace, largest coefficient per cell, sums of the ranges of split tiles
+    fmm::DevBuf m2l_ws, m2l_part;  // its workspace and the cells' largest coefficients; sums of the ranges of split tiles
     int m2l_nsplit = 1, m2l_chunk = 0;  // ranges per tile and their length (m2l_plan, rotation_plan)
     // tensor-core M2L on lattice levels: the rows of each such level in lattice
     // order (octant bits, then z, y, x of the halved position), one TMA tensor

@@ -280,7 +280,7 @@ __device__ __forceinline__ bool m2l_is_wide(unsigned wide, const M2LTile &t)
 // shared memory 32 coefficients at a time; thread (ty, tx) holds rows 8 ty .. 8 ty
 // + 7 and columns tx, tx + 16, .... Sums run over 8 vectors in FP32, as in tensor
 // memory, then into (hi, lo) pairs, and over the ranges of a tile as there. Slow
-// (4 us a vector at p = 8) and rare.
+// (29 ms for 10^6 particles, p = 8, against 5.2 on the tensor cores) and rare.
 constexpr int WD_T = 256, WD_KC = 32, WD_LD = 132, WD_V = 8;
 template <int NP>
 struct WideShared {
@@ -346,34 +346,26 @@ __device__ __noinline__ void m2l_wide_tile(const M2LJob &J, int p, int item, Wid
             for (int c0 = 0; c0 < PP; c0 += WD_KC) {
                 __syncthreads();  // the staged coefficients are used up
                 if (on) {
-                    // all loads in flight before the first store: 16 rows a warp, one
-                    // coefficient a lane, and 8 coefficients of one output a thread
-                    constexpr int RW = 128 / (WD_T / 32), TI = (NP * (WD_KC / 8) + WD_T - 1) / WD_T;
                     const float a = c0 + lane < PP ? m2l_norm(c0 + lane) : 0.f;
+                    constexpr int RW = 128 / (WD_T / 32);  // rows per warp, all loads in flight before the first store
                     float m[RW];
-                    uint4 th[TI], tl[TI];
 #pragma unroll
                     for (int i = 0; i < RW; i++) {
                         const int b = sh.src[k][warp + i * (WD_T / 32)];
                         m[i] = b >= 0 && c0 + lane < PP ? J.M[(size_t)b * PP + c0 + lane] * a : 0.f;
                     }
-                    const unsigned char *blk = op + (size_t)(c0 >> 6) * C::B_BYTES;
-#pragma unroll
-                    for (int t = 0; t < TI; t++) {
-                        const int i = tid + t * WD_T, r = i % NP;
-                        const int ch = ((c0 & 63) >> 3) + i / NP;  // its 16-byte chunk in the k-block's row
-                        if (i >= NP * (WD_KC / 8)) break;
-                        th[t] = *reinterpret_cast<const uint4 *>(blk + r * 128 + ((ch ^ (r & 7)) << 4));
-                        tl[t] = *reinterpret_cast<const uint4 *>(C::PACK ? blk + r * 128 + (((ch + 4) ^ (r & 7)) << 4)
-                                                                         : blk + (NP + r) * 128 + ((ch ^ ((NP + r) & 7)) << 4));
-                    }
 #pragma unroll
                     for (int i = 0; i < RW; i++) sh.A[lane][warp + i * (WD_T / 32)] = m[i];
-#pragma unroll
-                    for (int t = 0; t < TI; t++) {
-                        const int i = tid + t * WD_T, r = i % NP, q = i / NP;
-                        if (i >= NP * (WD_KC / 8)) break;
-                        const unsigned hw[4] = {th[t].x, th[t].y, th[t].z, th[t].w}, lw[4] = {tl[t].x, tl[t].y, tl[t].z, tl[t].w};
+                    // 8 coefficients of one output a thread
+                    for (int i = tid; i < NP * (WD_KC / 8); i += WD_T) {
+                        const int r = i % NP, q = i / NP;
+                        const int ch = ((c0 & 63) >> 3) + q;  // its 16-byte chunk in the k-block's row
+                        const unsigned char *blk = op + (size_t)(c0 >> 6) * C::B_BYTES;
+                        const unsigned char *ph = blk + r * 128 + ((ch ^ (r & 7)) << 4);
+                        const unsigned char *pl = C::PACK ? blk + r * 128 + (((ch + 4) ^ (r & 7)) << 4)
+                                                          : blk + (NP + r) * 128 + ((ch ^ ((NP + r) & 7)) << 4);
+                        const uint4 h4 = *reinterpret_cast<const uint4 *>(ph), l4 = *reinterpret_cast<const uint4 *>(pl);
+                        const unsigned hw[4] = {h4.x, h4.y, h4.z, h4.w}, lw[4] = {l4.x, l4.y, l4.z, l4.w};
 #pragma unroll
                         for (int n = 0; n < 8; n++) {
                             const unsigned short hb = (unsigned short)(hw[n / 2] >> (16 * (n & 1)));
@@ -1215,8 +1207,7 @@ M2LJob m2l_tensor_job(fmm_ctx *h, float *L)
     tensor_tables_update(h);
     const int nc = h->ncells;
     h->msplit.ensure(tc_row_bytes(h->p) * (size_t)nc);
-    h->m2l_ws.ensure(sizeof(unsigned) * (M2LW_CNT + (size_t)h->ntiles_max));
-    h->m2l_cmax.ensure(sizeof(unsigned) * (size_t)nc);
+    h->m2l_ws.ensure(sizeof(unsigned) * (M2LW_CNT + (size_t)h->ntiles_max + (size_t)nc));
     if (h->m2l_nsplit > 1)
         h->m2l_part.ensure(sizeof(float2) * (size_t)h->ntiles_max * h->m2l_nsplit * h->p * h->p * TcCfg<64>::M);
     M2LJob j;
@@ -1233,10 +1224,10 @@ M2LJob m2l_tensor_job(fmm_ctx *h, float *L)
     j.ttab = h->ttab->buf.as<unsigned char>();
     j.L = L;
     j.M = h->Mexp.as<float>();
-    j.cmax = h->m2l_cmax.as<unsigned>();
     j.ws = h->m2l_ws.as<unsigned>();
     j.tcnt = h->m2l_ws.as<unsigned>() + M2LW_CNT;
     j.ws_words = M2LW_CNT + h->ntiles_max;
+    j.cmax = h->m2l_ws.as<unsigned>() + j.ws_words;
     j.part = h->m2l_part.as<float2>();
     j.nsplit = h->m2l_nsplit;
     j.chunk = h->m2l_chunk;
@@ -1407,14 +1398,14 @@ void m2l_tensor(fmm_ctx *h, float *L, const float *M)
     }
     // a block walks 64 cells or more; 4 blocks per SM at most
     const unsigned gx = (unsigned)std::min((most + 63) / 64, 4 * h->nsm);
-    m2l_lmax_k<<<dim3(gx, (unsigned)h->depth - 1), 256, 0, s>>>(M, PP, lv, h->m2l_cmax.as<unsigned>(), h->m2l_ws.as<unsigned>());
+    m2l_lmax_k<<<dim3(gx, (unsigned)h->depth - 1), 256, 0, s>>>(M, PP, lv, const_cast<unsigned *>(j.cmax), h->m2l_ws.as<unsigned>());
     count_launch(h);
     M2LLattice lat;
     lat.levels = h->lat_levels;
     for (int l = 0; l <= FMM_MAXLEVEL; l++) lat.off[l] = h->lat_off[l];
 #define FMM_TC_CALL(NPV)                                                                                           \
     m2l_split_k<NPV><<<nblk((int64_t)(nc - c0) * (NPV / 8), 256), 256, 0, s>>>(                                     \
-        M, PP, h->c_xyz.as<int4>(), c0, nc, h->c_parent.as<int>(), h->m2l_cmax.as<unsigned>(),                       \
+        M, PP, h->c_xyz.as<int4>(), c0, nc, h->c_parent.as<int>(), j.cmax,                                           \
         h->m2l_ws.as<unsigned>(), lat, h->msplit.as<unsigned char>(), h->mlat.as<unsigned char>())
     FMM_TC_SWITCH(tc_np(h->p), FMM_TC_CALL)
 #undef FMM_TC_CALL
