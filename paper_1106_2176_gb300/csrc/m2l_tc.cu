@@ -433,6 +433,18 @@ __device__ __noinline__ void m2l_wide_tile(const M2LJob &J, int p, int item, Wid
     }
 }
 
+// the job that holds queue item `it` (the last one: also items past its end)
+__device__ __forceinline__ int job_of(const M2LJob *__restrict__ jobs, int njobs, int it)
+{
+    int lo = 0, hi = njobs - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (jobs[mid].item0 <= it) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
 template <int NP, bool PERSIST>
 __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     m2l_tc_k(int p, const __grid_constant__ M2LJob one, const M2LJob *__restrict__ jobs, int njobs,
@@ -460,12 +472,15 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     int *abort_flag = reinterpret_cast<int *>(tmem_slot + 1);
     int *s_item = abort_flag + 1;                 // this CTA's current item (-1: none left)
     int *s_last = s_item + 1;                     // this CTA finished its tile last
-    int *s_wide = s_last + 1;                     // the item's tile is wide
+    int *s_wide = s_last + 1;                     // (PERSIST) *any, once per CTA
     M2LJob *s_job = reinterpret_cast<M2LJob *>(reinterpret_cast<unsigned char *>(bar) + 512);  // its job
     static_assert(sizeof(uint64_t) * (3 * NS + 4 * C::AC + 2) + 20 <= 512 && 512 + sizeof(M2LJob) <= C::BAR, "barrier area");
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (!PERSIST) {
+    static_assert(sizeof(WideShared<NP>) <= NS * C::STAGE, "shared memory of a wide tile");
+    if (PERSIST) {
+        if (tid == 0) *s_wide = (int)*any;
+    } else {
         const unsigned wide = *any;
         if ((int)blockIdx.x >= *one.ntiles * one.nsplit) return;
         if (wide && m2l_is_wide(wide, one.tiles[(int)blockIdx.x / one.nsplit])) {
@@ -486,17 +501,12 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     for (int pass = 0; PERSIST || pass == 0; pass++) {
     if (tid == 0) {
         if (PERSIST) {
-            const int it = atomicAdd(queue, 1);
-            int lo = 0, hi = njobs - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (jobs[mid].item0 <= it) lo = mid;
-                else hi = mid - 1;
-            }
-            *s_job = jobs[lo];
-            const int t = it - s_job->item0;
-            *s_item = (t >= 0 && t < s_job->count) ? t : -1;
-            *s_wide = *any != 0u && *s_item >= 0 && m2l_is_wide(s_job->ws[M2LW_WIDE], s_job->tiles[t / s_job->nsplit]);
+            do {  // (wide tiles are left for the end)
+                const int it = atomicAdd(queue, 1);
+                *s_job = jobs[job_of(jobs, njobs, it)];
+                const int t = it - s_job->item0;
+                *s_item = (t >= 0 && t < s_job->count) ? t : -1;
+            } while (*s_wide && *s_item >= 0 && m2l_is_wide(s_job->ws[M2LW_WIDE], s_job->tiles[*s_item / s_job->nsplit]));
         } else {
             *s_item = (int)blockIdx.x;
         }
@@ -520,16 +530,6 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     const int item = *s_item;
     if (item < 0) break;
     const M2LJob &J = PERSIST ? *s_job : one;
-    if constexpr (PERSIST) {
-        static_assert(sizeof(WideShared<NP>) <= NS * C::STAGE, "shared memory of a wide tile");
-        if (*s_wide) {
-            m2l_wide_tile<NP>(J, p, item, *reinterpret_cast<WideShared<NP> *>(base));
-            // plain writes to the stages before the asynchronous copies of the next item
-            fence_proxy_async();
-            __syncthreads();
-            continue;
-        }
-    }
     const int nsplit = J.nsplit, tile = item / nsplit, split = item - tile * nsplit;
     const M2LTile td = J.tiles[tile];
     const int PP = p * p;
@@ -916,6 +916,13 @@ __global__ void __launch_bounds__(TcCfg<NP>::NT, 1)
     if (warp == C::MMA_WARP) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TCOLS));
     }
+    // the wide tiles of many systems, in turn over the CTAs
+    if (PERSIST && *s_wide)
+        for (int it = blockIdx.x; it < jobs[njobs - 1].item0 + jobs[njobs - 1].count; it += (int)gridDim.x) {
+            const M2LJob &J = jobs[job_of(jobs, njobs, it)];
+            if (m2l_is_wide(J.ws[M2LW_WIDE], J.tiles[(it - J.item0) / J.nsplit]))
+                m2l_wide_tile<NP>(J, p, it - J.item0, *reinterpret_cast<WideShared<NP> *>(base));
+        }
 }
 
 // ---------------------------------------------------------------------------
